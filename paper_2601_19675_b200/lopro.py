@@ -1,4 +1,7 @@
-"""ctypes binding of liblopro.so: the same entry points as include/lopro.h, argument marshalling only.
+"""Python binding of liblopro.so: the same entry points as include/lopro.h, argument marshalling only.
+
+What a program calls for every batch goes through the CPython extension built from csrc/binding.cpp (about 1 us of host
+time per call); sizes, checks and one-time steps go through ctypes.
 
 Tensors are torch tensors (torch supplies device memory and streams); every computation runs in the
 library's CUDA kernels.  The library must have been built (`python -m paper_2601_19675_b200.build`);
@@ -49,6 +52,11 @@ class LoproError(RuntimeError):
 
 
 _lib = None
+_native = None      # the CPython extension, bound to the library by lib()
+# the entry points it calls, by address
+_NATIVE_SYMBOLS = ["lopro_linear_fwd", "lopro_linear_fwd_host", "lopro_linear_fwd_noalloc", "lopro_linear_fwd_group",
+                   "lopro_linear_fwd_experts", "lopro_vq_linear_fwd", "lopro_rotate", "lopro_block_add_rmsnorm",
+                   "lopro_block_rope_append", "lopro_block_attention_decode", "lopro_block_silu_mul"]
 
 
 class VqDesc(ctypes.Structure):
@@ -59,8 +67,8 @@ class VqDesc(ctypes.Structure):
 
 
 def lib():
-    """The loaded library (loads it on first use)."""
-    global _lib
+    """The loaded library (loads it, and binds the CPython extension to it, on first use)."""
+    global _lib, _native
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(f"{LIB_PATH} is missing: build it with `python -m paper_2601_19675_b200.build`")
@@ -149,8 +157,21 @@ def lib():
         L.lopro_block_attention_decode.argtypes = [vp, i64, vp, vp, vp, vp, i64, i32, i32, i32, i32, f32, vp, sz, vp, vp]
         L.lopro_block_silu_mul.restype = ctypes.c_int
         L.lopro_block_silu_mul.argtypes = [vp, i64, vp, i64, vp, i64, i32, i32, vp]
+        try:
+            from . import _binding
+        except ImportError as e:
+            raise RuntimeError("the CPython extension is missing: build it with `python -m paper_2601_19675_b200.build`") from e
+        _binding.bind({name: ctypes.cast(getattr(L, name), vp).value for name in _NATIVE_SYMBOLS})
+        _native = _binding
         _lib = L
     return _lib
+
+
+def _calls():
+    """The extension's functions (loads the library on first use)."""
+    if _native is None:
+        lib()
+    return _native
 
 
 OPT_NO_WIDE, OPT_NO_TALL, OPT_NO_CHUNKS, OPT_NO_TCGEN05, OPT_PREFILL_PAIRS, OPT_ONE_KERNEL_SET, OPT_NO_CTA_PAIRS = range(7)
@@ -353,23 +374,16 @@ def quantize_layer(desc, W, perm, sketches=None, it=8, s=None, workspace=None):
 
 def block_add_rmsnorm(h, y, w, eps, out=None):
     """lopro_block_add_rmsnorm: h (bf16 [T][d], updated in place when y is given), y or None, w bf16 [d] -> out."""
-    T, d = h.shape
     if out is None:
-        out = torch.empty((T, d), dtype=torch.bfloat16, device=h.device)
-    st = lib().lopro_block_add_rmsnorm(_ptr(h), h.stride(0), _ptr(y), 0 if y is None else y.stride(0), _ptr(_dev(w, 2)), eps,
-                                       _ptr(out), out.stride(0), T, d, _stream())
-    _check(st, "lopro_block_add_rmsnorm")
+        out = torch.empty(tuple(h.shape), dtype=torch.bfloat16, device=h.device)
+    _check(_calls().block_add_rmsnorm(h, y, w, eps, out), "lopro_block_add_rmsnorm")
     return out
 
 
 def block_rope_append(q, k, v, pos, k_cache, v_cache, theta, status):
     """lopro_block_rope_append: q rotated in place; rotated k and v stored at entry pos[t] of the caches
     [T][heads][ctx_max][head_dim]."""
-    T, n_heads, ctx_max, head_dim = k_cache.shape
-    st = lib().lopro_block_rope_append(_ptr(q), q.stride(0), _ptr(k), k.stride(0), _ptr(v), v.stride(0), _ptr(_dev(pos, 4)),
-                                       _ptr(_dev(k_cache, 2)), _ptr(_dev(v_cache, 2)), T, n_heads, head_dim, ctx_max, theta,
-                                       _ptr(status), _stream())
-    _check(st, "lopro_block_rope_append")
+    _check(_calls().block_rope_append(q, k, v, pos, k_cache, v_cache, theta, status), "lopro_block_rope_append")
 
 
 def block_attention_workspace_bytes(T, n_heads, head_dim, ctx_max):
@@ -378,22 +392,17 @@ def block_attention_workspace_bytes(T, n_heads, head_dim, ctx_max):
 
 def block_attention_decode(q, k_cache, v_cache, ctx, scale, workspace, status, out=None):
     """lopro_block_attention_decode: q bf16 [T][heads * head_dim] against the caches; ctx int32 [T] valid entries."""
-    T, n_heads, ctx_max, head_dim = k_cache.shape
     if out is None:
+        T, n_heads, _, head_dim = k_cache.shape
         out = torch.empty((T, n_heads * head_dim), dtype=torch.bfloat16, device=q.device)
-    st = lib().lopro_block_attention_decode(_ptr(q), q.stride(0), _ptr(_dev(k_cache, 2)), _ptr(_dev(v_cache, 2)),
-                                            _ptr(_dev(ctx, 4)), _ptr(out), out.stride(0), T, n_heads, head_dim, ctx_max, scale,
-                                            _ptr(workspace), workspace.numel(), _ptr(status), _stream())
-    _check(st, "lopro_block_attention_decode")
+    _check(_calls().block_attention_decode(q, k_cache, v_cache, ctx, scale, workspace, status, out), "lopro_block_attention_decode")
     return out
 
 
 def block_silu_mul(gate, up, out=None):
-    T, d = gate.shape
     if out is None:
-        out = torch.empty((T, d), dtype=torch.bfloat16, device=gate.device)
-    st = lib().lopro_block_silu_mul(_ptr(gate), gate.stride(0), _ptr(up), up.stride(0), _ptr(out), out.stride(0), T, d, _stream())
-    _check(st, "lopro_block_silu_mul")
+        out = torch.empty(tuple(gate.shape), dtype=torch.bfloat16, device=gate.device)
+    _check(_calls().block_silu_mul(gate, up, out), "lopro_block_silu_mul")
     return out
 
 
@@ -415,16 +424,12 @@ def linear_fwd_experts_path(desc, row_offsets):
 def linear_fwd_experts(desc, blobs, row_offsets, x, out_dtype=OUT_BF16, workspace=None, y=None):
     """lopro_linear_fwd_experts: x bf16 [rows][d_in] grouped by expert (host list row_offsets of len(blobs) + 1 entries)."""
     n = len(blobs)
-    rows = x.shape[0]
-    max_rows = max([row_offsets[e + 1] - row_offsets[e] for e in range(n)] + [1])
     if workspace is None:
+        max_rows = max([row_offsets[e + 1] - row_offsets[e] for e in range(n)] + [1])
         workspace = torch.zeros(max(experts_workspace_bytes(desc, n, max_rows), 256), dtype=torch.uint8, device=x.device)
     if y is None:
-        y = torch.empty((rows, desc.d_out), dtype=torch.float32 if out_dtype == OUT_F32 else torch.bfloat16, device=x.device)
-    ptrs = (ctypes.c_void_p * n)(*[b.data_ptr() for b in blobs])
-    st = lib().lopro_linear_fwd_experts(ctypes.byref(desc), n, ptrs, _offsets(row_offsets), _ptr(x), x.stride(0), _ptr(y),
-                                        y.stride(0), out_dtype, _ptr(workspace), workspace.numel(), _stream())
-    _check(st, "lopro_linear_fwd_experts")
+        y = torch.empty((x.shape[0], desc.d_out), dtype=torch.float32 if out_dtype == OUT_F32 else torch.bfloat16, device=x.device)
+    _check(_calls().linear_fwd_experts(desc, blobs, row_offsets, x, out_dtype, workspace, y), "lopro_linear_fwd_experts")
     return y
 
 
@@ -456,15 +461,11 @@ def vq_pack(desc, idx, codebooks_bf16, perm, A_f16=None, B_f16=None):
 
 def vq_linear_fwd(desc, packed, x, out_dtype=OUT_BF16, workspace=None, y=None):
     """lopro_vq_linear_fwd: x bf16 [T][n] device -> y [T][m]."""
-    T = x.shape[0]
     if workspace is None:
-        workspace = torch.zeros(max(vq_workspace_bytes(desc, T), 256), dtype=torch.uint8, device=x.device)
+        workspace = torch.zeros(max(vq_workspace_bytes(desc, x.shape[0]), 256), dtype=torch.uint8, device=x.device)
     if y is None:
-        y = torch.empty((T, desc.d_out), dtype=torch.float32 if out_dtype == OUT_F32 else torch.bfloat16, device=x.device)
-    st = lib().lopro_vq_linear_fwd(ctypes.byref(desc), _ptr(packed), _ptr(x), x.stride(0) if T > 1 else max(x.stride(0), desc.d_in),
-                                   _ptr(y), y.stride(0) if T > 1 else max(y.stride(0), desc.d_out), out_dtype, T, _ptr(workspace),
-                                   workspace.numel(), _stream())
-    _check(st, "lopro_vq_linear_fwd")
+        y = torch.empty((x.shape[0], desc.d_out), dtype=torch.float32 if out_dtype == OUT_F32 else torch.bfloat16, device=x.device)
+    _check(_calls().vq_linear_fwd(desc, packed, x, out_dtype, workspace, y), "lopro_vq_linear_fwd")
     return y
 
 
@@ -513,41 +514,27 @@ def perm_of(desc, packed):
 
 def rotate(desc, perm, x, out=None):
     """lopro_rotate: x bf16 [T][n] (rows may be strided) -> rotated bf16 [T][n]."""
-    assert x.is_cuda and x.dim() == 2 and x.element_size() == 2 and x.stride(1) == 1
-    T = x.shape[0]
     if out is None:
-        out = torch.empty((T, desc.d_in), dtype=x.dtype, device=x.device)
-    st = lib().lopro_rotate(ctypes.byref(desc), _ptr(perm), _ptr(x), x.stride(0) if T > 1 else max(x.stride(0), desc.d_in),
-                            _ptr(out), out.stride(0) if T > 1 else max(out.stride(0), desc.d_in), T, _stream())
-    _check(st, "lopro_rotate")
+        out = torch.empty((x.shape[0], desc.d_in), dtype=x.dtype, device=x.device)
+    _check(_calls().rotate(desc, perm, x, out), "lopro_rotate")
     return out
 
 
 def linear_fwd(desc, packed, x, out_dtype=OUT_BF16, workspace=None, y=None):
     """lopro_linear_fwd: x bf16 [T][n] device -> y [T][m] (bf16 or fp32)."""
-    assert x.is_cuda and x.dim() == 2 and x.element_size() == 2 and x.stride(1) == 1
-    T = x.shape[0]
     if workspace is None:
-        workspace = torch.empty(max(workspace_bytes(desc, T), 256), dtype=torch.uint8, device=x.device)
+        workspace = torch.empty(max(workspace_bytes(desc, x.shape[0]), 256), dtype=torch.uint8, device=x.device)
     if y is None:
-        y = torch.empty((T, desc.d_out), dtype=torch.float32 if out_dtype == OUT_F32 else torch.bfloat16,
+        y = torch.empty((x.shape[0], desc.d_out), dtype=torch.float32 if out_dtype == OUT_F32 else torch.bfloat16,
                         device=x.device)
-    ldx = x.stride(0) if T > 1 else max(x.stride(0), desc.d_in)
-    ldy = y.stride(0) if T > 1 else max(y.stride(0), desc.d_out)
-    st = lib().lopro_linear_fwd(ctypes.byref(desc), _ptr(packed), _ptr(x), ldx, _ptr(y), ldy, int(out_dtype), T,
-                                _ptr(workspace), workspace.numel(), _stream())
-    _check(st, "lopro_linear_fwd")
+    _check(_calls().linear_fwd(desc, packed, x, out_dtype, workspace, y), "lopro_linear_fwd")
     return y
 
 
 def linear_fwd_host(desc, packed, x_host, y_host, workspace, out_dtype=OUT_BF16):
     """lopro_linear_fwd_host: x_host / y_host are HOST tensors (pinned for asynchronous copies); enqueues
     copy-in, forward and copy-out on the current stream and returns without synchronising."""
-    assert not x_host.is_cuda and not y_host.is_cuda and x_host.is_contiguous() and y_host.is_contiguous()
-    T = x_host.shape[0]
-    st = lib().lopro_linear_fwd_host(ctypes.byref(desc), _ptr(packed), _ptr(x_host), _ptr(y_host), int(out_dtype), T,
-                                     _ptr(workspace), workspace.numel(), _stream())
-    _check(st, "lopro_linear_fwd_host")
+    _check(_calls().linear_fwd_host(desc, packed, x_host, out_dtype, workspace, y_host), "lopro_linear_fwd_host")
     return y_host
 
 
@@ -571,20 +558,12 @@ def linear_fwd_group_path(descs, T):
 
 def linear_fwd_group(descs, packed, x, out_dtype=OUT_BF16, workspace=None, ys=None):
     """lopro_linear_fwd_group: sibling layers on the same x bf16 [T][n] -> list of y_i [T][m_i]."""
-    assert x.is_cuda and x.dim() == 2 and x.element_size() == 2 and x.stride(1) == 1
-    T, k = x.shape[0], len(descs)
     if workspace is None:
-        workspace = torch.empty(max(group_workspace_bytes(descs, T), 256), dtype=torch.uint8, device=x.device)
+        workspace = torch.empty(max(group_workspace_bytes(descs, x.shape[0]), 256), dtype=torch.uint8, device=x.device)
     if ys is None:
-        ys = [torch.empty((T, d.d_out), dtype=torch.float32 if out_dtype == OUT_F32 else torch.bfloat16, device=x.device)
+        ys = [torch.empty((x.shape[0], d.d_out), dtype=torch.float32 if out_dtype == OUT_F32 else torch.bfloat16, device=x.device)
               for d in descs]
-    ldx = x.stride(0) if T > 1 else max(x.stride(0), descs[0].d_in)
-    blobs = (ctypes.c_void_p * k)(*[b.data_ptr() for b in packed])
-    outs = (ctypes.c_void_p * k)(*[y.data_ptr() for y in ys])
-    ldys = (ctypes.c_int64 * k)(*[(y.stride(0) if T > 1 else max(y.stride(0), d.d_out)) for y, d in zip(ys, descs)])
-    st = lib().lopro_linear_fwd_group(k, _desc_array(descs), blobs, _ptr(x), ldx, outs, ldys, int(out_dtype), T, _ptr(workspace),
-                                      workspace.numel(), _stream())
-    _check(st, "lopro_linear_fwd_group")
+    _check(_calls().linear_fwd_group(descs, packed, x, out_dtype, workspace, ys), "lopro_linear_fwd_group")
     return ys
 
 
@@ -596,13 +575,7 @@ def linear_fwd_noalloc(desc, packed, x, y, out_dtype=OUT_BF16):
     device memory (the scratch is a fixed array inside the library).  The binding allocates nothing either:
     the caller passes the output tensor y [T][m].  Raises LoproError(ERR_BUFFER_TOO_SMALL) when the layer and
     token count need more than NOALLOC_SCRATCH_BYTES of scratch."""
-    assert x.is_cuda and x.dim() == 2 and x.element_size() == 2 and x.stride(1) == 1
-    T = x.shape[0]
-    ldx = x.stride(0) if T > 1 else max(x.stride(0), desc.d_in)
-    ldy = y.stride(0) if T > 1 else max(y.stride(0), desc.d_out)
-    st = lib().lopro_linear_fwd_noalloc(ctypes.byref(desc), _ptr(packed), _ptr(x), ldx, _ptr(y), ldy, int(out_dtype), T,
-                                        _stream())
-    _check(st, "lopro_linear_fwd_noalloc")
+    _check(_calls().linear_fwd_noalloc(desc, packed, x, out_dtype, y), "lopro_linear_fwd_noalloc")
     return y
 
 
