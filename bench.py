@@ -675,8 +675,8 @@ EXTRA_WORKLOADS = [("cfg2_T1", 5), ("cfg2_T32", 5), ("cfg4_T16", 5), ("cfg5_T1",
 def measure_offline(dev, peaks, reps=3):
     """The offline side (quantization of one layer on the GPU: rank-1 sketch with deflation at the paper's defaults,
     rank 16 and 8 iterations; residual, rotation, group grid) on the two matrix shapes of the 7B decoder stack.  Every
-    step is a memory-bound pass over the fp32 matrix; bytes = 4 m n (2 [scaling] + r (2 it + 4) [products, update]
-    + 1 [residual]) + m n [codes]."""
+    step is a memory-bound pass over the fp32 matrix; bytes = 4 m n (r (it + 1) [product pairs of the sketch] + 1 [residual])
+    + m n [codes]."""
     import torch
     from paper_2601_19675_b200 import lopro, synth
     out = {}
@@ -701,8 +701,8 @@ def measure_offline(dev, peaks, reps=3):
             torch.cuda.synchronize()
             times.append(e0.elapsed_time(e1))
         ms = statistics.median(times)
-        nbytes = 4 * m * n * (2 + r * (2 * it + 4) + 1) + m * n
-        launches = 1 + r * (1 + it * 3 + 2 + 2) + 2
+        nbytes = 4 * m * n * (r * (it + 1) + 1) + m * n
+        launches = 3   # sketch, factors, residual and grid
         per_shape[(n, m)] = ms
         out[f"quantize_{n}x{m}_r{r}_it{it}"] = dict(
             ms_per_layer=ms, algorithmic_bytes=nbytes, achieved_gbs=nbytes / (ms * 1e-3) / 1e9,

@@ -360,8 +360,8 @@ LOPRO_API lopro_status lopro_linear_fwd_experts(const lopro_desc* desc, int32_t 
  *     w        [m][n], IN: the matrix to decompose (W diag(s)); OUT: the deflated remainder
  *     sketches [r][n] Gaussian test vectors v_j (the call draws nothing)
  *     U [m][r], sigma [r], V [r][n] outputs; workspace of lopro_r1svd_workspace_bytes(m, n) bytes, 256-byte aligned
- *   m, n multiples of 4, 1 <= r <= 512, 0 <= it <= 64.  The work is 2 it + 2 matrix-vector products and one
- *   rank-1 update per rank: memory-bound passes over w.
+ *   m, n multiples of 4, 1 <= r <= 512, 0 <= it <= 64.  The work is it + 1 passes over w per rank, each
+ *   forming a product with W and one with W^T, and one closing pass that deflates w.
  *
  * lopro_residual_rotate -- R' = (W - Af Bf) P Q (Eq. 3 form ii, Eq. 5, Eq. 6), one row of W at a time: the residual
  *   against the STORED low-rank factors (Af [m][rank], Bf [rank][n] hold the stored values, e.g. fp16 numbers or
@@ -384,8 +384,7 @@ LOPRO_API lopro_status lopro_linear_fwd_experts(const lopro_desc* desc, int32_t 
  *     lr0..lr3: LOPRO_LOWRANK_FOLDED_F16: lr0 = A [m][r] fp16 = fp16(U Sigma), lr1 = B [r][n] fp16 = fp16(V diag(s)^-1);
  *               LOPRO_LOWRANK_FP8: lr0 = U [m][r] e4m3, lr1 = V [r][n] e4m3, lr2 = Sigma [r] fp16, lr3 = s [n] fp16
  *     -- exactly the arguments of lopro_pack / lopro_pack_lr8.  rank = 0: no factors, R = W.
- *   The first word of the workspace is the status word; workspace of lopro_quantize_workspace_bytes(desc) bytes
- *   (a copy of W among other things). */
+ *   The first word of the workspace is the status word; workspace of lopro_quantize_workspace_bytes(desc) bytes. */
 LOPRO_API size_t lopro_r1svd_workspace_bytes(int32_t m, int32_t n);
 LOPRO_API lopro_status lopro_r1svd(float* w, int32_t m, int32_t n, int32_t r, int32_t it, const float* sketches,
                                    int32_t cast, float* U, float* sigma, float* V, void* workspace,

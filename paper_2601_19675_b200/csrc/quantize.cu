@@ -4,6 +4,7 @@
 // plain coalesced loads, fp32 arithmetic, results independent of the launch shape (fixed summation orders, no atomics).
 #include "common.cuh"
 #include "ptx.cuh"
+#include "sketch.cuh"
 
 #include <cuda_fp16.h>
 
@@ -105,15 +106,6 @@ __global__ void __launch_bounds__(256) colsum_kernel(const float* __restrict__ p
     }
 }
 
-// fp32 -> nearest fp8 e4m3 value (ties to even, saturating), returned as fp32; bits optionally kept.
-__device__ __forceinline__ float round_e4m3(float x, unsigned char* bits) {
-    unsigned short pair;
-    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(pair) : "f"(0.0f), "f"(x));  // low byte = second operand
-    if (bits) *bits = (unsigned char)(pair & 0xffu);
-    const uint32_t h2 = e4m3x2_to_f16x2((unsigned short)(pair & 0xffu));
-    return __half2float(__ushort_as_half((unsigned short)(h2 & 0xffffu)));
-}
-
 // Rank j is done: U[:, j] = y / |y|, V[j, :] = p / |p| (cast to fp8 values when asked), sigma[j] = |p| where
 // p = W^T (y / |y|).  Every CTA forms the two norms itself (same order in every CTA, same bits).  A vanished y or p gives a zero triple.
 __global__ void __launch_bounds__(256) finish_rank_kernel(const float* __restrict__ y, const float* __restrict__ p,
@@ -154,13 +146,13 @@ __global__ void __launch_bounds__(256) finish_rank_kernel(const float* __restric
     const int i = blockIdx.x * 256 + threadIdx.x;
     if (i < m) {
         float u = dead ? 0.0f : y[i] * iy;
-        if (cast) u = round_e4m3(u, nullptr);
+        if (cast) u = round_e4m3(u);
         U[(size_t)i * r + j] = u;
         u1[i] = u;
     }
     if (i < n) {
         float v = dead ? 0.0f : p[i] * ip;
-        if (cast) v = round_e4m3(v, nullptr);
+        if (cast) v = round_e4m3(v);
         V[(size_t)j * n + i] = v;
         v1[i] = v;
     }
@@ -186,6 +178,7 @@ __global__ void __launch_bounds__(256) deflate_kernel(float* __restrict__ W, int
 
 struct R1Workspace {
     float *y, *p, *u1, *v1, *partial;
+    void* scratch;  // of the persistent kernel
     int slabs;
     size_t total;
 };
@@ -199,15 +192,20 @@ R1Workspace r1svd_workspace(int m, int n, uint8_t* base) {
         off += round_up_size(bytes, 256);
         return p;
     };
+    w.scratch = base;
     w.y = take((size_t)m * 4);
     w.p = take((size_t)n * 4);
     w.u1 = take((size_t)m * 4);
     w.v1 = take((size_t)n * 4);
     w.partial = take((size_t)w.slabs * n * 4);
+    // (the size does not depend on the rank: the largest that the persistent kernel takes)
+    const int ranks = sketch_supported(n, 128) ? 128 : 0;
+    if (ranks && sketch_scratch_bytes(m, n, ranks) > off) off = sketch_scratch_bytes(m, n, ranks);
     w.total = off;
     return w;
 }
 
+// Rows too long for the persistent kernel of sketch.cu: one launch per product.
 cudaError_t run_r1svd(float* w, int m, int n, int r, int it, const float* sketches, int cast, float* U, float* sigma,
                       float* V, const R1Workspace& ws, cudaStream_t s) {
     const dim3 g_rows((m + kGemvThreads / 32 - 1) / (kGemvThreads / 32));
@@ -249,8 +247,37 @@ struct RowJob {
     float inv_sqrt_bh;
 };
 
+// The group grid of Appendix A.2 from a group's minimum and maximum, and a column's code on it.  Every operation is one
+// IEEE single-precision operation, in the order of the definition.  A group with a non-finite entry, or whose range
+// underflows fp16, is bad: it is stored as zeros and reported by the caller.
+struct GroupGrid {
+    __half scale_h, zero_h;
+    float scale, zero;
+    bool bad;
+};
+__device__ __forceinline__ GroupGrid group_grid(float lo, float hi, bool bad, float qmax) {
+    const bool constant = hi == lo;
+    const float step = constant ? (lo != 0.0f ? fabsf(lo) : 1.0f) : __fdiv_rn(__fsub_rn(hi, lo), qmax);
+    GroupGrid q;
+    q.scale_h = __float2half_rn(step);
+    q.scale = __half2float(q.scale_h);
+    q.bad = bad || q.scale == 0.0f;
+    if (q.bad) {
+        q.scale_h = __float2half_rn(1.0f);
+        q.zero_h = __float2half_rn(0.0f);
+    } else {
+        q.zero_h = __float2half_rn(constant ? (lo < 0.0f ? 1.0f : 0.0f) : rintf(__fdiv_rn(-lo, q.scale)));
+    }
+    q.zero = __half2float(q.zero_h);
+    return q;
+}
+__device__ __forceinline__ uint32_t grid_code(const GroupGrid& q, float v, float qmax) {
+    if (q.bad) return 0u;
+    const float c = __fadd_rn(rintf(__fdiv_rn(v, q.scale)), q.zero);
+    return (uint32_t)fminf(fmaxf(c, 0.0f), qmax);
+}
+
 // The group grid on one row held in shared memory: a warp per group, lanes strided over its columns.
-// Every operation below is one IEEE single-precision operation, in the order of the definition.
 __device__ __forceinline__ void quantize_row(const float* row, int n, int g, int bits, uint8_t* codes, __half* scales,
                                              __half* zeros, int* status) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
@@ -270,31 +297,13 @@ __device__ __forceinline__ void quantize_row(const float* row, int n, int g, int
             lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
             hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
         }
-        bad = __any_sync(0xffffffffu, bad);
-        const bool constant = hi == lo;
-        const float step = constant ? (lo != 0.0f ? fabsf(lo) : 1.0f) : __fdiv_rn(__fsub_rn(hi, lo), qmax);
-        const __half step_h = __float2half_rn(step);
-        const float scale = __half2float(step_h);
-        if (bad || scale == 0.0f) {
-            // non-finite entry, or a range that underflows fp16: reported, the group stored as zeros
-            if (lane == 0) {
-                atomicCAS(status, LOPRO_OK, LOPRO_ERR_INVALID_DATA);
-                scales[grp] = __float2half_rn(1.0f);
-                zeros[grp] = __float2half_rn(0.0f);
-            }
-            for (int c = lane; c < g; c += 32) codes[grp * g + c] = 0;
-            continue;
-        }
-        const __half zero_h = __float2half_rn(constant ? (lo < 0.0f ? 1.0f : 0.0f) : rintf(__fdiv_rn(-lo, scale)));
-        const float zero = __half2float(zero_h);
+        const GroupGrid q = group_grid(lo, hi, __any_sync(0xffffffffu, bad), qmax);
         if (lane == 0) {
-            scales[grp] = step_h;
-            zeros[grp] = zero_h;
+            if (q.bad) atomicCAS(status, LOPRO_OK, LOPRO_ERR_INVALID_DATA);
+            scales[grp] = q.scale_h;
+            zeros[grp] = q.zero_h;
         }
-        for (int c = lane; c < g; c += 32) {
-            const float q = __fadd_rn(rintf(__fdiv_rn(v[c], scale)), zero);
-            codes[grp * g + c] = (uint8_t)fminf(fmaxf(q, 0.0f), qmax);
-        }
+        for (int c = lane; c < g; c += 32) codes[grp * g + c] = (uint8_t)grid_code(q, v[c], qmax);
     }
 }
 
@@ -349,6 +358,130 @@ __global__ void __launch_bounds__(256) residual_rotate_kernel(const RowJob p) {
     }
 }
 
+// The same for the common descriptors (b_H and g up to 256, b_I a multiple of b_H), R rows per CTA.  The kernel above
+// reads every rank's row of Bf once per row of W from L2 (2.9 GB for 11008 x 4096 at rank 16) and synchronises the CTA at
+// every level of the recursion; here R rows share each piece of Bf, and a warp takes 256 gathered columns of a row
+// through butterflies, group minimum and maximum and rounding in registers: eight columns per lane, levels 1 to 4 inside
+// the lane, the others between lanes.  Every operation and its operands are those of the kernel above, so the codes are
+// bit for bit the same.  11008 x 4096, rank 16, 4 bits: 648 -> 172 us.
+template <bool FUSED, int R>
+__global__ void __launch_bounds__(256) residual_rows_kernel(const RowJob p) {
+    extern __shared__ __align__(16) float rowbuf[];  // [R][n] residual rows, [R][rank] factors
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = p.n;
+    const int i0 = blockIdx.x * R, live = min(R, p.m - i0);
+    float* a_rows = rowbuf + (size_t)R * n;
+    for (int j = tid; j < live * p.rank; j += 256) a_rows[j] = p.Af[(size_t)i0 * p.rank + j];
+    __syncthreads();
+    for (int c4 = tid; c4 < n / 4; c4 += 256) {
+        float4 acc[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            acc[r] = r < live ? __ldg(reinterpret_cast<const float4*>(p.W + (size_t)(i0 + r) * n) + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int j = 0; j < p.rank; ++j) {
+            const float4 b = __ldg(reinterpret_cast<const float4*>(p.Bf + (size_t)j * n) + c4);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (r < live) {
+                    const float a = -a_rows[r * p.rank + j];
+                    acc[r].x = fmaf(a, b.x, acc[r].x);
+                    acc[r].y = fmaf(a, b.y, acc[r].y);
+                    acc[r].z = fmaf(a, b.z, acc[r].z);
+                    acc[r].w = fmaf(a, b.w, acc[r].w);
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (r < live) reinterpret_cast<float4*>(rowbuf + (size_t)r * n)[c4] = acc[r];
+    }
+    __syncthreads();
+    const float qmax = (float)((1 << p.bits) - 1);
+    const int glanes = p.g >> 3;  // lanes of a group
+    for (int chunk = warp; chunk * 256 < n; chunk += 8) {
+        const int col0 = chunk * 256 + lane * 8;
+        const bool on = col0 < n;
+        int src[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            src[e] = on ? __ldg(p.perm + col0 + e) : 0;
+            if ((unsigned)src[e] >= (unsigned)n) {
+                atomicCAS(p.status, LOPRO_OK, LOPRO_ERR_INVALID_DATA);
+                src[e] = 0;
+            }
+        }
+        for (int r = 0; r < live; ++r) {
+            const float* row = rowbuf + (size_t)r * n;
+            float x[8], v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = x[e] = row[src[e]];
+#pragma unroll
+            for (int h = 1; h < 8; h <<= 1) {
+                if (h < p.b_h) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        if ((e & h) == 0) {
+                            const float a = v[e], b = v[e + h];
+                            v[e] = a + b;
+                            v[e + h] = a - b;
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                if (d * 8 < p.b_h) {
+                    const bool upper = (lane & d) != 0;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const float other = __shfl_xor_sync(0xffffffffu, v[e], d);
+                        v[e] = upper ? other - v[e] : v[e] + other;
+                    }
+                }
+            }
+            const bool rot = col0 >= p.b_i;  // whole blocks lie on one side of b_I
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = rot ? v[e] * p.inv_sqrt_bh : x[e];
+            if constexpr (!FUSED) {
+                if (on) {
+                    float4* out = reinterpret_cast<float4*>(p.r_rot + (size_t)(i0 + r) * n + col0);
+                    out[0] = make_float4(v[0], v[1], v[2], v[3]);
+                    out[1] = make_float4(v[4], v[5], v[6], v[7]);
+                }
+            } else {
+                float lo = v[0], hi = v[0];
+                bool bad = !isfinite(v[0]);
+#pragma unroll
+                for (int e = 1; e < 8; ++e) {
+                    bad |= !isfinite(v[e]);
+                    lo = fminf(lo, v[e]);
+                    hi = fmaxf(hi, v[e]);
+                }
+                for (int o = 1; o < glanes; o <<= 1) {
+                    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+                    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+                }
+                const unsigned votes = __ballot_sync(0xffffffffu, bad);
+                const int l0 = lane & ~(glanes - 1);
+                bad = ((votes >> l0) & (glanes == 32 ? 0xffffffffu : (1u << glanes) - 1u)) != 0u;
+                const GroupGrid q = group_grid(lo, hi, bad, qmax);
+                if (on) {
+                    if (lane == l0) {
+                        const size_t at = (size_t)(i0 + r) * (n / p.g) + col0 / p.g;
+                        if (q.bad) atomicCAS(p.status, LOPRO_OK, LOPRO_ERR_INVALID_DATA);
+                        p.scales[at] = q.scale_h;
+                        p.zeros[at] = q.zero_h;
+                    }
+                    uint32_t out[2] = {0u, 0u};
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) out[e >> 2] |= grid_code(q, v[e], qmax) << (8 * (e & 3));
+                    *reinterpret_cast<uint2*>(p.codes + (size_t)(i0 + r) * n + col0) = make_uint2(out[0], out[1]);
+                }
+            }
+        }
+    }
+}
+
 __global__ void __launch_bounds__(256) rtn_kernel(const float* __restrict__ r_rot, int n, int g, int bits,
                                                    uint8_t* __restrict__ codes, __half* __restrict__ scales,
                                                    __half* __restrict__ zeros, int* status) {
@@ -361,8 +494,26 @@ __global__ void __launch_bounds__(256) rtn_kernel(const float* __restrict__ r_ro
 
 constexpr int kQuantMaxDin = 24576;  // two fp32 rows of the layer in one CTA's shared memory
 
+template <bool FUSED, int R>
+cudaError_t launch_residual_rows(const RowJob& job, cudaStream_t s) {
+    static unsigned long long attr_done = 0;
+    cudaError_t e = ensure_dynamic_smem(residual_rows_kernel<FUSED, R>, 220 * 1024, &attr_done);
+    if (e != cudaSuccess) return e;
+    const size_t smem = (size_t)R * (job.n + job.rank) * sizeof(float);
+    residual_rows_kernel<FUSED, R><<<(job.m + R - 1) / R, 256, smem, s>>>(job);
+    return cudaGetLastError();
+}
+
 template <bool FUSED>
 cudaError_t launch_residual_rotate(const RowJob& job, cudaStream_t s) {
+    // the kernel in registers: blocks and groups inside a warp's 256 columns, vector accesses
+    const bool vec = aligned_to(job.W, 16) && (job.rank == 0 || aligned_to(job.Bf, 16)) &&
+                     (FUSED ? aligned_to(job.codes, 8) : aligned_to(job.r_rot, 16));
+    if (vec && job.b_h <= 256 && job.b_i % job.b_h == 0 && job.b_i % 8 == 0 && (!FUSED || job.g <= 256)) {
+        // four rows while three CTAs of them fit a multiprocessor, else two (24576 columns: 196 KB)
+        if (job.n <= 4608) return launch_residual_rows<FUSED, 4>(job, s);
+        return launch_residual_rows<FUSED, 2>(job, s);
+    }
     static unsigned long long attr_done = 0;
     const int smem = 2 * job.n * (int)sizeof(float);
     cudaError_t e = ensure_dynamic_smem(residual_rotate_kernel<FUSED>, 2 * kQuantMaxDin * (int)sizeof(float), &attr_done);
@@ -462,7 +613,7 @@ QuantWorkspace quant_workspace(const lopro_desc& d, uint8_t* base) {
         return p;
     };
     q.status = reinterpret_cast<int*>(take(256));
-    q.Ws = reinterpret_cast<float*>(take(r ? m * n * 4 : 0));
+    q.Ws = reinterpret_cast<float*>(take(r && !sketch_supported((int)n, (int)r) ? m * n * 4 : 0));
     q.U = reinterpret_cast<float*>(take(m * r * 4));
     q.V = reinterpret_cast<float*>(take(r * n * 4));
     q.sigma = reinterpret_cast<float*>(take(r * 4));
@@ -504,6 +655,23 @@ lopro_status lopro_r1svd(float* w, int32_t m, int32_t n, int32_t r, int32_t it, 
     if (!aligned_to(w, 16) || !aligned_to(sketches, 16) || !aligned_to(workspace, 256)) return LOPRO_ERR_INVALID_ARG;
     if (workspace_bytes < lopro_r1svd_workspace_bytes(m, n)) return LOPRO_ERR_BUFFER_TOO_SMALL;
     const R1Workspace ws = r1svd_workspace(m, n, (uint8_t*)workspace);
+    if (sketch_supported(n, r) && aligned_to(V, 16)) {
+        SketchJob job = {};
+        job.w = w;
+        job.sketches = sketches;
+        job.U = U;
+        job.sigma = sigma;
+        job.V = V;
+        job.m = m;
+        job.n = n;
+        job.r = r;
+        job.it = it;
+        job.cast = cast;
+        if (launch_sketch(job, ws.scratch, (cudaStream_t)stream) != cudaSuccess ||
+            launch_deflate(w, m, n, r, U, sigma, V, (cudaStream_t)stream) != cudaSuccess)
+            return LOPRO_ERR_CUDA;
+        return LOPRO_OK;
+    }
     return run_r1svd(w, m, n, r, it, sketches, cast, U, sigma, V, ws, (cudaStream_t)stream) == cudaSuccess ? LOPRO_OK
                                                                                                            : LOPRO_ERR_CUDA;
 }
@@ -553,9 +721,29 @@ lopro_status lopro_quantize_layer(const lopro_desc* desc, const float* W, const 
     const int m = d.d_out, n = d.d_in, r = d.rank;
     if (cudaMemsetAsync(q.status, 0, 4, cs) != cudaSuccess) return LOPRO_ERR_CUDA;
     if (r > 0) {
-        scale_columns_kernel<<<m, 256, 0, cs>>>(W, s, n, fp8 ? 1 : 0, q.Ws, q.s_eff, fp8 ? (__half*)lr3 : nullptr);
         const R1Workspace ws = r1svd_workspace(m, n, q.r1);
-        if (run_r1svd(q.Ws, m, n, r, it, sketches, fp8 ? 1 : 0, q.U, q.sigma, q.V, ws, cs) != cudaSuccess) return LOPRO_ERR_CUDA;
+        if (sketch_supported(n, r)) {
+            SketchJob sk = {};
+            sk.w = W;
+            sk.sketches = sketches;
+            sk.s = s;
+            sk.s_eff = q.s_eff;
+            sk.s16 = fp8 ? (__half*)lr3 : nullptr;
+            sk.U = q.U;
+            sk.sigma = q.sigma;
+            sk.V = q.V;
+            sk.status = q.status;
+            sk.m = m;
+            sk.n = n;
+            sk.r = r;
+            sk.it = it;
+            sk.cast = fp8 ? 1 : 0;
+            if (launch_sketch(sk, ws.scratch, cs) != cudaSuccess) return LOPRO_ERR_CUDA;
+        } else {
+            scale_columns_kernel<<<m, 256, 0, cs>>>(W, s, n, fp8 ? 1 : 0, q.Ws, q.s_eff, fp8 ? (__half*)lr3 : nullptr);
+            if (run_r1svd(q.Ws, m, n, r, it, sketches, fp8 ? 1 : 0, q.U, q.sigma, q.V, ws, cs) != cudaSuccess)
+                return LOPRO_ERR_CUDA;
+        }
         const size_t items = (size_t)r * (size_t)(m > n ? m : n);
         factors_kernel<<<(unsigned)((items + 255) / 256), 256, 0, cs>>>(q.U, q.sigma, q.V, q.s_eff, m, n, r, fp8 ? 1 : 0, lr0,
                                                                         lr1, lr2, q.Af, q.Bf);
