@@ -613,7 +613,7 @@ QuantWorkspace quant_workspace(const lopro_desc& d, uint8_t* base) {
         return p;
     };
     q.status = reinterpret_cast<int*>(take(256));
-    q.Ws = reinterpret_cast<float*>(take(r && !sketch_supported((int)n, (int)r) ? m * n * 4 : 0));
+    q.Ws = reinterpret_cast<float*>(take(r ? m * n * 4 : 0));  // (rows too long for the persistent sketch; the size stays)
     q.U = reinterpret_cast<float*>(take(m * r * 4));
     q.V = reinterpret_cast<float*>(take(r * n * 4));
     q.sigma = reinterpret_cast<float*>(take(r * 4));
