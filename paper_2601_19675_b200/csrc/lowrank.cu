@@ -56,7 +56,7 @@ __device__ __forceinline__ void lowrank_body(unsigned char* smem_raw, int bx, in
 #pragma unroll
         for (int u = 0; u < kXPer; ++u) {
             const int i = tid + u * kLrThreads, r = i >> 3, c = i & 7;
-            xr[u] = tok0 + r < T ? __ldg(reinterpret_cast<const uint4*>(x + (size_t)(tok0 + r) * ldx + k0) + c)
+            xr[u] = tok0 + r < T ? __ldcg(reinterpret_cast<const uint4*>(x + (size_t)(tok0 + r) * ldx + k0) + c)
                                  : make_uint4(0, 0, 0, 0);
         }
 #pragma unroll

@@ -775,9 +775,9 @@ prefill_kparts_kernel(const float* __restrict__ kparts, void* __restrict__ y, in
     const int tok = (tile / row_tiles) * 512 + tok_l, row = (tile % row_tiles) * 256 + row_l;
     if (tok >= T || row >= m) return;
     const float* src = kparts + (((size_t)split_tile * k_parts) * kp_tokens + tok_l) * 256 + row_l;
-    float4 acc = *reinterpret_cast<const float4*>(src);
+    float4 acc = __ldcg(reinterpret_cast<const float4*>(src));
     for (int part = 1; part < k_parts; ++part) {
-        const float4 v = *reinterpret_cast<const float4*>(src + (size_t)part * kp_tokens * 256);
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(src + (size_t)part * kp_tokens * 256));
         acc.x += v.x;
         acc.y += v.y;
         acc.z += v.z;

@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(256) residual_rotate_kernel(const RowJob p) {
 // every level of the recursion; here R rows share each piece of Bf, and a warp takes 256 gathered columns of a row
 // through butterflies, group minimum and maximum and rounding in registers: eight columns per lane, levels 1 to 4 inside
 // the lane, the others between lanes.  Every operation and its operands are those of the kernel above, so the codes are
-// bit for bit the same.  11008 x 4096, rank 16, 4 bits: 648 -> 172 us.
+// bit for bit the same.  11008 x 4096, rank 16, 4 bits: 648 -> 146 us.
 template <bool FUSED, int R>
 __global__ void __launch_bounds__(256) residual_rows_kernel(const RowJob p) {
     extern __shared__ __align__(16) float rowbuf[];  // [R][n] residual rows, [R][rank] factors

@@ -48,7 +48,7 @@ lowrank_down_kernel(const __half* __restrict__ B, const __nv_bfloat16* __restric
 #pragma unroll
         for (int tk = 0; tk < 8; ++tk) {
             if (tok0 + tk < T) {
-                const uint4 xw = __ldg(reinterpret_cast<const uint4*>(x + (size_t)(tok0 + tk) * ldx) + c);
+                const uint4 xw = __ldcg(reinterpret_cast<const uint4*>(x + (size_t)(tok0 + tk) * ldx) + c);
                 const __nv_bfloat162* xh = reinterpret_cast<const __nv_bfloat162*>(&xw);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -108,7 +108,7 @@ __device__ __forceinline__ void lowrank_row(const __nv_bfloat16* __restrict__ x,
     auto load_x = [&](uint4 (&xw)[TPR], int k) {
 #pragma unroll
         for (int tk = 0; tk < TPR; ++tk)
-            xw[tk] = (k < n && tq + tk < T) ? __ldg(reinterpret_cast<const uint4*>(x + (size_t)(tq + tk) * ldx + k))
+            xw[tk] = (k < n && tq + tk < T) ? __ldcg(reinterpret_cast<const uint4*>(x + (size_t)(tq + tk) * ldx + k))
                                             : make_uint4(0, 0, 0, 0);
     };
     auto accumulate = [&](const uint4& bw, const uint4 (&xw)[TPR]) {
@@ -204,7 +204,7 @@ __device__ __forceinline__ void lowrank_row_lr8(const __nv_bfloat16* __restrict_
     auto load_x = [&](uint4 (&xw)[TPR], int k) {
 #pragma unroll
         for (int tk = 0; tk < TPR; ++tk)
-            xw[tk] = (k < n && tq + tk < T) ? __ldg(reinterpret_cast<const uint4*>(x + (size_t)(tq + tk) * ldx + k))
+            xw[tk] = (k < n && tq + tk < T) ? __ldcg(reinterpret_cast<const uint4*>(x + (size_t)(tq + tk) * ldx + k))
                                             : make_uint4(0, 0, 0, 0);
     };
     auto accumulate = [&](const uint2& vw, const uint4& sw, const uint4 (&xw)[TPR]) {
@@ -349,7 +349,9 @@ constexpr int kPrologueMaxSmem = 200 * 1024;  // one row of x: d_in <= 102400
 //  * a row CTA computes t[token][j] = sum_k B[j][k] x[token][k] for one row j of B and `tpr` of the 8 tokens
 //    (8 / tpr CTAs per row): the low-rank intermediate "Y = V X".
 // Launched with programmatic stream serialization: perm and B (layer data) are pulled into L2 before the
-// wait, everything is loaded after it.
+// wait, everything is loaded after it.  x is read through L2 (ld.global.cg): a CTA that was resident before its
+// predecessor wrote x may find an older copy of a reused buffer in L1 (seen in a decoder layer whose norms share one
+// output buffer: gate and up projections of the first norm's output).
 // A launch for a single layer carries no sibling table (several hundred bytes of kernel parameters less).
 struct NoPrologueSiblings {};
 __device__ __forceinline__ void select_prologue_sibling(const NoPrologueSiblings&, const int32_t*&, const __half*&,
@@ -431,9 +433,9 @@ prologue_kernel(const __nv_bfloat16* __restrict__ x0, int64_t ldx, const int32_t
         const int tok = tok0 + warp;
         if (tok < T) {
             float v[8];
-            const __nv_bfloat16* xrow = x + (size_t)tok * ldx;
+            const unsigned short* xrow = reinterpret_cast<const unsigned short*>(x + (size_t)tok * ldx);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = col0 < n ? __bfloat162float(xrow[pidx[e]]) : 0.0f;
+            for (int e = 0; e < 8; ++e) v[e] = col0 < n ? __bfloat162float(__ushort_as_bfloat16(__ldcg(xrow + pidx[e]))) : 0.0f;
             rotate_tail(v, act_image, n, b_i, b_h, inv_sqrt_bh, t_pad, tok, col0, lane, img);
         }
     } else {
@@ -459,7 +461,7 @@ prologue_kernel(const __nv_bfloat16* __restrict__ x0, int64_t ldx, const int32_t
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int k = base + i * 2048 + tid * 8;
-                if (k < n) w[i] = __ldg(reinterpret_cast<const uint4*>(xrow + k));
+                if (k < n) w[i] = __ldcg(reinterpret_cast<const uint4*>(xrow + k));
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {

@@ -32,7 +32,7 @@ __device__ __forceinline__ void rotate_body(unsigned char* smem_raw, int block, 
 
     for (int r = 0; r < nt; ++r) {
         const uint4* src = reinterpret_cast<const uint4*>(x + (size_t)(t0 + r) * ldx);
-        for (int i = tid; i < n / 8; i += kRotThreads) reinterpret_cast<uint4*>(xin + (size_t)r * n)[i] = __ldg(src + i);
+        for (int i = tid; i < n / 8; i += kRotThreads) reinterpret_cast<uint4*>(xin + (size_t)r * n)[i] = __ldcg(src + i);
     }
     __syncthreads();
 

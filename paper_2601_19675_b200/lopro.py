@@ -1,7 +1,7 @@
 """Python binding of liblopro.so: the same entry points as include/lopro.h, argument marshalling only.
 
-What a program calls for every batch goes through the CPython extension built from csrc/binding.cpp (about 1 us of host
-time per call); sizes, checks and one-time steps go through ctypes.
+What a program calls for every batch goes through the CPython extension built from csrc/binding.cpp (0.35 us of host
+time per call besides the launches); sizes, checks and one-time steps go through ctypes.
 
 Tensors are torch tensors (torch supplies device memory and streams); every computation runs in the
 library's CUDA kernels.  The library must have been built (`python -m paper_2601_19675_b200.build`);
