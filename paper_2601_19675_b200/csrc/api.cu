@@ -124,6 +124,49 @@ ImageOut image_out(const lopro_desc& d, uint8_t* ws, const WorkspaceLayout& W) {
 
 static bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 
+// Host buffers of small forwards are read and written by kernels over PCIe instead of by the copy engines: a change from
+// engine to kernel and back costs more than the copy (H2D, two kernels, D2H of 64 KB each: 18.4 us; the same with copy
+// kernels in one programmatic chain 10.2).  From about 1 MB on the two are equal (56.9 against 48.9 us at 1 MB each way,
+// 164.7 against 169.2 at 4 MB), so larger buffers stay with the engines.
+constexpr size_t kZeroCopyMax = (size_t)1 << 20;
+__global__ void __launch_bounds__(128) copy16_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, int n16) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    uint4 a, b;
+    if (i < n16) a = __ldcv(src + i);
+    if (i + 128 < n16) b = __ldcv(src + i + 128);
+    if (i < n16) __stcs(dst + i, a);
+    if (i + 128 < n16) __stcs(dst + i + 128, b);
+}
+static cudaError_t launch_copy16(const void* src, void* dst, size_t bytes, cudaStream_t s) {
+    const int n16 = (int)(bytes / 16);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((n16 + 255) / 256);
+    cfg.blockDim = dim3(128);
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, copy16_kernel, (const uint4*)src, (uint4*)dst, n16);
+}
+// The device's address of a host buffer whose first and last byte are pinned and mapped as one piece; null otherwise.
+// (0.06 us per lookup.)
+static void* mapped(const void* host, size_t bytes) {
+    if (bytes == 0 || bytes > kZeroCopyMax || (bytes % 16) || !aligned(host, 16)) return nullptr;
+    cudaPointerAttributes a, b;
+    if (cudaPointerGetAttributes(&a, host) != cudaSuccess || cudaPointerGetAttributes(&b, (const uint8_t*)host + bytes - 1) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer || !aligned(a.devicePointer, 16) ||
+        (uint8_t*)b.devicePointer - (uint8_t*)a.devicePointer != (ptrdiff_t)bytes - 1)
+        return nullptr;
+    return a.devicePointer;
+}
+
 namespace {
 int g_options[LOPRO_OPT_COUNT];
 int g_options_ready = 0;  // 0 = not read yet, 1 = being read, 2 = ready
@@ -834,13 +877,20 @@ lopro_status lopro_linear_fwd_host(const lopro_desc* desc, const void* packed, c
     const size_t esz = out_dtype == LOPRO_OUT_F32 ? 4 : 2;
     uint8_t* xd = (uint8_t*)workspace + W.total;
     uint8_t* yd = xd + round_up_size((size_t)T * desc->d_in * 2, 256);
-    if (cudaMemcpyAsync(xd, x_host, (size_t)T * desc->d_in * 2, cudaMemcpyHostToDevice, s) != cudaSuccess)
+    const size_t x_bytes = (size_t)T * desc->d_in * 2, y_bytes = (size_t)T * desc->d_out * esz;
+    if (const void* x_map = mapped(x_host, x_bytes)) {
+        if (launch_copy16(x_map, xd, x_bytes, s) != cudaSuccess) return LOPRO_ERR_CUDA;
+    } else if (cudaMemcpyAsync(xd, x_host, x_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) {
         return LOPRO_ERR_CUDA;
+    }
     st = lopro_linear_fwd(desc, packed, (const uint16_t*)xd, desc->d_in, yd, desc->d_out, out_dtype, T, workspace,
                           W.total, stream);
     if (st != LOPRO_OK) return st;
-    if (cudaMemcpyAsync(y_host, yd, (size_t)T * desc->d_out * esz, cudaMemcpyDeviceToHost, s) != cudaSuccess)
+    if (void* y_map = mapped(y_host, y_bytes)) {
+        if (launch_copy16(yd, y_map, y_bytes, s) != cudaSuccess) return LOPRO_ERR_CUDA;
+    } else if (cudaMemcpyAsync(y_host, yd, y_bytes, cudaMemcpyDeviceToHost, s) != cudaSuccess) {
         return LOPRO_ERR_CUDA;
+    }
     return LOPRO_OK;
 }
 
