@@ -7,6 +7,7 @@
 
 #include "common.cuh"
 #include "ptx.cuh"
+#include "vq_product.cuh"
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -87,8 +88,32 @@ lopro_desc as_scalar_desc(const lopro_vq_desc& d) {
     return s;
 }
 
+// How vq_product_kernel takes a layer (rb = 0: it does not, the codebooks' row groups are too short for it).
+struct VqPlan {
+    int rb, kind, max_books, stages, blocks, total, ctas;
+};
+VqPlan vq_plan(const lopro_vq_desc& d) {
+    VqPlan p = {};
+    const int dim = vq_dim(d);
+    // a row block lies inside one row group; with 2-D centroids a lane's indices split into two phases at most
+    for (int rb = 512; rb >= (dim == 4 ? 128 : 256) && p.rb == 0; rb /= 2)
+        if (d.cb_rows % rb == 0) p.rb = rb;
+    if (p.rb == 0) return p;
+    p.stages = (d.d_in + 255) / 256;
+    for (int s = 0; s < p.stages; ++s) {
+        const int end = s * 256 + 256 < d.d_in ? s * 256 + 256 : d.d_in;
+        const int books = (end - 1) / d.cb_cols - s * 256 / d.cb_cols + 1;
+        if (books > p.max_books) p.max_books = books;
+    }
+    p.kind = dim == 2 ? kVqDim2 : (p.max_books <= 2 ? kVqDim4 : kVqDim4Half);
+    p.blocks = (d.d_out + p.rb - 1) / p.rb;
+    p.total = p.blocks * p.stages;
+    p.ctas = p.total < sm_count() ? p.total : sm_count();
+    return p;
+}
+
 struct VqWorkspace {
-    size_t off_status, off_xrot, off_t, off_part, total;
+    size_t off_status, off_xrot, off_t, off_part, off_sums, total;
     int r_pad;
 };
 
@@ -99,11 +124,19 @@ VqWorkspace vq_workspace(const lopro_vq_desc& d, int T) {
     W.off_status = off;
     off += 256;
     W.off_xrot = off;
-    off += round_up_size((size_t)T * d.d_in * 2, 256);
+    {
+        // rotated rows, or the records that the small-batch prologue writes (a little larger)
+        size_t xb = (size_t)T * d.d_in * 2;
+        const size_t image = act_image_bytes(d.d_in, round_up_int(T < kDecodeMaxT ? T : kDecodeMaxT, 8));
+        off += round_up_size(xb > image ? xb : image, 256);
+    }
     W.off_t = off;
     off += round_up_size((size_t)T * (W.r_pad > 0 ? W.r_pad : 16) * 2, 256);
     W.off_part = off;
     off += d.rank > 0 && T > kDecodeMaxT ? round_up_size(lowrank_mma_scratch_bytes(as_scalar_desc(d), T), 256) : 0;
+    W.off_sums = off;
+    const VqPlan plan = vq_plan(d);
+    if (plan.rb) off += (size_t)(plan.ctas + plan.blocks) * 512 * (T <= 8 ? 8 : (T <= 16 ? 16 : 32)) * 4;
     W.total = off;
     return W;
 }
@@ -397,6 +430,51 @@ __global__ void __launch_bounds__(128) vq_decode_kernel(const VqParams p) {
         }
 }
 
+cudaError_t launch_programmatic(const void* kernel, dim3 grid, int threads, size_t smem, void** args, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, kernel, args);
+}
+
+template <int NT, int PH, int KIND>
+cudaError_t launch_vq_product_k(VqProduct p, cudaStream_t s) {
+    static unsigned long long attr_done = 0;
+    constexpr int kMost = kVqExpandedAt + 4 * 32768 + 3 * 4 * 4096;
+    cudaError_t e = ensure_dynamic_smem(vq_product_kernel<NT, PH, KIND>, kMost, &attr_done);
+    if (e != cudaSuccess) return e;
+    const size_t smem = (size_t)kVqExpandedAt + 2 * (size_t)p.max_books * vq_slot_bytes(KIND) + 3 * NT * 4096;
+    void* args[] = {&p};
+    return launch_programmatic((const void*)vq_product_kernel<NT, PH, KIND>, dim3(p.ctas), kVqThreads, smem, args, s);
+}
+template <int NT, int PH>
+cudaError_t launch_vq_product_p(const VqProduct& p, int kind, cudaStream_t s) {
+    if (kind == kVqDim4) return launch_vq_product_k<NT, PH, kVqDim4>(p, s);
+    if (kind == kVqDim4Half) return launch_vq_product_k<NT, PH, kVqDim4Half>(p, s);
+    if constexpr (PH <= 2) return launch_vq_product_k<NT, PH, kVqDim2>(p, s);
+    return cudaErrorInvalidValue;
+}
+template <int NT>
+cudaError_t launch_vq_product(VqProduct p, const VqPlan& plan, const __half* A, const __half* t, int r_pad, void* y, int64_t ldy,
+                              int out_f32, cudaStream_t s) {
+    cudaError_t e;
+    int phases = 512 / plan.rb, groups = NT * 2, rb = plan.rb;
+    if (phases == 1) e = launch_vq_product_p<NT, 1>(p, plan.kind, s);
+    else if (phases == 2) e = launch_vq_product_p<NT, 2>(p, plan.kind, s);
+    else e = launch_vq_product_p<NT, 4>(p, plan.kind, s);
+    if (e != cudaSuccess) return e;
+    void* args[] = {&p, &groups, &rb, &phases, &A, &t, &r_pad, &y, &ldy, &out_f32};
+    return launch_programmatic((const void*)vq_finish_kernel, dim3((p.m + 127) / 128, (p.T + 3) / 4), 128, 0, args, s);
+}
+
+// Codebooks whose row groups are no multiple of 128 rows (256 with 2-D centroids).
 template <int NT>
 cudaError_t launch_vq_decode(const VqParams& p, int dim, cudaStream_t s) {
     // two sections of codebooks; at the end the same memory holds the four warps' partial sums [4][NT][4][32] fp32
@@ -507,26 +585,68 @@ lopro_status lopro_vq_linear_fwd(const lopro_vq_desc* desc, const void* packed, 
     __nv_bfloat16* xrot = (__nv_bfloat16*)(ws + W.off_xrot);
     __half* tbuf = (__half*)(ws + W.off_t);
     int* status = (int*)(ws + W.off_status);
-    // the rotation kernels that write no column sums do not reset the status word themselves in every form: clear it here
-    if (cudaMemsetAsync(status, 0, 4, s) != cudaSuccess) return LOPRO_ERR_CUDA;
-    if (launch_rotate(sd, (const int32_t*)(blob + L.off_perm), (const __nv_bfloat16*)x_bf16, ldx, xrot, d.d_in, nullptr,
-                      status, T, s) != cudaSuccess)
-        return LOPRO_ERR_CUDA;
-    if (d.rank > 0) {
-        const __half* B = (const __half*)(blob + L.off_b);
-        cudaError_t e;
-        if (T > kDecodeMaxT) {
-            e = launch_lowrank_down_mma(sd, B, L.r_pad, (const __nv_bfloat16*)x_bf16, ldx, (float*)(ws + W.off_part), tbuf, T, s);
-        } else {
-            vq_lowrank_down_kernel<<<dim3(L.r_pad, (T + 7) / 8), 256, 0, s>>>(B, (const __nv_bfloat16*)x_bf16, ldx, tbuf, d.d_in,
-                                                                            L.r_pad, T);
-            e = cudaGetLastError();
+    // up to 32 tokens the small-batch prologue does both jobs in one launch of the programmatic chain; its records of
+    // 1024 columns and plain rows differ in their strides only
+    const VqPlan plan = vq_plan(d);
+    const bool records = plan.rb > 0 && T <= kDecodeMaxT && prologue_supported(sd, T);
+    const int t_pad = round_up_int(T, 8);
+    if (records) {
+        if (launch_prologue(sd, (const int32_t*)(blob + L.off_perm), (const __half*)(blob + L.off_b), L.r_pad,
+                            (const __nv_bfloat16*)x_bf16, ldx, ws + W.off_xrot, tbuf, t_pad, status, T, s) != cudaSuccess)
+            return LOPRO_ERR_CUDA;
+    } else {
+        // the rotation kernels that write no column sums do not reset the status word themselves in every form: clear it here
+        if (cudaMemsetAsync(status, 0, 4, s) != cudaSuccess) return LOPRO_ERR_CUDA;
+        if (launch_rotate(sd, (const int32_t*)(blob + L.off_perm), (const __nv_bfloat16*)x_bf16, ldx, xrot, d.d_in, nullptr,
+                          status, T, s) != cudaSuccess)
+            return LOPRO_ERR_CUDA;
+        if (d.rank > 0) {
+            const __half* B = (const __half*)(blob + L.off_b);
+            cudaError_t e;
+            if (T > kDecodeMaxT) {
+                e = launch_lowrank_down_mma(sd, B, L.r_pad, (const __nv_bfloat16*)x_bf16, ldx, (float*)(ws + W.off_part), tbuf, T, s);
+            } else {
+                vq_lowrank_down_kernel<<<dim3(L.r_pad, (T + 7) / 8), 256, 0, s>>>(B, (const __nv_bfloat16*)x_bf16, ldx, tbuf, d.d_in,
+                                                                                L.r_pad, T);
+                e = cudaGetLastError();
+            }
+            if (e != cudaSuccess) return LOPRO_ERR_CUDA;
         }
-        if (e != cudaSuccess) return LOPRO_ERR_CUDA;
     }
     const size_t esz = out_dtype == LOPRO_OUT_F32 ? 4 : 2;
     for (int t0 = 0; t0 < T; t0 += kDecodeMaxT) {
         const int tc = T - t0 < kDecodeMaxT ? T - t0 : kDecodeMaxT;
+        if (plan.rb > 0) {
+            VqProduct p;
+            p.idx = blob + L.off_idx;
+            p.books = blob + L.off_books;
+            p.x_stage = records ? (int64_t)t_pad * kActRecord : 2048;
+            p.x_token = records ? (int64_t)kActRecord : (int64_t)d.d_in * 2;
+            p.x = ws + W.off_xrot + (size_t)t0 * p.x_token;
+            p.partial = (float*)(ws + W.off_sums);
+            p.m = d.d_out;
+            p.n = d.d_in;
+            p.T = tc;
+            p.cb_rows = d.cb_rows;
+            p.cb_cols = d.cb_cols;
+            p.n_cg = L.n_cg;
+            p.max_books = plan.max_books;
+            p.stages = plan.stages;
+            p.total = plan.total;
+            p.ctas = plan.ctas;
+            p.inv_stages = vq_reciprocal(plan.stages);
+            p.inv_cb_cols = vq_reciprocal(d.cb_cols);
+            p.inv_group = vq_reciprocal(d.cb_rows / plan.rb);  // row blocks that share codebooks
+            const __half* A = (const __half*)(blob + L.off_a);
+            const __half* tt = tbuf + (size_t)t0 * L.r_pad;
+            void* yt = (uint8_t*)y + (size_t)t0 * ldy * esz;
+            const int r_pad = d.rank > 0 ? L.r_pad : 0, f32 = out_dtype == LOPRO_OUT_F32;
+            const cudaError_t e = tc <= 8 ? launch_vq_product<1>(p, plan, A, tt, r_pad, yt, ldy, f32, s)
+                                          : (tc <= 16 ? launch_vq_product<2>(p, plan, A, tt, r_pad, yt, ldy, f32, s)
+                                                      : launch_vq_product<4>(p, plan, A, tt, r_pad, yt, ldy, f32, s));
+            if (e != cudaSuccess) return LOPRO_ERR_CUDA;
+            continue;
+        }
         VqParams p;
         p.idx = blob + L.off_idx;
         p.books = blob + L.off_books;
