@@ -124,7 +124,7 @@ enum {
     LOPRO_OPT_NO_TCGEN05 = 3,    /* 1: never the tcgen05 prefill kernel (general register-ring product)        */
     LOPRO_OPT_PREFILL_PAIRS = 4, /* >= 0: number of two-block row tiles of the prefill grid; where two CTAs share a
                                      tile (512 tokens and more): number of K parts of the last wave's tiles, 0 or 1
-                                     = none, at most 4; -1: chosen by the library                              */
+                                     = none, at most 16; -1: chosen by the library                              */
     LOPRO_OPT_ONE_KERNEL_SET = 5, /* 1: single-layer forwards launch the same kernel variants as grouped ones
                                       (lopro_linear_fwd_group / _experts), which carry a table of sibling layers in
                                       their parameters.  By default a single-layer forward launches variants without
@@ -298,7 +298,9 @@ LOPRO_API lopro_status lopro_linear_fwd_host(const lopro_desc* desc, const void*
  * budget.  It computes exactly what lopro_linear_fwd computes, with the same arguments minus the
  * workspace: the scratch is a fixed array of LOPRO_NOALLOC_SCRATCH_BYTES inside the library itself
  * (every GPU that loads the library holds that memory until the process ends).
- *   - Accepted sizes: lopro_workspace_bytes(desc, T) <= LOPRO_NOALLOC_SCRATCH_BYTES, which covers
+ *   - Accepted sizes: whatever the forward can run in LOPRO_NOALLOC_SCRATCH_BYTES: every layer and token
+ *     count with lopro_workspace_bytes(desc, T) <= LOPRO_NOALLOC_SCRATCH_BYTES, and more of them with
+ *     fewer parallel parts than in a workspace of that size.  This covers
  *     the small-batch (decode) range of ordinary layers, e.g. d_in = 8192 with T <= 32.  Anything
  *     larger returns LOPRO_ERR_BUFFER_TOO_SMALL and does nothing.
  *   - The call allocates and frees nothing and does not synchronise.  The first call on each device

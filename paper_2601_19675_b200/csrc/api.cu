@@ -51,7 +51,7 @@ lopro_status blob_layout(const lopro_desc& d, BlobLayout* out) {
     return LOPRO_OK;
 }
 
-lopro_status workspace_layout(const lopro_desc& d, int T, WorkspaceLayout* W) {
+lopro_status workspace_layout(const lopro_desc& d, int T, WorkspaceLayout* W, bool compact) {
     lopro_status st = check_desc(d);
     if (st != LOPRO_OK) return st;
     if (T < 0) return LOPRO_ERR_INVALID_ARG;
@@ -59,6 +59,7 @@ lopro_status workspace_layout(const lopro_desc& d, int T, WorkspaceLayout* W) {
     const int r_pad = round_up_int(d.rank, 16);
     size_t off = 0;
     W->t_pad = t_pad;
+    W->compact = compact ? 1 : 0;
     W->off_status = off;
     off += 256;
     W->off_xrot = off;
@@ -73,9 +74,9 @@ lopro_status workspace_layout(const lopro_desc& d, int T, WorkspaceLayout* W) {
     W->off_t = off;
     off += round_up_size((size_t)t_pad * (r_pad > 0 ? r_pad : 16) * 2, 256);
     W->off_lrpart = off;
-    if (T > kDecodeMaxT && d.rank > 0) off += round_up_size(lowrank_mma_scratch_bytes(d, T), 256);
+    if (T > kDecodeMaxT && d.rank > 0) off += round_up_size(lowrank_mma_scratch_bytes(d, T, compact), 256);
     W->off_kparts = off;
-    off += round_up_size(prefill_kparts_bytes(d, T), 256);
+    off += round_up_size(prefill_kparts_bytes(d, T, compact), 256);
     // FP8 low-rank record on the tensor-core path: the fp16 factors it is folded into
     W->off_fold_a = W->off_fold_b = off;
     if (d.lowrank_format == LOPRO_LOWRANK_FP8 && T > kDecodeMaxT) {
@@ -395,9 +396,10 @@ static bool group_uses_tall(int32_t n, const lopro_desc* const* descs, int32_t T
 // the small-batch kernels when that costs less than the tensor-core path: a prefill CTA walks all of K for its
 // 128 or 256 rows whatever the token count, and a layer with few rows fills few SMs.  Both sides are estimated from
 // timings on B200 (microseconds, beyond a common 8 for the first launches): a chunk 3 + 0.45e-6 d_out d_in (10.9 for
-// 4096 x 4096, 23.4 for 4096 x 11008 either way round), the tensor-core product by prefill_estimate_us plus 0.0015 d_in
-// for the longer launches in front of it (4096 x 4096: chunks up to 64 tokens, 25.0 against 29.8; 11008 -> 4096: up to
-// 96, 77 against 84).  LOPRO_OPT_NO_CHUNKS turns this off (A/B runs, tests of the prefill kernels on small layers).
+// 4096 x 4096, 23.4 for 4096 x 11008 either way round), or 3 + 1.87e-3 d_in where that is more (a CTA's 32 rows walk all of
+// K: 18.2 for 8192 columns however few the rows), the tensor-core product by prefill_plan plus 0.0015 d_in for the longer
+// launches in front of it (4096 x 4096: chunks up to 64 tokens, 23.7 against 25.4; 11008 -> 4096 at 33 tokens 36.3 against
+// 44.0).  LOPRO_OPT_NO_CHUNKS turns this off (A/B runs, tests of the prefill kernels on small layers).
 static int small_batch_chunks(const lopro_desc& d, int T) {
     if (T <= kDecodeMaxT) return 0;
     // the FP8 low-rank record has no general path: chunks wherever the tensor-core kernels cannot take the layer
@@ -406,8 +408,9 @@ static int small_batch_chunks(const lopro_desc& d, int T) {
     if (option(LOPRO_OPT_NO_CHUNKS) == 1) return 0;
     if (!prefill_supported(d, T)) return 0;  // keep the general path's behaviour where there is no prefill kernel
     const int chunks = (T + kDecodeMaxT - 1) / kDecodeMaxT;
-    const double chunk_us = 3.0 + 0.45e-6 * (double)d.d_out * (double)d.d_in;
-    const double prefill_us = prefill_estimate_us(d, T, nullptr) + 0.0015 * (double)d.d_in;  // + its longer launches in front
+    const double by_weights = 0.45e-6 * (double)d.d_out * (double)d.d_in, by_columns = 1.87e-3 * (double)d.d_in;
+    const double chunk_us = 3.0 + (by_weights > by_columns ? by_weights : by_columns);
+    const double prefill_us = prefill_plan(d, T).us + 0.0015 * (double)d.d_in;  // + its longer launches in front
     if ((double)chunks * chunk_us >= prefill_us) return 0;
     if (!prologue_supported(d, kDecodeMaxT) || !stream_supported(d, kDecodeMaxT)) return 0;
     return chunks;
@@ -441,16 +444,15 @@ int32_t lopro_linear_fwd_path(const lopro_desc* desc, int32_t T, int32_t* launch
         path = use_tall(*desc, T) ? LOPRO_PATH_TALL : (stream_uses_wide(*desc, T) ? LOPRO_PATH_WIDE : LOPRO_PATH_STREAM);
         n = 2;
     } else {
-        const int pre = (T > kDecodeMaxT && rotate_lowrank_supported(*desc, T))
+        const int pre = (T > kDecodeMaxT && prefill_supported(*desc, T) && rotate_lowrank_supported(*desc, T))
                             ? 2
                             : 1 + (desc->rank > 0 ? (T > kDecodeMaxT ? 2 : 1) : 0);
         path = prefill_supported(*desc, T) ? LOPRO_PATH_PREFILL : LOPRO_PATH_GENERAL;
         n = pre + 1;
         if (desc->lowrank_format == LOPRO_LOWRANK_FP8) ++n;  // the record folded into fp16 factors
         if (path == LOPRO_PATH_PREFILL) {
-            bool use_pairs = false;
-            (void)prefill_estimate_us(*desc, T, &use_pairs);
-            if (use_pairs && pair_plan(*desc, T).split_tiles > 0) ++n;  // the sum of the K parts of the last wave's tiles
+            const PrefillPlan plan = prefill_plan(*desc, T);
+            if (plan.use_pairs ? plan.pair.split_tiles > 0 : plan.k_parts > 1) ++n;  // the sum of the K parts
         }
     }
     if (launches) *launches = n;
@@ -477,7 +479,11 @@ lopro_status lopro_linear_fwd(const lopro_desc* desc, const void* packed, const 
     WorkspaceLayout W;
     st = workspace_layout(*desc, T, &W);
     if (st != LOPRO_OK) return st;
-    if (workspace_bytes < W.total) return LOPRO_ERR_BUFFER_TOO_SMALL;
+    if (workspace_bytes < W.total) {
+        // (the fixed scratch of lopro_linear_fwd_noalloc: fewer K slices and K parts)
+        workspace_layout(*desc, T, &W, true);
+        if (workspace_bytes < W.total) return LOPRO_ERR_BUFFER_TOO_SMALL;
+    }
 
     cudaStream_t s = (cudaStream_t)stream;
     uint8_t* ws = (uint8_t*)workspace;
@@ -556,10 +562,11 @@ lopro_status lopro_linear_fwd(const lopro_desc* desc, const void* packed, const 
         B = fb;
         a_f16 = fa;
     }
-    if (T > kDecodeMaxT && rotate_lowrank_supported(*desc, T)) {
+    // (the one grid writes no 64-column sums, which the general product needs)
+    if (T > kDecodeMaxT && prefill_supported(*desc, T) && rotate_lowrank_supported(*desc, T)) {
         // many tokens: rotation and B x side by side in one grid, then the sum over K slices
         if (launch_rotate_lowrank(*desc, perm, (const __nv_bfloat16*)x_bf16, ldx, xrot, desc->d_in, s64, status, B, L.r_pad,
-                                  (float*)(ws + W.off_lrpart), (__half*)(ws + W.off_t), T, s) != cudaSuccess)
+                                  (float*)(ws + W.off_lrpart), (__half*)(ws + W.off_t), T, s, W.compact != 0) != cudaSuccess)
             return LOPRO_ERR_CUDA;
     } else {
     if (launch_rotate(*desc, perm, (const __nv_bfloat16*)x_bf16, ldx, xrot, desc->d_in, s64, status, T, s) !=
@@ -568,7 +575,7 @@ lopro_status lopro_linear_fwd(const lopro_desc* desc, const void* packed, const 
     if (desc->rank > 0) {
         cudaError_t e = T > kDecodeMaxT
                             ? launch_lowrank_down_mma(*desc, B, L.r_pad, (const __nv_bfloat16*)x_bf16, ldx,
-                                                      (float*)(ws + W.off_lrpart), (__half*)(ws + W.off_t), T, s)
+                                                      (float*)(ws + W.off_lrpart), (__half*)(ws + W.off_t), T, s, W.compact != 0)
                             : launch_lowrank_down(*desc, B, L.r_pad, (const __nv_bfloat16*)x_bf16, ldx,
                                                   (__half*)(ws + W.off_t), T, s);
         if (e != cudaSuccess) return LOPRO_ERR_CUDA;

@@ -76,6 +76,7 @@ inline size_t round_up_size(size_t v, size_t a) { return (v + a - 1) / a * a; }
 struct WorkspaceLayout {
     size_t off_status, off_xrot, off_s64, off_t, off_lrpart, off_kparts, off_fold_a, off_fold_b, total;
     int t_pad;  // tokens padded to a multiple of 8
+    int compact;  // 1: fewer K slices and K parts, the least that the forward runs in
     // row-block layout only: the operand image of the tcgen05 small-batch kernel (see ImageOut)
     size_t off_counters, off_ximg, off_sums, off_timg, off_partial;
     int np;        // tokens per image tile: 16 (T <= 16) or 32
@@ -92,7 +93,7 @@ inline int s64_stride(int n) { return ((n / 64 + 15) / 16) * 16; }
 // reads of eight tokens conflict-free).  One bulk copy then brings a stage's activations.
 constexpr int kActRecord = 2048 + 64 + 16;
 inline size_t act_image_bytes(int n, int t_pad) { return (size_t)((n + 1023) / 1024) * t_pad * kActRecord; }
-lopro_status workspace_layout(const lopro_desc& d, int T, WorkspaceLayout* out);
+lopro_status workspace_layout(const lopro_desc& d, int T, WorkspaceLayout* out, bool compact = false);
 
 // Operand image of the tcgen05 small-batch kernel, written by the prologue (or converted from the plain rotated
 // activations): per group of NP tokens and 64-column step one K-major tile [NP tokens][64 columns] of bf16 with the
@@ -206,14 +207,15 @@ cudaError_t launch_tall(const lopro_desc& d, const uint8_t* blob, const BlobLayo
                         const StreamSiblingArgs* more = nullptr);
 
 // t = B x on the tensor cores for many tokens; `partial` holds lowrank_mma_scratch_bytes of fp32 K-slice sums.
-size_t lowrank_mma_scratch_bytes(const lopro_desc& d, int T);
+int lowrank_mma_slices(const lopro_desc& d, int T, bool compact = false);
+size_t lowrank_mma_scratch_bytes(const lopro_desc& d, int T, bool compact = false);
 cudaError_t launch_lowrank_down_mma(const lopro_desc& d, const __half* B, int r_pad, const __nv_bfloat16* x, int64_t ldx,
-                                    float* partial, __half* t, int T, cudaStream_t s);
+                                    float* partial, __half* t, int T, cudaStream_t s, bool compact = false);
 // Rotation and t = B x of a many-token forward in one grid (plus the dependent launch that adds the K slices).
 bool rotate_lowrank_supported(const lopro_desc& d, int T);
 cudaError_t launch_rotate_lowrank(const lopro_desc& d, const int32_t* perm, const __nv_bfloat16* x, int64_t ldx,
                                   __nv_bfloat16* xrot, int64_t ldo, float* s64, int* status, const __half* B, int r_pad,
-                                  float* partial, __half* t, int T, cudaStream_t s);
+                                  float* partial, __half* t, int T, cudaStream_t s, bool compact = false);
 // Prefill forward (T > 32) on tcgen05 / TMEM, after launch_rotate and launch_lowrank_down.
 bool prefill_supported(const lopro_desc& d, int T);
 // Tiling of the prefill kernel that puts two CTAs on a tile (large batches): n_tiles tiles of 256 rows x 512 tokens, the
@@ -221,10 +223,17 @@ bool prefill_supported(const lopro_desc& d, int T);
 struct PairPlan {
     int use, row_tiles, n_tiles, split_tiles, k_parts;
 };
-PairPlan pair_plan(const lopro_desc& d, int T);
-size_t prefill_kparts_bytes(const lopro_desc& d, int T);
-// Estimated duration (microseconds) of the tensor-core product for T > 32 tokens and whether it runs two CTAs per tile
-double prefill_estimate_us(const lopro_desc& d, int T, bool* use_pairs);
+// How the tensor-core product of T > 32 tokens runs, and an estimate of its duration in microseconds.  One CTA per tile:
+// pair_tiles row tiles of two 128-row blocks and single_tiles of one, units token tiles of tile_n, every tile cut along K
+// into k_parts units.  compact: within the workspace of the compact layout.
+struct PrefillPlan {
+    int use_pairs;
+    PairPlan pair;
+    int tile_n, units, pair_tiles, single_tiles, k_parts;
+    double us;
+};
+PrefillPlan prefill_plan(const lopro_desc& d, int T, bool compact = false);
+size_t prefill_kparts_bytes(const lopro_desc& d, int T, bool compact = false);
 // FP8 low-rank record -> fp16 factors A = U Sigma [m][r_pad], B = V / s [r_pad][n] in the workspace (tensor-core path)
 cudaError_t launch_lr8_fold(const lopro_desc& d, int r_pad, const uint8_t* U, const uint8_t* V, const __half* sigma,
                             const __half* svec, __half* A, __half* B, cudaStream_t s);

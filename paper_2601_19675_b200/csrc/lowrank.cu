@@ -169,45 +169,60 @@ rotate_lowrank_kernel(const __nv_bfloat16* __restrict__ x, int64_t ldx, const in
     }
 }
 
-// Adds the K slices in order and rounds once to fp16.  Safe under a programmatic launch: waits for the producer.
+// Adds the K slices in order and rounds once to fp16; eight loads in flight (4096 -> 4096 at 512 tokens: 40.7 -> 39.4 us for
+// the whole forward).  Safe under a programmatic launch: waits for the producer.
 __global__ void lowrank_finish_kernel(const float* __restrict__ partial, __half* __restrict__ t, size_t count, int slices) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
     float s = 0.0f;
-    for (int k = 0; k < slices; ++k) s += partial[(size_t)k * count + i];
+#pragma unroll 8
+    for (int k = 0; k < slices; ++k) s += __ldcg(partial + (size_t)k * count + i);
     t[i] = __float2half_rn(s);
 }
 
 }  // namespace
 
-int lowrank_mma_slices(const lopro_desc& d, int T) {
-    const int tiles = (T + kLrTokens - 1) / kLrTokens;
-    int slices = 1;
-    while (slices < 32 && tiles * slices < 512 && d.d_in / (slices * 2) >= 256 && (d.d_in / 64) % (slices * 2) == 0) slices *= 2;
-    return slices;
+// K slices of the down-projection: four 64-column steps each, more where that would make over 512 CTAs; the last slice
+// may be shorter.  Slices need not divide the width: when they had to, a width of an odd number of steps had one CTA
+// walk all of K (5696 -> 4160 at 133 tokens: 150.8 us for the whole forward, most of it here).  Two steps per slice
+// are slower at 512 tokens (4096 -> 4096: 45.9 against 41.9 us), the sums then cost more than the steps.
+// compact: the old rule, for workspaces sized by it.
+int lowrank_mma_slices(const lopro_desc& d, int T, bool compact) {
+    const int tiles = (T + kLrTokens - 1) / kLrTokens, steps = d.d_in / kLrChunk;
+    if (compact) {
+        int slices = 1;
+        while (slices < 32 && tiles * slices < 512 && d.d_in / (slices * 2) >= 256 && steps % (slices * 2) == 0) slices *= 2;
+        return slices;
+    }
+    int per = (int)(((long long)steps * tiles + 511) / 512);
+    if (per < 4) per = 4;
+    return (steps + per - 1) / per;
 }
-
+static int lowrank_slice_cols(const lopro_desc& d, int slices) {
+    const int steps = d.d_in / kLrChunk;
+    return (steps + slices - 1) / slices * kLrChunk;
+}
 // Bytes reserved for the K-slice sums of up to T tokens.  The slice count falls as the token tiles grow, so the
 // need of a launch, slices(T) * T rows, is not monotone in T; the reservation is the largest need of any token
 // count up to T (the slice count is constant within a tile count, so the last T of each tile count decides).
-size_t lowrank_mma_scratch_bytes(const lopro_desc& d, int T) {
+size_t lowrank_mma_scratch_bytes(const lopro_desc& d, int T, bool compact) {
     const int r_pad = round_up_int(d.rank, 16);
     const int tiles = (T + kLrTokens - 1) / kLrTokens;
     size_t rows = 0;
     for (int tl = 1; tl <= tiles; ++tl) {
         const int t_last = tl * kLrTokens < T ? tl * kLrTokens : T;
-        const size_t need = (size_t)lowrank_mma_slices(d, t_last) * (size_t)t_last;
+        const size_t need = (size_t)lowrank_mma_slices(d, t_last, compact) * (size_t)t_last;
         if (need > rows) rows = need;
     }
     return rows * (size_t)r_pad * 4;
 }
 
 cudaError_t launch_lowrank_down_mma(const lopro_desc& d, const __half* B, int r_pad, const __nv_bfloat16* x, int64_t ldx,
-                                    float* partial, __half* t, int T, cudaStream_t s) {
-    const int slices = lowrank_mma_slices(d, T);
-    const int slice_cols = d.d_in / slices;
+                                    float* partial, __half* t, int T, cudaStream_t s, bool compact) {
+    const int slices = lowrank_mma_slices(d, T, compact);
+    const int slice_cols = lowrank_slice_cols(d, slices);
     dim3 grid((T + kLrTokens - 1) / kLrTokens, slices);
     for (int j0 = 0; j0 < r_pad; j0 += kLrMaxRank) {
         const int rows = r_pad - j0 < kLrMaxRank ? r_pad - j0 : kLrMaxRank;
@@ -242,9 +257,9 @@ namespace {
 template <int NJ>
 cudaError_t launch_rotate_lowrank_nj(const lopro_desc& d, const int32_t* perm, const __nv_bfloat16* x, int64_t ldx,
                                      __nv_bfloat16* xrot, int64_t ldo, float* s64, int* status, const __half* B, int r_pad,
-                                     float* partial, int T, cudaStream_t s) {
-    const int slices = lowrank_mma_slices(d, T);
-    const int slice_cols = d.d_in / slices;
+                                     float* partial, int T, cudaStream_t s, bool compact) {
+    const int slices = lowrank_mma_slices(d, T, compact);
+    const int slice_cols = lowrank_slice_cols(d, slices);
     // rotation CTAs: the tensor-core form of the recursion with 8 rows per CTA where that leaves room for three CTAs
     // per SM, with 4 rows otherwise; the register-and-shuffle form where the block size or prefix rules it out
     const bool mma_form = rotate_mma_shape_ok(d) && (reinterpret_cast<uintptr_t>(perm) % 16) == 0 &&
@@ -315,20 +330,20 @@ cudaError_t launch_lr8_fold(const lopro_desc& d, int r_pad, const uint8_t* U, co
 
 bool rotate_lowrank_supported(const lopro_desc& d, int T) {
     const int r_pad = round_up_int(d.rank, 16);
-    // from 64 tokens on the one grid beats rotation and B x as two launches (11008 columns, 128 tokens: 84.6 -> 75.5 us
-    // for the whole forward; 8192 columns: 145 -> 141)
-    return d.rank > 0 && r_pad <= kLrMaxRank && T >= 64 && d.block_size <= 256 && d.identity_cols % 64 == 0 &&
+    // the one grid beats rotation and B x as two launches at every token count (11008 columns, 128 tokens: 84.6 -> 75.5 us
+    // for the whole forward; 8192 columns: 145 -> 141; 4096 -> 11008 at 33 tokens: 41.0 -> 34.8)
+    return d.rank > 0 && r_pad <= kLrMaxRank && T > kDecodeMaxT && d.block_size <= 256 && d.identity_cols % 64 == 0 &&
            (size_t)d.d_in * 8 <= 160 * 1024;
 }
 
 cudaError_t launch_rotate_lowrank(const lopro_desc& d, const int32_t* perm, const __nv_bfloat16* x, int64_t ldx,
                                   __nv_bfloat16* xrot, int64_t ldo, float* s64, int* status, const __half* B, int r_pad,
-                                  float* partial, __half* t, int T, cudaStream_t s) {
+                                  float* partial, __half* t, int T, cudaStream_t s, bool compact) {
     cudaError_t e;
-    if (r_pad > 64) e = launch_rotate_lowrank_nj<16>(d, perm, x, ldx, xrot, ldo, s64, status, B, r_pad, partial, T, s);
-    else if (r_pad > 32) e = launch_rotate_lowrank_nj<8>(d, perm, x, ldx, xrot, ldo, s64, status, B, r_pad, partial, T, s);
-    else if (r_pad > 16) e = launch_rotate_lowrank_nj<4>(d, perm, x, ldx, xrot, ldo, s64, status, B, r_pad, partial, T, s);
-    else e = launch_rotate_lowrank_nj<2>(d, perm, x, ldx, xrot, ldo, s64, status, B, r_pad, partial, T, s);
+    if (r_pad > 64) e = launch_rotate_lowrank_nj<16>(d, perm, x, ldx, xrot, ldo, s64, status, B, r_pad, partial, T, s, compact);
+    else if (r_pad > 32) e = launch_rotate_lowrank_nj<8>(d, perm, x, ldx, xrot, ldo, s64, status, B, r_pad, partial, T, s, compact);
+    else if (r_pad > 16) e = launch_rotate_lowrank_nj<4>(d, perm, x, ldx, xrot, ldo, s64, status, B, r_pad, partial, T, s, compact);
+    else e = launch_rotate_lowrank_nj<2>(d, perm, x, ldx, xrot, ldo, s64, status, B, r_pad, partial, T, s, compact);
     if (e != cudaSuccess) return e;
     // the K slices are added by a dependent launch that waits for the grid above
     const size_t count = (size_t)T * r_pad;
@@ -341,7 +356,7 @@ cudaError_t launch_rotate_lowrank(const lopro_desc& d, const int32_t* perm, cons
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, lowrank_finish_kernel, (const float*)partial, t, count, lowrank_mma_slices(d, T));
+    return cudaLaunchKernelEx(&cfg, lowrank_finish_kernel, (const float*)partial, t, count, lowrank_mma_slices(d, T, compact));
 }
 
 }  // namespace lopro

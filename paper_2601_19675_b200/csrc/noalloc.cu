@@ -35,7 +35,8 @@ extern "C" lopro_status lopro_linear_fwd_noalloc(const lopro_desc* desc, const v
                                                  void* stream) {
     if (!desc) return LOPRO_ERR_INVALID_ARG;
     if (T < 0) return LOPRO_ERR_INVALID_ARG;
-    const size_t need = lopro_workspace_bytes(desc, T);
+    lopro::WorkspaceLayout W;
+    const size_t need = lopro::workspace_layout(*desc, T, &W, true) == LOPRO_OK ? W.total : 0;
     if (need == 0) return lopro_check_desc(desc) != LOPRO_OK ? lopro_check_desc(desc) : LOPRO_ERR_INVALID_ARG;
     if (need > (size_t)LOPRO_NOALLOC_SCRATCH_BYTES) return LOPRO_ERR_BUFFER_TOO_SMALL;  // layer x tokens too large
     if (T == 0) return LOPRO_OK;

@@ -59,6 +59,8 @@ struct PrefillParams {
     int single_tiles;  // row tiles of one block
     int units;         // token tiles
     int lr_stages;   // ceil(r_pad / 64)
+    int k_parts;     // units that a tile is cut into along K (1: whole tiles)
+    float* kparts;   // their fp32 partial sums, [unit][tile_n tokens][256 rows]
 };
 
 template <int BITS>
@@ -75,15 +77,20 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap map_x,
     // The grid is one-dimensional and lists every two-block CTA (256 rows, two accumulators) before the
     // one-block CTAs, so that the cheaper tiles fill the last wave: pair_tiles two-block row tiles and
     // single_tiles one-block row tiles per token tile.
+    // Where those do not fill the multiprocessors every tile is cut along K into k_parts CTAs.
     const int n_pair_ctas = p.pair_tiles * p.units;
-    const bool is_pair = (int)blockIdx.x < n_pair_ctas;
+    const int tile_id = (int)blockIdx.x / p.k_parts, part = (int)blockIdx.x - tile_id * p.k_parts;
+    const bool is_pair = tile_id < n_pair_ctas;
     const int n_acc = is_pair ? 2 : 1;
-    const int rest = (int)blockIdx.x - n_pair_ctas;
-    const int tile_x = is_pair ? (int)blockIdx.x % p.pair_tiles : p.pair_tiles + rest % p.single_tiles;
-    const int tile_y = is_pair ? (int)blockIdx.x / p.pair_tiles : rest / p.single_tiles;
+    const int rest = tile_id - n_pair_ctas;
+    const int tile_x = is_pair ? tile_id % p.pair_tiles : p.pair_tiles + rest % p.single_tiles;
+    const int tile_y = is_pair ? tile_id / p.pair_tiles : rest / p.single_tiles;
     const int row_base = (is_pair ? tile_x * 2 : p.pair_tiles + tile_x) * kTileM;
     const int tok_base = tile_y * p.tile_n;
-    const int total = p.nsteps + p.lr_stages;
+    // the CTA's stages [s_begin, s_begin + total) of the layer's weight stages and low-rank stages
+    const int all_stages = p.nsteps + p.lr_stages;
+    const int s_begin = all_stages * part / p.k_parts, total = all_stages * (part + 1) / p.k_parts - s_begin;
+    const int n_weight = p.nsteps - s_begin;  // stages from here on (counted from s_begin) are low-rank ones
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;  // swizzle atoms are 1024-byte aligned
     unsigned char* base_ptr = smem_raw + (base - raw);
@@ -152,10 +159,10 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap map_x,
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 const int s = vstride * v + 2 * g + j;
-                if (valid && s < p.nsteps) {
+                if (valid && s < total && s < n_weight) {
 #pragma unroll
-                    for (int q = 0; q < BITS; ++q) wbuf[buf][j][q] = __ldg(wbase + (size_t)s * 32 * BITS + q);
-                    const uint32_t* z = szbase + (size_t)(s >> p.gshift) * 16;
+                    for (int q = 0; q < BITS; ++q) wbuf[buf][j][q] = __ldg(wbase + (size_t)(s_begin + s) * 32 * BITS + q);
+                    const uint32_t* z = szbase + (size_t)((s_begin + s) >> p.gshift) * 16;
                     szbuf[buf][j][0] = __ldg(z);
                     szbuf[buf][j][1] = __ldg(z + 8);
                 }
@@ -198,7 +205,7 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap map_x,
                         if (s < total) {
                             const int slot = s & 3, use = s >> 2;
                             if (use >= 1) warp_wait(empty_a(slot), (uint32_t)(use - 1) & 1u);
-                            if (valid && s < p.nsteps)
+                            if (valid && s < n_weight)
                                 convert(wbuf[u][j], szbuf[u][j][0], szbuf[u][j][1], blk_ptr + slot * kABytes);
                         }
                     }
@@ -227,11 +234,11 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap map_x,
                 if (s >= kBStages) wait_phase(empty_b(sb), (uint32_t)((s / kBStages) - 1) & 1u);
                 const uint32_t a_tile = base + sa * kABytes, b_tile = b_ring + sb * kBBytes;
                 mbar_expect_tx(full_b(sb), b_bytes);
-                if (s < p.nsteps) {
-                    tma_load_2d(b_tile, &map_x, s * kStageK, tok_base, full_b(sb));
+                if (s < n_weight) {
+                    tma_load_2d(b_tile, &map_x, (s_begin + s) * kStageK, tok_base, full_b(sb));
                     mbar_arrive(full_a(sa));
                 } else {
-                    const int lr = s - p.nsteps;
+                    const int lr = s - n_weight;
                     tma_load_2d(b_tile, &map_t, lr * kStageK, tok_base, full_b(sb));
                     mbar_expect_tx(full_a(sa), (uint32_t)(n_acc * kABlock));
                     for (int acc = 0; acc < n_acc; ++acc)
@@ -274,8 +281,8 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap map_x,
                     ready_a = mbar_test_wait(full_a(sa), pa);
                     ready_b = mbar_test_wait(full_b(sb), pb);
                 }
-                const bool lowrank = s >= p.nsteps;
-                const int ksub = lowrank ? min(4, (p.r_pad - (s - p.nsteps) * kStageK) / 16) : 4;
+                const bool lowrank = s >= n_weight;
+                const int ksub = lowrank ? min(4, (p.r_pad - (s - n_weight) * kStageK) / 16) : 4;
                 const uint32_t idesc = lowrank ? idesc_lr : idesc_w;
                 for (int k = 0; k < ksub; ++k)  // 16 columns = 32 bytes = 2 descriptor address units
                     umma_f16(d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, (s > 0 || k > 0) ? 1u : 0u);
@@ -308,7 +315,12 @@ prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap map_x,
                     : "r"(taddr)
                     : "memory");
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (p.y_vec) {
+                if (p.k_parts > 1) {
+                    float* dst = p.kparts + ((size_t)blockIdx.x * p.tile_n + c0) * 256 + acc * kTileM + lane_base + lane;
+#pragma unroll
+                    for (int i = 0; i < 32; ++i)
+                        if (tok_base + c0 + i < p.T) dst[(size_t)i * 256] = __uint_as_float(v[i]);
+                } else if (p.y_vec) {
                     // bf16 rows of 32 tokens meet in shared memory (the rings are idle now), [token][32 rows], and
                     // leave as 16-byte pieces of eight consecutive rows
                     __nv_bfloat16* stg = reinterpret_cast<__nv_bfloat16*>(base_ptr + (warp - kDequantWarps) * 2048);
@@ -375,8 +387,9 @@ constexpr int kPairSmemBytes = kPairAStages * kPairABytes + kPairBStages * kPair
 #ifndef LOPRO_PAIR_MIN_T
 #define LOPRO_PAIR_MIN_T 512
 #endif
-constexpr int kPairMinT = LOPRO_PAIR_MIN_T;   // from here on always two CTAs per tile; below, by prefill_estimate_us
-constexpr int kMaxKParts = 4;    // K parts of a tile of the last wave
+constexpr int kPairMinT = LOPRO_PAIR_MIN_T;   // from here on always two CTAs per tile; below, by prefill_plan
+constexpr int kMaxKParts = 16;   // K parts of a tile (of the last wave of the two-CTA kernel)
+constexpr int kCompactKParts = 4;  // ... in a workspace of the compact layout
 
 struct PairParams {
     const uint32_t* codes;
@@ -762,34 +775,95 @@ cudaError_t launch_prefill_bits(const PrefillParams& p, const CUtensorMap& mx, c
 }
 
 // The partial sums of the units cut along K, added in a fixed order: y[token][row] = sum over parts.  One thread per
-// token and four rows.
-__global__ void __launch_bounds__(256)
-prefill_kparts_kernel(const float* __restrict__ kparts, void* __restrict__ y, int64_t ldy, int out_f32, int m, int T,
-                      int row_tiles, int first_tile, int k_parts, int kp_tokens) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int blocks_per_tile = kp_tokens >> 2;                  // blocks of 4 tokens x 256 rows
+// four rows of two tokens, eight 16-byte loads in flight and 8-byte stores (4096 -> 11008 at 203 tokens: 46.2 us for the
+// whole forward, 47.8 with one token per thread and 2-byte stores).  It must not release its successor early: the next
+// forward's rotation then takes the multiprocessors' shared memory before the product is out (48 -> 54 us).  Tiles from first_tile on, of tile_tokens tokens; the two-CTA kernel's are 256 rows in row-major order
+// (pair_ctas = -1), the one-CTA kernel's two-block tiles (pair_ctas of them) precede its one-block tiles.
+struct KPartsSum {
+    const float* kparts;
+    void* y;
+    int64_t ldy;
+    int out_f32, y_vec, m, T;
+    int first_tile, k_parts, kp_tokens, tile_tokens;
+    int row_tiles;                              // two-CTA kernel
+    int pair_ctas, pair_tiles, single_tiles;    // one-CTA kernel
+};
+__global__ void __launch_bounds__(256) prefill_kparts_kernel(const KPartsSum p) {
+    const int blocks_per_tile = p.kp_tokens >> 3;                // blocks of 8 tokens x 256 rows
     const int split_tile = (int)blockIdx.x / blocks_per_tile;
-    const int tok_l = (((int)blockIdx.x % blocks_per_tile) << 2) + ((int)threadIdx.x >> 6);
+    const int tok_l = (((int)blockIdx.x - split_tile * blocks_per_tile) << 3) + ((int)threadIdx.x >> 6);
     const int row_l = ((int)threadIdx.x & 63) << 2;
-    const int tile = first_tile + split_tile;
-    const int tok = (tile / row_tiles) * 512 + tok_l, row = (tile % row_tiles) * 256 + row_l;
-    if (tok >= T || row >= m) return;
-    const float* src = kparts + (((size_t)split_tile * k_parts) * kp_tokens + tok_l) * 256 + row_l;
-    float4 acc = __ldcg(reinterpret_cast<const float4*>(src));
-    for (int part = 1; part < k_parts; ++part) {
-        const float4 v = __ldcg(reinterpret_cast<const float4*>(src + (size_t)part * kp_tokens * 256));
-        acc.x += v.x;
-        acc.y += v.y;
-        acc.z += v.z;
-        acc.w += v.w;
+    const int tile = p.first_tile + split_tile;
+    int row0, tile_y, rows = 256;
+    if (p.pair_ctas < 0) {
+        row0 = (tile % p.row_tiles) * 256;
+        tile_y = tile / p.row_tiles;
+    } else if (tile < p.pair_ctas) {
+        row0 = (tile % p.pair_tiles) * 256;
+        tile_y = tile / p.pair_tiles;
+    } else {
+        const int rest = tile - p.pair_ctas;
+        row0 = p.pair_tiles * 256 + (rest % p.single_tiles) * kTileM;
+        tile_y = rest / p.single_tiles;
+        rows = kTileM;
     }
-    const float r[4] = {acc.x, acc.y, acc.z, acc.w};
-    const size_t o = (size_t)tok * ldy + row;
-    for (int e = 0; e < 4; ++e)
-        if (row + e < m) {  // d_out is a multiple of 64 today; the check keeps the kernel right for any m
-            if (out_f32) reinterpret_cast<float*>(y)[o + e] = r[e];
-            else reinterpret_cast<__nv_bfloat16*>(y)[o + e] = __float2bfloat16_rn(r[e]);
+    const int tok = tile_y * p.tile_tokens + tok_l, row = row0 + row_l;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (tok >= p.T || row >= p.m || row_l >= rows) return;
+    const float* src = p.kparts + (((size_t)split_tile * p.k_parts) * p.kp_tokens + tok_l) * 256 + row_l;
+    float acc[2][4] = {};
+    for (int p0 = 0; p0 < p.k_parts; p0 += 4) {   // eight loads in flight
+        float4 v[4][2];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j)   // the second token's sums are in the buffer although it may lie beyond T
+                if (p0 + i < p.k_parts)
+                    v[i][j] = __ldcg(reinterpret_cast<const float4*>(src + ((size_t)(p0 + i) * p.kp_tokens + j * 4) * 256));
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                if (p0 + i < p.k_parts) {
+                    acc[j][0] += v[i][j].x;
+                    acc[j][1] += v[i][j].y;
+                    acc[j][2] += v[i][j].z;
+                    acc[j][3] += v[i][j].w;
+                }
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        if (tok + j * 4 >= p.T) return;
+        const size_t o = (size_t)(tok + j * 4) * p.ldy + row;
+        if (p.y_vec && row + 3 < p.m) {
+            if (p.out_f32) {
+                *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.y) + o) = make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+            } else {
+                const __nv_bfloat162 lo = __floats2bfloat162_rn(acc[j][0], acc[j][1]), hi = __floats2bfloat162_rn(acc[j][2], acc[j][3]);
+                *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.y) + o) =
+                    make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+            }
+        } else {
+            for (int e = 0; e < 4; ++e)
+                if (row + e < p.m) {
+                    if (p.out_f32) reinterpret_cast<float*>(p.y)[o + e] = acc[j][e];
+                    else reinterpret_cast<__nv_bfloat16*>(p.y)[o + e] = __float2bfloat16_rn(acc[j][e]);
+                }
         }
+    }
+}
+cudaError_t launch_kparts_sum(KPartsSum p, int tiles, cudaStream_t s) {
+    p.y_vec = p.ldy % 4 == 0 && reinterpret_cast<uintptr_t>(p.y) % (p.out_f32 ? 16 : 8) == 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)tiles * (unsigned)(p.kp_tokens / 8));
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, prefill_kparts_kernel, p);
 }
 
 template <int BITS>
@@ -812,11 +886,20 @@ cudaError_t launch_pair_bits(PairParams p, const CUtensorMap& mx, const CUtensor
     cfg.numAttrs = 1;
     e = cudaLaunchKernelEx(&cfg, prefill_pair_kernel<BITS>, p, mx, ma, mt);
     if (e != cudaSuccess || plan.split_tiles == 0) return e;
-    cfg.gridDim = dim3((unsigned)plan.split_tiles * (unsigned)(p.kp_tokens / 4));
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
-    return cudaLaunchKernelEx(&cfg, prefill_kparts_kernel, (const float*)p.kparts, p.y, p.ldy, p.out_f32, p.m, p.T, p.row_tiles,
-                              plan.n_tiles - plan.split_tiles, plan.k_parts, p.kp_tokens);
+    KPartsSum k = {};
+    k.kparts = p.kparts;
+    k.y = p.y;
+    k.ldy = p.ldy;
+    k.out_f32 = p.out_f32;
+    k.m = p.m;
+    k.T = p.T;
+    k.first_tile = plan.n_tiles - plan.split_tiles;
+    k.k_parts = plan.k_parts;
+    k.kp_tokens = p.kp_tokens;
+    k.tile_tokens = 512;
+    k.row_tiles = p.row_tiles;
+    k.pair_ctas = -1;
+    return launch_kparts_sum(k, plan.split_tiles, s);
 }
 
 }  // namespace
@@ -828,9 +911,9 @@ bool prefill_supported(const lopro_desc& d, int T) {
 
 // Tiling of the two-CTA kernel: tiles of 256 rows x 512 tokens over the CTA pairs the device holds at once (one CTA
 // fills a multiprocessor).  The tiles of the last, partial wave are cut along K into as many parts as fill the idle
-// pairs (at most kMaxKParts, at least eight stages each), so that the wave ends early instead of running a full
+// pairs (at most kMaxKParts, at least four stages each), so that the wave ends early instead of running a full
 // tile's length on a few pairs.
-PairPlan pair_plan(const lopro_desc& d, int T) {
+static PairPlan pair_plan(const lopro_desc& d, int T, bool compact) {
     PairPlan plan = {};
     if (T <= kDecodeMaxT) return plan;
     plan.use = 1;
@@ -845,10 +928,11 @@ PairPlan pair_plan(const lopro_desc& d, int T) {
     const int rem = plan.n_tiles % slots;
     const int stages = d.d_in / kStageK + (round_up_int(d.rank, 16) + kStageK - 1) / kStageK;
     int parts = rem > 0 ? slots / rem : 1;
-    if (parts > kMaxKParts) parts = kMaxKParts;
-    if (parts > stages / 8) parts = stages / 8;
+    const int most = compact ? kCompactKParts : kMaxKParts, shortest = compact ? 8 : 4;
+    if (parts > most) parts = most;
+    if (parts > stages / shortest) parts = stages / shortest;
     const int forced = option(LOPRO_OPT_PREFILL_PAIRS);  // tuning and tests: K parts of the last wave, 0 or 1 = none
-    if (forced >= 0 && rem > 0) parts = forced < kMaxKParts ? forced : kMaxKParts;
+    if (forced >= 0 && rem > 0) parts = forced < most ? forced : most;
     if (rem > 0 && parts > slots / rem) parts = slots / rem;  // the units of the last wave fit the resident pairs
     if (parts > stages / 2) parts = stages / 2;  // every part holds at least two stages
     if (parts >= 2) {
@@ -861,47 +945,83 @@ PairPlan pair_plan(const lopro_desc& d, int T) {
     return plan;
 }
 
-// fp32 partial sums of the tiles cut along K: room for the most units any plan may use (one per resident pair, four
-// per tile), whatever the switches say -- a bound that does not decrease as T grows, unlike the plan's own count
+// fp32 partial sums of the tiles cut along K: room for the most units any plan may use (one per resident pair or
+// multiprocessor, kMaxKParts per tile), whatever the switches say -- a bound that does not decrease as T grows, unlike the
+// plan's own count
 static int kparts_tokens(int T) { return T >= 512 ? 512 : round_up_int(T, 32); }
-size_t prefill_kparts_bytes(const lopro_desc& d, int T) {
-    const PairPlan plan = pair_plan(d, T);
+static int single_tile_n(int T) { return T <= 64 ? 64 : (T <= 128 ? 128 : 256); }
+size_t prefill_kparts_bytes(const lopro_desc& d, int T, bool compact) {
+    const PairPlan plan = pair_plan(d, T, compact);
     if (!plan.use) return 0;
     const long long slots = sm_count() / 2 > 0 ? sm_count() / 2 : 1;
-    const long long by_tiles = (long long)plan.n_tiles * kMaxKParts;
-    return (size_t)(by_tiles < slots ? by_tiles : slots) * kparts_tokens(T) * 256 * sizeof(float);
+    const long long by_tiles = (long long)plan.n_tiles * (compact ? kCompactKParts : kMaxKParts);
+    size_t bytes = (size_t)(by_tiles < slots ? by_tiles : slots) * kparts_tokens(T) * 256 * sizeof(float);
+    if (!compact) {
+        // one CTA per tile, which serves fewer than kPairMinT tokens (one-block tiles count as two-block ones here)
+        const int t = T < kPairMinT ? T : kPairMinT - 1, tile_n = single_tile_n(t), units = (t + tile_n - 1) / tile_n;
+        const long long m_tiles = (d.d_out + kTileM - 1) / kTileM, most = m_tiles * units * kMaxKParts;
+        const size_t single = (size_t)(most < sm_count() ? most : sm_count()) * tile_n * 256 * sizeof(float);
+        if (single > bytes) bytes = single;
+    }
+    return bytes;
 }
 
-// Which of the two tensor-core kernels serves T tokens, and an estimate of its duration in microseconds (beyond the
-// launches in front of it), from timings on B200 per 64-column stage of one CTA: two CTAs on a tile 0.95 (two
-// accumulators) or 0.80 (one, T <= 256), one CTA per tile 0.78 (one 128-row block) or 1.03 (two); a tile cut along K
-// costs its share plus 9 (start-up of the shorter units and the kernel that adds them).  From 512 tokens on the
-// two-CTA kernel always; below, whichever is estimated faster: few row tiles favour the two-CTA kernel (its K parts
-// fill the machine), many row tiles and at most 256 tokens the other (twice the rows per CTA for the same conversion).
-double prefill_estimate_us(const lopro_desc& d, int T, bool* use_pairs) {
+// Which of the two tensor-core kernels serves T tokens, how it is tiled, and an estimate of its duration in microseconds
+// (beyond the launches in front of it), from timings on B200 per 64-column stage of one CTA: two CTAs on a tile 0.95 (two
+// accumulators) or 0.80 (one, T <= 256), one CTA per tile 0.78 (one 128-row block) or 1.03 (two).  Tiles that do not fill
+// the machine are cut along K: the one-CTA kernel's all of them, when that makes one wave (its share of the stages, plus 10
+// for the start-up of the units and the kernel that adds them, plus the traffic of the partial sums at 7 TB/s), the two-CTA
+// kernel's the tiles of the last wave (plus 9).  From 512 tokens on the two-CTA kernel always; below, whichever is estimated
+// faster: with 11008 rows, 4096 columns and 203 tokens 43 two-block tiles in three parts each, 22 stages instead of 65
+// (63.8 -> 45.5 us for the whole forward).
+PrefillPlan prefill_plan(const lopro_desc& d, int T, bool compact) {
+    PrefillPlan plan = {};
     const int stages = d.d_in / kStageK + (round_up_int(d.rank, 16) + kStageK - 1) / kStageK;
     // one CTA per tile
-    const int tile_n = T <= 64 ? 64 : (T <= 128 ? 128 : 256);
+    const int tile_n = single_tile_n(T);
     const int units = (T + tile_n - 1) / tile_n, m_tiles = (d.d_out + kTileM - 1) / kTileM;
     const int n_sm = sm_count() > 0 ? sm_count() : 1;
+    plan.tile_n = tile_n;
+    plan.units = units;
+    plan.k_parts = 1;
     const long long two_block = (long long)(m_tiles / 2) * units, one_block = (long long)(m_tiles % 2) * units;
     const long long waves2 = (two_block + n_sm - 1) / n_sm, all_single_waves = ((long long)m_tiles * units + n_sm - 1) / n_sm;
     double single_us = (double)stages * 0.78 * (double)all_single_waves;
     const double mixed_us = (double)stages * (1.03 * (double)waves2 + (one_block > 0 && two_block % n_sm == 0 ? 0.78 : 0.0));
     if (two_block > 0 && mixed_us < single_us) single_us = mixed_us;
     single_us += 4.0;  // start-up and read-out of a CTA
+    if (!compact && T < kPairMinT && option(LOPRO_OPT_PREFILL_PAIRS) < 0) {
+        for (int blocks = 1; blocks <= 2; ++blocks) {
+            const int pair_tiles = blocks == 2 ? m_tiles / 2 : 0, single_tiles = m_tiles - 2 * pair_tiles;
+            if (blocks == 2 && pair_tiles == 0) continue;
+            const long long tiles = (long long)(pair_tiles + single_tiles) * units;
+            long long parts = n_sm / tiles;
+            if (parts > kMaxKParts) parts = kMaxKParts;
+            if (parts > stages / 4) parts = stages / 4;
+            if (parts < 2) continue;
+            const double us = (double)((stages + parts - 1) / parts) * (blocks == 2 ? 1.03 : 0.78) + 10.0 +
+                              2.0 * (double)parts * (double)T * (double)d.d_out * 4.0 / 7e6;
+            if (us < single_us) {
+                single_us = us;
+                plan.k_parts = (int)parts;
+                plan.pair_tiles = pair_tiles;
+                plan.single_tiles = single_tiles;
+            }
+        }
+    }
     // two CTAs per tile
-    const PairPlan plan = pair_plan(d, T);
+    plan.pair = pair_plan(d, T, compact);
     double pair_us = 1e30;
-    if (plan.use && option(LOPRO_OPT_NO_CTA_PAIRS) != 1) {
+    if (plan.pair.use && option(LOPRO_OPT_NO_CTA_PAIRS) != 1) {
         const int slots = n_sm / 2 > 0 ? n_sm / 2 : 1;
         const double tile_us = (double)stages * (T > 256 ? 0.95 : 0.80) + 4.0;
-        const int whole_waves = (plan.n_tiles - plan.split_tiles + slots - 1) / slots;
-        pair_us = tile_us * (double)whole_waves + (plan.split_tiles > 0 ? tile_us / (double)plan.k_parts + 9.0 : 0.0);
+        const int whole_waves = (plan.pair.n_tiles - plan.pair.split_tiles + slots - 1) / slots;
+        pair_us = tile_us * (double)whole_waves + (plan.pair.split_tiles > 0 ? tile_us / (double)plan.pair.k_parts + 9.0 : 0.0);
     }
     const bool pairs = T >= kPairMinT ? pair_us < 1e29 : (T > 256 ? pair_us <= single_us * 1.05 : pair_us < single_us);
-    if (use_pairs) *use_pairs = pairs;
-    return pairs ? pair_us : single_us;
+    plan.use_pairs = pairs ? 1 : 0;
+    plan.us = pairs ? pair_us : single_us;
+    return plan;
 }
 
 cudaError_t launch_prefill(const lopro_desc& d, const uint8_t* blob, const BlobLayout& L, const uint8_t* ws,
@@ -925,12 +1045,13 @@ cudaError_t launch_prefill(const lopro_desc& d, const uint8_t* blob, const BlobL
     p.gshift = gshift;
     p.ng = d.d_in / d.group_size;
     p.r_pad = d.rank > 0 ? L.r_pad : 0;
-    p.tile_n = T <= 64 ? 64 : (T <= 128 ? 128 : 256);
     p.lr_stages = (p.r_pad + kStageK - 1) / kStageK;
-    const PairPlan plan = pair_plan(d, T);
-    bool use_pairs = false;
-    (void)prefill_estimate_us(d, T, &use_pairs);
-    if (use_pairs) {
+    const PrefillPlan whole_plan = prefill_plan(d, T, W.compact != 0);
+    const PairPlan& plan = whole_plan.pair;
+    p.tile_n = whole_plan.tile_n;
+    p.k_parts = whole_plan.k_parts;
+    p.kparts = reinterpret_cast<float*>(const_cast<uint8_t*>(ws) + W.off_kparts);
+    if (whole_plan.use_pairs) {
         // two CTAs per tile (each loads boxes of 128 tokens)
         PairParams q;
         q.codes = p.codes;
@@ -985,11 +1106,11 @@ cudaError_t launch_prefill(const lopro_desc& d, const uint8_t* blob, const BlobL
     // kernel is bound by that stream, so it costs little more than a CTA with one block), but coarser
     // tiles waste more of the last wave; pick the number of two-block CTAs that minimises the makespan of a
     // greedy schedule over the SMs (two-block CTAs are dispatched first, then the single blocks).
-    const int units = (T + p.tile_n - 1) / p.tile_n;
+    const int units = whole_plan.units;
     const int m_tiles = (d.d_out + kTileM - 1) / kTileM;
-    int best_pairs = m_tiles / 2;
+    int best_pairs = p.k_parts > 1 ? whole_plan.pair_tiles : m_tiles / 2;
     const int n_sm = sm_count() > 0 ? sm_count() : 1;
-    {
+    if (p.k_parts == 1) {
         // Makespan of the greedy schedule in closed form (the search runs on the host at every launch): the two-block
         // CTAs leave the SMs on at most two levels, and the one-block CTAs then fill the lower level a round at a time.
         auto makespan = [&](long long n_pairs, long long n_singles) {
@@ -1022,14 +1143,26 @@ cudaError_t launch_prefill(const lopro_desc& d, const uint8_t* blob, const BlobL
     p.pair_tiles = best_pairs;
     p.single_tiles = m_tiles - 2 * best_pairs;
     p.units = units;
-    const long long n_ctas = (long long)(p.pair_tiles + p.single_tiles) * units;
+    const long long n_ctas = (long long)(p.pair_tiles + p.single_tiles) * units * p.k_parts;
     if (n_ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
     dim3 grid((unsigned)n_ctas);
-    switch (d.bits) {
-        case 2: return launch_prefill_bits<2>(p, mx, ma, mt, grid, s);
-        case 3: return launch_prefill_bits<3>(p, mx, ma, mt, grid, s);
-        default: return launch_prefill_bits<4>(p, mx, ma, mt, grid, s);
-    }
+    const cudaError_t e = d.bits == 2 ? launch_prefill_bits<2>(p, mx, ma, mt, grid, s)
+                                      : (d.bits == 3 ? launch_prefill_bits<3>(p, mx, ma, mt, grid, s)
+                                                     : launch_prefill_bits<4>(p, mx, ma, mt, grid, s));
+    if (e != cudaSuccess || p.k_parts == 1) return e;
+    KPartsSum k = {};
+    k.kparts = p.kparts;
+    k.y = y;
+    k.ldy = ldy;
+    k.out_f32 = p.out_f32;
+    k.m = p.m;
+    k.T = T;
+    k.k_parts = p.k_parts;
+    k.kp_tokens = k.tile_tokens = p.tile_n;
+    k.pair_ctas = p.pair_tiles * units;
+    k.pair_tiles = p.pair_tiles;
+    k.single_tiles = p.single_tiles;
+    return launch_kparts_sum(k, (p.pair_tiles + p.single_tiles) * units, s);
 }
 
 }  // namespace lopro
