@@ -167,27 +167,34 @@ __global__ void rope_append_kernel(__nv_bfloat16* __restrict__ q, int64_t ldq, c
 constexpr int kAttnBatch = 4;                   // keys that a half-warp holds at once (and as many on their way)
 constexpr int kMaxCluster = 8;
 
-// Attention of one query over the keys of its sequence; grid (cluster, n_heads, T), one cluster of CTAs per (head,
-// sequence).  Bound by reading keys and values once.  The sequence's keys are shared out evenly over the cluster's CTAs,
+// Attention of one query over the keys of its sequence; grid cluster x pairs, one cluster of CTAs per (head, sequence) pair
+// from pair0 on.  Bound by reading keys and values once.  The sequence's keys are shared out evenly over the cluster's CTAs,
 // and within a CTA over its half-warps: sixteen lanes read a key's (value's) 256 bytes as one 16-byte piece each, so every
 // access is a whole row, and a half-warp needs nobody else until the end: it keeps its own running maximum, sum of weights
 // and weighted values.  Keys and values of the next four keys are requested before the present four are used.  The
 // half-warps' results meet in shared memory, the CTAs' in that of the cluster's first CTA: no second launch, no scratch
 // in global memory.
 // 32 sequences of 32 heads, context 2049 (1.07 GB): 217 us in two launches before, 165 us = 6.5 TB/s now.
-template <int THREADS>
+// kWhole: all pairs.  kFirst, kTail: the pairs of a short last wave run as a second launch in larger clusters, which starts
+// as the first launch's CTAs finish.  For that the first releases it when its own predecessor is complete, and the tail
+// reads without waiting and waits for the first launch before it ends, so that its successor waits for both.
+// 16 sequences of 40 heads, context 2540 (0.83 GB; 640 pairs over 592 slots): 180 us in one launch, 123 us = 6.8 TB/s.
+enum AttnPart { kWhole, kFirst, kTail };
+template <int THREADS, AttnPart PART>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS)
 attention_kernel(const __nv_bfloat16* __restrict__ q, int64_t ldq, const __nv_bfloat16* __restrict__ k_cache,
                  const __nv_bfloat16* __restrict__ v_cache, const int32_t* __restrict__ ctx, int n_heads, int ctx_max, float scale,
-                 __nv_bfloat16* __restrict__ out, int64_t ldo, int* status) {
+                 __nv_bfloat16* __restrict__ out, int64_t ldo, int* status, int size, int pair0) {
     constexpr int kAttnHalves = THREADS / 16;          // half-warps, each a stream of keys of its own
     __shared__ float acc_s[kAttnHalves][kHeadDim];
     __shared__ float2 ml_s[kAttnHalves];               // (maximum, sum) of a half-warp
     __shared__ __align__(16) float part_s[kMaxCluster][kHeadDim + 4];  // first CTA: the CTAs' weighted values, maximum, sum
-    const int size = gridDim.x, rank = blockIdx.x, hd = blockIdx.y, t = blockIdx.z, tid = threadIdx.x;
+    const int pair = pair0 + (int)blockIdx.x / size, rank = (int)blockIdx.x % size, tid = threadIdx.x;
+    const int t = pair / n_heads, hd = pair - t * n_heads;
     const int half = tid >> 4, piece = tid & 15;
     if (size > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // this CTA has started
-    wait_for_predecessor();
+    if (PART != kTail) wait_for_predecessor();
+    if (PART == kFirst) release_successor();
     const int n_all = __ldcg(ctx + t);
     const bool bad = n_all < 1 || n_all > ctx_max;
     if (bad && tid == 0 && hd == 0 && rank == 0) atomicCAS(status, LOPRO_OK, LOPRO_ERR_INVALID_DATA);
@@ -271,7 +278,7 @@ attention_kernel(const __nv_bfloat16* __restrict__ q, int64_t ldq, const __nv_bf
         fetch(ka, va, first + r + 2 * kStep);
         consume(kb, vb, first + r + kStep);
     }
-    release_successor();
+    if (PART != kFirst) release_successor();
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc_s[half][8 * piece + e] = acc[e];
     if (piece == 0) ml_s[half] = make_float2(m, l);
@@ -298,7 +305,10 @@ attention_kernel(const __nv_bfloat16* __restrict__ q, int64_t ldq, const __nv_bf
         }
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-        if (rank != 0) return;
+        if (rank != 0) {
+            if (PART == kTail) wait_for_predecessor();
+            return;
+        }
         top = -INFINITY;
         num = den = 0.0f;
         for (int c = 0; c < size; ++c) top = fmaxf(top, part_s[c][kHeadDim]);
@@ -309,6 +319,7 @@ attention_kernel(const __nv_bfloat16* __restrict__ q, int64_t ldq, const __nv_bf
         }
     }
     if (tid < kHeadDim) out[(size_t)t * ldo + (size_t)hd * kHeadDim + tid] = __float2bfloat16_rn(den > 0.0f ? num / den : 0.0f);
+    if (PART == kTail) wait_for_predecessor();
 }
 
 __global__ void __launch_bounds__(256) silu_mul_kernel(const __nv_bfloat16* __restrict__ gate, int64_t ldg,
@@ -410,10 +421,20 @@ lopro_status lopro_block_attention_decode(const uint16_t* q, int64_t ldq, const 
     int cluster = 1;
     while (cluster < kMaxCluster && pairs * cluster * 2 <= slots) cluster *= 2;
     const bool wide = pairs * cluster * 2 <= slots;
-    return launch(wide ? attention_kernel<256> : attention_kernel<128>, dim3(cluster, n_heads, T), wide ? 256 : 128, stream, cluster,
-                  reinterpret_cast<const __nv_bfloat16*>(q), ldq, reinterpret_cast<const __nv_bfloat16*>(k_cache),
-                  reinterpret_cast<const __nv_bfloat16*>(v_cache), ctx, n_heads, ctx_max, scale,
-                  reinterpret_cast<__nv_bfloat16*>(out), ldo, (int*)status_word);
+    auto run = [&](auto kernel, int size, int threads, int64_t first, int64_t count) {
+        return launch(kernel, dim3((unsigned)(count * size)), threads, stream, size, reinterpret_cast<const __nv_bfloat16*>(q), ldq,
+                      reinterpret_cast<const __nv_bfloat16*>(k_cache), reinterpret_cast<const __nv_bfloat16*>(v_cache), ctx, n_heads,
+                      ctx_max, scale, reinterpret_cast<__nv_bfloat16*>(out), ldo, (int*)status_word, size, (int)first);
+    };
+    if (pairs > 0x7fffffff) return LOPRO_ERR_UNSUPPORTED;   // (a cache of half a terabyte)
+    if (wide) return run(attention_kernel<256, kWhole>, cluster, 256, 0, pairs);
+    // A last wave that leaves half the slots idle or more: its pairs in clusters that fill them.
+    const int64_t rest = pairs % slots;
+    if (pairs < slots || rest == 0 || rest * 2 > slots) return run(attention_kernel<128, kWhole>, cluster, 128, 0, pairs);
+    const lopro_status st = run(attention_kernel<128, kFirst>, 1, 128, 0, pairs - rest);
+    if (st != LOPRO_OK) return st;
+    for (cluster = 2; cluster < kMaxCluster && rest * cluster * 2 <= slots; ) cluster *= 2;
+    return run(attention_kernel<128, kTail>, cluster, 128, pairs - rest, rest);
 }
 
 lopro_status lopro_block_silu_mul(const uint16_t* gate, int64_t ldg, const uint16_t* up, int64_t ldu, uint16_t* out,

@@ -46,7 +46,7 @@ def test_a_buffer_rewritten_inside_a_chain_is_read_as_last_written(T):
 
 
 # pairs of (sequence, head) on both sides of every cluster size the launch chooses
-@pytest.mark.parametrize("H", [1, 4, 8, 16, 32])
+@pytest.mark.parametrize("H", [1, 4, 8, 16, 32, 46, 57, 92])   # (from 46 on more pairs than one wave: 6, 149 and 12 in the last)
 def test_attention_at_the_edges_of_its_splits(H):
     ctx = np.array([1, 2, 7, 8, 9, 31, 32, 33, 64, 65, 255, 257, 300], dtype=np.int32)
     T, hd, ctx_max = len(ctx), 128, 300
