@@ -156,10 +156,14 @@ rotate_lowrank_kernel(const __nv_bfloat16* __restrict__ x, int64_t ldx, const in
     if (rot_through > rot_before) {
         const int rb = rot_before;
         // (no 64-column sums: the tensor-core product that follows dequantizes the weights and needs none)
-        if (rows_per_cta == 8)
+        if (mma_form && rows_per_cta == 8)
             rotate_mma_body<8>(smem_raw, rb, x, ldx, perm, xrot, ldo, status, n, b_i, b_h, inv_sqrt_bh, T);
-        else if (mma_form)
+        else if (mma_form && rows_per_cta == 4)
             rotate_mma_body<4>(smem_raw, rb, x, ldx, perm, xrot, ldo, status, n, b_i, b_h, inv_sqrt_bh, T);
+        else if (mma_form && rows_per_cta == 2)
+            rotate_mma_body<2>(smem_raw, rb, x, ldx, perm, xrot, ldo, status, n, b_i, b_h, inv_sqrt_bh, T);
+        else if (mma_form && rows_per_cta == 1)
+            rotate_mma_body<1>(smem_raw, rb, x, ldx, perm, xrot, ldo, status, n, b_i, b_h, inv_sqrt_bh, T);
         else
             rotate_body<8, 4, true>(smem_raw, rb, x, ldx, perm, xrot, ldo, s64, s64_ld, status, n, b_i, b_h,
                                     inv_sqrt_bh, T);
@@ -260,11 +264,11 @@ cudaError_t launch_rotate_lowrank_nj(const lopro_desc& d, const int32_t* perm, c
                                      float* partial, int T, cudaStream_t s, bool compact) {
     const int slices = lowrank_mma_slices(d, T, compact);
     const int slice_cols = lowrank_slice_cols(d, slices);
-    // rotation CTAs: the tensor-core form of the recursion with 8 rows per CTA where that leaves room for three CTAs
-    // per SM, with 4 rows otherwise; the register-and-shuffle form where the block size or prefix rules it out
+    // rotation CTAs: the tensor-core form of the recursion; the register-and-shuffle form where the block size or prefix
+    // rules it out
     const bool mma_form = rotate_mma_shape_ok(d) && (reinterpret_cast<uintptr_t>(perm) % 16) == 0 &&
                           rotate_mma_smem_bytes(4, d.d_in) <= 160 * 1024;
-    const int rows_per_cta = mma_form && rotate_mma_smem_bytes(8, d.d_in) <= 74 * 1024 ? 8 : 4;
+    const int rows_per_cta = mma_form ? rotate_mma_rows(d, T) : 4;
     const int n_rot = (T + rows_per_cta - 1) / rows_per_cta, lr_gx = (T + kLrTokens - 1) / kLrTokens;
     const size_t smem_rot = mma_form ? rotate_mma_smem_bytes(rows_per_cta, d.d_in) : (size_t)d.d_in * 8;
     const size_t smem_lr = (size_t)(kLrTokens + 2 * NJ * 8) * kLrStride * 2;

@@ -539,12 +539,16 @@ cudaError_t launch_rotate_mma(const lopro_desc& d, const int32_t* perm, const __
 
 cudaError_t launch_rotate(const lopro_desc& d, const int32_t* perm, const __nv_bfloat16* x, int64_t ldx,
                           __nv_bfloat16* xrot, int64_t ldo, float* s64, int* status, int T, cudaStream_t s) {
-    // many rows and no column sums wanted: the tensor-core form of the recursion, eight (or four) rows per CTA
+    // many rows and no column sums wanted: the tensor-core form of the recursion
     if (s64 == nullptr && T >= 16 && rotate_mma_shape_ok(d) && (reinterpret_cast<uintptr_t>(perm) % 16) == 0) {
-        if (rotate_mma_smem_bytes(8, d.d_in) <= (size_t)kRotMmaMaxSmem / 2)
-            return launch_rotate_mma<8>(d, perm, x, ldx, xrot, ldo, status, T, s);
-        if (rotate_mma_smem_bytes(4, d.d_in) <= (size_t)kRotMmaMaxSmem)
-            return launch_rotate_mma<4>(d, perm, x, ldx, xrot, ldo, status, T, s);
+        if (rotate_mma_smem_bytes(4, d.d_in) <= (size_t)kRotMmaMaxSmem) {
+            switch (rotate_mma_rows(d, T)) {
+                case 8: return launch_rotate_mma<8>(d, perm, x, ldx, xrot, ldo, status, T, s);
+                case 4: return launch_rotate_mma<4>(d, perm, x, ldx, xrot, ldo, status, T, s);
+                case 2: return launch_rotate_mma<2>(d, perm, x, ldx, xrot, ldo, status, T, s);
+                default: return launch_rotate_mma<1>(d, perm, x, ldx, xrot, ldo, status, T, s);
+            }
+        }
     }
     if (d.block_size <= 256) return launch_rotate_e<8>(d, perm, x, ldx, xrot, ldo, s64, status, T, s);
     if (d.block_size == 512) return launch_rotate_e<16>(d, perm, x, ldx, xrot, ldo, s64, status, T, s);

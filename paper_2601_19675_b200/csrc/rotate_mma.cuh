@@ -3,13 +3,13 @@
 //
 // H_b = H_{b/16} (x) H_16 in the natural (Kronecker) order: a block of b gathered entries is cut into tiles of 16;
 // every tile is multiplied by H_16 (entries +-1, exact in bf16; fp32 accumulation) with mma.m16n8k16 -- tokens are
-// the M dimension, so a warp rotates the same block of up to 8 token rows at once --, then the tiles are combined by
+// the M dimension, so a warp rotates one block of 8 token rows, or 2, 4, 8 blocks of 4, 2, 1 rows at once --, then the tiles are combined by
 // log2(b/16) levels of add / subtract, which pair registers of the SAME lane (no shuffles), one scaling by 1/sqrt(b)
 // and one rounding to bf16.  Against register-and-shuffle butterflies this is about a third of the instructions
 // per entry, which is what bounds the rotation of a prefill batch (the data is read and written exactly once).
 //
 // A CTA stages TOK token rows of x in shared memory (the permutation scatters over the whole row) and its warps
-// take the row's blocks in turn.  Lane l = 4 g + t: token g; of every 16-tile the gathered columns 2t, 2t+1, 2t+8,
+// take the row's blocks in turn.  Lane l = 4 g + t: token g % TOK, block g / TOK of those at once; of every 16-tile the gathered columns 2t, 2t+1, 2t+8,
 // 2t+9 (the A fragment) and, after the product, the outputs 2t, 2t+1, 8+2t, 8+2t+1 (the D fragments of the two
 // 8-column halves).  The identity prefix (b_I columns, Eq. 6) is gathered and stored by the same lanes.
 // Requires 16 <= b_H <= 256, b_I a multiple of 16.  Writes no column sums.
@@ -106,7 +106,8 @@ __device__ __forceinline__ void rotate_mma_body(unsigned char* smem_raw, int blo
                                                 int64_t ldx, const int32_t* __restrict__ perm,
                                                 __nv_bfloat16* __restrict__ xrot, int64_t ldo, int* __restrict__ status, int n,
                                                 int b_i, int b_h, float inv_sqrt_bh, int T) {
-    static_assert(TOK == 4 || TOK == 8, "token rows per CTA");
+    static_assert(TOK == 1 || TOK == 2 || TOK == 4 || TOK == 8, "token rows per CTA");
+    constexpr int kSub = 8 / TOK;   // blocks that a warp rotates at once, TOK rows of each
     unsigned short* xs = reinterpret_cast<unsigned short*>(smem_raw);  // [TOK][n + kRotMmaPad]
     const int stride = n + kRotMmaPad;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
@@ -134,15 +135,17 @@ __device__ __forceinline__ void rotate_mma_body(unsigned char* smem_raw, int blo
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     const int g = lane >> 2, t = lane & 3;
-    const bool live = g < nt;
-    const uint32_t xrow = (uint32_t)__cvta_generic_to_shared(xs + (size_t)(live ? g : 0) * stride);
+    const int tok = g % TOK, sub = g / TOK;
+    const bool live = tok < nt;
+    const uint32_t xrow = (uint32_t)__cvta_generic_to_shared(xs + (size_t)(live ? tok : 0) * stride);
     const uint32_t perm_s32 = (uint32_t)__cvta_generic_to_shared(off_tab);
-    __nv_bfloat16* orow = xrot + (size_t)(t0 + (live ? g : 0)) * ldo;
+    __nv_bfloat16* orow = xrot + (size_t)(t0 + (live ? tok : 0)) * ldo;
     // identity prefix: gathered entries go out as they are
-    for (int j = warp; j < (b_i >> 4); j += nwarps) {
+    for (int jj = warp; jj * kSub < (b_i >> 4); jj += nwarps) {
+        const int j = min(jj * kSub + sub, (b_i >> 4) - 1);
         uint32_t a0, a2;
         gather_tile(xrow, perm_s32, 16 * j, t, a0, a2);
-        if (live) {
+        if (live && j == jj * kSub + sub) {
             *reinterpret_cast<uint32_t*>(orow + 16 * j + 2 * t) = a0;
             *reinterpret_cast<uint32_t*>(orow + 16 * j + 8 + 2 * t) = a2;
         }
@@ -151,16 +154,27 @@ __device__ __forceinline__ void rotate_mma_body(unsigned char* smem_raw, int blo
     h16_fragment(t, g, h0);
     h16_fragment(t, g + 8, h1);
     const int n_blk = (n - b_i) / b_h;
-    for (int blk = warp; blk < n_blk; blk += nwarps) {
-        const int kb = b_i + blk * b_h;
+    for (int bb = warp; bb * kSub < n_blk; bb += nwarps) {
+        const int blk = min(bb * kSub + sub, n_blk - 1), kb = b_i + blk * b_h;
+        const bool keep = live && blk == bb * kSub + sub;
         switch (b_h) {
-            case 16: rotate_block_mma<1>(xrow, perm_s32, kb, t, live, h0, h1, inv_sqrt_bh, orow); break;
-            case 32: rotate_block_mma<2>(xrow, perm_s32, kb, t, live, h0, h1, inv_sqrt_bh, orow); break;
-            case 64: rotate_block_mma<4>(xrow, perm_s32, kb, t, live, h0, h1, inv_sqrt_bh, orow); break;
-            case 128: rotate_block_mma<8>(xrow, perm_s32, kb, t, live, h0, h1, inv_sqrt_bh, orow); break;
-            default: rotate_block_mma<16>(xrow, perm_s32, kb, t, live, h0, h1, inv_sqrt_bh, orow); break;
+            case 16: rotate_block_mma<1>(xrow, perm_s32, kb, t, keep, h0, h1, inv_sqrt_bh, orow); break;
+            case 32: rotate_block_mma<2>(xrow, perm_s32, kb, t, keep, h0, h1, inv_sqrt_bh, orow); break;
+            case 64: rotate_block_mma<4>(xrow, perm_s32, kb, t, keep, h0, h1, inv_sqrt_bh, orow); break;
+            case 128: rotate_block_mma<8>(xrow, perm_s32, kb, t, keep, h0, h1, inv_sqrt_bh, orow); break;
+            default: rotate_block_mma<16>(xrow, perm_s32, kb, t, keep, h0, h1, inv_sqrt_bh, orow); break;
         }
     }
+}
+
+// Token rows per CTA.  Eight where that leaves a CTA for every multiprocessor and room for three on each (a lookup's lanes
+// then read few columns of many rows, and the table of indices is built for eight rows at once); fewer rows where the chip
+// would idle (4096 -> 11008 at 203 tokens: 45.7 us for the whole forward with 8 rows, 42.0 with 4, 40.5 with 2, 43.9 with 1;
+// 4096 -> 4096 at 64: 25.8, 22.5, 21.5, 21.2; 4096 -> 4096 at 512: 40.1, 38.8, 40.1, 43.4; 4096 -> 2048 at 2048: 69.0, 72.4).
+inline int rotate_mma_rows(const lopro_desc& d, int T) {
+    const int unit = d.d_in <= 2048 ? sm_count() / 2 : sm_count();   // (2048 -> 2048 at 1024: 31.8 with 8 rows, 33.4 with 4)
+    if (T >= 8 * unit && rotate_mma_smem_bytes(8, d.d_in) <= 74 * 1024) return 8;
+    return T >= 2 * unit ? 4 : (T >= unit ? 2 : 1);
 }
 
 inline bool rotate_mma_shape_ok(const lopro_desc& d) {

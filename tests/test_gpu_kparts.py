@@ -1,12 +1,14 @@
 """More than 32 tokens with tiles cut along K: the one-CTA-per-tile tensor-core kernel (one- and two-block tiles, an odd
 number of row blocks, parts that hold low-rank stages only), more parts of the two-CTA kernel, and K slices of the low-rank
-product that do not divide the width; and the same layers in a workspace without room for the parts."""
+product that do not divide the width; the same layers in a workspace without room for the parts; and the rotation's CTAs."""
+import numpy as np
 import pytest
 import torch
 
 from paper_2601_19675_b200 import lopro, synth
 from tests._layers import bf16_bits_to_device, random_layer_np
 from tests.test_gpu_forward import GATE_A, GATE_B, _check_forward_once, _pack
+from tests.test_gpu_rotate import _run as _run_rotation, _ulp_bf16
 
 pytestmark = pytest.mark.gpu
 
@@ -56,3 +58,12 @@ def test_the_fixed_scratch_takes_fewer_parts(n, m, T):
     lopro.linear_fwd_noalloc(d, blob, x, y, lopro.OUT_F32)
     torch.cuda.synchronize()
     assert (y - want).abs().max().item() <= 1e-5 * want.abs().max().item()
+
+
+# 1, 2, 4 and 8 token rows per CTA of the rotation (148 multiprocessors, up to 2048 columns), odd numbers of 16-column tiles in the prefix and of
+# rotated blocks, and a last CTA with rows missing
+@pytest.mark.parametrize("n,b_i,b_h", [(832, 64, 64), (320, 80, 16), (1088, 64, 256), (512, 0, 32), (448, 64, 128)])
+@pytest.mark.parametrize("T", [16, 73, 75, 147, 149, 591, 593])
+def test_rotation_with_every_number_of_rows_per_cta(n, b_i, b_h, T):
+    got, exact, _, _ = _run_rotation(n, b_i, b_h, T, seed=T)
+    assert np.all(np.abs(got - exact) <= _ulp_bf16(exact) + 1e-6 * np.abs(exact).max())
