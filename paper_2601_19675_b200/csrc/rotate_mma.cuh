@@ -9,9 +9,10 @@
 // per entry, which is what bounds the rotation of a prefill batch (the data is read and written exactly once).
 //
 // A CTA stages TOK token rows of x in shared memory (the permutation scatters over the whole row) and its warps
-// take the row's blocks in turn.  Lane l = 4 g + t: token g % TOK, block g / TOK of those at once; of every 16-tile the gathered columns 2t, 2t+1, 2t+8,
-// 2t+9 (the A fragment) and, after the product, the outputs 2t, 2t+1, 8+2t, 8+2t+1 (the D fragments of the two
-// 8-column halves).  The identity prefix (b_I columns, Eq. 6) is gathered and stored by the same lanes.
+// take the row's blocks in turn.  Lane l = 4 g + t: token g % TOK, block g / TOK of those at
+// once; of every 16-tile the gathered columns 4t .. 4t + 3 and the outputs 4t .. 4t + 3 -- H_16's rows and columns are dealt to the fragments'
+// positions that way --, so that a lane's indices are one 8-byte load and its outputs one 8-byte store, four lanes a whole
+// 32-byte sector of the row (with the fragments' own order two half sectors: 4096 rows of 8192 63 -> 49 us).  The identity prefix (b_I columns, Eq. 6) is gathered and stored by the same lanes.
 // Requires 16 <= b_H <= 256, b_I a multiple of 16.  Writes no column sums.
 #pragma once
 
@@ -19,12 +20,14 @@
 
 namespace lopro {
 
-// +-1 fragments of H_16 for the B operand (k x n, "col" layout): b0 = rows 2t, 2t+1, b1 = rows 2t+8, 2t+9 of
-// column n = col; H_16[k][i] = (-1)^popcount(k & i).
-__device__ __forceinline__ void h16_fragment(int t, int col, uint32_t (&b)[2]) {
+// +-1 fragments of H_16 for the B operand (k x n, "col" layout) of the product whose column n = g is column 4 (g / 2) +
+// (g & 1) + 2 h of H_16: b0 = positions 2t, 2t+1 of k, rows 4t, 4t+1; b1 = positions 2t+8, 2t+9, rows 4t+2, 4t+3;
+// H_16[k][i] = (-1)^popcount(k & i).
+__device__ __forceinline__ void h16_fragment(int t, int g, int h, uint32_t (&b)[2]) {
+    const int col = 4 * (g >> 1) + (g & 1) + 2 * h;
     auto entry = [&](int k) { return (__popc(k & col) & 1) ? 0xBF80u : 0x3F80u; };
-    b[0] = entry(2 * t) | (entry(2 * t + 1) << 16);
-    b[1] = entry(2 * t + 8) | (entry(2 * t + 9) << 16);
+    b[0] = entry(4 * t) | (entry(4 * t + 1) << 16);
+    b[1] = entry(4 * t + 2) | (entry(4 * t + 3) << 16);
 }
 
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint32_t a2, const uint32_t (&b)[2]) {
@@ -41,8 +44,7 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint3
 // memory).
 __device__ __forceinline__ void gather_tile(uint32_t xrow_s, uint32_t off_s, int k0, int t, uint32_t& a0, uint32_t& a2) {
     uint32_t w0, w1;  // two 16-bit column indices each
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w0) : "r"(off_s + 2u * (uint32_t)(k0 + 2 * t)));
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w1) : "r"(off_s + 2u * (uint32_t)(k0 + 8 + 2 * t)));
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(w0), "=r"(w1) : "r"(off_s + 2u * (uint32_t)(k0 + 4 * t)));
     unsigned short v0, v1, v2, v3;
     asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v0) : "r"(xrow_s + 2u * (w0 & 0xFFFFu)));
     asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v1) : "r"(xrow_s + 2u * (w0 >> 16)));
@@ -84,9 +86,10 @@ __device__ __forceinline__ void rotate_block_mma(uint32_t xrow, uint32_t perm,
     if (live) {
 #pragma unroll
         for (int kt = 0; kt < KT; ++kt) {
-            __nv_bfloat16* o = orow + kb + 16 * kt + 2 * t;
-            *reinterpret_cast<__nv_bfloat162*>(o) = __floats2bfloat162_rn(z[kt][0] * inv_sqrt_bh, z[kt][1] * inv_sqrt_bh);
-            *reinterpret_cast<__nv_bfloat162*>(o + 8) = __floats2bfloat162_rn(z[kt][2] * inv_sqrt_bh, z[kt][3] * inv_sqrt_bh);
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(z[kt][0] * inv_sqrt_bh, z[kt][1] * inv_sqrt_bh);
+            const __nv_bfloat162 hi = __floats2bfloat162_rn(z[kt][2] * inv_sqrt_bh, z[kt][3] * inv_sqrt_bh);
+            *reinterpret_cast<uint2*>(orow + kb + 16 * kt + 4 * t) =
+                make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
         }
     }
 }
@@ -146,13 +149,12 @@ __device__ __forceinline__ void rotate_mma_body(unsigned char* smem_raw, int blo
         uint32_t a0, a2;
         gather_tile(xrow, perm_s32, 16 * j, t, a0, a2);
         if (live && j == jj * kSub + sub) {
-            *reinterpret_cast<uint32_t*>(orow + 16 * j + 2 * t) = a0;
-            *reinterpret_cast<uint32_t*>(orow + 16 * j + 8 + 2 * t) = a2;
+            *reinterpret_cast<uint2*>(orow + 16 * j + 4 * t) = make_uint2(a0, a2);
         }
     }
     uint32_t h0[2], h1[2];
-    h16_fragment(t, g, h0);
-    h16_fragment(t, g + 8, h1);
+    h16_fragment(t, g, 0, h0);
+    h16_fragment(t, g, 1, h1);
     const int n_blk = (n - b_i) / b_h;
     for (int bb = warp; bb * kSub < n_blk; bb += nwarps) {
         const int blk = min(bb * kSub + sub, n_blk - 1), kb = b_i + blk * b_h;
