@@ -400,7 +400,7 @@ class Workload:
                                          else lopro.linear_fwd_path(c[0][0], T)[1] for c in self.calls)
             if self.block:
                 self.bytes_per_pass += block_glue_bytes(T)
-                self.launches_per_pass += 6 * STACK_LAYERS      # 2 norms, rotary + append, attention (2), gating
+                self.launches_per_pass += 5 * STACK_LAYERS      # 2 norms, rotary + append, attention, gating
             self.c = None
             return
         c = synth.CONFIGS[cfg]

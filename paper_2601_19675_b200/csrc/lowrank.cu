@@ -36,17 +36,23 @@ __device__ __forceinline__ void lowrank_body(unsigned char* smem_raw, int bx, in
     const int kb = by * slice_cols, ke = min(n, kb + slice_cols);
     const int rows_b = min(NJ * 8, r_pad - j0);
 
-    float acc[NJ][4];
+    // Warps split the tile by 32 tokens and half of B's rows (16 tokens and all rows where there are only 16): the operands
+    // come from shared memory, whose reads bound this with 16 tokens per warp (8 ldmatrix of B for 16 products, now 8 for 32).
+    constexpr int WN = NJ == 4 || NJ == 16 ? 2 : 1, MT = WN, NW = NJ / WN;
+    const int wm = warp / WN * MT * 16, wn = warp % WN * NW * 8;   // the warp's first token and first row of B
+    float acc[MT][NW][4];
 #pragma unroll
-    for (int j = 0; j < NJ; ++j)
+    for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[j][i] = 0.0f;
+        for (int j = 0; j < NW; ++j)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[mt][j][i] = 0.0f;
 
     const uint32_t xs_u = (uint32_t)__cvta_generic_to_shared(xs);
     const uint32_t bh_u = (uint32_t)__cvta_generic_to_shared(bh), bl_u = (uint32_t)__cvta_generic_to_shared(bl);
     // ldmatrix lane addresses: A operand (16 tokens x 16 columns), B operand (16 rows of B x 16 columns)
-    const uint32_t a_off = (uint32_t)((warp * 16 + (lane & 7) + 8 * ((lane >> 3) & 1)) * kLrStride + 8 * (lane >> 4)) * 2u;
-    const uint32_t b_off = (uint32_t)(((lane & 7) + 8 * (lane >> 4)) * kLrStride + 8 * ((lane >> 3) & 1)) * 2u;
+    const uint32_t a_off = (uint32_t)((wm + (lane & 7) + 8 * ((lane >> 3) & 1)) * kLrStride + 8 * (lane >> 4)) * 2u;
+    const uint32_t b_off = (uint32_t)((wn + (lane & 7) + 8 * (lane >> 4)) * kLrStride + 8 * ((lane >> 3) & 1)) * 2u;
 
     // global loads of one 64-column chunk, kept in registers while the previous chunk is multiplied
     constexpr int kXPer = kLrTokens * 8 / kLrThreads;                     // 16-byte pieces of x per thread
@@ -100,29 +106,36 @@ __device__ __forceinline__ void lowrank_body(unsigned char* smem_raw, int bx, in
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < kLrChunk; kk += 16) {
-            uint32_t a[4];
-            ldmatrix_x4(a, xs_u + a_off + kk * 2);
+            uint32_t a[MT][4];
 #pragma unroll
-            for (int jp = 0; jp < NJ / 2; ++jp) {
-                uint32_t b[4];
-                ldmatrix_x4(b, bh_u + b_off + (uint32_t)(jp * 16 * kLrStride + kk) * 2u);
-                mma_bf16(acc[2 * jp], a, b[0], b[1]);
-                mma_bf16(acc[2 * jp + 1], a, b[2], b[3]);
-                ldmatrix_x4(b, bl_u + b_off + (uint32_t)(jp * 16 * kLrStride + kk) * 2u);
-                mma_bf16(acc[2 * jp], a, b[0], b[1]);
-                mma_bf16(acc[2 * jp + 1], a, b[2], b[3]);
-            }
+            for (int mt = 0; mt < MT; ++mt) ldmatrix_x4(a[mt], xs_u + a_off + (uint32_t)(mt * 16 * kLrStride + kk) * 2u);
+#pragma unroll
+            for (int jp = 0; jp < NW / 2; ++jp)
+#pragma unroll
+                for (int part = 0; part < 2; ++part) {
+                    uint32_t b[4];
+                    ldmatrix_x4(b, (part == 0 ? bh_u : bl_u) + b_off + (uint32_t)(jp * 16 * kLrStride + kk) * 2u);
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt) {
+                        mma_bf16(acc[mt][2 * jp], a[mt], b[0], b[1]);
+                        mma_bf16(acc[mt][2 * jp + 1], a[mt], b[2], b[3]);
+                    }
+                }
         }
     }
     // partial[slice][token][j]
     const int gq = lane >> 2, tg = lane & 3;
 #pragma unroll
-    for (int j = 0; j < NJ; ++j)
+    for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int tok = tok0 + warp * 16 + gq + 8 * (i >> 1), col = j0 + j * 8 + 2 * tg + (i & 1);
-            if (tok < T && col < r_pad) partial[((size_t)by * T + tok) * r_pad + col] = acc[j][i];
-        }
+        for (int j = 0; j < NW; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int tok = tok0 + wm + mt * 16 + gq + 8 * h, col = j0 + wn + j * 8 + 2 * tg;
+                if (tok < T && col < r_pad)   // (r_pad is even)
+                    *reinterpret_cast<float2*>(partial + ((size_t)by * T + tok) * r_pad + col) =
+                        make_float2(acc[mt][j][2 * h], acc[mt][j][2 * h + 1]);
+            }
 }
 
 template <int NJ>

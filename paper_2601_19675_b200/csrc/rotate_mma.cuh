@@ -12,7 +12,8 @@
 // take the row's blocks in turn.  Lane l = 4 g + t: token g % TOK, block g / TOK of those at
 // once; of every 16-tile the gathered columns 4t .. 4t + 3 and the outputs 4t .. 4t + 3 -- H_16's rows and columns are dealt to the fragments'
 // positions that way --, so that a lane's indices are one 8-byte load and its outputs one 8-byte store, four lanes a whole
-// 32-byte sector of the row (with the fragments' own order two half sectors: 4096 rows of 8192 63 -> 49 us).  The identity prefix (b_I columns, Eq. 6) is gathered and stored by the same lanes.
+// 32-byte sector of the row (with the fragments' own order two half sectors: 4096 rows of 8192 63 -> 49 us).  The identity
+// prefix (b_I columns, Eq. 6) is gathered and stored by the same lanes.
 // Requires 16 <= b_H <= 256, b_I a multiple of 16.  Writes no column sums.
 #pragma once
 
