@@ -75,50 +75,60 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
-// One row j of B against TPR tokens: t[token][j] = sum_k B[j][k] x[token][k], fp32 accumulation over all of K, one
+// One row j of B (or ROWS neighbouring ones) against TPR tokens: t[token][j] = sum_k B[j][k] x[token][k], fp32 accumulation over all of K, one
 // rounding to fp16.  The row of B is pulled into L2 before griddepcontrol.wait, every load of the first 4096 columns
 // is in flight before the first use.  Fewer tokens per CTA mean more CTAs and less to load per SM: this chain decides
 // when the prologue ends.
-template <int TPR>
+template <int TPR, int ROWS = 1>
 __device__ __forceinline__ void lowrank_row(const __nv_bfloat16* __restrict__ x, int64_t ldx, const __half* __restrict__ B,
                                             __half* __restrict__ t, int n, int r_pad, int T, int rb, int tok0,
                                             const ImageOut& img) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    __shared__ float part[8][TPR];
-    const int j = rb % r_pad, tq = tok0 + TPR * (rb / r_pad);
+    __shared__ float part[8][ROWS][TPR];
+    const int j = rb % (r_pad / ROWS) * ROWS, tq = tok0 + TPR * (rb / (r_pad / ROWS));
     const __half* brow = B + (size_t)j * n;
     const int npass = (n + 2047) >> 11;
     if ((tid & 7) == 0) {  // one request per 128-byte line of the first 4096 columns of the row
 #pragma unroll
         for (int ps = 0; ps < 2; ++ps) {
             const int k = ps * 2048 + tid * 8;
-            if (k < n) prefetch_l2(brow + k);
+            if (k < n) {
+#pragma unroll
+                for (int rw = 0; rw < ROWS; ++rw) prefetch_l2(brow + (size_t)rw * n + k);
+            }
         }
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    uint4 pre[2];
+    auto load_b = [&](uint4 (&bw)[ROWS], int k) {
 #pragma unroll
-    for (int ps = 0; ps < 2; ++ps) {
-        const int k = ps * 2048 + tid * 8;
-        pre[ps] = k < n ? __ldg(reinterpret_cast<const uint4*>(brow + k)) : make_uint4(0, 0, 0, 0);
-    }
-    float acc[TPR];
+        for (int rw = 0; rw < ROWS; ++rw)
+            bw[rw] = k < n ? __ldg(reinterpret_cast<const uint4*>(brow + (size_t)rw * n + k)) : make_uint4(0, 0, 0, 0);
+    };
+    uint4 pre0[ROWS], pre1[ROWS];
+    load_b(pre0, tid * 8);
+    load_b(pre1, 2048 + tid * 8);
+    float acc[ROWS][TPR];
 #pragma unroll
-    for (int tk = 0; tk < TPR; ++tk) acc[tk] = 0.0f;
+    for (int rw = 0; rw < ROWS; ++rw)
+#pragma unroll
+        for (int tk = 0; tk < TPR; ++tk) acc[rw][tk] = 0.0f;
     auto load_x = [&](uint4 (&xw)[TPR], int k) {
 #pragma unroll
         for (int tk = 0; tk < TPR; ++tk)
             xw[tk] = (k < n && tq + tk < T) ? __ldcg(reinterpret_cast<const uint4*>(x + (size_t)(tq + tk) * ldx + k))
                                             : make_uint4(0, 0, 0, 0);
     };
-    auto accumulate = [&](const uint4& bw, const uint4 (&xw)[TPR]) {
-        float bf[8];
-        const __half2* h = reinterpret_cast<const __half2*>(&bw);
+    auto accumulate = [&](const uint4 (&bw)[ROWS], const uint4 (&xw)[TPR]) {
+        float bf[ROWS][8];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 f = __half22float2(h[i]);
-            bf[2 * i] = f.x;
-            bf[2 * i + 1] = f.y;
+        for (int rw = 0; rw < ROWS; ++rw) {
+            const __half2* h = reinterpret_cast<const __half2*>(&bw[rw]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 f = __half22float2(h[i]);
+                bf[rw][2 * i] = f.x;
+                bf[rw][2 * i + 1] = f.y;
+            }
         }
 #pragma unroll
         for (int tk = 0; tk < TPR; ++tk) {
@@ -126,8 +136,11 @@ __device__ __forceinline__ void lowrank_row(const __nv_bfloat16* __restrict__ x,
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float2 f = __bfloat1622float2(xh[i]);
-                acc[tk] = fmaf(bf[2 * i], f.x, acc[tk]);
-                acc[tk] = fmaf(bf[2 * i + 1], f.y, acc[tk]);
+#pragma unroll
+                for (int rw = 0; rw < ROWS; ++rw) {
+                    acc[rw][tk] = fmaf(bf[rw][2 * i], f.x, acc[rw][tk]);
+                    acc[rw][tk] = fmaf(bf[rw][2 * i + 1], f.y, acc[rw][tk]);
+                }
             }
         }
     };
@@ -136,37 +149,41 @@ __device__ __forceinline__ void lowrank_row(const __nv_bfloat16* __restrict__ x,
         uint4 x0[TPR], x1[TPR];
         load_x(x0, tid * 8);
         load_x(x1, 2048 + tid * 8);
-        accumulate(pre[0], x0);
-        accumulate(pre[1], x1);
+        accumulate(pre0, x0);
+        accumulate(pre1, x1);
     }
     for (int ps = 2; ps < npass; ++ps) {
         const int k = ps * 2048 + tid * 8;
         if (k >= n) break;
-        uint4 xw[TPR];
+        uint4 xw[TPR], bw[ROWS];
         load_x(xw, k);
-        accumulate(__ldg(reinterpret_cast<const uint4*>(brow + k)), xw);
+        load_b(bw, k);
+        accumulate(bw, xw);
     }
 #pragma unroll
-    for (int tk = 0; tk < TPR; ++tk) {
-        float v = acc[tk];
+    for (int rw = 0; rw < ROWS; ++rw)
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-        if (lane == 0) part[warp][tk] = v;
-    }
+        for (int tk = 0; tk < TPR; ++tk) {
+            float v = acc[rw][tk];
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+            if (lane == 0) part[warp][rw][tk] = v;
+        }
     __syncthreads();
-    if (tid < TPR) {
+    if (tid < ROWS * TPR) {
+        const int jr = j + tid / TPR, tk = tid % TPR;
         float v = 0.0f;
 #pragma unroll
-        for (int w = 0; w < 8; ++w) v += part[w][tid];
-        if (tq + tid < T) {
-            const int tok = tq + tid;
+        for (int w = 0; w < 8; ++w) v += part[w][tid / TPR][tk];
+        if (tq + tk < T) {
+            const int tok = tq + tk;
             if (img.ximg == nullptr) {
-                t[(size_t)tok * r_pad + j] = __float2half_rn(v);
+                t[(size_t)tok * r_pad + jr] = __float2half_rn(v);
             } else {
                 // operand image: tile (token group, 64-column step of the rank), token row tl, swizzled 16-byte piece
                 const int tgp = tok >> img.np_shift, tl = tok & (img.np - 1);
-                unsigned char* tile = img.timg + ((size_t)tgp * img.lr_steps + (j >> 6)) * img.np * 128;
-                *reinterpret_cast<__half*>(tile + tl * 128 + ((((j & 63) >> 3) ^ (tl & 7)) << 4) + (j & 7) * 2) =
+                unsigned char* tile = img.timg + ((size_t)tgp * img.lr_steps + (jr >> 6)) * img.np * 128;
+                *reinterpret_cast<__half*>(tile + tl * 128 + ((((jr & 63) >> 3) ^ (tl & 7)) << 4) + (jr & 7) * 2) =
                     __float2half_rn(v);
             }
         }
@@ -373,7 +390,7 @@ __device__ __forceinline__ void select_prologue_sibling(const PrologueSiblings& 
     }
 }
 
-template <bool STAGED, typename SIBS>
+template <bool STAGED, typename SIBS, int ROWS = 1>
 __global__ void __launch_bounds__(256)
 prologue_kernel(const __nv_bfloat16* __restrict__ x0, int64_t ldx, const int32_t* __restrict__ perm0,
                 const __half* __restrict__ B0, unsigned char* __restrict__ act_image0, __half* __restrict__ t0,
@@ -397,6 +414,12 @@ prologue_kernel(const __nv_bfloat16* __restrict__ x0, int64_t ldx, const int32_t
     const int nrow = (int)gridDim.x - (STAGED ? live * ((nchunks + 7) >> 3) : nchunks);
     if ((int)blockIdx.x < nrow) {
         const int rb = (int)blockIdx.x;
+        if constexpr (ROWS == 2) {
+            if (tpr == 8) lowrank_row<8, 2>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
+            else if (tpr == 4) lowrank_row<4, 2>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
+            else lowrank_row<2, 2>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
+            return;
+        }
         if (lr8.V != nullptr) {
             if (tpr == 8) lowrank_row_lr8<8>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
             else if (tpr == 4) lowrank_row_lr8<4>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
@@ -579,12 +602,22 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
     // groups about one CTA per SM)
     const int want = T <= 8 ? 256 : 120;
     while (tpr > 1 && r_pad * ((live + tpr - 1) / tpr) * ((T + 7) / 8) < want) tpr >>= 1;
-    const int row_ctas = d.rank > 0 ? r_pad * ((live + tpr - 1) / tpr) : 0;
+    const int groups = (T + 7) / 8;
+    int row_ctas = d.rank > 0 ? r_pad * ((live + tpr - 1) / tpr) : 0;
     // rotation: a token's row of x is staged in shared memory and gathered from there; with very few (token,
     // chunk) pairs the gather straight from global memory, warp = token, is as fast (measured: 6.1 against 6.3 us
     // per layer forward for one token and 4096 columns, 15.4 against 16.9 us for 8 tokens and 11008 columns)
-    const int nchunks = (d.d_in + 255) / 256, groups = (T + 7) / 8;
+    const int nchunks = (d.d_in + 255) / 256;
     const bool staged = nchunks * live * groups > 64;
+    // More than eight tokens: two rows of B per CTA and half the tokens (as many CTAs as before), or all eight tokens where
+    // rows and tokens are plenty and all loads of x are in flight at once: fewer reads through L2.  Whole forwards: 4096 ->
+    // 4096, 64 rows, 32 tokens 14.6 -> 13.1 us; 8192 -> 28672, 128 rows, 16 tokens 53.6 -> 51.7 (54.7 with eight tokens);
+    // 11008 -> 4096, 64 rows, 24 tokens 24.8 -> 23.3.  A kernel of its own: it takes other numbers of registers.
+    const bool pairs = staged && groups > 1 && tpr >= 4 && lr8.V == nullptr;
+    if (pairs) {
+        if (tpr == 8 && d.d_in <= 4096 && row_ctas * groups * (1 + sibs.n) >= 240) row_ctas /= 2;
+        else tpr /= 2;
+    }
     const int rot_ctas = staged ? live * ((nchunks + 7) / 8) : nchunks;
     if (staged && (size_t)d.d_in * 2 > 48 * 1024) {  // a row of x beyond the default limit
         static unsigned long long attr_done = 0;
@@ -607,11 +640,17 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
     const int rp = d.rank > 0 ? r_pad : 0;
     if (sibs.n == 0 && !sibs.own_rows && option(LOPRO_OPT_ONE_KERNEL_SET) != 1) {
         const NoPrologueSiblings none;
+        if (pairs)
+            return cudaLaunchKernelEx(&cfg, prologue_kernel<true, NoPrologueSiblings, 2>, x, ldx, perm, B, act_image, t, status,
+                                      d.d_in, d.identity_cols, d.block_size, inv, rp, t_pad, T, tpr, img, none, lr8);
         return staged ? cudaLaunchKernelEx(&cfg, prologue_kernel<true, NoPrologueSiblings>, x, ldx, perm, B, act_image, t, status,
                                            d.d_in, d.identity_cols, d.block_size, inv, rp, t_pad, T, tpr, img, none, lr8)
                       : cudaLaunchKernelEx(&cfg, prologue_kernel<false, NoPrologueSiblings>, x, ldx, perm, B, act_image, t, status,
                                            d.d_in, d.identity_cols, d.block_size, inv, rp, t_pad, T, tpr, img, none, lr8);
     }
+    if (pairs)
+        return cudaLaunchKernelEx(&cfg, prologue_kernel<true, PrologueSiblings, 2>, x, ldx, perm, B, act_image, t, status, d.d_in,
+                                  d.identity_cols, d.block_size, inv, rp, t_pad, T, tpr, img, sibs, lr8);
     return staged ? cudaLaunchKernelEx(&cfg, prologue_kernel<true, PrologueSiblings>, x, ldx, perm, B, act_image, t, status, d.d_in,
                                        d.identity_cols, d.block_size, inv, rp, t_pad, T, tpr, img, sibs, lr8)
                   : cudaLaunchKernelEx(&cfg, prologue_kernel<false, PrologueSiblings>, x, ldx, perm, B, act_image, t, status, d.d_in,

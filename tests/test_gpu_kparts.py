@@ -67,3 +67,12 @@ def test_the_fixed_scratch_takes_fewer_parts(n, m, T):
 def test_rotation_with_every_number_of_rows_per_cta(n, b_i, b_h, T):
     got, exact, _, _ = _run_rotation(n, b_i, b_h, T, seed=T)
     assert np.all(np.abs(got - exact) <= _ulp_bf16(exact) + 1e-6 * np.abs(exact).max())
+
+
+# the prologue's row CTAs of B x with two rows and 8, 4 or 2 tokens (more than eight tokens, by rows, columns and tokens), the
+# last group of tokens short
+@pytest.mark.parametrize("n,r,T", [(1024, 128, 21), (4096, 64, 30), (4160, 64, 32), (4096, 32, 17), (2560, 16, 31), (1024, 17, 27)])
+def test_two_rows_of_the_down_factor_per_cta(n, r, T):
+    layer = random_layer_np(n, 272, 4, 64, r, seed=n + T)
+    d = lopro.make_desc(n, 272, 4, 64, 64, identity_cols=64, rank=r)
+    _check_forward_once(layer, d, synth.activations(T, n, seed=T, outlier_frac=0.01), None, GATE_A, GATE_B)
