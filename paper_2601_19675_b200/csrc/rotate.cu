@@ -77,9 +77,10 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 
 // One row j of B (or ROWS neighbouring ones) against TPR tokens: t[token][j] = sum_k B[j][k] x[token][k], fp32 accumulation over all of K, one
 // rounding to fp16.  The row of B is pulled into L2 before griddepcontrol.wait, every load of the first 4096 columns
-// is in flight before the first use.  Fewer tokens per CTA mean more CTAs and less to load per SM: this chain decides
-// when the prologue ends.
-template <int TPR, int ROWS = 1>
+// is in flight before the first use.  DEEP: four (two) further passes of 2048 columns at a time and the row's lines of the
+// first 16384 columns requested; each pass by itself is a memory round trip.  Fewer tokens per CTA mean more CTAs and less
+// to load per SM: this chain decides when the prologue ends.
+template <int TPR, int ROWS = 1, bool DEEP = false>
 __device__ __forceinline__ void lowrank_row(const __nv_bfloat16* __restrict__ x, int64_t ldx, const __half* __restrict__ B,
                                             __half* __restrict__ t, int n, int r_pad, int T, int rb, int tok0,
                                             const ImageOut& img) {
@@ -87,10 +88,9 @@ __device__ __forceinline__ void lowrank_row(const __nv_bfloat16* __restrict__ x,
     __shared__ float part[8][ROWS][TPR];
     const int j = rb % (r_pad / ROWS) * ROWS, tq = tok0 + TPR * (rb / (r_pad / ROWS));
     const __half* brow = B + (size_t)j * n;
-    const int npass = (n + 2047) >> 11;
-    if ((tid & 7) == 0) {  // one request per 128-byte line of the first 4096 columns of the row
+    if ((tid & 7) == 0) {  // one request per 128-byte line of the first columns of the row
 #pragma unroll
-        for (int ps = 0; ps < 2; ++ps) {
+        for (int ps = 0; ps < (DEEP ? 8 : 2); ++ps) {
             const int k = ps * 2048 + tid * 8;
             if (k < n) {
 #pragma unroll
@@ -152,13 +152,27 @@ __device__ __forceinline__ void lowrank_row(const __nv_bfloat16* __restrict__ x,
         accumulate(pre0, x0);
         accumulate(pre1, x1);
     }
-    for (int ps = 2; ps < npass; ++ps) {
-        const int k = ps * 2048 + tid * 8;
-        if (k >= n) break;
-        uint4 xw[TPR], bw[ROWS];
-        load_x(xw, k);
-        load_b(bw, k);
-        accumulate(bw, xw);
+    constexpr int DEPTH = !DEEP || TPR > 4 ? 1 : (TPR <= 2 ? 4 : 2);
+    if constexpr (DEPTH == 1) {
+        for (int ps = 2; ps < ((n + 2047) >> 11); ++ps) {
+            const int k = ps * 2048 + tid * 8;
+            if (k >= n) break;
+            uint4 xw[TPR], bw[ROWS];
+            load_x(xw, k);
+            load_b(bw, k);
+            accumulate(bw, xw);
+        }
+    } else {
+        for (int k = 4096 + tid * 8; k < n; k += DEPTH * 2048) {
+            uint4 xw[DEPTH][TPR], bw[DEPTH][ROWS];
+#pragma unroll
+            for (int q = 0; q < DEPTH; ++q) {
+                load_x(xw[q], k + q * 2048);
+                load_b(bw[q], k + q * 2048);
+            }
+#pragma unroll
+            for (int q = 0; q < DEPTH; ++q) accumulate(bw[q], xw[q]);
+        }
     }
 #pragma unroll
     for (int rw = 0; rw < ROWS; ++rw)
@@ -193,23 +207,23 @@ __device__ __forceinline__ void lowrank_row(const __nv_bfloat16* __restrict__ x,
 // The same row job for the FP8 low-rank record (U, V, Sigma, s) that Algorithm 1 saves:
 // t[token][j] = sigma[j] * sum_k V[j][k] * (x[token][k] / s[k]), V in fp8 e4m3 (exact in fp32), the quotient taken on
 // the layer's side as V[j][k] * (1 / s[k]) in fp32 (once for all tokens), fp32 accumulation, one rounding to fp16.
-template <int TPR>
+template <int TPR, bool DEEP>
 __device__ __forceinline__ void lowrank_row_lr8(const __nv_bfloat16* __restrict__ x, int64_t ldx, const Lr8Args lr8,
                                                 __half* __restrict__ t, int n, int r_pad, int T, int rb, int tok0) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __shared__ float part[8][TPR];
     const int j = rb % r_pad, tq = tok0 + TPR * (rb / r_pad);
     const uint8_t* vrow = lr8.V + (size_t)j * n;
-    if ((tid & 15) == 0) {  // one request per 128-byte line of the first 4096 columns of the row of V; s likewise
+    if ((tid & 15) == 0) {  // one request per 128-byte line of the first columns of the row of V; s likewise
 #pragma unroll
-        for (int ps = 0; ps < 2; ++ps) {
+        for (int ps = 0; ps < (DEEP ? 8 : 2); ++ps) {
             const int k = ps * 2048 + tid * 8;
             if (k < n) prefetch_l2(vrow + k);
         }
     }
     if ((tid & 7) == 0) {
 #pragma unroll
-        for (int ps = 0; ps < 2; ++ps) {
+        for (int ps = 0; ps < (DEEP ? 8 : 2); ++ps) {
             const int k = ps * 2048 + tid * 8;
             if (k < n) prefetch_l2(lr8.svec + k);
         }
@@ -265,10 +279,27 @@ __device__ __forceinline__ void lowrank_row_lr8(const __nv_bfloat16* __restrict_
         accumulate(v0, s0, x0);
         accumulate(v1, s1, x1);
     }
-    for (int k = 4096 + tid * 8; k < n; k += 2048) {
-        uint4 xw[TPR];
-        load_x(xw, k);
-        accumulate(__ldg(reinterpret_cast<const uint2*>(vrow + k)), __ldg(reinterpret_cast<const uint4*>(lr8.svec + k)), xw);
+    constexpr int DEPTH = !DEEP || TPR > 4 ? 1 : (TPR <= 2 ? 4 : 2);
+    if constexpr (DEPTH == 1) {
+        for (int k = 4096 + tid * 8; k < n; k += 2048) {
+            uint4 xw[TPR];
+            load_x(xw, k);
+            accumulate(__ldg(reinterpret_cast<const uint2*>(vrow + k)), __ldg(reinterpret_cast<const uint4*>(lr8.svec + k)), xw);
+        }
+    } else {
+        for (int k = 4096 + tid * 8; k < n; k += DEPTH * 2048) {
+            uint4 xw[DEPTH][TPR], sw[DEPTH];
+            uint2 vw[DEPTH];
+#pragma unroll
+            for (int q = 0; q < DEPTH; ++q) {
+                const int kq = k + q * 2048;
+                load_x(xw[q], kq);
+                vw[q] = kq < n ? __ldg(reinterpret_cast<const uint2*>(vrow + kq)) : make_uint2(0, 0);
+                sw[q] = kq < n ? __ldg(reinterpret_cast<const uint4*>(lr8.svec + kq)) : one;
+            }
+#pragma unroll
+            for (int q = 0; q < DEPTH; ++q) accumulate(vw[q], sw[q], xw[q]);
+        }
     }
 #pragma unroll
     for (int tk = 0; tk < TPR; ++tk) {
@@ -390,7 +421,9 @@ __device__ __forceinline__ void select_prologue_sibling(const PrologueSiblings& 
     }
 }
 
-template <bool STAGED, typename SIBS, int ROWS = 1>
+// KIND of the row CTAs: kRowsPlain, kRowsPaired (two rows of B each), kRowsDeep (few tokens, long rows).
+enum { kRowsPlain, kRowsPaired, kRowsDeep };
+template <bool STAGED, typename SIBS, int KIND = kRowsPlain>
 __global__ void __launch_bounds__(256)
 prologue_kernel(const __nv_bfloat16* __restrict__ x0, int64_t ldx, const int32_t* __restrict__ perm0,
                 const __half* __restrict__ B0, unsigned char* __restrict__ act_image0, __half* __restrict__ t0,
@@ -414,23 +447,24 @@ prologue_kernel(const __nv_bfloat16* __restrict__ x0, int64_t ldx, const int32_t
     const int nrow = (int)gridDim.x - (STAGED ? live * ((nchunks + 7) >> 3) : nchunks);
     if ((int)blockIdx.x < nrow) {
         const int rb = (int)blockIdx.x;
-        if constexpr (ROWS == 2) {
+        constexpr bool DEEP = KIND == kRowsDeep;
+        if constexpr (KIND == kRowsPaired) {
             if (tpr == 8) lowrank_row<8, 2>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
             else if (tpr == 4) lowrank_row<4, 2>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
             else lowrank_row<2, 2>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
             return;
         }
         if (lr8.V != nullptr) {
-            if (tpr == 8) lowrank_row_lr8<8>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
-            else if (tpr == 4) lowrank_row_lr8<4>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
-            else if (tpr == 2) lowrank_row_lr8<2>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
-            else lowrank_row_lr8<1>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
+            if (tpr == 8) lowrank_row_lr8<8, DEEP>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
+            else if (tpr == 4) lowrank_row_lr8<4, DEEP>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
+            else if (tpr == 2) lowrank_row_lr8<2, DEEP>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
+            else lowrank_row_lr8<1, DEEP>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
             return;
         }
-        if (tpr == 8) lowrank_row<8>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
-        else if (tpr == 4) lowrank_row<4>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
-        else if (tpr == 2) lowrank_row<2>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
-        else lowrank_row<1>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
+        if (tpr == 8) lowrank_row<8, 1, DEEP>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
+        else if (tpr == 4) lowrank_row<4, 1, DEEP>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
+        else if (tpr == 2) lowrank_row<2, 1, DEEP>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
+        else lowrank_row<1, 1, DEEP>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
         return;
     }
 
@@ -613,19 +647,23 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
     // rows and tokens are plenty and all loads of x are in flight at once: fewer reads through L2.  Whole forwards: 4096 ->
     // 4096, 64 rows, 32 tokens 14.6 -> 13.1 us; 8192 -> 28672, 128 rows, 16 tokens 53.6 -> 51.7 (54.7 with eight tokens);
     // 11008 -> 4096, 64 rows, 24 tokens 24.8 -> 23.3.  A kernel of its own: it takes other numbers of registers.
-    const bool pairs = staged && groups > 1 && tpr >= 4 && lr8.V == nullptr;
+    const bool pairs = staged && groups > 1 && tpr >= 4 && lr8.V == nullptr && (size_t)d.d_in * 2 <= 48 * 1024;
     if (pairs) {
         if (tpr == 8 && d.d_in <= 4096 && row_ctas * groups * (1 + sibs.n) >= 240) row_ctas /= 2;
         else tpr /= 2;
     }
+    // Few tokens of long rows: the passes over a row in flight together (11008 -> 4096 at 8 tokens 13.7 -> 13.4 us for the whole
+    // forward, FP8 record at 5 tokens 14.9 -> 14.5, 8192 columns 9.2 -> 9.1; 5120 columns 10.8 -> 11.0, so not there; also a kernel
+    // of its own, for its registers).
+    const bool deep = groups == 1 && d.d_in >= 8192;
     const int rot_ctas = staged ? live * ((nchunks + 7) / 8) : nchunks;
     if (staged && (size_t)d.d_in * 2 > 48 * 1024) {  // a row of x beyond the default limit
-        static unsigned long long attr_done = 0;
-        cudaError_t e = ensure_dynamic_smem(prologue_kernel<true, PrologueSiblings>, kPrologueMaxSmem, &attr_done);
-        if (e == cudaSuccess) {
-            static unsigned long long attr_done2 = 0;
-            e = ensure_dynamic_smem(prologue_kernel<true, NoPrologueSiblings>, kPrologueMaxSmem, &attr_done2);
-        }
+        static unsigned long long done[4] = {};
+        cudaError_t e = ensure_dynamic_smem(prologue_kernel<true, PrologueSiblings>, kPrologueMaxSmem, &done[0]);
+        if (e == cudaSuccess) e = ensure_dynamic_smem(prologue_kernel<true, NoPrologueSiblings>, kPrologueMaxSmem, &done[1]);
+        if (e == cudaSuccess) e = ensure_dynamic_smem(prologue_kernel<true, PrologueSiblings, kRowsDeep>, kPrologueMaxSmem, &done[2]);
+        if (e == cudaSuccess) e = ensure_dynamic_smem(prologue_kernel<true, NoPrologueSiblings, kRowsDeep>, kPrologueMaxSmem, &done[3]);
+        // rows this long do not run the paired kernel
         if (e != cudaSuccess) return e;
     }
     cfg.gridDim = dim3(row_ctas + rot_ctas, (T + 7) / 8, 1 + sibs.n);
@@ -641,20 +679,20 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
     if (sibs.n == 0 && !sibs.own_rows && option(LOPRO_OPT_ONE_KERNEL_SET) != 1) {
         const NoPrologueSiblings none;
         if (pairs)
-            return cudaLaunchKernelEx(&cfg, prologue_kernel<true, NoPrologueSiblings, 2>, x, ldx, perm, B, act_image, t, status,
+            return cudaLaunchKernelEx(&cfg, prologue_kernel<true, NoPrologueSiblings, kRowsPaired>, x, ldx, perm, B, act_image, t, status,
                                       d.d_in, d.identity_cols, d.block_size, inv, rp, t_pad, T, tpr, img, none, lr8);
-        return staged ? cudaLaunchKernelEx(&cfg, prologue_kernel<true, NoPrologueSiblings>, x, ldx, perm, B, act_image, t, status,
-                                           d.d_in, d.identity_cols, d.block_size, inv, rp, t_pad, T, tpr, img, none, lr8)
-                      : cudaLaunchKernelEx(&cfg, prologue_kernel<false, NoPrologueSiblings>, x, ldx, perm, B, act_image, t, status,
-                                           d.d_in, d.identity_cols, d.block_size, inv, rp, t_pad, T, tpr, img, none, lr8);
+        const auto kernel = deep ? (staged ? prologue_kernel<true, NoPrologueSiblings, kRowsDeep> : prologue_kernel<false, NoPrologueSiblings, kRowsDeep>)
+                                 : (staged ? prologue_kernel<true, NoPrologueSiblings> : prologue_kernel<false, NoPrologueSiblings>);
+        return cudaLaunchKernelEx(&cfg, kernel, x, ldx, perm, B, act_image, t, status, d.d_in, d.identity_cols, d.block_size, inv, rp,
+                                  t_pad, T, tpr, img, none, lr8);
     }
     if (pairs)
-        return cudaLaunchKernelEx(&cfg, prologue_kernel<true, PrologueSiblings, 2>, x, ldx, perm, B, act_image, t, status, d.d_in,
+        return cudaLaunchKernelEx(&cfg, prologue_kernel<true, PrologueSiblings, kRowsPaired>, x, ldx, perm, B, act_image, t, status, d.d_in,
                                   d.identity_cols, d.block_size, inv, rp, t_pad, T, tpr, img, sibs, lr8);
-    return staged ? cudaLaunchKernelEx(&cfg, prologue_kernel<true, PrologueSiblings>, x, ldx, perm, B, act_image, t, status, d.d_in,
-                                       d.identity_cols, d.block_size, inv, rp, t_pad, T, tpr, img, sibs, lr8)
-                  : cudaLaunchKernelEx(&cfg, prologue_kernel<false, PrologueSiblings>, x, ldx, perm, B, act_image, t, status, d.d_in,
-                                       d.identity_cols, d.block_size, inv, rp, t_pad, T, tpr, img, sibs, lr8);
+    const auto kernel = deep ? (staged ? prologue_kernel<true, PrologueSiblings, kRowsDeep> : prologue_kernel<false, PrologueSiblings, kRowsDeep>)
+                             : (staged ? prologue_kernel<true, PrologueSiblings> : prologue_kernel<false, PrologueSiblings>);
+    return cudaLaunchKernelEx(&cfg, kernel, x, ldx, perm, B, act_image, t, status, d.d_in, d.identity_cols, d.block_size, inv, rp, t_pad,
+                              T, tpr, img, sibs, lr8);
 }
 
 cudaError_t launch_lowrank_down(const lopro_desc& d, const __half* B, int r_pad, const __nv_bfloat16* x,

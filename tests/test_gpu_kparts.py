@@ -71,8 +71,10 @@ def test_rotation_with_every_number_of_rows_per_cta(n, b_i, b_h, T):
 
 # the prologue's row CTAs of B x with two rows and 8, 4 or 2 tokens (more than eight tokens, by rows, columns and tokens), the
 # last group of tokens short
-@pytest.mark.parametrize("n,r,T", [(1024, 128, 21), (4096, 64, 30), (4160, 64, 32), (4096, 32, 17), (2560, 16, 31), (1024, 17, 27)])
-def test_two_rows_of_the_down_factor_per_cta(n, r, T):
+# (25600 columns: past the default limit of shared memory; 8192 and 25600 at up to eight tokens: several passes at once)
+@pytest.mark.parametrize("n,r,T", [(1024, 128, 21), (4096, 64, 30), (4160, 64, 32), (4096, 32, 17), (2560, 16, 31), (1024, 17, 27),
+                                   (25600, 16, 17), (8192, 16, 1), (8256, 64, 3), (10304, 128, 8), (25600, 16, 2)])
+def test_row_ctas_of_the_down_factor(n, r, T):
     layer = random_layer_np(n, 272, 4, 64, r, seed=n + T)
     d = lopro.make_desc(n, 272, 4, 64, 64, identity_cols=64, rank=r)
     _check_forward_once(layer, d, synth.activations(T, n, seed=T, outlier_frac=0.01), None, GATE_A, GATE_B)
