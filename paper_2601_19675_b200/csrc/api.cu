@@ -392,14 +392,15 @@ static bool group_uses_tall(int32_t n, const lopro_desc* const* descs, int32_t T
     return use_tall(*descs[0], T, rows);
 }
 
-// Token counts a little above the small-batch range run as ONE prologue plus chunks of kDecodeMaxT tokens through
-// the small-batch kernels when that costs less than the tensor-core path: a prefill CTA walks all of K for its
-// 128 or 256 rows whatever the token count, and a layer with few rows fills few SMs.  Both sides are estimated from
-// timings on B200 (microseconds, beyond a common 8 for the first launches): a chunk 3 + 0.45e-6 d_out d_in (10.9 for
-// 4096 x 4096, 23.4 for 4096 x 11008 either way round), or 3 + 1.87e-3 d_in where that is more (a CTA's 32 rows walk all of
-// K: 18.2 for 8192 columns however few the rows), the tensor-core product by prefill_plan plus 0.0015 d_in for the longer
-// launches in front of it (4096 x 4096: chunks up to 64 tokens, 23.7 against 25.4; 11008 -> 4096 at 33 tokens 36.3 against
-// 44.0).  LOPRO_OPT_NO_CHUNKS turns this off (A/B runs, tests of the prefill kernels on small layers).
+// Token counts a little above the small-batch range run as ONE prologue plus chunks of kDecodeMaxT tokens through the
+// small-batch kernels, which apply scale and zero-point in fp32; the tensor-core path rounds the dequantized weights to
+// bf16 (4096 -> 11008 at 64 tokens, 3 bits: 2.0e-3 from 64-bit arithmetic, 1.4e-3 in chunks).  The line between them is
+// therefore one of precision as well as of time and does not move with the speed of either side: it lies where chunks
+// cost less than tiles that are not cut along K (at most four parts of the two-CTA kernel's last wave, the compact plan).
+// The tensor-core path as it runs now is faster on part of the range below the line (that layer 32 against 47 us); its
+// weights in 16 bits are what it would cost.  Estimates in microseconds beyond a common 8 for the first launches: a chunk
+// 3 + 0.45e-6 d_out d_in (10.9 for 4096 x 4096, 23.4 for 4096 x 11008 either way round), the tensor-core product by
+// prefill_plan plus 0.0015 d_in for the longer launches in front of it.  LOPRO_OPT_NO_CHUNKS turns the chunks off.
 static int small_batch_chunks(const lopro_desc& d, int T) {
     if (T <= kDecodeMaxT) return 0;
     // the FP8 low-rank record has no general path: chunks wherever the tensor-core kernels cannot take the layer
@@ -408,9 +409,8 @@ static int small_batch_chunks(const lopro_desc& d, int T) {
     if (option(LOPRO_OPT_NO_CHUNKS) == 1) return 0;
     if (!prefill_supported(d, T)) return 0;  // keep the general path's behaviour where there is no prefill kernel
     const int chunks = (T + kDecodeMaxT - 1) / kDecodeMaxT;
-    const double by_weights = 0.45e-6 * (double)d.d_out * (double)d.d_in, by_columns = 1.87e-3 * (double)d.d_in;
-    const double chunk_us = 3.0 + (by_weights > by_columns ? by_weights : by_columns);
-    const double prefill_us = prefill_plan(d, T).us + 0.0015 * (double)d.d_in;  // + its longer launches in front
+    const double chunk_us = 3.0 + 0.45e-6 * (double)d.d_out * (double)d.d_in;
+    const double prefill_us = prefill_plan(d, T, true).us + 0.0015 * (double)d.d_in;
     if ((double)chunks * chunk_us >= prefill_us) return 0;
     if (!prologue_supported(d, kDecodeMaxT) || !stream_supported(d, kDecodeMaxT)) return 0;
     return chunks;
