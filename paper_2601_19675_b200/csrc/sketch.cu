@@ -233,6 +233,7 @@ __global__ void __launch_bounds__(kThreads, 1) sketch_kernel(const SketchParams 
     uint32_t parity = 0;
     bool back = false;
     float ip = 0.0f;      // 1 / |p| of the rank before
+    bool rank_dead = false;  // the rank before is a zero triple: its p may hold NaN or infinities, which no factor 0 removes
     int pass = 0;
     for (int j = 0; j < p.r; ++j) {
         for (int k = 0; k <= p.it; ++k, ++pass) {
@@ -258,7 +259,8 @@ __global__ void __launch_bounds__(kThreads, 1) sketch_kernel(const SketchParams 
                     for (int c = 0; c < V; ++c) {
                         float4 x;
                         if (l == 0) x = v[c];
-                        else if (l == j) x = cast4(__ldcg(reinterpret_cast<const float4*>(p.p) + cidx[c]), ip, p.cast);
+                        else if (l == j) x = rank_dead ? make_float4(0.f, 0.f, 0.f, 0.f)
+                                                       : cast4(__ldcg(reinterpret_cast<const float4*>(p.p) + cidx[c]), ip, p.cast);
                         else x = __ldcg(reinterpret_cast<const float4*>(p.V + (size_t)(l - 1) * n) + cidx[c]);
                         dot4(d, x, v[c]);
                     }
@@ -512,13 +514,13 @@ __global__ void __launch_bounds__(kThreads, 1) sketch_kernel(const SketchParams 
         __syncthreads();
         const float iy = inv_norm(s_yy);
         ip = inv_norm(s_vv);
-        const bool dead = iy == 0.0f || ip == 0.0f;   // exhausted: a zero triple
-        if (dead) ip = 0.0f;
-        const float sigma = dead ? 0.0f : sqrtf(s_vv);
+        rank_dead = iy == 0.0f || ip == 0.0f;   // exhausted, or something not finite: a zero triple
+        const float sigma = rank_dead ? 0.0f : sqrtf(s_vv);
         for (int c = tid; c < c1 - c0; c += kThreads)
-            reinterpret_cast<float4*>(p.V + (size_t)j * n)[c0 + c] = cast4(own[c], ip, p.cast);
+            reinterpret_cast<float4*>(p.V + (size_t)j * n)[c0 + c] =
+                rank_dead ? make_float4(0.f, 0.f, 0.f, 0.f) : cast4(own[c], ip, p.cast);
         for (int i = tid; i < rows; i += kThreads) {
-            float u = dead ? 0.0f : p.y[row0 + i] * iy;
+            float u = rank_dead ? 0.0f : p.y[row0 + i] * iy;
             if (p.cast) u = round_e4m3(u);
             p.U[(size_t)(row0 + i) * p.r + j] = u;
         }

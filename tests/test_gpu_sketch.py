@@ -1,0 +1,66 @@
+"""The persistent rank-1 sketch: what is not finite gives zero triples and touches nothing else."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import lopro_oracle as o
+from paper_2601_19675_b200 import lopro, synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("m,n", [(200, 512), (72, 2052)])
+def test_an_entry_that_is_not_finite_gives_zero_triples_and_leaves_the_matrix(m, n, bad):
+    w = synth.weights(m, n, seed=n)
+    w[m // 2, 17] = bad
+    for cast in (False, True):
+        wd = _dev(w.copy())
+        U, sigma, V = lopro.r1svd(wd, 3, 2, _dev(synth.sketches(3, n, seed=1).astype(np.float32)), cast=cast)
+        torch.cuda.synchronize()
+        assert not U.any() and not sigma.any() and not V.any()
+        np.testing.assert_array_equal(wd.cpu().numpy(), w)
+
+
+def test_a_sketch_vector_that_is_not_finite_costs_its_own_rank_only():
+    m, n, r, it = 160, 1536, 5, 4
+    w = synth.weights(m, n, seed=4, spikes=8)
+    sk = synth.sketches(r, n, seed=2).astype(np.float32)
+    keep = [0, 2, 4]
+    sk[1, 5], sk[3, 9] = np.nan, np.inf
+    U, sigma, V = lopro.r1svd(_dev(w.copy()), r, it, _dev(sk))
+    torch.cuda.synchronize()
+    assert not U[:, [1, 3]].any() and not sigma[[1, 3]].any() and not V[[1, 3]].any()
+    u_ref, s_ref, v_ref = o.r1svd(w.astype(np.float64), len(keep), it, sk[keep].astype(np.float64))
+    np.testing.assert_allclose(sigma.cpu().numpy()[keep], s_ref, rtol=2e-4)   # tolerances of the oracle test of r1svd
+    assert np.max(np.abs(U.cpu().numpy()[:, keep] - u_ref)) <= 5e-4 and np.max(np.abs(V.cpu().numpy()[keep] - v_ref)) <= 5e-4
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("fp8", [False, True])
+def test_a_bad_weight_spoils_its_own_group_only(fp8, bad):
+    n, m, g = 512, 64, 64
+    d = lopro.make_desc(n, m, 4, g, 64, identity_cols=n, rank=4,
+                        lowrank_format=lopro.LOWRANK_FP8 if fp8 else lopro.LOWRANK_FOLDED_F16)
+    w = synth.weights(m, n, seed=9)
+    w[11, 200] = bad
+    perm, sk = np.arange(n, dtype=np.int32), synth.sketches(4, n, seed=3).astype(np.float32)
+    out = lopro.quantize_layer(d, _dev(w), _dev(perm), _dev(sk), it=2)
+    torch.cuda.synchronize()
+    assert lopro.workspace_status(out["workspace"]) == lopro.ERR_INVALID_DATA
+    for name in ("U", "V", "sigma") if fp8 else ("A", "B"):
+        assert not out[name].any()
+    # without a low-rank part the residual is the matrix itself (no rotation here): the other groups are its grid
+    codes, scales, zeros = (out[k].cpu().numpy() for k in ("codes", "scales", "zeros"))
+    w[11, 192:256] = 0.0
+    c_ref, s_ref, z_ref = o.rtn_quantize(w, 4, g, dtype=np.float32)
+    ok = np.ones((m, n // g), dtype=bool)
+    ok[11, 200 // g] = False
+    np.testing.assert_array_equal(codes.reshape(m, -1, g)[ok], c_ref.reshape(m, -1, g)[ok])
+    np.testing.assert_array_equal(scales.view(np.float16).astype(np.float64)[ok], s_ref[ok])
+    np.testing.assert_array_equal(zeros.view(np.float16).astype(np.float64)[ok], z_ref[ok])
+    assert not codes.reshape(m, -1, g)[~ok].any()
