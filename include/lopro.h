@@ -361,7 +361,9 @@ LOPRO_API lopro_status lopro_linear_fwd_experts(const lopro_desc* desc, int32_t 
  *   W overflows.  A rank whose y or p vanishes (matrix exhausted) and all later ones come out as zeros.
  *     w        [m][n], IN: the matrix to decompose (W diag(s)); OUT: the deflated remainder
  *     sketches [r][n] Gaussian test vectors v_j (the call draws nothing)
- *     U [m][r], sigma [r], V [r][n] outputs; workspace of lopro_r1svd_workspace_bytes(m, n) bytes, 256-byte aligned
+ *     U [m][r], sigma [r], V [r][n] outputs; workspace of lopro_r1svd_workspace_bytes(m, n) bytes, 256-byte aligned; its
+ *     first word is a status word: LOPRO_OK, or LOPRO_ERR_TIMEOUT if a bounded wait ran out (w is then unchanged, the
+ *     outputs are unfinished)
  *   m, n multiples of 4, 1 <= r <= 512, 0 <= it <= 64.  The work is it + 1 passes over w per rank, each
  *   forming a product with W and one with W^T, and one closing pass that deflates w.
  *

@@ -177,8 +177,9 @@ __global__ void __launch_bounds__(256) deflate_kernel(float* __restrict__ W, int
 }
 
 struct R1Workspace {
+    int* status;    // first word
     float *y, *p, *u1, *v1, *partial;
-    void* scratch;  // of the persistent kernel
+    void* scratch;  // of the persistent kernel, from the status word on
     int slabs;
     size_t total;
 };
@@ -193,6 +194,7 @@ R1Workspace r1svd_workspace(int m, int n, uint8_t* base) {
         return p;
     };
     w.scratch = base;
+    w.status = reinterpret_cast<int*>(take(256));
     w.y = take((size_t)m * 4);
     w.p = take((size_t)n * 4);
     w.u1 = take((size_t)m * 4);
@@ -662,16 +664,18 @@ lopro_status lopro_r1svd(float* w, int32_t m, int32_t n, int32_t r, int32_t it, 
         job.U = U;
         job.sigma = sigma;
         job.V = V;
+        job.status = sketch_status(ws.scratch);
         job.m = m;
         job.n = n;
         job.r = r;
         job.it = it;
         job.cast = cast;
         if (launch_sketch(job, ws.scratch, (cudaStream_t)stream) != cudaSuccess ||
-            launch_deflate(w, m, n, r, U, sigma, V, (cudaStream_t)stream) != cudaSuccess)
+            launch_deflate(w, m, n, r, U, sigma, V, job.status, (cudaStream_t)stream) != cudaSuccess)
             return LOPRO_ERR_CUDA;
         return LOPRO_OK;
     }
+    if (cudaMemsetAsync(ws.status, 0, 4, (cudaStream_t)stream) != cudaSuccess) return LOPRO_ERR_CUDA;
     return run_r1svd(w, m, n, r, it, sketches, cast, U, sigma, V, ws, (cudaStream_t)stream) == cudaSuccess ? LOPRO_OK
                                                                                                            : LOPRO_ERR_CUDA;
 }

@@ -20,7 +20,8 @@
 // 31 us pass in the two barriers and the sums between them; 4096 x 4096 3.9 -> 2.0 ms.
 //
 // All sums have a fixed order (threads, rows of a CTA, CTAs): the result depends on the number of CTAs, never on timing.
-// Every wait is bounded: one that runs out raises a flag on which all CTAs leave, and stores LOPRO_ERR_TIMEOUT.
+// Every wait is bounded.  One that runs out raises the abort flag before its CTA arrives at the next grid barrier; every CTA
+// reads the flag behind the barrier, so all leave at the same one, store LOPRO_ERR_TIMEOUT and let w be.
 #include "common.cuh"
 #include "ptx.cuh"
 #include "sketch.cuh"
@@ -51,7 +52,7 @@ struct SketchParams {
     float* ext_rows;        // [1 + r][gridDim]: |y|^2, u_l y   (sums over rows)
     float* ext_cols;        // [1 + r][gridDim]: |p|^2, v_l p   (sums over columns)
     unsigned* sync;         // [0] arrivals, [1] abort flag; both zero at launch
-    int* status;            // may be null
+    int* status;
     int m, n, r, it, cast;
     int slots;              // ring slots per group
     int resident;           // every group's stages fit its slots
@@ -204,7 +205,7 @@ __global__ void __launch_bounds__(kThreads, 1) sketch_kernel(const SketchParams 
             }
         }
 
-    bool dead_wait = false;
+    bool dead_wait = false;    // this thread's wait for a stage ran out: it waits for no other
     unsigned generation = 0;
     auto grid_sync = [&]() {  // false: some CTA gave up, all leave
         __syncthreads();
@@ -216,10 +217,11 @@ __global__ void __launch_bounds__(kThreads, 1) sketch_kernel(const SketchParams 
             while (load_acquire(p.sync) < target) {
                 if ((++i & 255u) == 0u && (load_acquire(p.sync + 1) != 0u || i > kGridSpin)) {
                     atomicExch(p.sync + 1, 1u);
-                    s_abort = 1;
                     break;
                 }
             }
+            // (raised by a CTA before it arrived, or by this one above)
+            if (load_acquire(p.sync + 1) != 0u) s_abort = 1;
         }
         __syncthreads();
         return s_abort == 0;
@@ -532,17 +534,20 @@ __global__ void __launch_bounds__(kThreads, 1) sketch_kernel(const SketchParams 
     }
 leave:
     // no copy may be in flight when the CTA leaves: after an aborted barrier, wait for those of this group
-    if (s_abort || dead_wait) {
+    if (s_abort) {
         if (tg == 0)
             for (int x = q; x < min(q + p.slots, n_loads); ++x)
                 (void)mbar_wait(bar0 + 8u * (uint32_t)(x % p.slots), (uint32_t)(x / p.slots) & 1u);
-        if (tid == 0 && p.status != nullptr) atomicExch(p.status, (int)LOPRO_ERR_TIMEOUT);
+        if (tid == 0) atomicExch(p.status, (int)LOPRO_ERR_TIMEOUT);
     }
 }
 
-// W <- W - sum_l sigma_l u_l v_l^T, ranks in ascending order: four rows per CTA share each piece of V.
+// W <- W - sum_l sigma_l u_l v_l^T, ranks in ascending order: four rows per CTA share each piece of V.  Nothing if the
+// sketch gave up (*status).
 __global__ void __launch_bounds__(256) deflate_kernel(float* __restrict__ W, int m, int n, int r, const float* __restrict__ U,
-                                                      const float* __restrict__ sigma, const float* __restrict__ V) {
+                                                      const float* __restrict__ sigma, const float* __restrict__ V,
+                                                      const int* __restrict__ status) {
+    if (*status != (int)LOPRO_OK) return;
     constexpr int R = 4;
     const int i0 = blockIdx.x * R, live = min(R, m - i0), c4 = blockIdx.y * 256 + threadIdx.x;
     if (c4 >= n / 4) return;
@@ -575,7 +580,7 @@ cudaError_t launch(SketchParams p, cudaStream_t s) {
     const int rows = (p.m + ctas - 1) / ctas, stages = ((rows + R - 1) / R + G - 1) / G;
     p.slots = (int)slots;
     p.resident = stages <= slots;
-    e = cudaMemsetAsync(p.sync, 0, 8, s);
+    e = cudaMemsetAsync(p.sync - 2, 0, 16, s);  // the status word of the scratch with them
     if (e != cudaSuccess) return e;
     void* args[] = {&p};
     return cudaLaunchCooperativeKernel(sketch_kernel<TR, V, R>, dim3(ctas), dim3(kThreads), args, (size_t)kRingBytes, s);
@@ -619,7 +624,7 @@ cudaError_t launch_sketch(const SketchJob& job, void* scratch, cudaStream_t s) {
         return at;
     };
     const size_t ctas = (size_t)sm_count();
-    p.sync = (unsigned*)take(256);
+    p.sync = (unsigned*)take(256) + 2;  // (sketch_status in front)
     p.partial = (float*)take(ctas * p.n * 4);
     p.ext_rows = (float*)take(ctas * (1 + (size_t)p.r) * 4);
     p.ext_cols = (float*)take(ctas * (1 + (size_t)p.r) * 4);
@@ -633,8 +638,9 @@ cudaError_t launch_sketch(const SketchJob& job, void* scratch, cudaStream_t s) {
     return launch<512, 6, 1>(p, s);
 }
 
-cudaError_t launch_deflate(float* w, int m, int n, int r, const float* U, const float* sigma, const float* V, cudaStream_t s) {
-    deflate_kernel<<<dim3((m + 3) / 4, (n / 4 + 255) / 256), 256, 0, s>>>(w, m, n, r, U, sigma, V);
+cudaError_t launch_deflate(float* w, int m, int n, int r, const float* U, const float* sigma, const float* V, const int* status,
+                           cudaStream_t s) {
+    deflate_kernel<<<dim3((m + 3) / 4, (n / 4 + 255) / 256), 256, 0, s>>>(w, m, n, r, U, sigma, V, status);
     return cudaGetLastError();
 }
 

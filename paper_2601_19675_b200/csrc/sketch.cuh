@@ -13,15 +13,17 @@ struct SketchJob {
     float* s_eff;            // [n] the scale as applied, or null
     __half* s16;             // [n] the scale rounded to fp16 (then applied in that form), or null
     float *U, *sigma, *V;    // outputs [m][r], [r], [r][n]; V 16-byte aligned
-    int* status;             // or null
+    int* status;             // LOPRO_ERR_TIMEOUT where a wait ran out (the launch clears the scratch's own word only)
     int m, n, r, it, cast;
 };
 
 bool sketch_supported(int n, int r);
 size_t sketch_scratch_bytes(int m, int n, int r);
+inline int* sketch_status(void* scratch) { return (int*)scratch; }  // a status word that the launch clears
 cudaError_t launch_sketch(const SketchJob& job, void* scratch, cudaStream_t s);
-// w <- w - U diag(sigma) V
-cudaError_t launch_deflate(float* w, int m, int n, int r, const float* U, const float* sigma, const float* V, cudaStream_t s);
+// w <- w - U diag(sigma) V, unless *status is an error
+cudaError_t launch_deflate(float* w, int m, int n, int r, const float* U, const float* sigma, const float* V, const int* status,
+                           cudaStream_t s);
 
 // fp32 -> nearest fp8 e4m3 value (ties to even, saturating), returned as fp32; bits optionally kept.
 __device__ __forceinline__ float round_e4m3(float x, unsigned char* bits = nullptr) {

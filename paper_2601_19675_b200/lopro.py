@@ -301,14 +301,21 @@ def pack_lr8(desc, codes, scales_f16, zeros_f16, perm, U_e4m3, V_e4m3, sigma_f16
     return out
 
 
-def r1svd(w, r, it, sketches, cast=False):
-    """lopro_r1svd on a device fp32 matrix w [m][n] (deflated IN PLACE); returns (U [m][r], sigma [r], V [r][n]) fp32."""
+def r1svd_workspace_bytes(m, n):
+    return int(lib().lopro_r1svd_workspace_bytes(m, n))
+
+
+def r1svd(w, r, it, sketches, cast=False, workspace=None):
+    """lopro_r1svd on a device fp32 matrix w [m][n] (deflated IN PLACE); returns (U [m][r], sigma [r], V [r][n]) fp32.
+    The first word of the workspace (of r1svd_workspace_bytes) is the status word."""
     m, n = w.shape
     dev = w.device
     U = torch.empty((m, r), dtype=torch.float32, device=dev)
     sigma = torch.empty((r,), dtype=torch.float32, device=dev)
     V = torch.empty((r, n), dtype=torch.float32, device=dev)
-    ws = torch.empty(max(lib().lopro_r1svd_workspace_bytes(m, n), 256), dtype=torch.uint8, device=dev)
+    ws = workspace
+    if ws is None:
+        ws = torch.empty(max(r1svd_workspace_bytes(m, n), 256), dtype=torch.uint8, device=dev)
     st = lib().lopro_r1svd(_ptr(_dev(w, 4)), m, n, r, it, _ptr(_dev(sketches, 4)), 1 if cast else 0, _ptr(U), _ptr(sigma),
                            _ptr(V), _ptr(ws), ws.numel(), _stream())
     _check(st, "lopro_r1svd")

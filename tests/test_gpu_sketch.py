@@ -1,4 +1,7 @@
-"""The persistent rank-1 sketch: what is not finite gives zero triples and touches nothing else."""
+"""The persistent rank-1 sketch: what is not finite gives zero triples and touches nothing else; a wait that gives up is
+reported and leaves the matrix."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -64,3 +67,30 @@ def test_a_bad_weight_spoils_its_own_group_only(fp8, bad):
     np.testing.assert_array_equal(scales.view(np.float16).astype(np.float64)[ok], s_ref[ok])
     np.testing.assert_array_equal(zeros.view(np.float16).astype(np.float64)[ok], z_ref[ok])
     assert not codes.reshape(m, -1, g)[~ok].any()
+
+
+@pytest.mark.parametrize("m,n,r,it", [(4096, 4096, 64, 64), (16384, 512, 64, 64)])   # one and four groups of threads per CTA
+def test_a_sketch_that_gives_up_reports_it_and_leaves_the_matrix(m, n, r, it):
+    # what a wait that ran out does -- raise the abort flag, word 3 of the workspace -- is done from another stream while the
+    # kernel runs (some 100 ms if nothing stops it): every CTA leaves at its next barrier
+    w = torch.randn((m, n), device="cuda")
+    keep, sk = w.clone(), torch.randn((r, n), device="cuda")
+    ws = torch.zeros(lopro.r1svd_workspace_bytes(m, n), dtype=torch.uint8, device="cuda")
+    one = torch.ones(1, dtype=torch.int32).pin_memory()
+    other = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    done = torch.cuda.Event()
+    lopro.r1svd(w, r, it, sk, workspace=ws)
+    done.record()
+    time.sleep(0.02)
+    assert not done.query()
+    with torch.cuda.stream(other):
+        ws[12:16].view(torch.int32).copy_(one, non_blocking=True)
+    torch.cuda.synchronize()
+    assert lopro.workspace_status(ws) == lopro.ERR_TIMEOUT
+    assert torch.equal(w, keep)
+    # the next call on the same workspace starts over
+    U, sigma, V = lopro.r1svd(w, 2, 1, sk[:2], workspace=ws)
+    torch.cuda.synchronize()
+    assert lopro.workspace_status(ws) == lopro.OK
+    assert torch.dist(w + (U * sigma) @ V, keep).item() <= 1e-5 * keep.norm().item()
