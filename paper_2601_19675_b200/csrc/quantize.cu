@@ -207,7 +207,8 @@ R1Workspace r1svd_workspace(int m, int n, uint8_t* base) {
     return w;
 }
 
-// Rows too long for the persistent kernel of sketch.cu: one launch per product.
+// What the persistent kernel of sketch.cu does not take -- rows beyond 12288 columns, ranks above 128, a context that holds
+// fewer CTAs at once than the device has multiprocessors --: one launch per product.
 cudaError_t run_r1svd(float* w, int m, int n, int r, int it, const float* sketches, int cast, float* U, float* sigma,
                       float* V, const R1Workspace& ws, cudaStream_t s) {
     const dim3 g_rows((m + kGemvThreads / 32 - 1) / (kGemvThreads / 32));
@@ -232,6 +233,12 @@ cudaError_t run_r1svd(float* w, int m, int n, int r, int it, const float* sketch
     return cudaGetLastError();
 }
 
+// The persistent kernel; cudaErrorCooperativeLaunchTooLarge (cleared) where this context cannot hold its CTAs at once.
+cudaError_t try_sketch(const SketchJob& job, void* scratch, cudaStream_t s) {
+    const cudaError_t e = launch_sketch(job, scratch, s);
+    if (e == cudaErrorCooperativeLaunchTooLarge) (void)cudaGetLastError();
+    return e;
+}
 
 // ---- residual, R' = R P Q, group grid ------------------------------------------------------------
 
@@ -615,7 +622,7 @@ QuantWorkspace quant_workspace(const lopro_desc& d, uint8_t* base) {
         return p;
     };
     q.status = reinterpret_cast<int*>(take(256));
-    q.Ws = reinterpret_cast<float*>(take(r ? m * n * 4 : 0));  // (rows too long for the persistent sketch; the size stays)
+    q.Ws = reinterpret_cast<float*>(take(r ? m * n * 4 : 0));  // (the launches that stand in for the persistent sketch)
     q.U = reinterpret_cast<float*>(take(m * r * 4));
     q.V = reinterpret_cast<float*>(take(r * n * 4));
     q.sigma = reinterpret_cast<float*>(take(r * 4));
@@ -670,10 +677,11 @@ lopro_status lopro_r1svd(float* w, int32_t m, int32_t n, int32_t r, int32_t it, 
         job.r = r;
         job.it = it;
         job.cast = cast;
-        if (launch_sketch(job, ws.scratch, (cudaStream_t)stream) != cudaSuccess ||
-            launch_deflate(w, m, n, r, U, sigma, V, job.status, (cudaStream_t)stream) != cudaSuccess)
-            return LOPRO_ERR_CUDA;
-        return LOPRO_OK;
+        const cudaError_t e = try_sketch(job, ws.scratch, (cudaStream_t)stream);
+        if (e == cudaSuccess)
+            return launch_deflate(w, m, n, r, U, sigma, V, job.status, (cudaStream_t)stream) == cudaSuccess ? LOPRO_OK
+                                                                                                            : LOPRO_ERR_CUDA;
+        if (e != cudaErrorCooperativeLaunchTooLarge) return LOPRO_ERR_CUDA;
     }
     if (cudaMemsetAsync(ws.status, 0, 4, (cudaStream_t)stream) != cudaSuccess) return LOPRO_ERR_CUDA;
     return run_r1svd(w, m, n, r, it, sketches, cast, U, sigma, V, ws, (cudaStream_t)stream) == cudaSuccess ? LOPRO_OK
@@ -726,6 +734,7 @@ lopro_status lopro_quantize_layer(const lopro_desc* desc, const float* W, const 
     if (cudaMemsetAsync(q.status, 0, 4, cs) != cudaSuccess) return LOPRO_ERR_CUDA;
     if (r > 0) {
         const R1Workspace ws = r1svd_workspace(m, n, q.r1);
+        cudaError_t e = cudaErrorCooperativeLaunchTooLarge;
         if (sketch_supported(n, r)) {
             SketchJob sk = {};
             sk.w = W;
@@ -742,8 +751,10 @@ lopro_status lopro_quantize_layer(const lopro_desc* desc, const float* W, const 
             sk.r = r;
             sk.it = it;
             sk.cast = fp8 ? 1 : 0;
-            if (launch_sketch(sk, ws.scratch, cs) != cudaSuccess) return LOPRO_ERR_CUDA;
-        } else {
+            e = try_sketch(sk, ws.scratch, cs);
+            if (e != cudaSuccess && e != cudaErrorCooperativeLaunchTooLarge) return LOPRO_ERR_CUDA;
+        }
+        if (e != cudaSuccess) {
             scale_columns_kernel<<<m, 256, 0, cs>>>(W, s, n, fp8 ? 1 : 0, q.Ws, q.s_eff, fp8 ? (__half*)lr3 : nullptr);
             if (run_r1svd(q.Ws, m, n, r, it, sketches, fp8 ? 1 : 0, q.U, q.sigma, q.V, ws, cs) != cudaSuccess)
                 return LOPRO_ERR_CUDA;

@@ -1,5 +1,6 @@
-"""The persistent rank-1 sketch: what is not finite gives zero triples and touches nothing else; a wait that gives up is
-reported and leaves the matrix."""
+"""The persistent rank-1 sketch: every number of threads per row, resident rows and rows that stream, and the launches that
+stand in for it, against the oracle; what is not finite gives zero triples and touches nothing else; a wait that gives up
+is reported and leaves the matrix."""
 import time
 
 import numpy as np
@@ -14,6 +15,28 @@ pytestmark = pytest.mark.gpu
 
 def _dev(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def _check_against_the_oracle(m, n, r, it):
+    w = synth.weights(m, n, seed=m + n, spikes=r + 2)
+    sk = synth.sketches(r, n, seed=5).astype(np.float32)
+    wd = _dev(w.copy())
+    ws = torch.zeros(lopro.r1svd_workspace_bytes(m, n), dtype=torch.uint8, device="cuda")
+    U, sigma, V = lopro.r1svd(wd, r, it, _dev(sk), workspace=ws)
+    torch.cuda.synchronize()
+    assert lopro.workspace_status(ws) == lopro.OK
+    u_ref, s_ref, v_ref = o.r1svd(w.astype(np.float64), r, it, sk.astype(np.float64))
+    # the tolerances of the oracle test of r1svd: unit vectors absolutely, the remainder in the Frobenius norm
+    np.testing.assert_allclose(sigma.cpu().numpy(), s_ref, rtol=2e-4)
+    assert np.max(np.abs(U.cpu().numpy() - u_ref)) <= 5e-4 and np.max(np.abs(V.cpu().numpy() - v_ref)) <= 5e-4
+    rem_ref = w.astype(np.float64) - (u_ref * s_ref[None, :]) @ v_ref
+    assert np.linalg.norm(wd.cpu().numpy() - rem_ref) <= 1e-4 * np.linalg.norm(w)
+
+
+# rows past the persistent kernel's 12288 columns, ranks past its 128
+@pytest.mark.parametrize("m,n,r,it", [(96, 12292, 3, 2), (160, 256, 129, 1)])
+def test_the_launches_that_stand_in_for_the_persistent_kernel(m, n, r, it):
+    _check_against_the_oracle(m, n, r, it)
 
 
 @pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
