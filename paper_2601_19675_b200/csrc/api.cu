@@ -2,7 +2,10 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <cuda.h>
+
 #include "common.cuh"
+#include "hostmem.h"
 
 namespace lopro {
 
@@ -153,19 +156,33 @@ static cudaError_t launch_copy16(const void* src, void* dst, size_t bytes, cudaS
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, copy16_kernel, (const uint4*)src, (uint4*)dst, n16);
 }
-// The device's address of a host buffer whose first and last byte are pinned and mapped as one piece; null otherwise.
-// (0.06 us per lookup.)
+using PointerAttributesFn = CUresult (*)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+static PointerAttributesFn pointer_attributes_fn() {
+    static PointerAttributesFn fn = nullptr;
+    if (fn == nullptr) {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<PointerAttributesFn>(p);
+    }
+    return fn;
+}
+// The device's address of a host buffer that lies inside one pinned and mapped piece; null otherwise.
 static void* mapped(const void* host, size_t bytes) {
     if (bytes == 0 || bytes > kZeroCopyMax || (bytes % 16) || !aligned(host, 16)) return nullptr;
-    cudaPointerAttributes a, b;
-    if (cudaPointerGetAttributes(&a, host) != cudaSuccess || cudaPointerGetAttributes(&b, (const uint8_t*)host + bytes - 1) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return nullptr;
-    }
-    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer || !aligned(a.devicePointer, 16) ||
-        (uint8_t*)b.devicePointer - (uint8_t*)a.devicePointer != (ptrdiff_t)bytes - 1)
-        return nullptr;
-    return a.devicePointer;
+    const PointerAttributesFn fn = pointer_attributes_fn();
+    if (fn == nullptr) return nullptr;
+    unsigned type = 0, managed = 0;
+    HostRange r = {};
+    CUdeviceptr device = 0, start = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* into[] = {&type, &managed, &device, &start, &r.size};
+    if (fn(5, what, into, (CUdeviceptr)(uintptr_t)host) != CUDA_SUCCESS) return nullptr;
+    r.device = device;
+    r.start = start;
+    if (type != CU_MEMORYTYPE_HOST || managed || (device % 16) || !holds_whole_buffer(r, bytes)) return nullptr;
+    return (void*)(uintptr_t)device;
 }
 
 namespace {
