@@ -5,10 +5,10 @@
 //
 // At small batches each of these is a few microseconds of latency and a launch gap.  They are launched with programmatic
 // stream serialization: a kernel's CTAs are resident when its predecessor ends and wait there (every kernel executes
-// griddepcontrol.wait, so completion is transitive).  What a predecessor wrote is read through L2 (ld.global.cg): a CTA
-// that was resident before the data existed may find an older copy of a reused buffer in L1.  The small ones release their successor at once, attention only when
-// its CTAs are done with their keys: a successor that takes shared memory and thread slots while attention still has CTAs
-// to start costs more than the gap.
+// griddepcontrol.wait, so completion is transitive).  What a predecessor wrote is never read by __ldg: its non-coherent path
+// promises nothing about data written while the kernel was resident already.  The small kernels release their successor
+// at once, attention only when its CTAs are done with their keys: a successor that takes shared memory and thread slots
+// while attention still has CTAs to start costs more than the gap.
 #include "lopro_block.h"
 
 #include <cuda_bf16.h>

@@ -48,7 +48,7 @@ lowrank_down_kernel(const __half* __restrict__ B, const __nv_bfloat16* __restric
 #pragma unroll
         for (int tk = 0; tk < 8; ++tk) {
             if (tok0 + tk < T) {
-                const uint4 xw = __ldcg(reinterpret_cast<const uint4*>(x + (size_t)(tok0 + tk) * ldx) + c);
+                const uint4 xw = __ldg(reinterpret_cast<const uint4*>(x + (size_t)(tok0 + tk) * ldx) + c);
                 const __nv_bfloat162* xh = reinterpret_cast<const __nv_bfloat162*>(&xw);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -66,6 +66,28 @@ lowrank_down_kernel(const __half* __restrict__ B, const __nv_bfloat16* __restric
         for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
         if (lane == 0 && tok0 + tk < T) t[(size_t)(tok0 + tk) * r_pad + j] = __float2half_rn(s);
     }
+}
+
+// Activations that the launch in front may still be writing when this one starts.  After griddepcontrol.wait an ordinary
+// load sees them; __ldg and its non-coherent path do not have to, and the compiler may move them in front of the wait (three
+// rows of a reused buffer per layer, 16 and 32 tokens: wrong in every repetition).  Loads past L1 (ld.global.cg) are right
+// too, but the row CTAs of a multiprocessor share these rows through L1: 4096 -> 1024, 64 rows, 4 tokens 6.2 against 5.7 us.
+__device__ __forceinline__ uint4 load_coherent(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 load_coherent(const uint4* p, bool on) {   // zeros where not on
+    uint4 v = make_uint4(0, 0, 0, 0);
+    asm volatile("{\n\t.reg .pred on;\n\tsetp.ne.u32 on, %5, 0;\n\t@on ld.global.v4.u32 {%0, %1, %2, %3}, [%4];\n\t}"
+                 : "+r"(v.x), "+r"(v.y), "+r"(v.z), "+r"(v.w)
+                 : "l"(p), "r"((unsigned)on));
+    return v;
+}
+__device__ __forceinline__ unsigned short load_coherent(const unsigned short* p) {
+    unsigned short v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
 }
 
 // Pulls the 128-byte line at p into L2.  Layer data (perm, B) is requested this way before griddepcontrol.wait and
@@ -115,8 +137,7 @@ __device__ __forceinline__ void lowrank_row(const __nv_bfloat16* __restrict__ x,
     auto load_x = [&](uint4 (&xw)[TPR], int k) {
 #pragma unroll
         for (int tk = 0; tk < TPR; ++tk)
-            xw[tk] = (k < n && tq + tk < T) ? __ldcg(reinterpret_cast<const uint4*>(x + (size_t)(tq + tk) * ldx + k))
-                                            : make_uint4(0, 0, 0, 0);
+            xw[tk] = load_coherent(reinterpret_cast<const uint4*>(x + (size_t)(tq + tk) * ldx + k), k < n && tq + tk < T);
     };
     auto accumulate = [&](const uint4 (&bw)[ROWS], const uint4 (&xw)[TPR]) {
         float bf[ROWS][8];
@@ -235,8 +256,7 @@ __device__ __forceinline__ void lowrank_row_lr8(const __nv_bfloat16* __restrict_
     auto load_x = [&](uint4 (&xw)[TPR], int k) {
 #pragma unroll
         for (int tk = 0; tk < TPR; ++tk)
-            xw[tk] = (k < n && tq + tk < T) ? __ldcg(reinterpret_cast<const uint4*>(x + (size_t)(tq + tk) * ldx + k))
-                                            : make_uint4(0, 0, 0, 0);
+            xw[tk] = load_coherent(reinterpret_cast<const uint4*>(x + (size_t)(tq + tk) * ldx + k), k < n && tq + tk < T);
     };
     auto accumulate = [&](const uint2& vw, const uint4& sw, const uint4 (&xw)[TPR]) {
         float vs[8];  // V[j][k] / s[k]
@@ -397,9 +417,7 @@ constexpr int kPrologueMaxSmem = 200 * 1024;  // one row of x: d_in <= 102400
 //  * a row CTA computes t[token][j] = sum_k B[j][k] x[token][k] for one row j of B and `tpr` of the 8 tokens
 //    (8 / tpr CTAs per row): the low-rank intermediate "Y = V X".
 // Launched with programmatic stream serialization: perm and B (layer data) are pulled into L2 before the
-// wait, everything is loaded after it.  x is read through L2 (ld.global.cg): a CTA that was resident before its
-// predecessor wrote x may find an older copy of a reused buffer in L1 (seen in a decoder layer whose norms share one
-// output buffer: gate and up projections of the first norm's output).
+// wait, everything is loaded after it, x by load_coherent.
 // A launch for a single layer carries no sibling table (several hundred bytes of kernel parameters less).
 struct NoPrologueSiblings {};
 __device__ __forceinline__ void select_prologue_sibling(const NoPrologueSiblings&, const int32_t*&, const __half*&,
@@ -492,7 +510,7 @@ prologue_kernel(const __nv_bfloat16* __restrict__ x0, int64_t ldx, const int32_t
             float v[8];
             const unsigned short* xrow = reinterpret_cast<const unsigned short*>(x + (size_t)tok * ldx);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = col0 < n ? __bfloat162float(__ushort_as_bfloat16(__ldcg(xrow + pidx[e]))) : 0.0f;
+            for (int e = 0; e < 8; ++e) v[e] = col0 < n ? __bfloat162float(__ushort_as_bfloat16(load_coherent(xrow + pidx[e]))) : 0.0f;
             rotate_tail(v, act_image, n, b_i, b_h, inv_sqrt_bh, t_pad, tok, col0, lane, img);
         }
     } else {
@@ -518,7 +536,7 @@ prologue_kernel(const __nv_bfloat16* __restrict__ x0, int64_t ldx, const int32_t
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int k = base + i * 2048 + tid * 8;
-                if (k < n) w[i] = __ldcg(reinterpret_cast<const uint4*>(xrow + k));
+                if (k < n) w[i] = load_coherent(reinterpret_cast<const uint4*>(xrow + k));
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -644,12 +662,13 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
     const int nchunks = (d.d_in + 255) / 256;
     const bool staged = nchunks * live * groups > 64;
     // More than eight tokens: two rows of B per CTA and half the tokens (as many CTAs as before), or all eight tokens where
-    // rows and tokens are plenty and all loads of x are in flight at once: fewer reads through L2.  Whole forwards: 4096 ->
-    // 4096, 64 rows, 32 tokens 14.6 -> 13.1 us; 8192 -> 28672, 128 rows, 16 tokens 53.6 -> 51.7 (54.7 with eight tokens);
-    // 11008 -> 4096, 64 rows, 24 tokens 24.8 -> 23.3.  A kernel of its own: it takes other numbers of registers.
+    // that leaves more than one CTA per multiprocessor and all loads of x are in flight at once: fewer reads of x.  Whole
+    // forwards with one row, two rows and half the tokens, two rows and all of them: 2048 -> 1024, 128 rows, 32 tokens 11.9 us,
+    // 11.3, 10.6; 16 tokens (128 CTAs in the last form) 6.8, 6.5, 7.4; 4096 -> 4096, 64 rows, 32 tokens 14.3, 13.5, 13.4.  A
+    // kernel of its own: it takes other numbers of registers.
     const bool pairs = staged && groups > 1 && tpr >= 4 && lr8.V == nullptr && (size_t)d.d_in * 2 <= 48 * 1024;
     if (pairs) {
-        if (tpr == 8 && d.d_in <= 4096 && row_ctas * groups * (1 + sibs.n) >= 240) row_ctas /= 2;
+        if (tpr == 8 && d.d_in <= 4096 && row_ctas * groups * (1 + sibs.n) > 2 * sm_count()) row_ctas /= 2;
         else tpr /= 2;
     }
     // Few tokens of long rows: the passes over a row in flight together (11008 -> 4096 at 8 tokens 13.7 -> 13.4 us for the whole
