@@ -474,7 +474,13 @@ cudaError_t launch_vq_product(VqProduct p, const VqPlan& plan, const __half* A, 
     return launch_programmatic((const void*)vq_finish_kernel, dim3((p.m + 127) / 128, (p.T + 3) / 4), 128, 0, args, s);
 }
 
-// Codebooks whose row groups are no multiple of 128 rows (256 with 2-D centroids).
+// More than 32 tokens run in chunks of 32, and a chunk of vq_product_kernel is two launches and its partial sums.  On a
+// layer of few stages per multiprocessor that is more than a launch of vq_decode_kernel: 512 -> 512 at 96 tokens 40.5 us
+// against 27.8, 4096 -> 4096 at 64 tokens 49.7 against 42.5 (4096 -> 2048 at 96: 51.7, 53.5).  Long rows and large layers
+// are the other way: 8192 -> 1024 at 64 tokens 57 against 66, 4096 -> 8192 at 33 tokens, 2-D, 48 against 62.
+bool vq_row_blocks_pay(const lopro_vq_desc& d) { return d.d_in > 4096 || (int64_t)d.d_in * d.d_out > (1 << 24); }
+
+// Codebooks whose row groups are no multiple of 128 rows (256 with 2-D centroids), and chunks of small layers.
 template <int NT>
 cudaError_t launch_vq_decode(const VqParams& p, int dim, cudaStream_t s) {
     // two sections of codebooks; at the end the same memory holds the four warps' partial sums [4][NT][4][32] fp32
@@ -587,7 +593,8 @@ lopro_status lopro_vq_linear_fwd(const lopro_vq_desc* desc, const void* packed, 
     int* status = (int*)(ws + W.off_status);
     // up to 32 tokens the small-batch prologue does both jobs in one launch of the programmatic chain; its records of
     // 1024 columns and plain rows differ in their strides only
-    const VqPlan plan = vq_plan(d);
+    VqPlan plan = vq_plan(d);
+    if (T > kDecodeMaxT && !vq_row_blocks_pay(d)) plan.rb = 0;
     const bool records = plan.rb > 0 && T <= kDecodeMaxT && prologue_supported(sd, T);
     const int t_pad = round_up_int(T, 8);
     if (records) {
