@@ -33,6 +33,16 @@ def _check_against_the_oracle(m, n, r, it):
     assert np.linalg.norm(wd.cpu().numpy() - rem_ref) <= 1e-4 * np.linalg.norm(w)
 
 
+# threads per row and float4 columns per thread by width (512, 1024, 2048, 4096, 8192, 12288 columns at most), the last four
+# columns alone in theirs, fewer rows than CTAs, rows that stay in the ring and rows that stream, one group of threads and
+# several, ranks in a second and a fourth warp of a row's threads
+@pytest.mark.parametrize("m,n,r,it", [(60, 512, 20, 2), (15000, 512, 3, 2), (300, 516, 40, 1), (7500, 1024, 3, 2), (148, 1536, 40, 1),
+                                      (4000, 2048, 3, 2), (300, 2052, 5, 2), (1800, 4096, 3, 1), (1000, 5000, 3, 2), (200, 8192, 20, 1),
+                                      (700, 11008, 3, 2), (160, 12288, 33, 1), (256, 512, 128, 1), (256, 1536, 128, 0)])
+def test_every_form_of_the_persistent_kernel(m, n, r, it):
+    _check_against_the_oracle(m, n, r, it)
+
+
 # rows past the persistent kernel's 12288 columns, ranks past its 128
 @pytest.mark.parametrize("m,n,r,it", [(96, 12292, 3, 2), (160, 256, 129, 1)])
 def test_the_launches_that_stand_in_for_the_persistent_kernel(m, n, r, it):
