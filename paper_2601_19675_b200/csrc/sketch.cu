@@ -20,8 +20,9 @@
 // 31 us pass in the two barriers and the sums between them; 4096 x 4096 3.9 -> 2.0 ms.
 //
 // All sums have a fixed order (threads, rows of a CTA, CTAs): the result depends on the number of CTAs, never on timing.
-// Every wait is bounded.  One that runs out raises the abort flag before its CTA arrives at the next grid barrier; every CTA
-// reads the flag behind the barrier, so all leave at the same one, store LOPRO_ERR_TIMEOUT and let w be.
+// Every wait is bounded.  One that runs out raises the abort flag before its CTA arrives at the next grid barrier.  The flag
+// is a bit of the word that counts the arrivals, so no CTA gets past that barrier without it (a word of its own, read behind
+// every barrier, cost 0.25 us each: 4096 x 512 at rank 8 327 -> 348 us).  All leave there, store LOPRO_ERR_TIMEOUT and let w be.
 #include "common.cuh"
 #include "ptx.cuh"
 #include "sketch.cuh"
@@ -38,6 +39,7 @@ constexpr int kMaxSlots = 64;                  // ring slots of all groups toget
 constexpr int kMaxRank = 128;                  // one thread of a row per rank before
 constexpr int kMaxOwn = 32;                    // float4 columns of p a CTA sums
 constexpr uint32_t kGridSpin = 1u << 24;       // polls of a grid barrier before it gives up
+constexpr unsigned kAbort = 1u << 31;          // in the count of arrivals (2 (it + 1) r barriers of at most 192 CTAs: 22 bits)
 
 struct SketchParams {
     const float* w;         // [m][n]
@@ -51,7 +53,7 @@ struct SketchParams {
     float* partial;         // [gridDim][n] sums of y_i w_i
     float* ext_rows;        // [1 + r][gridDim]: |y|^2, u_l y   (sums over rows)
     float* ext_cols;        // [1 + r][gridDim]: |p|^2, v_l p   (sums over columns)
-    unsigned* sync;         // [0] arrivals, [1] abort flag; both zero at launch
+    unsigned* sync;         // arrivals and the abort flag; zero at launch
     int* status;
     int m, n, r, it, cast;
     int slots;              // ring slots per group
@@ -213,15 +215,14 @@ __global__ void __launch_bounds__(kThreads, 1) sketch_kernel(const SketchParams 
         if (tid == 0) {
             asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.sync) : "memory");
             const unsigned target = generation * (unsigned)ctas;
-            uint32_t i = 0;
-            while (load_acquire(p.sync) < target) {
-                if ((++i & 255u) == 0u && (load_acquire(p.sync + 1) != 0u || i > kGridSpin)) {
-                    atomicExch(p.sync + 1, 1u);
+            unsigned seen;
+            for (uint32_t i = 0; (seen = load_acquire(p.sync)) < target; ++i) {   // (the flag ends the wait too)
+                if (i > kGridSpin) {
+                    seen = kAbort | atomicOr(p.sync, kAbort);
                     break;
                 }
             }
-            // (raised by a CTA before it arrived, or by this one above)
-            if (load_acquire(p.sync + 1) != 0u) s_abort = 1;
+            if (seen & kAbort) s_abort = 1;
         }
         __syncthreads();
         return s_abort == 0;
@@ -308,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, 1) sketch_kernel(const SketchParams 
                 if (p.resident) slot = st / G;
                 if (!dead_wait && !mbar_wait(bar0 + 8u * (uint32_t)slot, parity)) {
                     dead_wait = true;
-                    atomicExch(p.sync + 1, 1u);
+                    atomicOr(p.sync, kAbort);
                 }
                 const Quad* sm = reinterpret_cast<const Quad*>(ring + (size_t)slot * stage_bytes);
 #pragma unroll

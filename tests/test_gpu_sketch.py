@@ -104,12 +104,12 @@ def test_a_bad_weight_spoils_its_own_group_only(fp8, bad):
 
 @pytest.mark.parametrize("m,n,r,it", [(4096, 4096, 64, 64), (16384, 512, 64, 64)])   # one and four groups of threads per CTA
 def test_a_sketch_that_gives_up_reports_it_and_leaves_the_matrix(m, n, r, it):
-    # what a wait that ran out does -- raise the abort flag, word 3 of the workspace -- is done from another stream while the
-    # kernel runs (some 100 ms if nothing stops it): every CTA leaves at its next barrier
+    # what a wait that ran out does -- raise the abort flag, the highest bit of word 2 of the workspace -- is done from another
+    # stream while the kernel runs (some 100 ms if nothing stops it): every CTA leaves at its next barrier
     w = torch.randn((m, n), device="cuda")
     keep, sk = w.clone(), torch.randn((r, n), device="cuda")
     ws = torch.zeros(lopro.r1svd_workspace_bytes(m, n), dtype=torch.uint8, device="cuda")
-    one = torch.ones(1, dtype=torch.int32).pin_memory()
+    flag = torch.tensor([-2 ** 31], dtype=torch.int32).pin_memory()
     other = torch.cuda.Stream()
     torch.cuda.synchronize()
     done = torch.cuda.Event()
@@ -118,7 +118,7 @@ def test_a_sketch_that_gives_up_reports_it_and_leaves_the_matrix(m, n, r, it):
     time.sleep(0.02)
     assert not done.query()
     with torch.cuda.stream(other):
-        ws[12:16].view(torch.int32).copy_(one, non_blocking=True)
+        ws[8:12].view(torch.int32).copy_(flag, non_blocking=True)
     torch.cuda.synchronize()
     assert lopro.workspace_status(ws) == lopro.ERR_TIMEOUT
     assert torch.equal(w, keep)
