@@ -4,10 +4,11 @@ marshals arguments for it) with the host compiler, in-tree.
 Usage:  python -m paper_2601_19675_b200.build [--force]
 Both are written next to this file; the library links the CUDA runtime statically and does not
 depend on the driver library at load time, so it can be loaded (not run) on a machine without
-a GPU.
+a GPU.  The library needs no torch; without one it is built alone.
 """
 from __future__ import annotations
 
+import importlib.metadata
 import os
 import shutil
 import subprocess
@@ -18,6 +19,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblopro.so")
 BINDING = os.path.join(HERE, "_binding.so")
+STAMP = os.path.join(HERE, "_build", "binding.txt")
 SOURCES = ["api.cu", "pack.cu", "rotate.cu", "decode.cu", "stream.cu", "tall.cu", "noalloc.cu", "prefill.cu", "lowrank.cu", "rowblock.cu", "quantize.cu", "sketch.cu", "block.cu", "vq.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden"]
@@ -30,9 +32,25 @@ def _nvcc():
     return exe
 
 
+def _torch_version():
+    try:
+        return importlib.metadata.version("torch")
+    except importlib.metadata.PackageNotFoundError:
+        return None
+
+
+def _binding_for():
+    """What the extension is compiled against: it is good for this Python and this torch only."""
+    return f"{sys.implementation.cache_tag} torch {_torch_version()}"
+
+
 def _stale():
     if not os.path.exists(LIB) or not os.path.exists(BINDING):
         return True
+    if os.path.exists(STAMP):
+        with open(STAMP) as f:
+            if f.read() != _binding_for():
+                return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
     inc = os.path.join(ROOT, "include")
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(inc, f) for f in os.listdir(inc)] + [__file__]
@@ -61,7 +79,11 @@ def build(force=False, verbose=False):
     os.makedirs(objdir, exist_ok=True)
     nvcc = _nvcc()
     objs = []
-    procs = [("binding.cpp", subprocess.Popen(_binding_command(), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True))]
+    procs = []
+    if _torch_version() is None:
+        sys.stderr.write("torch is not installed: liblopro.so is built without the Python extension\n")
+    else:
+        procs.append(("binding.cpp", subprocess.Popen(_binding_command(), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
     for src in SOURCES:
         obj = os.path.join(objdir, src.replace(".cu", ".o"))
         cmd = [nvcc, *NVCC_FLAGS, "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-c", os.path.join(CSRC, src), "-o", obj]
@@ -77,6 +99,9 @@ def build(force=False, verbose=False):
             raise RuntimeError(f"the compiler failed on {src}")
     cmd = [nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", LIB, *objs]
     subprocess.run(cmd, check=True)
+    if _torch_version() is not None:
+        with open(STAMP, "w") as f:
+            f.write(_binding_for())
     return LIB
 
 

@@ -160,7 +160,9 @@ def lib():
         try:
             from . import _binding
         except ImportError as e:
-            raise RuntimeError("the CPython extension is missing: build it with `python -m paper_2601_19675_b200.build`") from e
+            path = os.path.join(os.path.dirname(LIB_PATH), "_binding.so")
+            what = f"cannot be loaded here ({e})" if os.path.exists(path) else "is missing"
+            raise RuntimeError(f"{path} {what}: build it with `python -m paper_2601_19675_b200.build`") from e
         _binding.bind({name: ctypes.cast(getattr(L, name), vp).value for name in _NATIVE_SYMBOLS})
         _native = _binding
         _lib = L
