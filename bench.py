@@ -633,7 +633,7 @@ def measure(args, name, steps, warmup, rank, world, local, dev, dist, with_e2e=T
     note = ("duration = step time / layer forwards (includes the prologue kernels of each forward): an upper bound on the "
             "product kernel's own duration, a lower bound on `achieved`")
     if getattr(w, "block", False):
-        kernel += " + attention_split_kernel"
+        kernel += " + attention_kernel"
         note = ("whole decode step: bytes = packed weights + key/value cache, duration = step time / 224 linears (every kernel of "
                 "the step included)")
     if w.T <= 64:

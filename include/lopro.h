@@ -225,9 +225,13 @@ LOPRO_API lopro_status lopro_rotate(const lopro_desc* desc, const int32_t* perm,
  *             after synchronising).  Calls that share a workspace must be ordered on one stream.
  * Arithmetic: rotated activations rounded to bf16; B x accumulated in fp32 and rounded to fp16; A
  * times that accumulated in fp32 into the same sum as the quantized part; one final rounding to the
- * output type.  Quantized part, T <= 32: code-times-activation products accumulated in fp32 on the
- * tensor cores, scales and zero-points applied in fp32 (the weights are never rounded).  T > 32:
- * weights dequantized in fp32 and rounded once to bf16, bf16 x bf16 products accumulated in fp32.
+ * output type.  Quantized part, T <= 32 and longer calls that run as chunks of 32 (lopro_linear_fwd_path):
+ * code-times-activation products accumulated in fp32 on the tensor cores, scales and zero-points
+ * applied in fp32 (the weights are never rounded).  Other calls with T > 32: weights dequantized in
+ * fp32 and rounded once to bf16, bf16 x bf16 products accumulated in fp32.
+ * A workspace smaller than lopro_workspace_bytes(desc, T) is refused with LOPRO_ERR_BUFFER_TOO_SMALL
+ * unless it holds the least the forward can run in (see lopro_linear_fwd_noalloc): then fewer parts of
+ * K run side by side, the sums are taken in another order and the call is slower.
  * T = 0 is a no-op. */
 LOPRO_API lopro_status lopro_linear_fwd(const lopro_desc* desc, const void* packed, const uint16_t* x_bf16, int64_t ldx,
                               void* y, int64_t ldy, int32_t out_dtype, int32_t T, void* workspace,
@@ -242,9 +246,9 @@ LOPRO_API lopro_status lopro_linear_fwd(const lopro_desc* desc, const void* pack
  *   LOPRO_PATH_GENERAL  rotation, B x, register-ring product (any shape the descriptor allows)
  *   LOPRO_PATH_PREFILL  rotation, B x (2 launches), tcgen05 product (one CTA per tile, or two with a launch more
  *                       where the last wave's tiles are cut along K), T > 32
- * For T a little above 32, where the library estimates it to be faster than the tensor-core path (layers with
- * few output rows; e.g. up to 64 tokens for 4096 x 4096), the forward runs as chunks of 32 tokens through the
- * small-batch kernels: STREAM or TALL with one prologue launch and one launch per chunk.
+ * For T a little above 32 (layers with few output rows; e.g. up to 64 tokens for 4096 x 4096) the forward runs as
+ * chunks of 32 tokens through the small-batch kernels, whose weights are not rounded: STREAM or TALL with one
+ * prologue launch and one launch per chunk.  The answer is that of a workspace of lopro_workspace_bytes.
  * Returns the path (> 0) and stores the number of kernel launches in *launches (may be NULL), or
  * returns 0 for a bad descriptor or T < 1. */
 typedef enum {
@@ -295,14 +299,13 @@ LOPRO_API lopro_status lopro_linear_fwd_host(const lopro_desc* desc, const void*
  * driver for memory is not an option: a plug-in inside a host program that owns the whole device
  * heap and hands out none of it, a latency-critical serving loop in which cudaMalloc's implicit
  * device synchronisation would stall every other stream, or a process started with a fixed memory
- * budget.  It computes exactly what lopro_linear_fwd computes, with the same arguments minus the
- * workspace: the scratch is a fixed array of LOPRO_NOALLOC_SCRATCH_BYTES inside the library itself
+ * budget.  It computes what lopro_linear_fwd computes (fp32 sums in another order where its workspace is
+ * larger than this scratch), with the same arguments minus the workspace: the scratch is a fixed array of LOPRO_NOALLOC_SCRATCH_BYTES inside the library itself
  * (every GPU that loads the library holds that memory until the process ends).
- *   - Accepted sizes: whatever the forward can run in LOPRO_NOALLOC_SCRATCH_BYTES: every layer and token
- *     count with lopro_workspace_bytes(desc, T) <= LOPRO_NOALLOC_SCRATCH_BYTES, and more of them with
- *     fewer parallel parts than in a workspace of that size.  This covers
- *     the small-batch (decode) range of ordinary layers, e.g. d_in = 8192 with T <= 32.  Anything
- *     larger returns LOPRO_ERR_BUFFER_TOO_SMALL and does nothing.
+ *   - Accepted sizes: whatever the forward can run in LOPRO_NOALLOC_SCRATCH_BYTES with the fewest parallel
+ *     parts.  lopro_workspace_bytes(desc, T) may be larger than that from 33 tokens on.  This covers the
+ *     small-batch (decode) range of ordinary layers, e.g. d_in = 8192 with T <= 32.  Anything larger
+ *     returns LOPRO_ERR_BUFFER_TOO_SMALL and does nothing.
  *   - The call allocates and frees nothing and does not synchronise.  The first call on each device
  *     looks up the array's device address (once per device, with that device current); make that
  *     first call before any stream capture begins.
@@ -357,8 +360,9 @@ LOPRO_API lopro_status lopro_linear_fwd_experts(const lopro_desc* desc, int32_t 
  * lopro_r1svd -- rank-1 randomized sketch with deflation (Sec. 3.3, Eq. 10-12; inner loop of Algorithm 1).  Per rank
  *   j: y = (W W^T)^it W v_j, p = W^T y, U_j = y / |y|, V_j = p / |p|, sigma_j = |p| / |y|, optionally U_j, V_j
  *   rounded to fp8 e4m3 (cast = 1; the values are then those fp8 numbers, held in fp32), then W <- W - sigma_j U_j V_j^T.
- *   The vector is renormalised after every product (a scaling that cancels in U_j, V_j and sigma_j), so no power of
- *   W overflows.  A rank whose y or p vanishes (matrix exhausted) and all later ones come out as zeros.
+ *   The vector is renormalised after every product with W and one with W^T (a scaling that cancels in U_j, V_j and
+ *   sigma_j), so no power of W overflows.  A rank whose y or p vanishes (matrix exhausted) or has a norm that is not
+ *   finite (an entry of w or a sketch that is not) comes out as zeros and leaves w as it is.
  *     w        [m][n], IN: the matrix to decompose (W diag(s)); OUT: the deflated remainder
  *     sketches [r][n] Gaussian test vectors v_j (the call draws nothing)
  *     U [m][r], sigma [r], V [r][n] outputs; workspace of lopro_r1svd_workspace_bytes(m, n) bytes, 256-byte aligned; its
@@ -388,7 +392,8 @@ LOPRO_API lopro_status lopro_linear_fwd_experts(const lopro_desc* desc, int32_t 
  *     lr0..lr3: LOPRO_LOWRANK_FOLDED_F16: lr0 = A [m][r] fp16 = fp16(U Sigma), lr1 = B [r][n] fp16 = fp16(V diag(s)^-1);
  *               LOPRO_LOWRANK_FP8: lr0 = U [m][r] e4m3, lr1 = V [r][n] e4m3, lr2 = Sigma [r] fp16, lr3 = s [n] fp16
  *     -- exactly the arguments of lopro_pack / lopro_pack_lr8.  rank = 0: no factors, R = W.
- *   The first word of the workspace is the status word; workspace of lopro_quantize_workspace_bytes(desc) bytes. */
+ *   The first word of the workspace is the status word; workspace of lopro_quantize_workspace_bytes(desc) bytes (a copy of
+ *   W among them, for the launches that stand in for the persistent sketch where that does not run). */
 LOPRO_API size_t lopro_r1svd_workspace_bytes(int32_t m, int32_t n);
 LOPRO_API lopro_status lopro_r1svd(float* w, int32_t m, int32_t n, int32_t r, int32_t it, const float* sketches,
                                    int32_t cast, float* U, float* sigma, float* V, void* workspace,

@@ -35,9 +35,11 @@ LOPRO_API lopro_status lopro_block_rope_append(uint16_t* q, int64_t ldq, const u
                                                void* status_word, void* stream);
 
 /* out[t, h] = sum_j softmax_j(q[t, h] . K[t, h, j] * scale) V[t, h, j] over j < ctx[t] (1 <= ctx[t] <= ctx_max, else
- * LOPRO_ERR_INVALID_DATA in *status_word and zeros).  One launch: the keys of a (sequence, head) pair are shared out over a
- * cluster of CTAs.  head_dim = 128.  workspace: lopro_block_attention_workspace_bytes(...) bytes of
- * device memory, 256-byte aligned.  out [T][n_heads * head_dim] (ldo). */
+ * LOPRO_ERR_INVALID_DATA in *status_word and zeros).  The keys of a (sequence, head) pair are shared out over a
+ * cluster of CTAs; one launch, or a second one for the pairs of a short last wave.  head_dim = 128.  workspace:
+ * lopro_block_attention_workspace_bytes(...) bytes of device memory, 256-byte aligned: still asked for and checked,
+ * neither read nor written by the present kernels.  k_cache and v_cache 16-byte aligned.
+ * out [T][n_heads * head_dim] (ldo). */
 LOPRO_API size_t lopro_block_attention_workspace_bytes(int32_t T, int32_t n_heads, int32_t head_dim, int32_t ctx_max);
 LOPRO_API lopro_status lopro_block_attention_decode(const uint16_t* q, int64_t ldq, const uint16_t* k_cache,
                                                     const uint16_t* v_cache, const int32_t* ctx, uint16_t* out, int64_t ldo,

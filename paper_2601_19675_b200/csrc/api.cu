@@ -497,7 +497,7 @@ lopro_status lopro_linear_fwd(const lopro_desc* desc, const void* packed, const 
     st = workspace_layout(*desc, T, &W);
     if (st != LOPRO_OK) return st;
     if (workspace_bytes < W.total) {
-        // (the fixed scratch of lopro_linear_fwd_noalloc: fewer K slices and K parts)
+        // (the fixed scratch of lopro_linear_fwd_noalloc, or a workspace of that least size: fewer K slices and K parts)
         workspace_layout(*desc, T, &W, true);
         if (workspace_bytes < W.total) return LOPRO_ERR_BUFFER_TOO_SMALL;
     }

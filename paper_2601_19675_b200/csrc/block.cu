@@ -172,8 +172,8 @@ constexpr int kMaxCluster = 8;
 // and within a CTA over its half-warps: sixteen lanes read a key's (value's) 256 bytes as one 16-byte piece each, so every
 // access is a whole row, and a half-warp needs nobody else until the end: it keeps its own running maximum, sum of weights
 // and weighted values.  Keys and values of the next four keys are requested before the present four are used.  The
-// half-warps' results meet in shared memory, the CTAs' in that of the cluster's first CTA: no second launch, no scratch
-// in global memory.
+// half-warps' results meet in shared memory, the CTAs' in that of the cluster's first CTA: no merging launch, no scratch
+// in global memory (the workspace of the entry point is not touched).
 // 32 sequences of 32 heads, context 2049 (1.07 GB): 217 us in two launches before, 165 us = 6.5 TB/s now.
 // kWhole: all pairs.  kFirst, kTail: the pairs of a short last wave run as a second launch in larger clusters, which starts
 // as the first launch's CTAs finish.  For that the first releases it when its own predecessor is complete, and the tail

@@ -777,8 +777,9 @@ cudaError_t launch_prefill_bits(const PrefillParams& p, const CUtensorMap& mx, c
 // The partial sums of the units cut along K, added in a fixed order: y[token][row] = sum over parts.  One thread per
 // four rows of two tokens, eight 16-byte loads in flight and 8-byte stores (4096 -> 11008 at 203 tokens: 46.2 us for the
 // whole forward, 47.8 with one token per thread and 2-byte stores).  It must not release its successor early: the next
-// forward's rotation then takes the multiprocessors' shared memory before the product is out (48 -> 54 us).  Tiles from first_tile on, of tile_tokens tokens; the two-CTA kernel's are 256 rows in row-major order
-// (pair_ctas = -1), the one-CTA kernel's two-block tiles (pair_ctas of them) precede its one-block tiles.
+// forward's rotation then takes the multiprocessors' shared memory before the product is out (48 -> 54 us).  Tiles from
+// first_tile on, of tile_tokens tokens; the two-CTA kernel's are 256 rows in row-major order (pair_ctas = -1), the one-CTA
+// kernel's two-block tiles (pair_ctas of them) precede its one-block tiles.
 struct KPartsSum {
     const float* kparts;
     void* y;

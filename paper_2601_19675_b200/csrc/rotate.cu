@@ -97,8 +97,8 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
-// One row j of B (or ROWS neighbouring ones) against TPR tokens: t[token][j] = sum_k B[j][k] x[token][k], fp32 accumulation over all of K, one
-// rounding to fp16.  The row of B is pulled into L2 before griddepcontrol.wait, every load of the first 4096 columns
+// One row j of B (or ROWS neighbouring ones) against TPR tokens: t[token][j] = sum_k B[j][k] x[token][k], fp32 accumulation
+// over all of K, one rounding to fp16.  The row of B is pulled into L2 before griddepcontrol.wait, every load of the first 4096 columns
 // is in flight before the first use.  DEEP: four (two) further passes of 2048 columns at a time and the row's lines of the
 // first 16384 columns requested; each pass by itself is a memory round trip.  Fewer tokens per CTA mean more CTAs and less
 // to load per SM: this chain decides when the prologue ends.

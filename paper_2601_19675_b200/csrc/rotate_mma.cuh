@@ -3,14 +3,14 @@
 //
 // H_b = H_{b/16} (x) H_16 in the natural (Kronecker) order: a block of b gathered entries is cut into tiles of 16;
 // every tile is multiplied by H_16 (entries +-1, exact in bf16; fp32 accumulation) with mma.m16n8k16 -- tokens are
-// the M dimension, so a warp rotates one block of 8 token rows, or 2, 4, 8 blocks of 4, 2, 1 rows at once --, then the tiles are combined by
-// log2(b/16) levels of add / subtract, which pair registers of the SAME lane (no shuffles), one scaling by 1/sqrt(b)
+// the M dimension, so a warp rotates one block of 8 token rows, or 2, 4, 8 blocks of 4, 2, 1 rows at once --, then the
+// tiles are combined by log2(b/16) levels of add / subtract, which pair registers of the SAME lane (no shuffles), one scaling by 1/sqrt(b)
 // and one rounding to bf16.  Against register-and-shuffle butterflies this is about a third of the instructions
 // per entry, which is what bounds the rotation of a prefill batch (the data is read and written exactly once).
 //
 // A CTA stages TOK token rows of x in shared memory (the permutation scatters over the whole row) and its warps
-// take the row's blocks in turn.  Lane l = 4 g + t: token g % TOK, block g / TOK of those at
-// once; of every 16-tile the gathered columns 4t .. 4t + 3 and the outputs 4t .. 4t + 3 -- H_16's rows and columns are dealt to the fragments'
+// take the row's blocks in turn.  Lane l = 4 g + t: token g % TOK, block g / TOK of those at once; of every 16-tile the
+// gathered columns 4t .. 4t + 3 and the outputs 4t .. 4t + 3 -- H_16's rows and columns are dealt to the fragments'
 // positions that way --, so that a lane's indices are one 8-byte load and its outputs one 8-byte store, four lanes a whole
 // 32-byte sector of the row (with the fragments' own order two half sectors: 4096 rows of 8192 63 -> 49 us).  The identity
 // prefix (b_I columns, Eq. 6) is gathered and stored by the same lanes.
