@@ -104,7 +104,7 @@ struct Struct {
     Struct(const Struct&) = delete;
     ~Struct() { PyBuffer_Release(&view); }
     const T* operator->() const { return static_cast<const T*>(view.buf); }
-    operator const T*() const { return static_cast<const T*>(view.buf); }
+    const T* get() const { return static_cast<const T*>(view.buf); }
 };
 
 // A list or tuple for the length of a call.
@@ -121,13 +121,20 @@ struct Sequence {
 
 void* current_stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
-// Calls into the library with the interpreter lock released: a launch may wait for room in the driver's queue.
-template <typename F>
-PyObject* status_of(F&& call) {
+// Calls into the library with the interpreter lock released: a launch may wait for room in the driver's queue.  Nothing but
+// the call runs in there: a tensor's address may be refused with an exception (a batched or a fake tensor has none), and
+// whoever catches that needs the lock.
+template <typename F, typename... Args>
+PyObject* status_of(F* call, Args... args) {
+    struct Unlocked {
+        PyThreadState* state = PyEval_SaveThread();
+        ~Unlocked() { PyEval_RestoreThread(state); }
+    };
     lopro_status st;
-    Py_BEGIN_ALLOW_THREADS
-    st = call();
-    Py_END_ALLOW_THREADS
+    {
+        Unlocked unlocked;
+        st = call(args...);
+    }
     return PyLong_FromLong((long)st);
 }
 
@@ -158,10 +165,8 @@ PyObject* linear_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int32_t T = (int32_t)x.size(0), out = int32(a[3]);
         const void* packed = address(a[1]);
         void* s = current_stream();
-        return status_of([&] {
-            return api.linear_fwd(d, packed, (const uint16_t*)x.data_ptr(), leading(x, T, d->d_in), y.data_ptr(),
-                                  leading(y, T, d->d_out), out, T, ws.data_ptr(), (size_t)ws.numel(), s);
-        });
+        return status_of(api.linear_fwd, d.get(), packed, (const uint16_t*)x.data_ptr(), leading(x, T, d->d_in),
+                         y.data_ptr(), leading(y, T, d->d_out), out, T, ws.data_ptr(), (size_t)ws.numel(), s);
     });
 }
 
@@ -175,10 +180,8 @@ PyObject* linear_fwd_host(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int32_t T = (int32_t)x.size(0), out = int32(a[3]);
         const void* packed = address(a[1]);
         void* s = current_stream();
-        return status_of([&] {
-            return api.linear_fwd_host(d, packed, (const uint16_t*)x.data_ptr(), y.data_ptr(), out, T, ws.data_ptr(),
-                                       (size_t)ws.numel(), s);
-        });
+        return status_of(api.linear_fwd_host, d.get(), packed, (const uint16_t*)x.data_ptr(), y.data_ptr(), out, T,
+                         ws.data_ptr(), (size_t)ws.numel(), s);
     });
 }
 
@@ -191,10 +194,8 @@ PyObject* linear_fwd_noalloc(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int32_t T = (int32_t)x.size(0), out = int32(a[3]);
         const void* packed = address(a[1]);
         void* s = current_stream();
-        return status_of([&] {
-            return api.linear_fwd_noalloc(d, packed, (const uint16_t*)x.data_ptr(), leading(x, T, d->d_in), y.data_ptr(),
-                                          leading(y, T, d->d_out), out, T, s);
-        });
+        return status_of(api.linear_fwd_noalloc, d.get(), packed, (const uint16_t*)x.data_ptr(), leading(x, T, d->d_in),
+                         y.data_ptr(), leading(y, T, d->d_out), out, T, s);
     });
 }
 
@@ -221,11 +222,9 @@ PyObject* linear_fwd_group(PyObject*, PyObject* const* a, Py_ssize_t n) {
             ldy[i] = leading(y, T, d[i].d_out);
         }
         void* s = current_stream();
-        return status_of([&] {
-            return api.linear_fwd_group((int32_t)k, dp.data(), blobs.data(), (const uint16_t*)x.data_ptr(),
-                                        leading(x, T, d[0].d_in), outs.data(), ldy.data(), out, T, ws.data_ptr(),
-                                        (size_t)ws.numel(), s);
-        });
+        return status_of(api.linear_fwd_group, (int32_t)k, dp.data(), blobs.data(), (const uint16_t*)x.data_ptr(),
+                         leading(x, T, d[0].d_in), outs.data(), ldy.data(), out, T, ws.data_ptr(), (size_t)ws.numel(),
+                         s);
     });
 }
 
@@ -244,10 +243,9 @@ PyObject* linear_fwd_experts(PyObject*, PyObject* const* a, Py_ssize_t n) {
         for (Py_ssize_t i = 0; i < k; ++i) ptrs[i] = address(blobs[i]);
         for (Py_ssize_t i = 0; i <= k; ++i) offs[i] = int32(rows[i]);
         void* s = current_stream();
-        return status_of([&] {
-            return api.linear_fwd_experts(d, (int32_t)k, ptrs.data(), offs.data(), (const uint16_t*)x.data_ptr(), x.stride(0),
-                                          y.data_ptr(), y.stride(0), out, ws.data_ptr(), (size_t)ws.numel(), s);
-        });
+        return status_of(api.linear_fwd_experts, d.get(), (int32_t)k, ptrs.data(), offs.data(),
+                         (const uint16_t*)x.data_ptr(), x.stride(0), y.data_ptr(), y.stride(0), out, ws.data_ptr(),
+                         (size_t)ws.numel(), s);
     });
 }
 
@@ -260,10 +258,8 @@ PyObject* vq_linear_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int32_t T = (int32_t)x.size(0), out = int32(a[3]);
         const void* packed = address(a[1]);
         void* s = current_stream();
-        return status_of([&] {
-            return api.vq_linear_fwd(d, packed, (const uint16_t*)x.data_ptr(), leading(x, T, d->d_in), y.data_ptr(),
-                                     leading(y, T, d->d_out), out, T, ws.data_ptr(), (size_t)ws.numel(), s);
-        });
+        return status_of(api.vq_linear_fwd, d.get(), packed, (const uint16_t*)x.data_ptr(), leading(x, T, d->d_in),
+                         y.data_ptr(), leading(y, T, d->d_out), out, T, ws.data_ptr(), (size_t)ws.numel(), s);
     });
 }
 
@@ -276,10 +272,8 @@ PyObject* rotate(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int32_t T = (int32_t)x.size(0);
         const void* perm = address(a[1]);
         void* s = current_stream();
-        return status_of([&] {
-            return api.rotate(d, (const int32_t*)perm, (const uint16_t*)x.data_ptr(), leading(x, T, d->d_in),
-                              (uint16_t*)out.data_ptr(), leading(out, T, d->d_in), T, s);
-        });
+        return status_of(api.rotate, d.get(), (const int32_t*)perm, (const uint16_t*)x.data_ptr(), leading(x, T, d->d_in),
+                         (uint16_t*)out.data_ptr(), leading(out, T, d->d_in), T, s);
     });
 }
 
@@ -293,11 +287,9 @@ PyObject* block_add_rmsnorm(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const void* w = contiguous_device(a[2], 2);
         const float eps = (float)number(a[3]);
         void* s = current_stream();
-        return status_of([&] {
-            return api.add_rmsnorm((uint16_t*)h.data_ptr(), h.stride(0), y ? (const uint16_t*)y->data_ptr() : nullptr,
-                                   y ? y->stride(0) : 0, (const uint16_t*)w, eps, (uint16_t*)out.data_ptr(), out.stride(0),
-                                   (int32_t)h.size(0), (int32_t)h.size(1), s);
-        });
+        return status_of(api.add_rmsnorm, (uint16_t*)h.data_ptr(), h.stride(0),
+                         y ? (const uint16_t*)y->data_ptr() : nullptr, y ? y->stride(0) : 0, (const uint16_t*)w, eps,
+                         (uint16_t*)out.data_ptr(), out.stride(0), (int32_t)h.size(0), (int32_t)h.size(1), s);
     });
 }
 
@@ -311,12 +303,10 @@ PyObject* block_rope_append(PyObject*, PyObject* const* a, Py_ssize_t n) {
         void *kp = contiguous_device(a[4], 2), *vp = contiguous_device(a[5], 2), *status = address(a[7]);
         const float theta = (float)number(a[6]);
         void* s = current_stream();
-        return status_of([&] {
-            return api.rope_append((uint16_t*)q.data_ptr(), q.stride(0), (const uint16_t*)k.data_ptr(), k.stride(0),
-                                   (const uint16_t*)v.data_ptr(), v.stride(0), (const int32_t*)pos, (uint16_t*)kp, (uint16_t*)vp,
-                                   (int32_t)kc.size(0), (int32_t)kc.size(1), (int32_t)kc.size(3), (int32_t)kc.size(2), theta,
-                                   status, s);
-        });
+        return status_of(api.rope_append, (uint16_t*)q.data_ptr(), q.stride(0), (const uint16_t*)k.data_ptr(),
+                         k.stride(0), (const uint16_t*)v.data_ptr(), v.stride(0), (const int32_t*)pos, (uint16_t*)kp,
+                         (uint16_t*)vp, (int32_t)kc.size(0), (int32_t)kc.size(1), (int32_t)kc.size(3),
+                         (int32_t)kc.size(2), theta, status, s);
     });
 }
 
@@ -330,12 +320,10 @@ PyObject* block_attention_decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
         void* status = address(a[6]);
         const float scale = (float)number(a[4]);
         void* s = current_stream();
-        return status_of([&] {
-            return api.attention_decode((const uint16_t*)q.data_ptr(), q.stride(0), (const uint16_t*)kp, (const uint16_t*)vp,
-                                        (const int32_t*)ctx, (uint16_t*)out.data_ptr(), out.stride(0), (int32_t)kc.size(0),
-                                        (int32_t)kc.size(1), (int32_t)kc.size(3), (int32_t)kc.size(2), scale, ws.data_ptr(),
-                                        (size_t)ws.numel(), status, s);
-        });
+        return status_of(api.attention_decode, (const uint16_t*)q.data_ptr(), q.stride(0), (const uint16_t*)kp,
+                         (const uint16_t*)vp, (const int32_t*)ctx, (uint16_t*)out.data_ptr(), out.stride(0),
+                         (int32_t)kc.size(0), (int32_t)kc.size(1), (int32_t)kc.size(3), (int32_t)kc.size(2), scale,
+                         ws.data_ptr(), (size_t)ws.numel(), status, s);
     });
 }
 
@@ -346,10 +334,9 @@ PyObject* block_silu_mul(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const at::Tensor &g = tensor(a[0]), &u = tensor(a[1]), &out = tensor(a[2]);
         require(g.dim() == 2, "gate: two dimensions");
         void* s = current_stream();
-        return status_of([&] {
-            return api.silu_mul((const uint16_t*)g.data_ptr(), g.stride(0), (const uint16_t*)u.data_ptr(), u.stride(0),
-                                (uint16_t*)out.data_ptr(), out.stride(0), (int32_t)g.size(0), (int32_t)g.size(1), s);
-        });
+        return status_of(api.silu_mul, (const uint16_t*)g.data_ptr(), g.stride(0), (const uint16_t*)u.data_ptr(),
+                         u.stride(0), (uint16_t*)out.data_ptr(), out.stride(0), (int32_t)g.size(0),
+                         (int32_t)g.size(1), s);
     });
 }
 
