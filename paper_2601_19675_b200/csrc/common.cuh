@@ -62,6 +62,18 @@ inline cudaError_t ensure_dynamic_smem(Kernel kernel, int bytes, unsigned long l
     return e;
 }
 
+// Asks, once per device, for a split of the multiprocessor's memory between L1 and shared memory (percent of shared memory)
+// when `kernel` runs.  A hint: an error is not one of the launch.
+template <typename Kernel>
+inline void prefer_shared_memory(Kernel kernel, int percent, unsigned long long* done) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (__atomic_load_n(done, __ATOMIC_ACQUIRE) & bit) return;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, percent) != cudaSuccess) (void)cudaGetLastError();
+    __atomic_fetch_or(done, bit, __ATOMIC_RELEASE);
+}
+
 // Tuning switches (lopro_configure; initial values from the environment, read once per process).
 int option(int id);
 // Multiprocessors of the current device (cached per device; 148 if the query fails).
