@@ -2,6 +2,7 @@
 // waits, warp-level tensor-core instructions, and the expansion of packed codes into bf16 operands.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <stdint.h>
 
 namespace lopro {
@@ -154,6 +155,111 @@ __device__ __forceinline__ void expand_codes(uint32_t (&a)[16], const uint32_t (
 #pragma unroll
         for (int pi = 0; pi < 15; ++pi) a[pi] = and_or(w[pi / 5] >> (3 * (pi % 5)), mask, magic);
         a[15] = ((w[0] >> 15) & 0x00010001u) | ((w[1] >> 14) & 0x00020002u) | ((w[2] >> 13) & 0x00040004u) | kMagic128;
+    }
+}
+
+// The same with fewer shifts for the kernels that scale rows afterwards: the odd pairs, which are the rows gq + 8 of a tile,
+// come out as 128 + kOdd c, their bits left where a shift that an even pair needs anyway puts them (2 bits: 6 shifts instead of
+// 14 per tile step, 3 bits: 10 instead of 15).  kOdd is a power of two and goes into the rows' scale exactly.  The loops these
+serve are bound by instruction issue with the integer pipe next; with the packed multiply-adds below 8192 -> 28672 at 2 bits,
+16 tokens 51.4 -> 48.4 us, eight experts 4096 -> 14336 at 2 bits 69.9 -> 65.8, 11008 -> 4096 at 3 bits, 5 tokens 14.5 -> 13.8.
+template <int BITS>
+struct OddRows {
+    static constexpr float factor = BITS == 4 ? 1.0f : (BITS == 2 ? 4.0f : 8.0f);
+};
+template <int BITS>
+__device__ __forceinline__ void expand_codes_by_rows(uint32_t (&a)[16], const uint32_t (&w)[BITS]) {
+    const uint32_t magic = kMagic128;
+    if constexpr (BITS == 4) {
+        expand_codes<4>(a, w);
+    } else if constexpr (BITS == 2) {
+        // word h holds pairs 8h .. 8h + 7 at bits 2p: two pairs per shift by 4
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t v = w[h] >> (4 * k);
+                a[8 * h + 2 * k] = and_or(v, 0x00030003u, magic);
+                a[8 * h + 2 * k + 1] = and_or(v, 0x000C000Cu, magic);
+            }
+    } else {
+        // words 0 and 2: even pairs at bits 0, 6, 12, odd ones at 3, 9; word 1: odd pairs at 0, 6, 12, even ones at 3, 9
+        const uint32_t even = 0x00070007u, odd = 0x00380038u;
+#pragma unroll
+        for (int h = 0; h < 3; h += 2) {
+            const uint32_t v = w[h] >> 6;
+            a[5 * h] = and_or(w[h], even, magic);
+            a[5 * h + 1] = and_or(w[h], odd, magic);
+            a[5 * h + 2] = and_or(v, even, magic);
+            a[5 * h + 3] = and_or(v, odd, magic);
+            a[5 * h + 4] = and_or(w[h] >> 12, even, magic);
+        }
+        const uint32_t v3 = w[1] >> 3, v9 = w[1] >> 9;
+        a[5] = and_or(w[1] << 3, odd, magic);
+        a[6] = and_or(v3, even, magic);
+        a[7] = and_or(v3, odd, magic);
+        a[8] = and_or(v9, even, magic);
+        a[9] = and_or(v9, odd, magic);
+        // pair 15: bit b at bit 15 (and 31) of word b, wanted at bit 3 + b
+        a[15] = and_or(w[2] >> 10, 0x00200020u, and_or(w[1] >> 11, 0x00100010u, and_or(w[0] >> 12, 0x00080008u, magic)));
+    }
+}
+
+// Two fp32 multiply-adds in one issue slot; the halves of a register pair are two tokens of a row.
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+    unsigned long long v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ void unpack2(unsigned long long v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// Scale and zero-point of a group for the rows gq (.x) and gq + 8 (.y) of a tile, as the sums of a tile step meet them:
+// y += s (acc - (128 + z) sum x~), with acc = sum (128 + kOdd c) x~ for the odd rows, whose y carries the factor kOdd.
+template <int BITS>
+struct RowScales {
+    float s[2], z[2];
+    __device__ __forceinline__ RowScales(uint32_t sz_lo, uint32_t sz_hi) {
+        const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&sz_lo));
+        const float2 hi = __half22float2(*reinterpret_cast<const __half2*>(&sz_hi));
+        s[0] = lo.x;
+        s[1] = hi.x;
+        z[0] = -128.0f - lo.y;
+        z[1] = fmaf(hi.y, -OddRows<BITS>::factor, -128.0f);
+    }
+};
+// Adds the products of one step to the sums of a tile: acc and y in the accumulator layout of m16n8k16 (rows gq, gq + 8,
+// tokens 2 tg and 2 tg + 1 of NT token tiles), sx the step's column sums of those tokens.
+template <int BITS, int NT>
+__device__ __forceinline__ void add_scaled(float (&y)[NT][4], const float (&acc)[NT][4], const float (&sx)[NT][2], const RowScales<BITS>& r) {
+    if constexpr (NT == 1) {   // (packed operands would cost the registers' copies that they save)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) y[0][i] = fmaf(r.s[i >> 1], fmaf(r.z[i >> 1], sx[0][i & 1], acc[0][i]), y[0][i]);
+    } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const unsigned long long s2 = pack2(r.s[h], r.s[h]), z2 = pack2(r.z[h], r.z[h]);
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                const unsigned long long t = fma2(z2, pack2(sx[nt][0], sx[nt][1]), pack2(acc[nt][2 * h], acc[nt][2 * h + 1]));
+                unpack2(fma2(s2, t, pack2(y[nt][2 * h], y[nt][2 * h + 1])), y[nt][2 * h], y[nt][2 * h + 1]);
+            }
+        }
+    }
+}
+// The factor of the odd rows put on (the low-rank term that starts the sums) or taken off again.
+template <int NT>
+__device__ __forceinline__ void scale_odd_rows(float (&y)[NT][4], float f) {
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+        y[nt][2] *= f;
+        y[nt][3] *= f;
     }
 }
 

@@ -174,6 +174,7 @@ stream_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
                 mma_f16(acc[nt], a, *reinterpret_cast<const uint32_t*>(trow), *reinterpret_cast<const uint32_t*>(trow + 8));
             }
         }
+        scale_odd_rows(acc, OddRows<BITS>::factor);
     };
     if (warp == kConsumerWarps) {
         // ---------------- producer warp ----------------
@@ -277,23 +278,16 @@ stream_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
                             for (int q = 0; q < BITS; ++q) w[q] = wp[q];
                         }
                         uint32_t a[16];
-                        expand_codes<BITS>(a, w);
-                        const uint32_t sz_lo = szp[r * sz_tile], sz_hi = szp[r * sz_tile + 8];
-                        const float2 f_lo = __half22float2(*reinterpret_cast<const __half2*>(&sz_lo));
-                        const float2 f_hi = __half22float2(*reinterpret_cast<const __half2*>(&sz_hi));
-                        const float nsz_lo = -f_lo.x * (128.0f + f_lo.y), nsz_hi = -f_hi.x * (128.0f + f_hi.y);
+                        expand_codes_by_rows<BITS>(a, w);
+                        float acc[NT][4];
 #pragma unroll
                         for (int nt = 0; nt < NT; ++nt) {
-                            float acc[4];
-                            mma_bf16_first(acc, &a[0], b[nt][0], b[nt][1]);
-                            mma_bf16(acc, &a[4], b[nt][2], b[nt][3]);
-                            mma_bf16(acc, &a[8], b[nt][4], b[nt][5]);
-                            mma_bf16(acc, &a[12], b[nt][6], b[nt][7]);
-                            yacc[r][nt][0] = fmaf(f_lo.x, acc[0], fmaf(nsz_lo, sx[nt][0], yacc[r][nt][0]));
-                            yacc[r][nt][1] = fmaf(f_lo.x, acc[1], fmaf(nsz_lo, sx[nt][1], yacc[r][nt][1]));
-                            yacc[r][nt][2] = fmaf(f_hi.x, acc[2], fmaf(nsz_hi, sx[nt][0], yacc[r][nt][2]));
-                            yacc[r][nt][3] = fmaf(f_hi.x, acc[3], fmaf(nsz_hi, sx[nt][1], yacc[r][nt][3]));
+                            mma_bf16_first(acc[nt], &a[0], b[nt][0], b[nt][1]);
+                            mma_bf16(acc[nt], &a[4], b[nt][2], b[nt][3]);
+                            mma_bf16(acc[nt], &a[8], b[nt][4], b[nt][5]);
+                            mma_bf16(acc[nt], &a[12], b[nt][6], b[nt][7]);
                         }
+                        add_scaled<BITS, NT>(yacc[r], acc, sx, RowScales<BITS>(szp[r * sz_tile], szp[r * sz_tile + 8]));
                     }
                 }
             }
@@ -320,6 +314,8 @@ stream_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
     constexpr int kRows = RT * 16, kRowsP = kRows + kRedPad;
     float* red = reinterpret_cast<float*>(smem + p.off_ring);
     if (warp < kConsumerWarps) {
+#pragma unroll
+        for (int r = 0; r < RT; ++r) scale_odd_rows(yacc[r], 1.0f / OddRows<BITS>::factor);
 #pragma unroll
         for (int r = 0; r < RT; ++r)
 #pragma unroll
@@ -441,7 +437,7 @@ stream_wide_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
     const uint32_t* szs = reinterpret_cast<const uint32_t*>(smem + p.off_sz) + r * p.ng * 16 + gq;
     bool timed_out = false;
 
-    float yacc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    float yacc[1][4] = {{0.0f, 0.0f, 0.0f, 0.0f}};
     if (!mbar_wait(cbar, 0)) timed_out = true;
     if (p.r_pad > 0 && step == 0) {
         // low-rank term A t of row tile r starts the sums of its step-0 warp
@@ -453,8 +449,9 @@ stream_wide_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
                 uint32_t a[4];
                 load_up_fragment(a, as, p.r_pad, gq, tg, jj, p.lr8 != 0);
                 const __half* trow = ts + gq * p.r_pad + jj + 2 * tg;
-                mma_f16(yacc, a, *reinterpret_cast<const uint32_t*>(trow), *reinterpret_cast<const uint32_t*>(trow + 8));
+                mma_f16(yacc[0], a, *reinterpret_cast<const uint32_t*>(trow), *reinterpret_cast<const uint32_t*>(trow + 8));
             }
+            scale_odd_rows(yacc, OddRows<BITS>::factor);
         }
     }
 #pragma unroll
@@ -479,21 +476,15 @@ stream_wide_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
             for (int q = 0; q < BITS; ++q) w[q] = wp[q];
         }
         uint32_t a[16];
-        expand_codes<BITS>(a, w);
+        expand_codes_by_rows<BITS>(a, w);
         const uint32_t* szp = szs + ((s * kStageSteps + step) >> p.gshift) * 16;  // the step's group
-        const uint32_t sz_lo = szp[0], sz_hi = szp[8];
-        const float2 f_lo = __half22float2(*reinterpret_cast<const __half2*>(&sz_lo));
-        const float2 f_hi = __half22float2(*reinterpret_cast<const __half2*>(&sz_hi));
-        const float nsz_lo = -f_lo.x * (128.0f + f_lo.y), nsz_hi = -f_hi.x * (128.0f + f_hi.y);
-        float acc[4];
-        mma_bf16_first(acc, &a[0], b[0], b[1]);
-        mma_bf16(acc, &a[4], b[2], b[3]);
-        mma_bf16(acc, &a[8], b[4], b[5]);
-        mma_bf16(acc, &a[12], b[6], b[7]);
-        yacc[0] = fmaf(f_lo.x, acc[0], fmaf(nsz_lo, sx0, yacc[0]));
-        yacc[1] = fmaf(f_lo.x, acc[1], fmaf(nsz_lo, sx1, yacc[1]));
-        yacc[2] = fmaf(f_hi.x, acc[2], fmaf(nsz_hi, sx0, yacc[2]));
-        yacc[3] = fmaf(f_hi.x, acc[3], fmaf(nsz_hi, sx1, yacc[3]));
+        float acc[1][4];
+        mma_bf16_first(acc[0], &a[0], b[0], b[1]);
+        mma_bf16(acc[0], &a[4], b[2], b[3]);
+        mma_bf16(acc[0], &a[8], b[4], b[5]);
+        mma_bf16(acc[0], &a[12], b[6], b[7]);
+        const float sx[1][2] = {{sx0, sx1}};
+        add_scaled<BITS, 1>(yacc, acc, sx, RowScales<BITS>(szp[0], szp[8]));
     }
     if (timed_out && lane == 0) atomicExch(p.status, (int)LOPRO_ERR_TIMEOUT);
     // Every stage has a step-0 warp that waited for it, so after this barrier every copy has landed and the ring
@@ -502,10 +493,11 @@ stream_wide_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
 
     static_assert(kStageSteps * kRedStep * 4 <= kStageBytes, "the partial sums fit one stage of the ring");
     float* red = reinterpret_cast<float*>(smem + p.off_ring);
+    scale_odd_rows(yacc, 1.0f / OddRows<BITS>::factor);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int tk = 2 * tg + (i & 1), rl = r * 16 + gq + 8 * (i >> 1);
-        red[step * kRedStep + tk * kRedTok + rl] = yacc[i];
+        red[step * kRedStep + tk * kRedTok + rl] = yacc[0][i];
     }
     __syncthreads();
     // four threads per output: each adds four of the 16 partial sums, two shuffles finish

@@ -143,23 +143,16 @@ __device__ __forceinline__ void tile_step(const uint32_t* wp, uint32_t xaddr, co
         for (int q = 0; q < BITS; ++q) w[q] = wp[q];
     }
     uint32_t a[16];
-    expand_codes<BITS>(a, w);
-    const uint32_t sz_lo = szp[0], sz_hi = szp[8];
-    const float2 f_lo = __half22float2(*reinterpret_cast<const __half2*>(&sz_lo));
-    const float2 f_hi = __half22float2(*reinterpret_cast<const __half2*>(&sz_hi));
-    const float nsz_lo = -f_lo.x * (128.0f + f_lo.y), nsz_hi = -f_hi.x * (128.0f + f_hi.y);
+    expand_codes_by_rows<BITS>(a, w);
+    float acc[NT][4];
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
-        float acc[4];
-        mma_bf16_first(acc, &a[0], b[nt][0], b[nt][1]);
-        mma_bf16(acc, &a[4], b[nt][2], b[nt][3]);
-        mma_bf16(acc, &a[8], b[nt][4], b[nt][5]);
-        mma_bf16(acc, &a[12], b[nt][6], b[nt][7]);
-        yacc[nt][0] = fmaf(f_lo.x, acc[0], fmaf(nsz_lo, sx[nt][0], yacc[nt][0]));
-        yacc[nt][1] = fmaf(f_lo.x, acc[1], fmaf(nsz_lo, sx[nt][1], yacc[nt][1]));
-        yacc[nt][2] = fmaf(f_hi.x, acc[2], fmaf(nsz_hi, sx[nt][0], yacc[nt][2]));
-        yacc[nt][3] = fmaf(f_hi.x, acc[3], fmaf(nsz_hi, sx[nt][1], yacc[nt][3]));
+        mma_bf16_first(acc[nt], &a[0], b[nt][0], b[nt][1]);
+        mma_bf16(acc[nt], &a[4], b[nt][2], b[nt][3]);
+        mma_bf16(acc[nt], &a[8], b[nt][4], b[nt][5]);
+        mma_bf16(acc[nt], &a[12], b[nt][6], b[nt][7]);
     }
+    add_scaled<BITS, NT>(yacc, acc, sx, RowScales<BITS>(szp[0], szp[8]));
 }
 
 // Byte offsets, from the start of a stage, of what a warp reads in its first step (step kq of tile slot r); they
@@ -170,8 +163,8 @@ struct WarpOffsets {
 
 // The steps kq, kq + KQ, ... of one stage for tile slot r (KQ = 16 >> RBITS phases), unrolled with constant
 // strides; gs = min(gshift, 4): a stage starts on a group boundary or lies inside one group, so the group of
-// step st within the stage's (scale, zero) block is st >> gs.
-template <int BITS, int NT, int RBITS>
+// step st within the stage's (scale, zero) block is st >> gs.  WHOLE: a stage of sixteen steps (no test in front of each).
+template <int BITS, int NT, int RBITS, bool WHOLE>
 __device__ __forceinline__ void consume_stage(const unsigned char* stage, uint32_t stage_u32, const WarpOffsets& o, int kq,
                                               int gs, int steps, float (&yacc)[NT][4]) {
     constexpr int KQ = kConsumerWarps >> RBITS, PER = kStageSteps / KQ;
@@ -182,7 +175,7 @@ __device__ __forceinline__ void consume_stage(const unsigned char* stage, uint32
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
         const int st = kq + i * KQ;
-        if (st < steps)
+        if (WHOLE || st < steps)
             tile_step<BITS, NT>(reinterpret_cast<const uint32_t*>(wbase + i * KQ * kStepBytes),
                                 stage_u32 + o.x + (uint32_t)(i * KQ * 128), sxbase + i * KQ, szbase + (st >> gs) * 16,
                                 yacc);
@@ -344,6 +337,7 @@ tall_kernel(const TallParams p_in, const __grid_constant__ SIBS sibs) {
                                 *reinterpret_cast<const uint32_t*>(trow + 8));
                     }
                 }
+                scale_odd_rows(yacc, OddRows<BITS>::factor);
             }
         }
 
@@ -360,9 +354,12 @@ tall_kernel(const TallParams p_in, const __grid_constant__ SIBS sibs) {
             }
             if (active) {
                 const int steps = steps_of(s);
-                if (rbits == 2) consume_stage<BITS, NT, 2>(stage, stage_u32, wo, kq, gs, steps, yacc);
-                else if (rbits == 1) consume_stage<BITS, NT, 1>(stage, stage_u32, wo, kq, gs, steps, yacc);
-                else consume_stage<BITS, NT, 0>(stage, stage_u32, wo, kq, gs, steps, yacc);
+                const bool whole = steps == kStageSteps;
+                if (rbits == 2 && whole) consume_stage<BITS, NT, 2, true>(stage, stage_u32, wo, kq, gs, steps, yacc);
+                else if (rbits == 2) consume_stage<BITS, NT, 2, false>(stage, stage_u32, wo, kq, gs, steps, yacc);
+                else if (rbits == 1 && whole) consume_stage<BITS, NT, 1, true>(stage, stage_u32, wo, kq, gs, steps, yacc);
+                else if (rbits == 1) consume_stage<BITS, NT, 1, false>(stage, stage_u32, wo, kq, gs, steps, yacc);
+                else consume_stage<BITS, NT, 0, false>(stage, stage_u32, wo, kq, gs, steps, yacc);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(empty(slot));
@@ -399,6 +396,7 @@ tall_kernel(const TallParams p_in, const __grid_constant__ SIBS sibs) {
             }
             if (KQ > 1) named_arrive(2);
             if (active) {
+                scale_odd_rows(yacc, 1.0f / OddRows<BITS>::factor);
 #pragma unroll
                 for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
