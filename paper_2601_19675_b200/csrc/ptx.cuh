@@ -161,8 +161,8 @@ __device__ __forceinline__ void expand_codes(uint32_t (&a)[16], const uint32_t (
 // The same with fewer shifts for the kernels that scale rows afterwards: the odd pairs, which are the rows gq + 8 of a tile,
 // come out as 128 + kOdd c, their bits left where a shift that an even pair needs anyway puts them (2 bits: 6 shifts instead of
 // 14 per tile step, 3 bits: 10 instead of 15).  kOdd is a power of two and goes into the rows' scale exactly.  The loops these
-serve are bound by instruction issue with the integer pipe next; with the packed multiply-adds below 8192 -> 28672 at 2 bits,
-16 tokens 51.4 -> 48.4 us, eight experts 4096 -> 14336 at 2 bits 69.9 -> 65.8, 11008 -> 4096 at 3 bits, 5 tokens 14.5 -> 13.8.
+// serve are bound by instruction issue with the integer pipe next; with the packed multiply-adds below 8192 -> 28672 at 2 bits,
+// 16 tokens 51.4 -> 48.4 us, eight experts 4096 -> 14336 at 2 bits 69.9 -> 65.8, 11008 -> 4096 at 3 bits, 5 tokens 14.5 -> 13.8.
 template <int BITS>
 struct OddRows {
     static constexpr float factor = BITS == 4 ? 1.0f : (BITS == 2 ? 4.0f : 8.0f);
