@@ -2,8 +2,8 @@
 // by bulk asynchronous copies (steps "Dequant(W_q) X" and "U (Sigma Y)" of Appendix A.3, summed as
 // in Eq. 8).
 //
-// One CTA owns 32 or 64 output rows (two or four 16-row tiles of the fragment layout) over the WHOLE K range, so
-// no partial sums ever cross CTAs.  A producer warp fills a ring of shared-memory stages with
+// One CTA owns 32 or 64 output rows (two or four 16-row tiles of the fragment layout; up to eight in runs, see plan_run)
+// over the WHOLE K range, so no partial sums ever cross CTAs.  A producer warp fills a ring of shared-memory stages with
 // cp.async.bulk copies (16 steps of 64 columns per stage): the layer's own data -- codes,
 // (scale, zero) pairs, the rows of A -- is requested before griddepcontrol.wait, i.e. while the
 // prologue kernel of the same forward still runs; the rotated activations and their 64-column
@@ -48,6 +48,7 @@ struct StreamParams {
     int n_stages;  // ring depth
     int total_stages;
     int lr8;       // the up-projection factor is fp8 e4m3 (U of the FP8 low-rank record), one byte per entry
+    int run_ctas;  // not 0: the layer's row tiles are shared out evenly over so many CTAs (else RT tiles each)
     // shared-memory layout (bytes from the dynamic base)
     int off_sz, off_a, off_t, off_ring, stage_bytes, off_stage_x;
 };
@@ -107,8 +108,14 @@ stream_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int gq = lane >> 2, tg = lane & 3;
-    const int rt0 = bx * RT;                             // first 16-row tile of this CTA
-    const int n_rt = min(RT, (p.m >> 4) - rt0);          // live row tiles
+    // this CTA's first 16-row tile and its live row tiles (runs differ by at most one tile)
+    const int tiles = p.m >> 4;
+    int rt0 = bx * RT, n_rt = min(RT, tiles - rt0);
+    if (RT > 2 && p.run_ctas != 0) {
+        const int base = tiles / p.run_ctas, extra = tiles - base * p.run_ctas;
+        rt0 = bx * base + min(bx, extra);
+        n_rt = base + (bx < extra ? 1 : 0);
+    }
     const int tc = min(kTok, p.T);                                  // live tokens
     const uint32_t bar0 = smem_u32(bars);
     auto wfull = [&](int s) { return bar0 + 8u * (uint32_t)s; };
@@ -567,6 +574,10 @@ cudaError_t launch_stream_k(const StreamParams& p, const StreamSiblings& sibs, i
 template <int BITS>
 cudaError_t launch_stream_bits(const StreamParams& p, const StreamSiblings& sibs, int grid, int nt, int rt, int smem_bytes,
                                cudaStream_t s) {
+    if (nt == 1 && rt == 5) return launch_stream_k<BITS, 1, 5>(p, sibs, grid, smem_bytes, s);
+    if (nt == 1 && rt == 6) return launch_stream_k<BITS, 1, 6>(p, sibs, grid, smem_bytes, s);
+    if (nt == 1 && rt == 8) return launch_stream_k<BITS, 1, 8>(p, sibs, grid, smem_bytes, s);
+    if (nt == 2 && rt == 5) return launch_stream_k<BITS, 2, 5>(p, sibs, grid, smem_bytes, s);
     if (nt == 1)
         return rt == 4 ? launch_stream_k<BITS, 1, 4>(p, sibs, grid, smem_bytes, s) : launch_stream_k<BITS, 1, 2>(p, sibs, grid, smem_bytes, s);
     if (nt == 2)
@@ -623,7 +634,35 @@ bool plan_layout(const lopro_desc& d, StreamPlan* pl, int r_pad, int ng, int kto
     return pl->smem_bytes <= kStreamMaxSmem;
 }
 
+// A taller layer in runs: every CTA of one even wave takes up to six row tiles (five with 16 tokens) over all of K, so that a
+// warp multiplies the step it has fetched with all of them and hands its sums over once; the persistent kernel gives a warp one
+// tile, reads the activations again and hands over per group of four.  Bound by the expansion (integer pipe) at about 80 cycles
+// per tile step and scheduler.  Persistent kernel against runs: 4096 -> 11008, 4 bits, 1 and 8 tokens 12.2 and 13.1 us against
+// 11.2 and 12.0; 5120 -> 5120 at 4 tokens 9.6 and 8.6; 2 bits at 12 tokens 13.6 and 12.2.  A second wave pays a start-up of
+// its own (4096 -> 22016 18.9 and 19.3), so only where K has eight stages or more, and with 8 tokens at most: 8192 -> 28672,
+// 2 bits, 4 tokens 37.9 and 34.0, 16 tokens 41.7 and 46.1.  Layers that share a launch stay with the persistent kernel: three
+// layers 4096 -> 4096 alone gained (13.8 and 12.2), the decoder layer of one sequence around them lost (85.1 and 89.4).
+bool plan_run(const lopro_desc& d, int T, StreamPlan* pl, int* ctas) {
+    if (T < 1 || T > 16) return false;
+    pl->nt = T <= 8 ? 1 : 2;
+    const int r_pad = d.rank > 0 ? round_up_int(d.rank, 16) : 0, ng = d.d_in / d.group_size, tiles = d.d_out / 16;
+    for (int waves = 1; waves <= (pl->nt == 1 && d.d_in >= 8192 ? 2 : 1); ++waves) {
+        *ctas = sm_count() * waves;
+        const int most = (tiles + *ctas - 1) / *ctas;   // the longest run
+        if (most > (pl->nt == 2 ? 5 : (waves == 2 ? 8 : 6))) continue;
+        pl->rt = most <= 4 ? 4 : (most <= 6 ? most : 8);
+        if (plan_layout(d, pl, r_pad, ng, pl->nt * 8)) return true;
+    }
+    return false;
+}
+
 }  // namespace
+
+bool run_supported(const lopro_desc& d, int T) {
+    StreamPlan pl;
+    int ctas;
+    return plan_run(d, T, &pl, &ctas);
+}
 
 // The 32-warp variant runs for up to 8 tokens when all of K fits the ring; LOPRO_OPT_NO_WIDE keeps it off (A/B
 // comparison and tests).
@@ -645,9 +684,10 @@ bool stream_supported(const lopro_desc& d, int T) {
 
 cudaError_t launch_stream(const lopro_desc& d, const uint8_t* blob, const BlobLayout& L, const uint8_t* ws,
                           const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s, int t0,
-                          const StreamSiblingArgs* more) {
+                          const StreamSiblingArgs* more, bool in_runs) {
     StreamPlan pl;
-    if (!plan_stream(d, T, &pl)) return cudaErrorInvalidValue;
+    int run_ctas = 0;
+    if (!(in_runs ? plan_run(d, T, &pl, &run_ctas) : plan_stream(d, T, &pl))) return cudaErrorInvalidValue;
     StreamParams p;
     p.codes = reinterpret_cast<const uint32_t*>(blob + L.off[LOPRO_SEC_CODES]);
     p.sz = reinterpret_cast<const uint32_t*>(blob + L.off[LOPRO_SEC_SCALEZERO]);
@@ -678,9 +718,10 @@ cudaError_t launch_stream(const lopro_desc& d, const uint8_t* blob, const BlobLa
     p.off_ring = pl.off_ring;
     p.stage_bytes = pl.stage_bytes;
     p.off_stage_x = pl.off_stage_x;
-    const bool wide = wide_variant(d, pl);
+    const bool wide = !in_runs && wide_variant(d, pl);
     const int rows_per_cta = wide ? 32 : pl.rt * 16;
-    int grid = (d.d_out + rows_per_cta - 1) / rows_per_cta;
+    int grid = in_runs ? run_ctas : (d.d_out + rows_per_cta - 1) / rows_per_cta;
+    p.run_ctas = run_ctas;
     // sibling layers: the CTAs of each follow those of the one before
     StreamSiblings sibs = {};
     if (more != nullptr) {

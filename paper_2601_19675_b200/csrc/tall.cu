@@ -3,6 +3,9 @@
 // "U (Sigma Y)" of Appendix A.3, summed as in Eq. 8), after the prologue kernel that writes the
 // rotated activations x~ (as the stage image), their 64-column sums and t = B x.
 //
+// A single layer of up to 16 tokens whose tiles make one even wave of short runs goes through the kernel of stream.cu instead
+// (plan_run there): longer runs, more tokens and layers that share a launch run here.
+//
 // Persistent: one CTA per SM, each owning a contiguous run of 16-row tiles (the runs differ by at
 // most one tile) and walking it in groups of up to four tiles (two with 32 tokens).  A producer warp keeps one ring of
 // shared-memory stages full ACROSS the groups (16 steps of 64 columns per stage: the packed codes
@@ -499,6 +502,7 @@ cudaError_t launch_tall(const lopro_desc& d, const uint8_t* blob, const BlobLayo
     long long total_rows = d.d_out;
     if (more != nullptr)
         for (int i = 0; i < more->n; ++i) total_rows += more->d_out[i];
+    if ((more == nullptr || more->n == 0) && run_supported(d, T)) return launch_stream(d, blob, L, ws, W, y, ldy, out_dtype, T, s, t0, more, true);
     if (!plan_tall(d, T, &pl, total_rows)) return cudaErrorInvalidValue;
     TallParams p;
     p.codes = blob + L.off[LOPRO_SEC_CODES];
