@@ -43,12 +43,11 @@ struct StreamParams {
     void* y;
     int64_t ldy;
     int out_f32;
-    int m, n, T, t_pad;
+    int m, run_ctas, T, t_pad;  // run_ctas not 0: the layer's row tiles are shared out evenly over so many CTAs (else RT tiles each)
     int nsteps, gshift, ng, r_pad;
     int n_stages;  // ring depth
     int total_stages;
     int lr8;       // the up-projection factor is fp8 e4m3 (U of the FP8 low-rank record), one byte per entry
-    int run_ctas;  // not 0: the layer's row tiles are shared out evenly over so many CTAs (else RT tiles each)
     // shared-memory layout (bytes from the dynamic base)
     int off_sz, off_a, off_t, off_ring, stage_bytes, off_stage_x;
 };
@@ -485,13 +484,13 @@ stream_wide_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
         uint32_t a[16];
         expand_codes_by_rows<BITS>(a, w);
         const uint32_t* szp = szs + ((s * kStageSteps + step) >> p.gshift) * 16;  // the step's group
-        float acc[1][4];
-        mma_bf16_first(acc[0], &a[0], b[0], b[1]);
-        mma_bf16(acc[0], &a[4], b[2], b[3]);
-        mma_bf16(acc[0], &a[8], b[4], b[5]);
-        mma_bf16(acc[0], &a[12], b[6], b[7]);
-        const float sx[1][2] = {{sx0, sx1}};
-        add_scaled<BITS, 1>(yacc, acc, sx, RowScales<BITS>(szp[0], szp[8]));
+        const RowScales<BITS> scales(szp[0], szp[8]);
+        float acc[4];
+        mma_bf16_first(acc, &a[0], b[0], b[1]);
+        mma_bf16(acc, &a[4], b[2], b[3]);
+        mma_bf16(acc, &a[8], b[4], b[5]);
+        mma_bf16(acc, &a[12], b[6], b[7]);
+        add_scaled_early<BITS>(yacc[0], acc, sx0, sx1, scales);
     }
     if (timed_out && lane == 0) atomicExch(p.status, (int)LOPRO_ERR_TIMEOUT);
     // Every stage has a step-0 warp that waited for it, so after this barrier every copy has landed and the ring
@@ -700,7 +699,6 @@ cudaError_t launch_stream(const lopro_desc& d, const uint8_t* blob, const BlobLa
     p.ldy = ldy;
     p.out_f32 = out_dtype == LOPRO_OUT_F32;
     p.m = d.d_out;
-    p.n = d.d_in;
     p.T = T;
     p.t_pad = W.t_pad;
     p.nsteps = d.d_in / 64;
