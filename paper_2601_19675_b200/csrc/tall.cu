@@ -564,8 +564,8 @@ cudaError_t launch_tall(const lopro_desc& d, const uint8_t* blob, const BlobLayo
             sibs.m[i] = more->d_out[i];
             sibs.T[i] = more->own_rows ? more->T_of[i + 1] : T;
         }
-        if (more->own_rows) p.T = more->T_of[0];
     }
+    if (more != nullptr && more->own_rows) p.T = more->T_of[0];  // also where this expert is the only one of its launch
     switch (d.bits) {
         case 2: return launch_tall_bits<2>(p, sibs, pl.nt, pl.grid, pl.smem_bytes, s);
         case 3: return launch_tall_bits<3>(p, sibs, pl.nt, pl.grid, pl.smem_bytes, s);

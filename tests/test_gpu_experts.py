@@ -79,6 +79,30 @@ def test_experts_through_the_persistent_kernel():
     _check_experts(d, layers, blobs, [8, 0, 3, 20, 1], seed=9, shared=True, bit_equal=False)
 
 
+@pytest.mark.parametrize("per_sm,extra,counts", [(7, 3, [8] * 8 + [3]),           # persistent kernel, up to 8 rows
+                                                 (2, 5, [20] + [1] * 7 + [2]),    # and more than 16
+                                                 (2, 5, [8] * 8 + [1])])          # the last layer alone: in runs of row tiles
+def test_an_expert_alone_in_the_last_launch_writes_its_own_rows_only(per_sm, extra, counts):
+    # eight experts share a pair of launches, the ninth has one of its own, shaped for the largest row count: its rows end
+    # where y ends, and the rows behind keep their pattern
+    n, m = 512, 16 * (torch.cuda.get_device_properties(0).multi_processor_count * per_sm + extra)
+    d, _, blobs = _experts(n, m, 4, 128, 128, 16, 1, seed=per_sm)
+    blobs = blobs * len(counts)                                   # what an expert's weights are does not matter here
+    offs = np.concatenate([[0], np.cumsum(counts)]).tolist()
+    total, spare = offs[-1], max(counts)
+    x = bf16_bits_to_device(synth.activations(total, n, seed=total))
+    assert lopro.linear_fwd_path(d, max(counts))[0] == lopro.PATH_TALL
+    buf = torch.full((total + spare, m), 7.0, dtype=torch.float32, device="cuda")
+    y = lopro.linear_fwd_experts(d, blobs, offs, x, lopro.OUT_F32, y=buf[:total])
+    torch.cuda.synchronize()
+    assert torch.all(buf[total:] == 7.0)
+    for e in (0, len(counts) - 1):
+        rows = slice(offs[e], offs[e + 1])
+        alone = lopro.linear_fwd(d, blobs[e], x[rows], lopro.OUT_F32)
+        # the same products in fp32 in another order
+        assert (alone - y[rows]).abs().max().item() <= 2e-5 * alone.abs().max().item()
+
+
 def test_experts_with_many_rows_run_one_after_the_other():
     n, m, r = 1024, 256, 16
     d, layers, blobs = _experts(n, m, 4, 128, 128, r, 3, seed=4)
