@@ -502,7 +502,9 @@ cudaError_t launch_tall(const lopro_desc& d, const uint8_t* blob, const BlobLayo
     long long total_rows = d.d_out;
     if (more != nullptr)
         for (int i = 0; i < more->n; ++i) total_rows += more->d_out[i];
-    if ((more == nullptr || more->n == 0) && run_supported(d, T)) return launch_stream(d, blob, L, ws, W, y, ldy, out_dtype, T, s, t0, more, true);
+    // (a caller that asks for one set of kernels gets the one that sibling layers use)
+    if ((more == nullptr || more->n == 0) && option(LOPRO_OPT_ONE_KERNEL_SET) != 1 && run_supported(d, T))
+        return launch_stream(d, blob, L, ws, W, y, ldy, out_dtype, T, s, t0, more, true);
     if (!plan_tall(d, T, &pl, total_rows)) return cudaErrorInvalidValue;
     TallParams p;
     p.codes = blob + L.off[LOPRO_SEC_CODES];

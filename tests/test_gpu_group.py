@@ -108,6 +108,19 @@ def test_sibling_layers_through_the_persistent_kernel(T, bits, g, extra):
     _check_group(layers, descs, blobs, synth.activations(T, n, seed=T + 50, outlier_frac=0.01), shared=True, bit_equal=False)
 
 
+@pytest.mark.parametrize("T", [1, 8, 16])
+def test_one_kernel_set_gives_single_layers_the_sums_of_a_group(T):
+    # four row tiles per multiprocessor and layer: a CTA owns four alone and eight in the group of two, i.e. whole groups of
+    # four tiles either way, so the persistent kernel adds a row's products in one order -- and another kernel would not
+    n, m = 1024, 16 * 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    layers, descs, blobs = _siblings(n, (m, m), 4, 128, 128, 16, seed=T)
+    x = bf16_bits_to_device(synth.activations(T, n, seed=T + 3))
+    with lopro.configured(lopro.OPT_ONE_KERNEL_SET, 1):
+        together = lopro.linear_fwd_group(descs, blobs, x, lopro.OUT_F32)
+        for d, blob, y in zip(descs, blobs, together):
+            assert torch.equal(lopro.linear_fwd(d, blob, x, lopro.OUT_F32), y)
+
+
 @pytest.mark.parametrize("T", [1, 32])
 def test_mlp_projections_of_the_stack_at_full_size(T):
     # gate, up of the 32-layer stack configuration: two 4096 -> 11008 layers, 4-bit g128, block 128, rank 32
