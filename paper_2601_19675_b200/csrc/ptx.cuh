@@ -160,7 +160,9 @@ __device__ __forceinline__ void expand_codes(uint32_t (&a)[16], const uint32_t (
 
 // The same with fewer shifts for the kernels that scale rows afterwards: the odd pairs, which are the rows gq + 8 of a tile,
 // come out as 128 + kOdd c, their bits left where a shift that an even pair needs anyway puts them (2 bits: 6 shifts instead of
-// 14 per tile step, 3 bits: 10 instead of 15).  kOdd is a power of two and goes into the rows' scale exactly.  The loops these
+// 14 per tile step, 3 bits: 10 instead of 15).  kOdd is a power of two and comes off with the rows' scale, exactly.  The
+// operands of those rows reach 140 (2 bits) and 184 (3 bits) instead of 131 and 135: the products of one step leave the fp32
+// range from sums of 64 |x~| of 1.8e36 on, where they did from 2.5e36 on.  The loops these
 // serve are bound by instruction issue with the integer pipe next; with the packed multiply-adds below 8192 -> 28672 at 2 bits,
 // 16 tokens 51.4 -> 48.4 us, eight experts 4096 -> 14336 at 2 bits 69.9 -> 65.8, 11008 -> 4096 at 3 bits, 5 tokens 14.5 -> 13.8.
 template <int BITS>
@@ -221,7 +223,7 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
 }
 
 // Scale and zero-point of a group for the rows gq (.x) and gq + 8 (.y) of a tile, as the sums of a tile step meet them:
-// y += s (acc - (128 + z) sum x~), with acc = sum (128 + kOdd c) x~ for the odd rows, whose y carries the factor kOdd.
+// y += s (acc - (128 + z) sum x~); for the odd rows acc = sum (128 + kOdd c) x~, and s and z are those of kOdd c.
 template <int BITS>
 struct RowScales {
     float s[2], z[2];
@@ -229,7 +231,7 @@ struct RowScales {
         const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&sz_lo));
         const float2 hi = __half22float2(*reinterpret_cast<const __half2*>(&sz_hi));
         s[0] = lo.x;
-        s[1] = hi.x;
+        s[1] = hi.x * (1.0f / OddRows<BITS>::factor);
         z[0] = -128.0f - lo.y;
         z[1] = fmaf(hi.y, -OddRows<BITS>::factor, -128.0f);
     }
@@ -261,14 +263,4 @@ __device__ __forceinline__ void add_scaled_early(float (&y)[4], const float (&ac
 #pragma unroll
     for (int i = 0; i < 4; ++i) y[i] = fmaf(r.s[i >> 1], acc[i], fmaf(r.s[i >> 1] * r.z[i >> 1], sx[i & 1], y[i]));
 }
-// The factor of the odd rows put on (the low-rank term that starts the sums) or taken off again.
-template <int NT>
-__device__ __forceinline__ void scale_odd_rows(float (&y)[NT][4], float f) {
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-        y[nt][2] *= f;
-        y[nt][3] *= f;
-    }
-}
-
 }  // namespace lopro

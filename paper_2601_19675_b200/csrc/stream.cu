@@ -180,7 +180,6 @@ stream_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
                 mma_f16(acc[nt], a, *reinterpret_cast<const uint32_t*>(trow), *reinterpret_cast<const uint32_t*>(trow + 8));
             }
         }
-        scale_odd_rows(acc, OddRows<BITS>::factor);
     };
     if (warp == kConsumerWarps) {
         // ---------------- producer warp ----------------
@@ -321,8 +320,6 @@ stream_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
     float* red = reinterpret_cast<float*>(smem + p.off_ring);
     if (warp < kConsumerWarps) {
 #pragma unroll
-        for (int r = 0; r < RT; ++r) scale_odd_rows(yacc[r], 1.0f / OddRows<BITS>::factor);
-#pragma unroll
         for (int r = 0; r < RT; ++r)
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt)
@@ -457,7 +454,6 @@ stream_wide_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
                 const __half* trow = ts + gq * p.r_pad + jj + 2 * tg;
                 mma_f16(yacc[0], a, *reinterpret_cast<const uint32_t*>(trow), *reinterpret_cast<const uint32_t*>(trow + 8));
             }
-            scale_odd_rows(yacc, OddRows<BITS>::factor);
         }
     }
 #pragma unroll
@@ -499,7 +495,6 @@ stream_wide_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
 
     static_assert(kStageSteps * kRedStep * 4 <= kStageBytes, "the partial sums fit one stage of the ring");
     float* red = reinterpret_cast<float*>(smem + p.off_ring);
-    scale_odd_rows(yacc, 1.0f / OddRows<BITS>::factor);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int tk = 2 * tg + (i & 1), rl = r * 16 + gq + 8 * (i >> 1);

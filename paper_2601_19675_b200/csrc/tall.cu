@@ -340,7 +340,6 @@ tall_kernel(const TallParams p_in, const __grid_constant__ SIBS sibs) {
                                 *reinterpret_cast<const uint32_t*>(trow + 8));
                     }
                 }
-                scale_odd_rows(yacc, OddRows<BITS>::factor);
             }
         }
 
@@ -399,7 +398,6 @@ tall_kernel(const TallParams p_in, const __grid_constant__ SIBS sibs) {
             }
             if (KQ > 1) named_arrive(2);
             if (active) {
-                scale_odd_rows(yacc, 1.0f / OddRows<BITS>::factor);
 #pragma unroll
                 for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
