@@ -207,6 +207,18 @@ __device__ __forceinline__ void expand_codes_by_rows(uint32_t (&a)[16], const ui
     }
 }
 
+// The products of one step with NT token tiles, the tiles of a quarter step one after the other: products that follow each
+// other then do not wait for one another (8192 -> 4096 at 4 bits, 24 tokens: 25.3 us tile by tile, 24.8 this way).
+template <int NT>
+__device__ __forceinline__ void multiply_step(float (&acc)[NT][4], const uint32_t (&a)[16], const uint32_t (&b)[NT][8]) {
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) mma_bf16_first(acc[nt], &a[0], b[nt][0], b[nt][1]);
+#pragma unroll
+    for (int k = 1; k < 4; ++k)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) mma_bf16(acc[nt], &a[4 * k], b[nt][2 * k], b[nt][2 * k + 1]);
+}
+
 // Two fp32 multiply-adds in one issue slot; the halves of a register pair are two tokens of a row.
 __device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
     unsigned long long v;

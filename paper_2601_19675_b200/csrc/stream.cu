@@ -285,13 +285,7 @@ stream_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
                         uint32_t a[16];
                         expand_codes_by_rows<BITS>(a, w);
                         float acc[NT][4];
-#pragma unroll
-                        for (int nt = 0; nt < NT; ++nt) {
-                            mma_bf16_first(acc[nt], &a[0], b[nt][0], b[nt][1]);
-                            mma_bf16(acc[nt], &a[4], b[nt][2], b[nt][3]);
-                            mma_bf16(acc[nt], &a[8], b[nt][4], b[nt][5]);
-                            mma_bf16(acc[nt], &a[12], b[nt][6], b[nt][7]);
-                        }
+                        multiply_step<NT>(acc, a, b);
                         add_scaled<BITS, NT>(yacc[r], acc, sx, RowScales<BITS>(szp[r * sz_tile], szp[r * sz_tile + 8]));
                     }
                 }

@@ -148,13 +148,7 @@ __device__ __forceinline__ void tile_step(const uint32_t* wp, uint32_t xaddr, co
     uint32_t a[16];
     expand_codes_by_rows<BITS>(a, w);
     float acc[NT][4];
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-        mma_bf16_first(acc[nt], &a[0], b[nt][0], b[nt][1]);
-        mma_bf16(acc[nt], &a[4], b[nt][2], b[nt][3]);
-        mma_bf16(acc[nt], &a[8], b[nt][4], b[nt][5]);
-        mma_bf16(acc[nt], &a[12], b[nt][6], b[nt][7]);
-    }
+    multiply_step<NT>(acc, a, b);
     add_scaled<BITS, NT>(yacc, acc, sx, RowScales<BITS>(szp[0], szp[8]));
 }
 
@@ -356,7 +350,9 @@ tall_kernel(const TallParams p_in, const __grid_constant__ SIBS sibs) {
             }
             if (active) {
                 const int steps = steps_of(s);
-                const bool whole = steps == kStageSteps;
+                // (one token tile only: the second copy of the loop costs registers, and with more tiles they were spilled --
+                // 17 to 32 tokens of 512 -> 8192, 3 bits, 9.63 us against 9.01, 3072 -> 22016, 2 bits, 35.8 against 34.3)
+                const bool whole = NT == 1 && steps == kStageSteps;
                 if (rbits == 2 && whole) consume_stage<BITS, NT, 2, true>(stage, stage_u32, wo, kq, gs, steps, yacc);
                 else if (rbits == 2) consume_stage<BITS, NT, 2, false>(stage, stage_u32, wo, kq, gs, steps, yacc);
                 else if (rbits == 1 && whole) consume_stage<BITS, NT, 1, true>(stage, stage_u32, wo, kq, gs, steps, yacc);
