@@ -424,10 +424,13 @@ lopro_status lopro_block_attention_decode(const uint16_t* q, int64_t ldq, const 
     // The loads in flight land in L1.  A programmatic launch puts the first CTAs beside those of a product kernel that holds
     // 220 KB of shared memory, and as long as the multiprocessor is never empty its split stays: 28 KB of L1 for all waves of
     // this grid.  With a split of its own asked for, the grid starts on multiprocessors that have it: 32 sequences of 32 heads
-    // after the q/k/v projections of a decoder layer 202 us without, 160 with (163 alone); 10 to 75 percent are alike.
+    // after the q/k/v projections of a decoder layer 202 us without, 160 with (163 alone).  Three quarters of shared memory,
+    // which leave 57 KB of L1, do as well as one for grids of several waves (decoder layer, 19 sequences of 40 heads, context
+    // 1705: 294 us without, 270 and 270), and cost a grid of one wave nothing, where the smaller share did (10 sequences of 32
+    // heads, context 2410: 156 us without, 161 with a quarter, 157 with three).
     static unsigned long long split_whole = 0, split_first = 0;
-    lopro::prefer_shared_memory(attention_kernel<128, kWhole>, 25, &split_whole);
-    lopro::prefer_shared_memory(attention_kernel<128, kFirst>, 25, &split_first);
+    lopro::prefer_shared_memory(attention_kernel<128, kWhole>, 75, &split_whole);
+    lopro::prefer_shared_memory(attention_kernel<128, kFirst>, 75, &split_first);
     auto run = [&](auto kernel, int size, int threads, int64_t first, int64_t count) {
         return launch(kernel, dim3((unsigned)(count * size)), threads, stream, size, reinterpret_cast<const __nv_bfloat16*>(q), ldq,
                       reinterpret_cast<const __nv_bfloat16*>(k_cache), reinterpret_cast<const __nv_bfloat16*>(v_cache), ctx, n_heads,
