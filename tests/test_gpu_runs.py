@@ -33,3 +33,15 @@ def test_runs_of_row_tiles(n, per_sm, extra, bits, g, T):
         y_short = lopro.linear_fwd(d, blob, x, lopro.OUT_F32)
     torch.cuda.synchronize()
     assert (y - y_short).abs().max().item() <= 2e-5 * y_short.abs().max().item()
+
+
+def test_short_rows_of_more_than_eight_tokens_stay_with_the_persistent_kernel():
+    # with a whole stage of K the two kernels add a row's products in different orders, so equal sums name the kernel
+    for n, same in ((512, True), (960, True), (1024, False)):
+        m = _rows(3, 5)
+        layer = random_layer_np(n, m, 4, 64, 16, seed=n)
+        d = lopro.make_desc(n, m, 4, 64, 64, identity_cols=64, rank=16)
+        blob, x = _pack(layer, d), bf16_bits_to_device(synth.activations(12, n, seed=n))
+        y = lopro.linear_fwd(d, blob, x, lopro.OUT_F32)
+        with lopro.configured(lopro.OPT_ONE_KERNEL_SET, 1):
+            assert torch.equal(lopro.linear_fwd(d, blob, x, lopro.OUT_F32), y) == same
