@@ -267,12 +267,5 @@ __device__ __forceinline__ void add_scaled(float (&y)[NT][4], const float (&acc)
         }
     }
 }
-// The same for one token tile where latency counts: the zero-point's part is added while the products are on their way, one
-// multiply-add follows them (4096 -> 4096 at one token 5.83 us with two, 5.74 with one).
-template <int BITS>
-__device__ __forceinline__ void add_scaled_early(float (&y)[4], const float (&acc)[4], float sx0, float sx1, const RowScales<BITS>& r) {
-    const float sx[2] = {sx0, sx1};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) y[i] = fmaf(r.s[i >> 1], acc[i], fmaf(r.s[i >> 1] * r.z[i >> 1], sx[i & 1], y[i]));
-}
+
 }  // namespace lopro

@@ -454,11 +454,10 @@ stream_wide_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
     for (int s = 0; s < kMaxStages; ++s) {
         if (s >= my_stages) break;
         if (!mbar_wait(full(s), 0)) timed_out = true;
-        uint32_t b[8];
-        ldmatrix_x4(*reinterpret_cast<uint32_t(*)[4]>(&b[0]), xaddr + s * kStageBytes);
-        ldmatrix_x4(*reinterpret_cast<uint32_t(*)[4]>(&b[4]), xaddr + s * kStageBytes + 64u);
-        const float sx0 = sxp[s * (kStageBytes / 4)];
-        const float sx1 = sxp[s * (kStageBytes / 4) + kActRecord / 4];
+        uint32_t b[1][8];
+        ldmatrix_x4(*reinterpret_cast<uint32_t(*)[4]>(&b[0][0]), xaddr + s * kStageBytes);
+        ldmatrix_x4(*reinterpret_cast<uint32_t(*)[4]>(&b[0][4]), xaddr + s * kStageBytes + 64u);
+        const float sx[1][2] = {{sxp[s * (kStageBytes / 4)], sxp[s * (kStageBytes / 4) + kActRecord / 4]}};
         uint32_t w[BITS];
         const uint32_t* wp = reinterpret_cast<const uint32_t*>(wptr + s * kStageBytes);
         if constexpr (BITS == 4) {
@@ -474,13 +473,9 @@ stream_wide_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
         uint32_t a[16];
         expand_codes_by_rows<BITS>(a, w);
         const uint32_t* szp = szs + ((s * kStageSteps + step) >> p.gshift) * 16;  // the step's group
-        const RowScales<BITS> scales(szp[0], szp[8]);
-        float acc[4];
-        mma_bf16_first(acc, &a[0], b[0], b[1]);
-        mma_bf16(acc, &a[4], b[2], b[3]);
-        mma_bf16(acc, &a[8], b[4], b[5]);
-        mma_bf16(acc, &a[12], b[6], b[7]);
-        add_scaled_early<BITS>(yacc[0], acc, sx0, sx1, scales);
+        float acc[1][4];
+        multiply_step<1>(acc, a, b);
+        add_scaled<BITS, 1>(yacc, acc, sx, RowScales<BITS>(szp[0], szp[8]));
     }
     if (timed_out && lane == 0) atomicExch(p.status, (int)LOPRO_ERR_TIMEOUT);
     // Every stage has a step-0 warp that waited for it, so after this barrier every copy has landed and the ring
