@@ -251,22 +251,24 @@ stream_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
                 if (lane == 0) atomicExch(p.status, (int)LOPRO_ERR_TIMEOUT);
             }
             if (warp < steps_left) {
-                // B operand: the 64 columns of step `warp`, all token tiles
-                uint32_t b[NT][8];
-#pragma unroll
-                for (int nt = 0; nt < NT; ++nt) {
-                    const uint32_t base = stage_u32 + xofs + (uint32_t)(nt * 8 * kXsStride) * 2u;
-                    ldmatrix_x4(*reinterpret_cast<uint32_t(*)[4]>(&b[nt][0]), base);
-                    ldmatrix_x4(*reinterpret_cast<uint32_t(*)[4]>(&b[nt][4]), base + 64u);
-                }
+                // B operand and column sums: the 64 columns of step `warp`, all token tiles.  With four token tiles they are read
+                // anew for every row tile: kept beside two tiles' sums they did not fit the registers (17 to 32 tokens of up to
+                // 2752 rows, 64 to 80 drawn layers per number of bits: with the spills 10 percent slower).
                 const float* sxp = reinterpret_cast<const float*>(stage + sxofs);
                 const uint32_t* szp = szs + (kstep >> p.gshift) * 16;
+                uint32_t b[NT][8];
                 float sx[NT][2];
+                auto read_activations = [&] {
 #pragma unroll
-                for (int nt = 0; nt < NT; ++nt) {
-                    sx[nt][0] = sxp[nt * 8 * (kActRecord / 4)];
-                    sx[nt][1] = sxp[(nt * 8 + 1) * (kActRecord / 4)];
-                }
+                    for (int nt = 0; nt < NT; ++nt) {
+                        const uint32_t base = stage_u32 + xofs + (uint32_t)(nt * 8 * kXsStride) * 2u;
+                        ldmatrix_x4(*reinterpret_cast<uint32_t(*)[4]>(&b[nt][0]), base);
+                        ldmatrix_x4(*reinterpret_cast<uint32_t(*)[4]>(&b[nt][4]), base + 64u);
+                        sx[nt][0] = sxp[nt * 8 * (kActRecord / 4)];
+                        sx[nt][1] = sxp[(nt * 8 + 1) * (kActRecord / 4)];
+                    }
+                };
+                if (NT < 4) read_activations();
 #pragma unroll
                 for (int r = 0; r < RT; ++r) {
                     if (r < n_rt) {
@@ -284,6 +286,7 @@ stream_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
                         }
                         uint32_t a[16];
                         expand_codes_by_rows<BITS>(a, w);
+                        if (NT == 4) read_activations();
                         float acc[NT][4];
                         multiply_step<NT>(acc, a, b);
                         add_scaled<BITS, NT>(yacc[r], acc, sx, RowScales<BITS>(szp[r * sz_tile], szp[r * sz_tile + 8]));
