@@ -627,18 +627,18 @@ bool plan_layout(const lopro_desc& d, StreamPlan* pl, int r_pad, int ng, int kto
 // 11.2 and 12.0; 5120 -> 5120 at 4 tokens 9.6 and 8.6; 2 bits at 12 tokens 13.6 and 12.2.  A second wave pays a start-up of
 // its own (4096 -> 22016 18.9 and 19.3), so only where K has eight stages or more, and with 8 tokens at most: 8192 -> 28672,
 // 2 bits, 4 tokens 37.9 and 34.0, 16 tokens 41.7 and 46.1.  With less than a whole stage of K some of the sixteen warps have no
-// step at all; nine tokens and more then stay with the persistent kernel (512 -> 8192, 2 bits, 9 tokens 5.8 and 6.0; 1024 ->
-// 8192, 3 bits, 12 tokens 6.9 and 6.7).  Layers that share a launch stay with the persistent kernel: three
+// step at all; with nine tokens and more, runs of up to four tiles, which the persistent kernel takes as one group, then stay there
+// (512 -> 8192, 2 bits, 9 tokens 5.8 and 6.0; with five tiles 512 -> 11008, 12 tokens 8.7 and 8.2).  Layers that share a launch stay with the persistent kernel: three
 // layers 4096 -> 4096 alone gained (13.8 and 12.2), the decoder layer of one sequence around them lost (85.1 and 89.4).
 bool plan_run(const lopro_desc& d, int T, StreamPlan* pl, int* ctas) {
     if (T < 1 || T > 16) return false;
     pl->nt = T <= 8 ? 1 : 2;
-    if (pl->nt == 2 && d.d_in < 1024) return false;
     const int r_pad = d.rank > 0 ? round_up_int(d.rank, 16) : 0, ng = d.d_in / d.group_size, tiles = d.d_out / 16;
     for (int waves = 1; waves <= (pl->nt == 1 && d.d_in >= 8192 ? 2 : 1); ++waves) {
         *ctas = sm_count() * waves;
         const int most = (tiles + *ctas - 1) / *ctas;   // the longest run
         if (most > (pl->nt == 2 ? 5 : (waves == 2 ? 8 : 6))) continue;
+        if (pl->nt == 2 && d.d_in < 1024 && most <= 4) continue;
         pl->rt = most <= 4 ? 4 : (most <= 6 ? most : 8);
         if (plan_layout(d, pl, r_pad, ng, pl->nt * 8)) return true;
     }

@@ -37,8 +37,8 @@ def test_runs_of_row_tiles(n, per_sm, extra, bits, g, T):
 
 def test_short_rows_of_more_than_eight_tokens_stay_with_the_persistent_kernel():
     # with a whole stage of K the two kernels add a row's products in different orders, so equal sums name the kernel
-    for n, same in ((512, True), (960, True), (1024, False)):
-        m = _rows(3, 5)
+    for n, per_sm, same in ((512, 3, True), (960, 3, True), (1024, 3, False), (512, 4, False)):
+        m = _rows(per_sm, 5)      # 3 or 4 tiles per CTA; 4 or 5
         layer = random_layer_np(n, m, 4, 64, 16, seed=n)
         d = lopro.make_desc(n, m, 4, 64, 64, identity_cols=64, rank=16)
         blob, x = _pack(layer, d), bf16_bits_to_device(synth.activations(12, n, seed=n))
