@@ -627,6 +627,7 @@ def measure(args, name, steps, warmup, rank, world, local, dev, dist, with_e2e=T
     ms_per_pass = ms_per_step / passes
     value = w.tokens_per_pass * passes * world / (ms_per_step * 1e-3)
     per_forward_s = ms_per_pass * 1e-3 / w.forwards
+    # ("tall": none of the workloads is a layer that runs of row tiles take)
     kernel = " + ".join({"stream": "stream_kernel", "wide": "stream_wide_kernel", "tall": "tall_kernel", "general": "decode_kernel",
                          "prefill": "prefill_pair_kernel" if w.T >= 512 else "prefill_kernel",
                          "rowblock": "rowblock_kernel"}.get(n, n) for n in w.paths)

@@ -119,7 +119,7 @@ enum {
  * (LOPRO_NO_WIDE=1, ...); 0 = default behaviour. */
 enum {
     LOPRO_OPT_NO_WIDE = 0,       /* 1: never the 32-warp variant of the streaming kernel                       */
-    LOPRO_OPT_NO_TALL = 1,       /* 1: never the persistent streaming kernel for layers with many rows         */
+    LOPRO_OPT_NO_TALL = 1,       /* 1: never the kernels for layers with many rows (persistent, runs of row tiles) */
     LOPRO_OPT_NO_CHUNKS = 2,     /* 1: token counts above 32 always take the tensor-core (prefill) kernel      */
     LOPRO_OPT_NO_TCGEN05 = 3,    /* 1: never the tcgen05 prefill kernel (general register-ring product)        */
     LOPRO_OPT_PREFILL_PAIRS = 4, /* >= 0: number of two-block row tiles of the prefill grid; where two CTAs share a
@@ -127,7 +127,8 @@ enum {
                                      = none, at most 16; -1: chosen by the library                              */
     LOPRO_OPT_ONE_KERNEL_SET = 5, /* 1: single-layer forwards launch the same kernel variants as grouped ones
                                       (lopro_linear_fwd_group / _experts), which carry a table of sibling layers in
-                                      their parameters.  By default a single-layer forward launches variants without
+                                      their parameters; layers with many rows then always take the persistent kernel,
+                                      never runs of row tiles, as no group does.  By default a single-layer forward launches variants without
                                       that table (0.15-0.4 us less per launch of a small layer); a caller that
                                       alternates single and grouped forwards -- a decoder stack -- then alternates
                                       between two copies of every kernel, which costs more than the table does
@@ -242,7 +243,9 @@ LOPRO_API lopro_status lopro_linear_fwd(const lopro_desc* desc, const void* pack
  * measure; the paper's Appendix A.3 lists the steps, not their grouping into launches).
  *   LOPRO_PATH_STREAM   2 launches: prologue (permutation, rotation, B x) + streaming product, T <= 32
  *   LOPRO_PATH_WIDE     the same with the 32-warp variant of the streaming kernel (T <= 8, all of K in the ring)
- *   LOPRO_PATH_TALL     the same with the persistent streaming kernel for layers with many output rows
+ *   LOPRO_PATH_TALL     the same with a kernel for layers with many output rows: the persistent streaming kernel or, for
+ *                       up to 16 tokens where the rows make even waves of short runs, the streaming kernel with longer
+ *                       runs of rows per CTA (not with LOPRO_OPT_ONE_KERNEL_SET)
  *   LOPRO_PATH_GENERAL  rotation, B x, register-ring product (any shape the descriptor allows)
  *   LOPRO_PATH_PREFILL  rotation, B x (2 launches), tcgen05 product (one CTA per tile, or two with a launch more
  *                       where the last wave's tiles are cut along K), T > 32

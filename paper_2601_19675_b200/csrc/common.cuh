@@ -211,7 +211,7 @@ struct StreamSiblingArgs {
 cudaError_t launch_stream(const lopro_desc& d, const uint8_t* blob, const BlobLayout& L, const uint8_t* ws,
                           const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s, int t0 = 0,
                           const StreamSiblingArgs* more = nullptr, bool in_runs = false);
-// The same kernel for a taller layer, in even waves of longer runs of rows (no siblings).
+// The same kernel for a taller layer alone, in one or two even waves of longer runs of row tiles.
 bool run_supported(const lopro_desc& d, int T);
 
 // Small-batch forward for tall layers after launch_prologue: persistent CTAs, one ring across tile groups.

@@ -162,9 +162,9 @@ __device__ __forceinline__ void expand_codes(uint32_t (&a)[16], const uint32_t (
 // come out as 128 + kOdd c, their bits left where a shift that an even pair needs anyway puts them (2 bits: 6 shifts instead of
 // 14 per tile step, 3 bits: 10 instead of 15).  kOdd is a power of two and comes off with the rows' scale, exactly.  The
 // operands of those rows reach 140 (2 bits) and 184 (3 bits) instead of 131 and 135: the products of one step leave the fp32
-// range from sums of 64 |x~| of 1.8e36 on, where they did from 2.5e36 on.  The loops these
+// range where its 64 |x~| add up to 1.8e36 or more (2.5e36 with operands up to 135).  The loops these
 // serve are bound by instruction issue with the integer pipe next; with the packed multiply-adds below 8192 -> 28672 at 2 bits,
-// 16 tokens 51.4 -> 48.4 us, eight experts 4096 -> 14336 at 2 bits 69.9 -> 65.8, 11008 -> 4096 at 3 bits, 5 tokens 14.5 -> 13.8.
+// 16 tokens 51.4 -> 48.8 us, eight experts 4096 -> 14336 at 2 bits 81.4 -> 76.3, 11008 -> 4096 at 3 bits, 5 tokens 14.5 -> 14.0.
 template <int BITS>
 struct OddRows {
     static constexpr float factor = BITS == 4 ? 1.0f : (BITS == 2 ? 4.0f : 8.0f);
@@ -208,7 +208,7 @@ __device__ __forceinline__ void expand_codes_by_rows(uint32_t (&a)[16], const ui
 }
 
 // The products of one step with NT token tiles, the tiles of a quarter step one after the other: products that follow each
-// other then do not wait for one another (8192 -> 4096 at 4 bits, 24 tokens: 25.3 us tile by tile, 24.8 this way).
+// other then do not wait for one another (8192 -> 4096 at 4 bits, 24 tokens: 25.2 us tile by tile, 24.8 this way).
 template <int NT>
 __device__ __forceinline__ void multiply_step(float (&acc)[NT][4], const uint32_t (&a)[16], const uint32_t (&b)[NT][8]) {
 #pragma unroll

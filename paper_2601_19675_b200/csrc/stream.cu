@@ -12,7 +12,8 @@
 // from the low-rank term A t); one shared-memory reduction over the warps at the end, then the store.
 //
 // Arithmetic: as in the general path, sum_k s (c_k - z) x~_k = s (sum_k (128 + c_k) x~_k
-// - (128 + z) sum_k x~_k), the first sum on the tensor cores with exact bf16 operands 128 + c_k,
+// - (128 + z) sum_k x~_k), the first sum on the tensor cores with exact bf16 operands 128 + c_k
+// (128 + 4 c_k or 128 + 8 c_k for half of the rows of 2- and 3-bit codes, see expand_codes_by_rows),
 // fp32 accumulation, scale and zero-point applied in fp32 once per 64 columns.
 //
 // Every wait on an mbarrier is bounded; a wait that runs out stores LOPRO_ERR_TIMEOUT in the
@@ -560,15 +561,25 @@ cudaError_t launch_stream_k(const StreamParams& p, const StreamSiblings& sibs, i
 template <int BITS>
 cudaError_t launch_stream_bits(const StreamParams& p, const StreamSiblings& sibs, int grid, int nt, int rt, int smem_bytes,
                                cudaStream_t s) {
-    if (nt == 1 && rt == 5) return launch_stream_k<BITS, 1, 5>(p, sibs, grid, smem_bytes, s);
-    if (nt == 1 && rt == 6) return launch_stream_k<BITS, 1, 6>(p, sibs, grid, smem_bytes, s);
-    if (nt == 1 && rt == 8) return launch_stream_k<BITS, 1, 8>(p, sibs, grid, smem_bytes, s);
-    if (nt == 2 && rt == 5) return launch_stream_k<BITS, 2, 5>(p, sibs, grid, smem_bytes, s);
     if (nt == 1)
         return rt == 4 ? launch_stream_k<BITS, 1, 4>(p, sibs, grid, smem_bytes, s) : launch_stream_k<BITS, 1, 2>(p, sibs, grid, smem_bytes, s);
     if (nt == 2)
         return rt == 4 ? launch_stream_k<BITS, 2, 4>(p, sibs, grid, smem_bytes, s) : launch_stream_k<BITS, 2, 2>(p, sibs, grid, smem_bytes, s);
     return launch_stream_k<BITS, 4, 2>(p, sibs, grid, smem_bytes, s);
+}
+
+// Runs of row tiles (plan_run): a layer alone, so only the kernels without a table of siblings.
+template <int BITS>
+cudaError_t launch_stream_run(const StreamParams& p, int grid, int nt, int rt, int smem_bytes, cudaStream_t s) {
+    const NoSiblings none{};
+    if (nt == 2)
+        return rt == 4 ? launch_stream_ks<BITS, 2, 4>(p, none, grid, smem_bytes, s) : launch_stream_ks<BITS, 2, 5>(p, none, grid, smem_bytes, s);
+    if (rt == 4) return launch_stream_ks<BITS, 1, 4>(p, none, grid, smem_bytes, s);
+    if (rt == 5) return launch_stream_ks<BITS, 1, 5>(p, none, grid, smem_bytes, s);
+    if (rt == 6) return launch_stream_ks<BITS, 1, 6>(p, none, grid, smem_bytes, s);
+    if constexpr (BITS < 4)  // three stages of eight 4-bit tiles do not fit
+        if (rt == 8) return launch_stream_ks<BITS, 1, 8>(p, none, grid, smem_bytes, s);
+    return cudaErrorInvalidValue;
 }
 
 struct StreamPlan {
@@ -622,14 +633,15 @@ bool plan_layout(const lopro_desc& d, StreamPlan* pl, int r_pad, int ng, int kto
 
 // A taller layer in runs: every CTA of one even wave takes up to six row tiles (five with 16 tokens) over all of K, so that a
 // warp multiplies the step it has fetched with all of them and hands its sums over once; the persistent kernel gives a warp one
-// tile, reads the activations again and hands over per group of four.  Bound by the expansion (integer pipe) at about 80 cycles
-// per tile step and scheduler.  Persistent kernel against runs: 4096 -> 11008, 4 bits, 1 and 8 tokens 12.2 and 13.1 us against
-// 11.2 and 12.0; 5120 -> 5120 at 4 tokens 9.6 and 8.6; 2 bits at 12 tokens 13.6 and 12.2.  A second wave pays a start-up of
-// its own (4096 -> 22016 18.9 and 19.3), so only where K has eight stages or more, and with 8 tokens at most: 8192 -> 28672,
-// 2 bits, 4 tokens 37.9 and 34.0, 16 tokens 41.7 and 46.1.  With less than a whole stage of K some of the sixteen warps have no
-// step at all; with nine tokens and more, runs of up to four tiles, which the persistent kernel takes as one group, then stay there
-// (512 -> 8192, 2 bits, 9 tokens 5.8 and 6.0; with five tiles 512 -> 11008, 12 tokens 8.7 and 8.2).  Layers that share a launch stay with the persistent kernel: three
-// layers 4096 -> 4096 alone gained (13.8 and 12.2), the decoder layer of one sequence around them lost (85.1 and 89.4).
+// tile, reads the activations again and hands over per group of four.  Persistent kernel against runs: 4096 -> 11008, 4 bits,
+// 1 and 8 tokens 12.2 and 13.1 us against 11.2 and 12.0; 5120 -> 5120 at 4 tokens 9.6 and 8.6; 2 bits at 12 tokens 13.6 and
+// 12.2.  A second wave pays a start-up of its own (4096 -> 22016 18.9 and 19.3), so two waves, with up to eight tiles, only where
+// K has eight stages or more, and with 8 tokens at most: 8192 -> 28672, 2 bits, rank 32, block 128, 4 tokens 37.9 and 34.0,
+// 16 tokens 41.7 and 46.1.  With less than a whole stage of K some of the sixteen warps have no step at all; with nine tokens and
+// more, runs of up to four tiles, which the persistent kernel takes as one group, then stay there (512 -> 8192, 2 bits, 9 tokens
+// 5.8 and 6.0; with five tiles 512 -> 11008, 12 tokens 8.7 and 8.2).  Layers that share a launch stay with the persistent kernel:
+// three layers 4096 -> 4096 alone gained (13.8 and 12.2), the decoder layer of one sequence around them lost (85.1 and 89.4; the
+// reason is not known).
 bool plan_run(const lopro_desc& d, int T, StreamPlan* pl, int* ctas) {
     if (T < 1 || T > 16) return false;
     pl->nt = T <= 8 ? 1 : 2;
@@ -706,10 +718,18 @@ cudaError_t launch_stream(const lopro_desc& d, const uint8_t* blob, const BlobLa
     p.off_ring = pl.off_ring;
     p.stage_bytes = pl.stage_bytes;
     p.off_stage_x = pl.off_stage_x;
-    const bool wide = !in_runs && wide_variant(d, pl);
-    const int rows_per_cta = wide ? 32 : pl.rt * 16;
-    int grid = in_runs ? run_ctas : (d.d_out + rows_per_cta - 1) / rows_per_cta;
     p.run_ctas = run_ctas;
+    if (in_runs) {
+        if (more != nullptr && more->own_rows) p.T = more->T_of[0];
+        switch (d.bits) {
+            case 2: return launch_stream_run<2>(p, run_ctas, pl.nt, pl.rt, pl.smem_bytes, s);
+            case 3: return launch_stream_run<3>(p, run_ctas, pl.nt, pl.rt, pl.smem_bytes, s);
+            default: return launch_stream_run<4>(p, run_ctas, pl.nt, pl.rt, pl.smem_bytes, s);
+        }
+    }
+    const bool wide = wide_variant(d, pl);
+    const int rows_per_cta = wide ? 32 : pl.rt * 16;
+    int grid = (d.d_out + rows_per_cta - 1) / rows_per_cta;
     // sibling layers: the CTAs of each follow those of the one before
     StreamSiblings sibs = {};
     if (more != nullptr) {

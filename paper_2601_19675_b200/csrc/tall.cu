@@ -3,8 +3,9 @@
 // "U (Sigma Y)" of Appendix A.3, summed as in Eq. 8), after the prologue kernel that writes the
 // rotated activations x~ (as the stage image), their 64-column sums and t = B x.
 //
-// A single layer of up to 16 tokens whose tiles make one even wave of short runs goes through the kernel of stream.cu instead
-// (plan_run there): longer runs, more tokens and layers that share a launch run here.
+// A single layer of up to 16 tokens whose tiles make an even wave of runs of up to six goes through the kernel of stream.cu
+// instead (plan_run there; two waves of runs of up to eight for long rows): longer runs, more tokens, layers that share a launch
+// and callers that ask for one set of kernels run here.
 //
 // Persistent: one CTA per SM, each owning a contiguous run of 16-row tiles (the runs differ by at
 // most one tile) and walking it in groups of up to four tiles (two with 32 tokens).  A producer warp keeps one ring of
@@ -23,8 +24,8 @@
 // takes part in them.
 //
 // Arithmetic as in stream.cu: sum_k s (c_k - z) x~_k = s (sum_k (128 + c_k) x~_k - (128 + z) sum_k x~_k),
-// exact bf16 operands 128 + c_k on the tensor cores, fp32 accumulation, scale and zero-point
-// applied in fp32 once per 64 columns.
+// exact bf16 operands 128 + c_k on the tensor cores (rows gq + 8 of a tile: see expand_codes_by_rows), fp32 accumulation,
+// scale and zero-point applied in fp32 once per 64 columns.
 //
 // Every mbarrier wait is bounded; a wait that runs out stores LOPRO_ERR_TIMEOUT in the workspace
 // status word and the CTA stops waiting (its outputs are then unspecified).

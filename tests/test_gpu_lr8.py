@@ -157,11 +157,12 @@ def _tall_rows(tiles_per_sm, extra):
 
 
 @pytest.mark.parametrize("T", [1, 3, 8, 16, 32, 40, 100])
-@pytest.mark.parametrize("bits,g,r,m", [(4, 128, 32, 272), (2, 64, 128, 144), (3, 64, 17, None)])
+@pytest.mark.parametrize("bits,g,r,m", [(4, 128, 32, 272), (2, 64, 128, 144), (3, 64, 17, 3), (3, 64, 17, 7)])
 def test_forward_with_the_fp8_record(T, bits, g, r, m):
-    # the 32-warp, the 16-warp and the persistent small-batch kernel, and more than 32 tokens as chunks of 32
+    # the 32-warp and the 16-warp kernel, runs of row tiles and the persistent kernel (m below 16: tiles per multiprocessor, and
+    # a few), and more than 32 tokens as chunks of 32
     n = 2048
-    m = _tall_rows(3, 5) if m is None else m
+    m = _tall_rows(m, 5) if m < 16 else m
     layer = random_layer_np(n, m, bits, g, 0, seed=T + bits)
     rec = synth.lowrank_record(m, n, r, seed=T + r)
     # Sigma large enough for the rank-r term to matter next to the synthetic quantized part
