@@ -127,8 +127,9 @@ enum {
                                      = none, at most 16; -1: chosen by the library                              */
     LOPRO_OPT_ONE_KERNEL_SET = 5, /* 1: single-layer forwards launch the same kernel variants as grouped ones
                                       (lopro_linear_fwd_group / _experts), which carry a table of sibling layers in
-                                      their parameters; layers with many rows then always take the persistent kernel,
-                                      never runs of row tiles, as no group does.  By default a single-layer forward launches variants without
+                                      their parameters, and which kernel a layer with many rows takes does not depend on
+                                      who shares its launch: those that alone could go in runs of row tiles always take the
+                                      persistent kernel.  By default a single-layer forward launches variants without
                                       that table (0.15-0.4 us less per launch of a small layer); a caller that
                                       alternates single and grouped forwards -- a decoder stack -- then alternates
                                       between two copies of every kernel, which costs more than the table does

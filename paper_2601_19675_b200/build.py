@@ -20,7 +20,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblopro.so")
 BINDING = os.path.join(HERE, "_binding.so")
 STAMP = os.path.join(HERE, "_build", "binding.txt")
-SOURCES = ["api.cu", "pack.cu", "rotate.cu", "decode.cu", "stream.cu", "tall.cu", "noalloc.cu", "prefill.cu", "lowrank.cu", "rowblock.cu", "quantize.cu", "sketch.cu", "block.cu", "vq.cu"]
+SOURCES = ["api.cu", "pack.cu", "rotate.cu", "decode.cu", "stream.cu", "tall.cu", "warps.cu", "noalloc.cu", "prefill.cu", "lowrank.cu", "rowblock.cu", "quantize.cu", "sketch.cu", "block.cu", "vq.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden"]
 

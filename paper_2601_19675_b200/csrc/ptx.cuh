@@ -101,6 +101,26 @@ __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
                  : "r"(addr));
 }
 
+// Loads from shared memory by 32-bit address, kept behind the waits in front of them.
+__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ float lds_f32(uint32_t addr) { return __uint_as_float(lds32(addr)); }
+// a lane's words of one tile step: one 16- or 8-byte load, three words one by one
+template <int BITS>
+__device__ __forceinline__ void lds_words(uint32_t (&w)[BITS], uint32_t addr) {
+    if constexpr (BITS == 4) {
+        asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(addr) : "memory");
+    } else if constexpr (BITS == 2) {
+        asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "r"(addr) : "memory");
+    } else {
+#pragma unroll
+        for (int q = 0; q < BITS; ++q) w[q] = lds32(addr + 4u * q);
+    }
+}
+
 // two fp8 e4m3 values (low byte first) -> two fp16 values (exact)
 __device__ __forceinline__ uint32_t e4m3x2_to_f16x2(uint16_t v) {
     uint32_t d;

@@ -3,9 +3,9 @@
 // "U (Sigma Y)" of Appendix A.3, summed as in Eq. 8), after the prologue kernel that writes the
 // rotated activations x~ (as the stage image), their 64-column sums and t = B x.
 //
-// A single layer of up to 16 tokens whose tiles make an even wave of runs of up to six goes through the kernel of stream.cu
-// instead (plan_run there; two waves of runs of up to eight for long rows): longer runs, more tokens, layers that share a launch
-// and callers that ask for one set of kernels run here.
+// Up to 16 tokens most such layers go elsewhere (launch_tall): every warp on a run of tile steps of its own where the activations
+// fit shared memory (warps.cu), runs of row tiles for a layer alone with few steps per CTA (plan_run in stream.cu).  More tokens, longer
+// rows and, where callers ask for one set of kernels, the layers that alone might go in runs of row tiles run here.
 //
 // Persistent: one CTA per SM, each owning a contiguous run of 16-row tiles (the runs differ by at
 // most one tile) and walking it in groups of up to four tiles (two with 32 tokens).  A producer warp keeps one ring of
@@ -121,8 +121,9 @@ __device__ __forceinline__ void named_arrive(int id) {
 // wp: the lane's words of the step; xaddr: the lane's ldmatrix row of the step (shared-space address);
 // sxp: the step's 64-column sum of token 2 * tg; szp: the (scale, zero) pair of row gq in the step's group.
 template <int BITS, int NT>
-__device__ __forceinline__ void tile_step(const uint32_t* wp, uint32_t xaddr, const float* sxp, const uint32_t* szp,
-                                          float (&yacc)[NT][4]) {
+__device__ __forceinline__ void tile_step(uint32_t waddr, uint32_t xaddr, uint32_t sxaddr, uint32_t szaddr, float (&yacc)[NT][4]) {
+    uint32_t w[BITS];
+    lds_words<BITS>(w, waddr);
     uint32_t b[NT][8];
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
@@ -132,25 +133,15 @@ __device__ __forceinline__ void tile_step(const uint32_t* wp, uint32_t xaddr, co
     float sx[NT][2];
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
-        sx[nt][0] = sxp[nt * 8 * (kActRecord / 4)];
-        sx[nt][1] = sxp[(nt * 8 + 1) * (kActRecord / 4)];
+        sx[nt][0] = lds_f32(sxaddr + nt * 8 * kActRecord);
+        sx[nt][1] = lds_f32(sxaddr + (nt * 8 + 1) * kActRecord);
     }
-    uint32_t w[BITS];
-    if constexpr (BITS == 4) {
-        const uint4 v = *reinterpret_cast<const uint4*>(wp);
-        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
-    } else if constexpr (BITS == 2) {
-        const uint2 v = *reinterpret_cast<const uint2*>(wp);
-        w[0] = v.x; w[1] = v.y;
-    } else {
-#pragma unroll
-        for (int q = 0; q < BITS; ++q) w[q] = wp[q];
-    }
+    const uint32_t sz0 = lds32(szaddr), sz1 = lds32(szaddr + 32u);
     uint32_t a[16];
     expand_codes_by_rows<BITS>(a, w);
     float acc[NT][4];
     multiply_step<NT>(acc, a, b);
-    add_scaled<BITS, NT>(yacc, acc, sx, RowScales<BITS>(szp[0], szp[8]));
+    add_scaled<BITS, NT>(yacc, acc, sx, RowScales<BITS>(sz0, sz1));
 }
 
 // Byte offsets, from the start of a stage, of what a warp reads in its first step (step kq of tile slot r); they
@@ -163,20 +154,15 @@ struct WarpOffsets {
 // strides; gs = min(gshift, 4): a stage starts on a group boundary or lies inside one group, so the group of
 // step st within the stage's (scale, zero) block is st >> gs.  WHOLE: a stage of sixteen steps (no test in front of each).
 template <int BITS, int NT, int RBITS, bool WHOLE>
-__device__ __forceinline__ void consume_stage(const unsigned char* stage, uint32_t stage_u32, const WarpOffsets& o, int kq,
-                                              int gs, int steps, float (&yacc)[NT][4]) {
+__device__ __forceinline__ void consume_stage(uint32_t stage, const WarpOffsets& o, int kq, int gs, int steps, float (&yacc)[NT][4]) {
     constexpr int KQ = kConsumerWarps >> RBITS, PER = kStageSteps / KQ;
     constexpr int kStepBytes = 128 * BITS;
-    const unsigned char* wbase = stage + o.w;
-    const float* sxbase = reinterpret_cast<const float*>(stage + o.sx);
-    const uint32_t* szbase = reinterpret_cast<const uint32_t*>(stage + o.sz);
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
         const int st = kq + i * KQ;
         if (WHOLE || st < steps)
-            tile_step<BITS, NT>(reinterpret_cast<const uint32_t*>(wbase + i * KQ * kStepBytes),
-                                stage_u32 + o.x + (uint32_t)(i * KQ * 128), sxbase + i * KQ, szbase + (st >> gs) * 16,
-                                yacc);
+            tile_step<BITS, NT>(stage + o.w + (uint32_t)(i * KQ * kStepBytes), stage + o.x + (uint32_t)(i * KQ * 128),
+                                stage + o.sx + (uint32_t)(i * KQ * 4), stage + o.sz + (uint32_t)((st >> gs) * 64), yacc);
     }
 }
 
@@ -295,7 +281,6 @@ tall_kernel(const TallParams p_in, const __grid_constant__ SIBS sibs) {
     // the ring slot of the next stage, its parity and its address
     int slot = 0;
     uint32_t phase = 0;
-    const unsigned char* stage = smem + p.off_ring;
     uint32_t stage_u32 = smem0 + (uint32_t)p.off_ring;
     for (int gi = 0; gi < n_groups; ++gi) {
         const int tile0 = my_start + gi * p.gt;
@@ -354,22 +339,20 @@ tall_kernel(const TallParams p_in, const __grid_constant__ SIBS sibs) {
                 // (one token tile only: the second copy of the loop costs registers, and with more tiles they were spilled --
                 // 17 to 32 tokens of 512 -> 8192, 3 bits, 9.63 us against 9.01, 3072 -> 22016, 2 bits, 35.8 against 34.3)
                 const bool whole = NT == 1 && steps == kStageSteps;
-                if (rbits == 2 && whole) consume_stage<BITS, NT, 2, true>(stage, stage_u32, wo, kq, gs, steps, yacc);
-                else if (rbits == 2) consume_stage<BITS, NT, 2, false>(stage, stage_u32, wo, kq, gs, steps, yacc);
-                else if (rbits == 1 && whole) consume_stage<BITS, NT, 1, true>(stage, stage_u32, wo, kq, gs, steps, yacc);
-                else if (rbits == 1) consume_stage<BITS, NT, 1, false>(stage, stage_u32, wo, kq, gs, steps, yacc);
-                else consume_stage<BITS, NT, 0, false>(stage, stage_u32, wo, kq, gs, steps, yacc);
+                if (rbits == 2 && whole) consume_stage<BITS, NT, 2, true>(stage_u32, wo, kq, gs, steps, yacc);
+                else if (rbits == 2) consume_stage<BITS, NT, 2, false>(stage_u32, wo, kq, gs, steps, yacc);
+                else if (rbits == 1 && whole) consume_stage<BITS, NT, 1, true>(stage_u32, wo, kq, gs, steps, yacc);
+                else if (rbits == 1) consume_stage<BITS, NT, 1, false>(stage_u32, wo, kq, gs, steps, yacc);
+                else consume_stage<BITS, NT, 0, false>(stage_u32, wo, kq, gs, steps, yacc);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(empty(slot));
             // next slot of the ring
             ++slot;
-            stage += p.stage_bytes;
             stage_u32 += (uint32_t)p.stage_bytes;
             if (slot == p.n_stages) {
                 slot = 0;
                 phase ^= 1u;
-                stage = smem + p.off_ring;
                 stage_u32 = smem0 + (uint32_t)p.off_ring;
             }
         }
@@ -497,9 +480,27 @@ cudaError_t launch_tall(const lopro_desc& d, const uint8_t* blob, const BlobLayo
     long long total_rows = d.d_out;
     if (more != nullptr)
         for (int i = 0; i < more->n; ++i) total_rows += more->d_out[i];
+    const bool alone = more == nullptr || more->n == 0, one_set = option(LOPRO_OPT_ONE_KERNEL_SET) == 1;
+    const bool row_runs = run_supported(d, T);
+    if (const int steps = warp_run_steps(d, T, more)) {
+        // Every warp on a run of its own wherever the activations fit: against this kernel 8192 -> 28672, 2 bits, 1 token 39.0 and
+        // 29.2 us, 4096 -> 28672, 3 bits, 9 tokens 25.0 and 22.4, 1024 -> 28672, 8 tokens 12.5 and 9.0, eight experts of the 2-bit layer 69.8
+        // and 52.9; two layers 1024 -> 2816 of 16 tokens (48 tile steps per CTA) lost 2 percent of their decoder layer.  Against runs of
+        // row tiles it pays its longer way in and out (1.3 us) back with enough steps per CTA: 4096 -> 11008 at 8 and 16 tokens (320) 12.2
+        // and 11.2, 15.8 and 13.5, 5120 -> 5120 at 4 (240) 9.3 and 9.5, 2048 -> 11008 at 16 (160) 9.7 and 9.9, 2048 -> 8192 at 4 (128)
+        // 6.7 and 7.3.  One set of kernels must not depend on who shares the launch: layers that alone may go in runs of row tiles then
+        // stay with this kernel.
+        const int least = T <= 8 ? (row_runs && alone ? 288 : 1) : (row_runs && alone ? 200 : 64);
+        bool take = steps >= least && !(one_set && row_runs);
+        for (int i = 0; one_set && i < (alone ? 0 : more->n); ++i) {
+            lopro_desc di = d;
+            di.d_out = more->d_out[i];
+            take = take && !run_supported(di, T);
+        }
+        if (take) return launch_warp_runs(d, blob, L, ws, W, y, ldy, out_dtype, T, s, t0, more);
+    }
     // (a caller that asks for one set of kernels gets the one that sibling layers use)
-    if ((more == nullptr || more->n == 0) && option(LOPRO_OPT_ONE_KERNEL_SET) != 1 && run_supported(d, T))
-        return launch_stream(d, blob, L, ws, W, y, ldy, out_dtype, T, s, t0, more, true);
+    if (alone && !one_set && row_runs) return launch_stream(d, blob, L, ws, W, y, ldy, out_dtype, T, s, t0, more, true);
     if (!plan_tall(d, T, &pl, total_rows)) return cudaErrorInvalidValue;
     TallParams p;
     p.codes = blob + L.off[LOPRO_SEC_CODES];
