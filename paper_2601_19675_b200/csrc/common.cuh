@@ -220,9 +220,9 @@ cudaError_t launch_tall(const lopro_desc& d, const uint8_t* blob, const BlobLayo
                         const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s, int t0 = 0,
                         const StreamSiblingArgs* more = nullptr);
 
-// The same for up to 16 tokens where the activations fit shared memory: every warp on a run of tile steps of its own.  The first
-// answers how many 16 x 64 tile steps a CTA gets at most, 0 where the kernel does not take the layers.
-int warp_run_steps(const lopro_desc& d, int T, const StreamSiblingArgs* more = nullptr);
+// The same where the activations, or a half of them, fit shared memory: every warp on a run of tile steps of its own.  The first
+// answers how many 16 x 64 tile steps a CTA gets at most, 0 where the kernel does not take the layers, and how many CTAs share K.
+int warp_run_steps(const lopro_desc& d, int T, const StreamSiblingArgs* more, int* cluster);
 cudaError_t launch_warp_runs(const lopro_desc& d, const uint8_t* blob, const BlobLayout& L, const uint8_t* ws,
                              const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s, int t0 = 0,
                              const StreamSiblingArgs* more = nullptr);

@@ -732,8 +732,9 @@ cudaError_t launch_stream(const lopro_desc& d, const uint8_t* blob, const BlobLa
     // of them idle here: 8192 -> 1024, 4 tokens 9.4 and 8.0 us, 8192 -> 2048 9.3 and 8.4) or rows of ten stages and more (11008 -> 4096,
     // 1 token 12.1 and 11.7, 3 bits with the FP8 record, 5 tokens 14.1 and 13.6): every warp on a run of its own.  Shorter rows of more
     // tiles are as fast here (8192 -> 4096, 8 tokens 11.0 and 10.9, 2 bits 9.0 and 9.6).
+    int cluster = 1;
     if (!in_runs && !wide && more == nullptr && T <= 8 && option(LOPRO_OPT_NO_TALL) != 1 && option(LOPRO_OPT_ONE_KERNEL_SET) != 1 &&
-        (d.d_out / 16 <= sm_count() || d.d_in >= 10240) && warp_run_steps(d, T) > 0)
+        (d.d_out / 16 <= sm_count() || d.d_in >= 10240) && warp_run_steps(d, T, nullptr, &cluster) > 0 && cluster == 1)
         return launch_warp_runs(d, blob, L, ws, W, y, ldy, out_dtype, T, s, t0);
     const int rows_per_cta = wide ? 32 : pl.rt * 16;
     int grid = (d.d_out + rows_per_cta - 1) / rows_per_cta;

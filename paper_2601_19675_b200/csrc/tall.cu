@@ -482,15 +482,22 @@ cudaError_t launch_tall(const lopro_desc& d, const uint8_t* blob, const BlobLayo
         for (int i = 0; i < more->n; ++i) total_rows += more->d_out[i];
     const bool alone = more == nullptr || more->n == 0, one_set = option(LOPRO_OPT_ONE_KERNEL_SET) == 1;
     const bool row_runs = run_supported(d, T);
-    if (const int steps = warp_run_steps(d, T, more)) {
-        // Every warp on a run of its own wherever the activations fit: against this kernel 8192 -> 28672, 2 bits, 1 token 39.0 and
-        // 29.2 us, 4096 -> 28672, 3 bits, 9 tokens 25.0 and 22.4, 1024 -> 28672, 8 tokens 12.5 and 9.0, eight experts of the 2-bit layer 69.8
-        // and 52.9; two layers 1024 -> 2816 of 16 tokens (48 tile steps per CTA) lost 2 percent of their decoder layer.  Against runs of
-        // row tiles it pays its longer way in and out (1.3 us) back with enough steps per CTA: 4096 -> 11008 at 8 and 16 tokens (320) 12.2
-        // and 11.2, 15.8 and 13.5, 5120 -> 5120 at 4 (240) 9.3 and 9.5, 2048 -> 11008 at 16 (160) 9.7 and 9.9, 2048 -> 8192 at 4 (128)
-        // 6.7 and 7.3.  One set of kernels must not depend on who shares the launch: layers that alone may go in runs of row tiles then
-        // stay with this kernel.
-        const int least = T <= 8 ? (row_runs && alone ? 288 : 1) : (row_runs && alone ? 200 : 64);
+    int cluster = 1;
+    if (const int steps = warp_run_steps(d, T, more, &cluster)) {
+        // Every warp on a run of its own wherever the activations fit.  Against this kernel: 8192 -> 28672, 2 bits, 1 token 39.0 and
+        // 29.2 us, 4096 -> 28672, 3 bits, 9 tokens 25.0 and 22.4, 1024 -> 28672, 8 tokens 12.5 and 9.0, 32 tokens 21.9 and 14.4, 512 -> 8192,
+        // 32 tokens 9.4 and 7.6, eight experts of the 2-bit layer 69.8 and 52.9; two layers 1024 -> 2816 of 16 tokens (48 tile steps per
+        // CTA) lost 2 percent of their decoder layer.  Against runs of row tiles it pays its longer way in and out (1.3 us) back with enough
+        // steps per CTA: 4096 -> 11008 at 8 and 16 tokens (320) 12.2 and 11.2, 15.8 and 13.5, 5120 -> 5120 at 4 (240) 9.3 and 9.5, 2048 ->
+        // 11008 at 16 (160) 9.7 and 9.9, 2048 -> 8192 at 4 (128) 6.7 and 7.3.  Two CTAs that share K pay another 2 us: 4096 -> 11008 at 32
+        // tokens (320 steps) 23.8 and 19.8, 3072 -> 8192 at 24 (168) 15.5 and 13.3, 4096 -> 4096 at 32 (128) 12.2 and 13.4; 8192 -> 28672,
+        // 2 bits, 16 tokens (1600) 48.8 and 42, 5120 -> 13824 at 16 (480) 19.9 and 18.7, 8192 -> 8192 at 16 (448) 17.3 and 18.1.
+        // One set of kernels must not depend on who shares the launch: layers that alone may go in runs of row tiles then stay with
+        // this kernel.
+        int least = T <= 8 ? 1 : (T <= 16 ? 64 : 1);
+        // (activations beyond 64 records of token and stage arrive too late: 8192 -> 8192, 2 bits, 9 tokens 16.3 and 16.9)
+        if (row_runs && alone) least = T * ((d.d_in + 1023) / 1024) > 64 ? 1 << 30 : (T <= 8 ? 288 : 200);
+        if (cluster > 1) least = T <= 8 ? 640 : (T <= 16 ? 464 : 160);
         bool take = steps >= least && !(one_set && row_runs);
         for (int i = 0; one_set && i < (alone ? 0 : more->n); ++i) {
             lopro_desc di = d;

@@ -1,4 +1,4 @@
-// Small-batch forward (decode, T <= 16) with every warp on a run of its own: y = W^ x~ + A t  (steps "Dequant(W_q) X" and
+// Small-batch forward (decode, T <= 32) with every warp on a run of its own: y = W^ x~ + A t  (steps "Dequant(W_q) X" and
 // "U (Sigma Y)" of Appendix A.3, summed as in Eq. 8), after the prologue kernel that writes the rotated activations x~ (as the
 // stage image), their 64-column sums and t = B x.
 //
@@ -31,6 +31,7 @@ namespace {
 
 constexpr int kWarps = 16;
 constexpr int kMaxX = 32;   // stages of the activation image that a CTA may hold
+constexpr int kRunMaxSmem = 226 * 1024;   // dynamic shared memory of a CTA
 
 struct RunParams {
     const unsigned char* codes;
@@ -45,13 +46,13 @@ struct RunParams {
     int m, T, t_pad;
     int nsteps, gshift, r_pad;
     int lr8;       // the up-projection factor is fp8 e4m3 (U of the FP8 low-rank record), one byte per entry
-    int n_stages;  // of the activation image
+    int n_clusters, cluster;   // units that the layers are shared out to: clusters of CTAs, each CTA a part of K
     // shared-memory layout (bytes from the dynamic base)
     int off_t, off_red, off_x, x_bytes, off_ring;
 };
 
-// Sibling layers of a grouped launch: the grid's CTAs from cta0[i] on work on sibling i (the layer of RunParams
-// owns the CTAs before cta0[0]); each sibling walks its own rows with its own share of the persistent CTAs.
+// Sibling layers of a grouped launch: the grid's clusters from cta0[i] on work on sibling i (the layer of RunParams
+// owns those before cta0[0]); each sibling walks its own rows with its own share of the persistent CTAs.
 struct RunSiblings {
     int n;
     int cta0[kMaxSiblings - 1];
@@ -68,20 +69,18 @@ struct RunSiblings {
 
 // A launch of a single layer carries no table (several hundred bytes of kernel parameters less).
 struct NoRunSiblings {};
-__device__ __forceinline__ int2 select_sibling(RunParams&, const NoRunSiblings&) {
-    return make_int2((int)blockIdx.x, (int)gridDim.x);
-}
+__device__ __forceinline__ int2 select_sibling(RunParams& p, int unit, const NoRunSiblings&) { return make_int2(unit, p.n_clusters); }
 
-// The layer a CTA works on: patches the per-layer fields, returns the CTA's index among the layer's CTAs and
-// their number.
-__device__ __forceinline__ int2 select_sibling(RunParams& p, const RunSiblings& sibs) {
+// The layer that a cluster (a CTA where they are alone) works on: patches the per-layer fields, returns the cluster's index among
+// the layer's and their number.
+__device__ __forceinline__ int2 select_sibling(RunParams& p, int unit, const RunSiblings& sibs) {
     int idx = -1;
 #pragma unroll
     for (int i = 0; i < kMaxSiblings - 1; ++i)
-        if (i < sibs.n && (int)blockIdx.x >= sibs.cta0[i]) idx = i;
-    if (idx < 0) return make_int2((int)blockIdx.x, sibs.n > 0 ? sibs.cta0[0] : (int)gridDim.x);
+        if (i < sibs.n && unit >= sibs.cta0[i]) idx = i;
+    if (idx < 0) return make_int2(unit, sibs.n > 0 ? sibs.cta0[0] : p.n_clusters);
     // (a __grid_constant__ parameter: one constant-bank load per field at a computed index)
-    const int first = sibs.cta0[idx], end = idx + 1 < sibs.n ? sibs.cta0[idx + 1] : (int)gridDim.x;
+    const int first = sibs.cta0[idx], end = idx + 1 < sibs.n ? sibs.cta0[idx + 1] : p.n_clusters;
     p.codes = sibs.codes[idx];
     p.sz = sibs.sz[idx];
     p.A = sibs.A[idx];
@@ -91,7 +90,7 @@ __device__ __forceinline__ int2 select_sibling(RunParams& p, const RunSiblings& 
     p.ldy = sibs.ldy[idx];
     p.m = sibs.m[idx];
     p.T = sibs.T[idx];
-    return make_int2((int)blockIdx.x - first, end - first);
+    return make_int2(unit - first, end - first);
 }
 
 __device__ __forceinline__ void copy16(uint32_t dst, const void* src) {
@@ -132,66 +131,93 @@ __host__ __device__ constexpr int slot_bytes() {
     return PER * (128 * BITS + 64);
 }
 
-template <int BITS, int NT, int PER, int D>
+__device__ __forceinline__ float4 load_from_rank(uint32_t addr, uint32_t rank) {
+    uint32_t there;
+    float4 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(there) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 load_shared(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+
+// CLUSTER: the CTAs of a cluster share their tiles and take a part of K each (rank r of C the batches nb r / C .. nb (r + 1) / C of every
+// tile), so that each holds its part of the activations only; at the end tile t is added up by rank t mod C.
+template <int BITS, int NT, int PER, int D, bool CLUSTER>
 __device__ __forceinline__ void run_body(const RunParams& p, const int2 cta) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t bars[kMaxX + 1];  // full per stage of activations; t
     constexpr int kTok = NT * 8;
     constexpr int kStepBytes = 128 * BITS;               // codes of one 16-row tile and one 64-column step
     constexpr int kSlot = slot_bytes<BITS, PER>(), kBatch = PER * kStepBytes;
-    constexpr int kSum = NT * 128;                       // floats of a warp's sums of a tile
+    static_assert(D * kSlot >= NT * 512, "a warp's last sums go where its ring was");
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int gq = lane >> 2, tg = lane & 3;
-    // this CTA's run of 16-row tiles: the first `extra` CTAs hold one tile more
+    const int C = CLUSTER ? p.cluster : 1, rank = CLUSTER ? (int)blockIdx.x % C : 0;
+    // this cluster's run of 16-row tiles: the first `extra` ones hold one tile more
     const int tiles = p.m >> 4;
     const int base = tiles / cta.y, extra = tiles - base * cta.y;
     const int my_cnt = base + (cta.x < extra ? 1 : 0);
     const int my_start = cta.x * base + min(cta.x, extra);
-    // the warp's batches of PER tile steps, counted along the run
-    const int per_tile = p.nsteps / PER, total = my_cnt * per_tile;
+    // the warp's batches of PER tile steps, counted along the run; k0: the CTA's first step of a tile
+    const int nb = p.nsteps / PER;
+    const int k0 = CLUSTER ? nb * rank / C * PER : 0, per_tile = CLUSTER ? nb * (rank + 1) / C - nb * rank / C : nb, k1 = k0 + per_tile * PER, total = my_cnt * per_tile;
+    const int stage0 = k0 >> 4, n_stages = ((k1 + 15) >> 4) - stage0;
     const int b0 = total * warp / kWarps, b1 = total * (warp + 1) / kWarps;
     const uint32_t bar0 = smem_u32(bars), smem0 = smem_u32(smem);
     const uint32_t tbar = bar0 + 8u * (uint32_t)kMaxX;
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (tid < p.n_stages) mbar_init(bar0 + 8u * (uint32_t)tid, 1);
+    if (tid < n_stages) mbar_init(bar0 + 8u * (uint32_t)tid, 1);
     if (tid == kMaxX) mbar_init(tbar, 1);
     if (tid <= kMaxX) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 
     // ---- the warp's ring ----
-    const uint32_t ring = smem0 + (uint32_t)(p.off_ring + warp * (D * kSlot)), ring_end = ring + D * kSlot;
-    const unsigned char* codes = p.codes + ((size_t)my_start * p.nsteps + (size_t)b0 * PER) * kStepBytes + lane * 16;
+    const uint32_t ring0 = smem0 + (uint32_t)p.off_ring;
+    const uint32_t ring = ring0 + (uint32_t)(warp * (D * kSlot)), ring_end = ring + D * kSlot;
+    int tile = b0 / per_tile, k = k0 + (b0 - tile * per_tile) * PER;   // tile of the run, step of the tile
+    int next = b0, pos = tile * p.nsteps + k, left = per_tile - (b0 - tile * per_tile);   // the next request: its batch, step of the run, batches to the tile's end
+    const unsigned char* codes = p.codes + ((size_t)my_start * p.nsteps + pos) * kStepBytes + lane * 16;
     const unsigned char* sz = p.sz + (size_t)my_start * (size_t)(p.nsteps >> p.gshift) * 64 + lane * 16;
     uint32_t dst = ring + (uint32_t)lane * 16u;
-    int next = b0;
     const bool sz_lane = lane < 4 * (PER >> min(p.gshift, PER == 4 ? 2 : 1));   // the pairs of PER steps: a group or more
     auto request = [&] {
         if (next < b1) {
 #pragma unroll
-            for (int k = 0; k < kBatch; k += 512)
-                if (k + 512 <= kBatch || lane * 16 < kBatch - k) copy16(dst + (uint32_t)k, codes + k);
-            if (sz_lane) copy16(dst + kBatch, sz + (uint32_t)(((next * PER) >> p.gshift) << 6));
+            for (int q = 0; q < kBatch; q += 512)
+                if (q + 512 <= kBatch || lane * 16 < kBatch - q) copy16(dst + (uint32_t)q, codes + q);
+            if (sz_lane) copy16(dst + kBatch, sz + (uint32_t)((pos >> p.gshift) << 6));
             codes += kBatch;
+            pos += PER;
             ++next;
+            if (CLUSTER && --left == 0) {   // on to the next tile's part of K
+                left = per_tile;
+                pos += p.nsteps - (k1 - k0);
+                codes += (p.nsteps - (k1 - k0)) * kStepBytes;
+            }
             dst += kSlot;
             if (dst >= ring_end) dst -= D * kSlot;
         }
         copy_commit();
     };
 #pragma unroll 1
-    for (int k = 0; k < D; ++k) request();
+    for (int q = 0; q < D; ++q) request();
+    const int t0 = rank + C * warp, t_step = C * kWarps;   // the tiles that this warp adds up at the end
     if (lane == 0 && p.r_pad > 0) {   // the rows of A, needed at the end, are on their way to L2
         const uint32_t tile_bytes = (uint32_t)(16 * p.r_pad * (p.lr8 ? 1 : 2));
-        for (int tl = warp; tl < my_cnt; tl += kWarps) prefetch_l2(p.A + (size_t)(my_start + tl) * tile_bytes, tile_bytes);
+        for (int tl = t0; tl < my_cnt; tl += t_step) prefetch_l2(p.A + (size_t)(my_start + tl) * tile_bytes, tile_bytes);
     }
     __syncthreads();
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (lane == 0 && my_cnt > 0) {
         const uint32_t bytes = (uint32_t)(min(kTok, p.T) * kActRecord);
-        for (int s = warp; s < p.n_stages; s += kWarps) {
-            mbar_expect_tx(bar0 + 8u * (uint32_t)s, bytes);
-            bulk_g2s(smem0 + p.off_x + (uint32_t)(s * p.x_bytes), p.act + (size_t)s * p.t_pad * kActRecord, bytes, bar0 + 8u * (uint32_t)s);
+        for (int q = warp; q < n_stages; q += kWarps) {
+            mbar_expect_tx(bar0 + 8u * (uint32_t)q, bytes);
+            bulk_g2s(smem0 + p.off_x + (uint32_t)(q * p.x_bytes), p.act + (size_t)(stage0 + q) * p.t_pad * kActRecord, bytes, bar0 + 8u * (uint32_t)q);
         }
         if (warp == kWarps - 1 && p.r_pad > 0) {  // low-rank intermediate of the live tokens
             const uint32_t t_bytes = (uint32_t)(min(kTok, p.T) * p.r_pad * 2);
@@ -208,17 +234,21 @@ __device__ __forceinline__ void run_body(const RunParams& p, const int2 cta) {
             if (lane == 0) atomicExch(p.status, (int)LOPRO_ERR_TIMEOUT);
         }
     };
-    // sums of a tile: slot (tile of the run) + warp, so that every (warp, tile) pair has one of its own
-    float* red = reinterpret_cast<float*>(smem + p.off_red);
+    // Sums of a tile [token tile][lane] float4: a warp that goes on to the next tile leaves them in the slot of the tile that it ends
+    // (one warp does, at most), a warp that is done where its ring was.
+    auto put = [&](uint32_t to, const float (&v)[NT][4]) {
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+            asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(to + (uint32_t)((nt * 32 + lane) * 16)), "f"(v[nt][0]), "f"(v[nt][1]), "f"(v[nt][2]), "f"(v[nt][3]) : "memory");
+    };
     // from a stage of activations: the lane's ldmatrix row, the column sums of token 2 tg
-    const uint32_t x_ofs = smem0 + (uint32_t)(p.off_x + (lane & 7) * kActRecord + (lane >> 3) * 16);
-    const uint32_t sx_ofs = smem0 + (uint32_t)(p.off_x + 2048 + 2 * tg * kActRecord);
+    const uint32_t x_ofs = smem0 + (uint32_t)(p.off_x + (lane & 7) * kActRecord + (lane >> 3) * 16 - stage0 * p.x_bytes);
+    const uint32_t sx_ofs = smem0 + (uint32_t)(p.off_x + 2048 + 2 * tg * kActRecord - stage0 * p.x_bytes);
     // bytes from the (scale, zero) pairs of a slot's first step to those of the others
     const uint32_t g1 = p.gshift == 0 ? 64u : 0u, g2 = p.gshift == 0 ? 128u : (p.gshift == 1 ? 64u : 0u), g3 = p.gshift == 0 ? 192u : (p.gshift == 1 ? 64u : 0u);
     uint32_t src = ring;   // the slot that is consumed next
     float yacc[NT][4];
-    int tile = b0 / per_tile, k = (b0 - tile * per_tile) * PER;   // tile of the run, step of the tile
-    if (b0 < b1) wait(bar0 + 8u * (uint32_t)(k >> 4));
+    if (b0 < b1) wait(bar0 + 8u * (uint32_t)((k >> 4) - stage0));
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -255,23 +285,22 @@ __device__ __forceinline__ void run_body(const RunParams& p, const int2 cta) {
         __syncwarp();
         request();
         k += PER;
-        if (k == p.nsteps || b == b1 - 1) {
-            // the warp leaves the tile
-            float4* mine = reinterpret_cast<float4*>(red + (tile + warp) * kSum) + lane;
+        if (b == b1 - 1) break;
+        if (k == k1) {
+            put(smem0 + (uint32_t)(p.off_red + tile * (NT * 512)), yacc);
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-                mine[nt * 32] = make_float4(yacc[nt][0], yacc[nt][1], yacc[nt][2], yacc[nt][3]);
+            for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) yacc[nt][i] = 0.0f;
-            }
-            if (k == p.nsteps) {
-                k = 0;
-                ++tile;
-            }
+            k = k0;
+            ++tile;
+            if (k & 15) wait(bar0);
         }
-        if ((k & 15) == 0 && b < b1 - 1) wait(bar0 + 8u * (uint32_t)(k >> 4));
+        if ((k & 15) == 0) wait(bar0 + 8u * (uint32_t)((k >> 4) - stage0));
     }
     copy_wait<0>();
+    __syncwarp();
+    if (b0 < b1) put(ring, yacc);
 
     // ---- a warp per tile adds the warps' sums in order, with the low-rank term A t (fp16 tensor-core product), and stores the rows ----
     const int rp = p.r_pad, row_bytes = rp * (p.lr8 ? 1 : 2);
@@ -292,22 +321,55 @@ __device__ __forceinline__ void run_body(const RunParams& p, const int2 cta) {
         }
     };
     uint32_t a0[4][4];   // the first tile's factor is on its way while the last warps finish
-    if (warp < my_cnt)
+    if (t0 < my_cnt)
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            if (q * 16 < rp) load_a(a0[q], warp, q * 16);
+            if (q * 16 < rp) load_a(a0[q], t0, q * 16);
     __syncthreads();
-    if (rp > 0 && warp < my_cnt) wait(tbar);
+    // this CTA's sums of tile tl, warp by warp
+    auto add_warps = [&](float (&sum)[NT][4], int tl) {
+        const int first = tl * per_tile, last = first + per_tile - 1;
+        int w = first * kWarps / total;
+        while (w > 0 && total * w / kWarps > first) --w;
+        while (total * (w + 1) / kWarps <= first) ++w;
+#pragma unroll 1
+        for (; w < kWarps && total * w / kWarps <= last; ++w) {
+            const int end = total * (w + 1) / kWarps;
+            if (total * w / kWarps == end) continue;   // (a warp without a batch)
+            const uint32_t theirs = (end > last + 1 ? smem0 + (uint32_t)(p.off_red + tl * (NT * 512)) : ring0 + (uint32_t)(w * (D * kSlot))) + (uint32_t)(lane * 16);
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                const float4 v = load_shared(theirs + nt * 512u);
+                sum[nt][0] += v.x;
+                sum[nt][1] += v.y;
+                sum[nt][2] += v.z;
+                sum[nt][3] += v.w;
+            }
+        }
+    };
+    if (CLUSTER) {   // one sum per tile, where the CTA that stores it finds it
+        for (int tl = warp; tl < my_cnt; tl += kWarps) {
+            float sum[NT][4];
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) sum[nt][i] = 0.0f;
+            add_warps(sum, tl);
+            put(smem0 + (uint32_t)(p.off_red + tl * (NT * 512)), sum);
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    if (rp > 0 && t0 < my_cnt) wait(tbar);
     const __half* ts = reinterpret_cast<const __half*>(smem + p.off_t);
 #pragma unroll 1
-    for (int tl = warp; tl < my_cnt; tl += kWarps) {
+    for (int tl = t0; tl < my_cnt; tl += t_step) {
         float sum[NT][4];
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
             for (int i = 0; i < 4; ++i) sum[nt][i] = 0.0f;
         for (int j0 = 0; j0 < rp; j0 += 64) {
-            if (tl != warp || j0 > 0)
+            if (tl != t0 || j0 > 0)
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     if (j0 + q * 16 < rp) load_a(a0[q], tl, j0 + q * 16);
@@ -321,21 +383,17 @@ __device__ __forceinline__ void run_body(const RunParams& p, const int2 cta) {
                     }
                 }
         }
-        // the warps whose pieces meet the tile's batches
-        const int first = tl * per_tile, last = first + per_tile - 1;
-        int w = first * kWarps / total;
-        while (w > 0 && total * w / kWarps > first) --w;
-        while (total * (w + 1) / kWarps <= first) ++w;
-        for (; w < kWarps && total * w / kWarps <= last; ++w) {
-            if (total * w / kWarps == total * (w + 1) / kWarps) continue;   // (a warp without a batch)
-            const float4* theirs = reinterpret_cast<const float4*>(red + (tl + w) * kSum) + lane;
+        if (!CLUSTER) add_warps(sum, tl);
+        for (int r = 0; CLUSTER && r < C; ++r) {
+            float4 v[NT];
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) v[nt] = load_from_rank(smem0 + (uint32_t)(p.off_red + tl * (NT * 512) + (nt * 32 + lane) * 16), (uint32_t)r);
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) {
-                const float4 v = theirs[nt * 32];
-                sum[nt][0] += v.x;
-                sum[nt][1] += v.y;
-                sum[nt][2] += v.z;
-                sum[nt][3] += v.w;
+                sum[nt][0] += v[nt].x;
+                sum[nt][1] += v[nt].y;
+                sum[nt][2] += v[nt].z;
+                sum[nt][3] += v[nt].w;
             }
         }
 #pragma unroll
@@ -350,26 +408,28 @@ __device__ __forceinline__ void run_body(const RunParams& p, const int2 cta) {
                 }
             }
     }
+    // (no CTA leaves while another reads its sums)
+    if (CLUSTER) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-template <int BITS, int NT, int PER, int D, typename SIBS>
+template <int BITS, int NT, int PER, int D, bool CLUSTER, typename SIBS>
 __global__ void __launch_bounds__(kWarps * 32, 1)
 run_kernel(const RunParams p_in, const __grid_constant__ SIBS sibs) {
     RunParams p = p_in;
-    const int2 cta = select_sibling(p, sibs);  // x: index among the layer's CTAs, y: their number
+    const int2 cta = select_sibling(p, CLUSTER ? (int)blockIdx.x / p.cluster : (int)blockIdx.x, sibs);
     // experts of a mixture layer: those with at most eight rows take one token tile although another of the launch needs two
-    if (NT == 2 && sizeof(SIBS) > 1 && p.T <= 8) run_body<BITS, 1, PER, D>(p, cta);
-    else run_body<BITS, NT, PER, D>(p, cta);
+    if (NT == 2 && !CLUSTER && sizeof(SIBS) > 1 && p.T <= 8) run_body<BITS, 1, PER, D, CLUSTER>(p, cta);
+    else run_body<BITS, NT, PER, D, CLUSTER>(p, cta);
 }
 
 struct RunPlan {
-    int nt, per, depth, grid, n_stages, most;   // most: row tiles of a CTA
+    int nt, per, depth, units, cluster, most;   // units: clusters of the grid; most: row tiles of a cluster
     int off_t, off_red, off_x, x_bytes, off_ring, smem_bytes;
     int cta0[kMaxSiblings];
 };
 
 // The persistent CTAs are shared out in proportion to the layers' row tiles (at least one CTA each), a tile with two token tiles
-// counting one and a half: the first CTA of layers 1 .. n and, returned, the most tiles of a CTA.
+// counting one and a half: the first CTA (cluster) of layers 1 .. n and, returned, the most tiles of one.
 int share_ctas(const lopro_desc& d, const StreamSiblingArgs* more, int grid, int* cta0) {
     const int n = more != nullptr ? more->n : 0;
     auto tiles = [&](int i) { return (i == 0 ? d.d_out : more->d_out[i - 1]) / 16; };
@@ -395,74 +455,102 @@ int share_ctas(const lopro_desc& d, const StreamSiblingArgs* more, int grid, int
 }
 
 bool plan_run(const lopro_desc& d, int T, const StreamSiblingArgs* more, RunPlan* pl) {
-    if (T < 1 || T > 16) return false;
-    pl->nt = T <= 8 ? 1 : 2;
-    pl->grid = sm_count();
+    if (T < 1 || T > kDecodeMaxT) return false;
+    pl->nt = T <= 8 ? 1 : (T <= 16 ? 2 : 4);
     const int r_pad = d.rank > 0 ? round_up_int(d.rank, 16) : 0, ktok = pl->nt * 8, nsteps = d.d_in / 64;
-    pl->n_stages = (nsteps + 15) / 16;
-    if (pl->n_stages > kMaxX) return false;
-    pl->most = share_ctas(d, more, pl->grid, pl->cta0);
     pl->x_bytes = T * kActRecord;   // (rows beyond the tokens are read, not used: the last stage has room behind it)
-    const int forms[3][2] = {{4, 3}, {4, 2}, {2, 3}};
-    for (const auto& f : forms) {
-        pl->per = f[0];
-        pl->depth = f[1];
-        if (nsteps % pl->per != 0) continue;
-        int off = 0;
-        pl->off_t = off;
-        off += round_up_int(ktok * r_pad * 2, 128);
-        pl->off_red = off;
-        off += (pl->most + kWarps - 1) * pl->nt * 512;
-        pl->off_ring = off;
-        off += round_up_int(kWarps * pl->depth * pl->per * (128 * d.bits + 64), 128);
-        pl->off_x = off;
-        off += pl->n_stages * pl->x_bytes + (ktok - T) * kActRecord;
-        pl->smem_bytes = off;
-        if (off <= kStreamMaxSmem) return true;
+    const int forms[2][3][2] = {{{4, 3}, {4, 2}, {2, 3}}, {{2, 4}, {2, 3}, {2, 2}}};   // (steps of a batch, batches of a ring)
+    for (int c = 1; c <= 2; c *= 2) {   // CTAs of a cluster: as few as it takes to hold the activations
+        pl->cluster = c;
+        pl->units = sm_count() / c;
+        if (more != nullptr && more->n + 1 > pl->units) continue;
+        pl->most = share_ctas(d, more, pl->units, pl->cta0);
+        for (const auto& f : forms[pl->nt == 4]) {
+            pl->per = f[0];
+            pl->depth = f[1];
+            if (nsteps % pl->per != 0 || nsteps / pl->per < c) continue;
+            if (pl->depth * pl->per * (128 * d.bits + 64) < pl->nt * 512) continue;   // a warp's last sums go where its ring was
+            int stages = 0;   // of activations that a CTA's part of K touches, at most
+            for (int r = 0; r < c; ++r) {
+                const int nb = nsteps / pl->per, k0 = nb * r / c * pl->per, k1 = nb * (r + 1) / c * pl->per, n = (k1 + 15) / 16 - k0 / 16;
+                if (n > stages) stages = n;
+            }
+            if (stages > kMaxX) continue;
+            int off = 0;
+            pl->off_t = off;
+            off += round_up_int(ktok * r_pad * 2, 128);
+            pl->off_red = off;
+            off += pl->most * pl->nt * 512;
+            pl->off_ring = off;
+            off += round_up_int(kWarps * pl->depth * pl->per * (128 * d.bits + 64), 128);
+            pl->off_x = off;
+            off += stages * pl->x_bytes + (ktok - T) * kActRecord;
+            pl->smem_bytes = off;
+            if (off <= kRunMaxSmem) return true;
+        }
     }
     return false;
 }
 
-template <int BITS, int NT, int PER, int D, typename SIBS>
-cudaError_t launch_run_ks(const RunParams& p, const SIBS& sibs, int grid, int smem_bytes, cudaStream_t s) {
+template <int BITS, int NT, int PER, int D, bool CLUSTER, typename SIBS>
+cudaError_t launch_run_ks(const RunParams& p, const SIBS& sibs, const RunPlan& pl, cudaStream_t s) {
     static unsigned long long attr_done = 0;
-    const auto kernel = run_kernel<BITS, NT, PER, D, SIBS>;
-    cudaError_t e = ensure_dynamic_smem(kernel, kStreamMaxSmem, &attr_done);
+    const auto kernel = run_kernel<BITS, NT, PER, D, CLUSTER, SIBS>;
+    cudaError_t e = ensure_dynamic_smem(kernel, kRunMaxSmem, &attr_done);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = dim3(pl.units * pl.cluster);
     cfg.blockDim = dim3(kWarps * 32);
-    cfg.dynamicSmemBytes = smem_bytes;
+    cfg.dynamicSmemBytes = pl.smem_bytes;
     cfg.stream = s;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = pl.cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = CLUSTER ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, p, sibs);
 }
 
+template <int BITS, int NT, int PER, int D, bool CLUSTER>
+cudaError_t launch_run_c(const RunParams& p, const RunSiblings& sibs, const RunPlan& pl, cudaStream_t s) {
+    return sibs.n == 0 && option(LOPRO_OPT_ONE_KERNEL_SET) != 1 ? launch_run_ks<BITS, NT, PER, D, CLUSTER, NoRunSiblings>(p, NoRunSiblings{}, pl, s)
+                       : launch_run_ks<BITS, NT, PER, D, CLUSTER, RunSiblings>(p, sibs, pl, s);
+}
 template <int BITS, int NT, int PER, int D>
-cudaError_t launch_run_k(const RunParams& p, const RunSiblings& sibs, int grid, int smem_bytes, cudaStream_t s) {
-    return sibs.n == 0 && option(LOPRO_OPT_ONE_KERNEL_SET) != 1 ? launch_run_ks<BITS, NT, PER, D, NoRunSiblings>(p, NoRunSiblings{}, grid, smem_bytes, s)
-                       : launch_run_ks<BITS, NT, PER, D, RunSiblings>(p, sibs, grid, smem_bytes, s);
+cudaError_t launch_run_k(const RunParams& p, const RunSiblings& sibs, const RunPlan& pl, cudaStream_t s) {
+    return pl.cluster > 1 ? launch_run_c<BITS, NT, PER, D, true>(p, sibs, pl, s) : launch_run_c<BITS, NT, PER, D, false>(p, sibs, pl, s);
 }
 
 template <int BITS>
 cudaError_t launch_run_bits(const RunParams& p, const RunSiblings& sibs, const RunPlan& pl, cudaStream_t s) {
     if (pl.nt == 1) {
-        if (pl.per == 2) return launch_run_k<BITS, 1, 2, 3>(p, sibs, pl.grid, pl.smem_bytes, s);
-        return pl.depth == 3 ? launch_run_k<BITS, 1, 4, 3>(p, sibs, pl.grid, pl.smem_bytes, s) : launch_run_k<BITS, 1, 4, 2>(p, sibs, pl.grid, pl.smem_bytes, s);
+        if (pl.per == 2) return launch_run_k<BITS, 1, 2, 3>(p, sibs, pl, s);
+        return pl.depth == 3 ? launch_run_k<BITS, 1, 4, 3>(p, sibs, pl, s) : launch_run_k<BITS, 1, 4, 2>(p, sibs, pl, s);
     }
-    if (pl.per == 2) return launch_run_k<BITS, 2, 2, 3>(p, sibs, pl.grid, pl.smem_bytes, s);
-    return pl.depth == 3 ? launch_run_k<BITS, 2, 4, 3>(p, sibs, pl.grid, pl.smem_bytes, s) : launch_run_k<BITS, 2, 4, 2>(p, sibs, pl.grid, pl.smem_bytes, s);
+    if (pl.nt == 2) {
+        if (pl.per == 2) return launch_run_k<BITS, 2, 2, 3>(p, sibs, pl, s);
+        return pl.depth == 3 ? launch_run_k<BITS, 2, 4, 3>(p, sibs, pl, s) : launch_run_k<BITS, 2, 4, 2>(p, sibs, pl, s);
+    }
+    // (a ring has room for the sums of four token tiles)
+    if (pl.depth == 4) return launch_run_k<BITS, 4, 2, 4>(p, sibs, pl, s);
+    if constexpr (3 * slot_bytes<BITS, 2>() >= 2048)
+        if (pl.depth == 3) return launch_run_k<BITS, 4, 2, 3>(p, sibs, pl, s);
+    if constexpr (2 * slot_bytes<BITS, 2>() >= 2048)
+        if (pl.depth == 2) return launch_run_k<BITS, 4, 2, 2>(p, sibs, pl, s);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
-int warp_run_steps(const lopro_desc& d, int T, const StreamSiblingArgs* more) {
+int warp_run_steps(const lopro_desc& d, int T, const StreamSiblingArgs* more, int* cluster) {
     RunPlan pl;
-    return plan_run(d, T, more, &pl) ? pl.most * (d.d_in / 64) : 0;
+    if (!plan_run(d, T, more, &pl)) return 0;
+    *cluster = pl.cluster;
+    return pl.most * (d.d_in / 64) / pl.cluster;
 }
 
 cudaError_t launch_warp_runs(const lopro_desc& d, const uint8_t* blob, const BlobLayout& L, const uint8_t* ws,
@@ -490,7 +578,8 @@ cudaError_t launch_warp_runs(const lopro_desc& d, const uint8_t* blob, const Blo
     p.gshift = gshift;
     p.r_pad = d.rank > 0 ? L.r_pad : 0;
     p.lr8 = d.lowrank_format == LOPRO_LOWRANK_FP8 ? 1 : 0;
-    p.n_stages = pl.n_stages;
+    p.n_clusters = pl.units;
+    p.cluster = pl.cluster;
     p.off_t = pl.off_t;
     p.off_red = pl.off_red;
     p.off_x = pl.off_x;

@@ -29,6 +29,14 @@ def _rows(per_sm, extra):
     (4096, 7, 9, 4, 128, 32, 13),     # four bits and two token tiles: batches of two
     (8192, 13, 3, 2, 64, 64, 2),      # eight stages of activations
     (4096, 40, 11, 2, 2048, 16, 4),   # forty tiles per CTA, groups longer than a stage
+    (512, 2, 3, 4, 64, 16, 32),       # four token tiles
+    (1024, 8, 3, 2, 64, 32, 17),      # two bits: a ring of four batches, where the sums of four token tiles fit
+    (2048, 3, 1, 3, 128, 0, 25),      # no low-rank term
+    (2304, 5, 3, 3, 64, 40, 32),      # two CTAs share K and the second begins in the middle of a stage
+    (4096, 4, 77, 4, 128, 32, 31),    # a ring of two batches of two
+    (4224, 4, 9, 4, 128, 17, 24),     # an odd number of batches of two: the CTAs' parts of K differ
+    (8192, 7, 5, 2, 64, 128, 16),     # two token tiles, eight stages shared by two CTAs
+    (11008, 8, 1, 3, 128, 16, 8),     # one token tile, eleven stages shared by two CTAs
 ])
 def test_runs_of_tile_steps(n, per_sm, extra, bits, g, r, T):
     m = _rows(per_sm, extra)
@@ -58,10 +66,9 @@ def test_long_rows_of_few_tiles(n, m, bits, T):
     _check_forward(layer, d, synth.activations(T, n, seed=T, outlier_frac=0.01), rows=np.arange(0, m, 7))
 
 
-@pytest.mark.parametrize("T", [1, 8, 11])
-def test_siblings_of_unequal_rows(T):
-    # the smallest layer gets a CTA or two, the tallest most of them
-    n = 1024
+@pytest.mark.parametrize("n,T", [(1024, 1), (1024, 8), (1024, 11), (1024, 32), (3072, 30)])
+def test_siblings_of_unequal_rows(n, T):
+    # the smallest layer gets a CTA (at 3072 columns and 30 tokens two that share K) or two, the tallest most of them
     layers, descs, blobs = _siblings(n, (64, _rows(9, 3), 272), 4, 128, 128, 17, seed=T)
     rows = np.arange(0, 64, 5)
     _check_group(layers, descs, blobs, synth.activations(T, n, seed=T + 50, outlier_frac=0.01), rows=rows, shared=True, bit_equal=False)
