@@ -3,6 +3,8 @@
 // down-projection t = B x (Appendix A.3, "Y = V X").
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "ptx.cuh"
 #include "rotate_body.cuh"
@@ -441,8 +443,9 @@ __device__ __forceinline__ void select_prologue_sibling(const PrologueSiblings& 
 
 // KIND of the row CTAs: kRowsPlain, kRowsPaired (two rows of B each), kRowsDeep (few tokens, long rows).
 enum { kRowsPlain, kRowsPaired, kRowsDeep };
-template <bool STAGED, typename SIBS, int KIND = kRowsPlain>
-__global__ void __launch_bounds__(256)
+// TPR: tokens of a row CTA, 0 where they are an argument (one kernel for all, with the registers of eight).
+template <bool STAGED, typename SIBS, int KIND, int TPR>
+__global__ void __launch_bounds__(256, KIND == kRowsPlain ? 1 : 2)
 prologue_kernel(const __nv_bfloat16* __restrict__ x0, int64_t ldx, const int32_t* __restrict__ perm0,
                 const __half* __restrict__ B0, unsigned char* __restrict__ act_image0, __half* __restrict__ t0,
                 int* __restrict__ status, int n, int b_i, int b_h, float inv_sqrt_bh, int r_pad, int t_pad, int T_grid,
@@ -465,24 +468,18 @@ prologue_kernel(const __nv_bfloat16* __restrict__ x0, int64_t ldx, const int32_t
     const int nrow = (int)gridDim.x - (STAGED ? live * ((nchunks + 7) >> 3) : nchunks);
     if ((int)blockIdx.x < nrow) {
         const int rb = (int)blockIdx.x;
-        constexpr bool DEEP = KIND == kRowsDeep;
-        if constexpr (KIND == kRowsPaired) {
-            if (tpr == 8) lowrank_row<8, 2>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
-            else if (tpr == 4) lowrank_row<4, 2>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
-            else lowrank_row<2, 2>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
-            return;
-        }
-        if (lr8.V != nullptr) {
-            if (tpr == 8) lowrank_row_lr8<8, DEEP>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
-            else if (tpr == 4) lowrank_row_lr8<4, DEEP>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
-            else if (tpr == 2) lowrank_row_lr8<2, DEEP>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
-            else lowrank_row_lr8<1, DEEP>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
-            return;
-        }
-        if (tpr == 8) lowrank_row<8, 1, DEEP>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
-        else if (tpr == 4) lowrank_row<4, 1, DEEP>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
-        else if (tpr == 2) lowrank_row<2, 1, DEEP>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
-        else lowrank_row<1, 1, DEEP>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
+        auto rows = [&](auto tokens) {
+            constexpr int N = decltype(tokens)::value;
+            bool fp8 = false;
+            if constexpr (KIND != kRowsPaired) fp8 = lr8.V != nullptr;
+            if (fp8) lowrank_row_lr8<N, KIND == kRowsDeep>(x, ldx, lr8, t, n, r_pad, T, rb, tok0);
+            else lowrank_row<N, KIND == kRowsPaired ? 2 : 1, KIND == kRowsDeep>(x, ldx, B, t, n, r_pad, T, rb, tok0, img);
+        };
+        if constexpr (TPR > 0) rows(std::integral_constant<int, TPR>{});
+        else if (tpr == 8) rows(std::integral_constant<int, 8>{});
+        else if (tpr == 4) rows(std::integral_constant<int, 4>{});
+        else if (tpr == 2) rows(std::integral_constant<int, 2>{});
+        else rows(std::integral_constant<int, 1>{});
         return;
     }
 
@@ -653,7 +650,7 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
     // (measured: with one group of tokens a CTA per (row, token) is best -- 256 CTAs for cfg2 --, with several
     // groups about one CTA per SM)
     const int want = T <= 8 ? 256 : 120;
-    while (tpr > 1 && r_pad * ((live + tpr - 1) / tpr) * ((T + 7) / 8) < want) tpr >>= 1;
+    while (tpr > 1 && r_pad * ((live + tpr - 1) / tpr) * ((T + 7) / 8) * (1 + sibs.n) < want) tpr >>= 1;
     const int groups = (T + 7) / 8;
     int row_ctas = d.rank > 0 ? r_pad * ((live + tpr - 1) / tpr) : 0;
     // rotation: a token's row of x is staged in shared memory and gathered from there; with very few (token,
@@ -676,15 +673,6 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
     // of its own, for its registers).
     const bool deep = groups == 1 && d.d_in >= 8192;
     const int rot_ctas = staged ? live * ((nchunks + 7) / 8) : nchunks;
-    if (staged && (size_t)d.d_in * 2 > 48 * 1024) {  // a row of x beyond the default limit
-        static unsigned long long done[4] = {};
-        cudaError_t e = ensure_dynamic_smem(prologue_kernel<true, PrologueSiblings>, kPrologueMaxSmem, &done[0]);
-        if (e == cudaSuccess) e = ensure_dynamic_smem(prologue_kernel<true, NoPrologueSiblings>, kPrologueMaxSmem, &done[1]);
-        if (e == cudaSuccess) e = ensure_dynamic_smem(prologue_kernel<true, PrologueSiblings, kRowsDeep>, kPrologueMaxSmem, &done[2]);
-        if (e == cudaSuccess) e = ensure_dynamic_smem(prologue_kernel<true, NoPrologueSiblings, kRowsDeep>, kPrologueMaxSmem, &done[3]);
-        // rows this long do not run the paired kernel
-        if (e != cudaSuccess) return e;
-    }
     cfg.gridDim = dim3(row_ctas + rot_ctas, (T + 7) / 8, 1 + sibs.n);
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = staged ? (size_t)d.d_in * 2 : 0;
@@ -695,23 +683,43 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     const int rp = d.rank > 0 ? r_pad : 0;
-    if (sibs.n == 0 && !sibs.own_rows && option(LOPRO_OPT_ONE_KERNEL_SET) != 1) {
-        const NoPrologueSiblings none;
-        if (pairs)
-            return cudaLaunchKernelEx(&cfg, prologue_kernel<true, NoPrologueSiblings, kRowsPaired>, x, ldx, perm, B, act_image, t, status,
-                                      d.d_in, d.identity_cols, d.block_size, inv, rp, t_pad, T, tpr, img, none, lr8);
-        const auto kernel = deep ? (staged ? prologue_kernel<true, NoPrologueSiblings, kRowsDeep> : prologue_kernel<false, NoPrologueSiblings, kRowsDeep>)
-                                 : (staged ? prologue_kernel<true, NoPrologueSiblings> : prologue_kernel<false, NoPrologueSiblings>);
+    auto launch = [&](auto kernel, const auto& siblings_of, unsigned long long* done) -> cudaError_t {
+        if (cfg.dynamicSmemBytes > 48 * 1024) {   // a row of x beyond the default limit
+            const cudaError_t e = ensure_dynamic_smem(kernel, kPrologueMaxSmem, done);
+            if (e != cudaSuccess) return e;
+        }
         return cudaLaunchKernelEx(&cfg, kernel, x, ldx, perm, B, act_image, t, status, d.d_in, d.identity_cols, d.block_size, inv, rp,
-                                  t_pad, T, tpr, img, none, lr8);
-    }
-    if (pairs)
-        return cudaLaunchKernelEx(&cfg, prologue_kernel<true, PrologueSiblings, kRowsPaired>, x, ldx, perm, B, act_image, t, status, d.d_in,
-                                  d.identity_cols, d.block_size, inv, rp, t_pad, T, tpr, img, sibs, lr8);
-    const auto kernel = deep ? (staged ? prologue_kernel<true, PrologueSiblings, kRowsDeep> : prologue_kernel<false, PrologueSiblings, kRowsDeep>)
-                             : (staged ? prologue_kernel<true, PrologueSiblings> : prologue_kernel<false, PrologueSiblings>);
-    return cudaLaunchKernelEx(&cfg, kernel, x, ldx, perm, B, act_image, t, status, d.d_in, d.identity_cols, d.block_size, inv, rp, t_pad,
-                              T, tpr, img, sibs, lr8);
+                                  t_pad, T, tpr, img, siblings_of, lr8);
+    };
+    // A kernel per number of tokens of a row CTA: with one or two it takes 44 to 72 registers instead of 98 to 128, and the CTAs of the
+    // next launch find room beside it (with kernels of their own throughout: decoder layer 4096, 4 sequences 69.4 -> 60.3 us, 2048, 6
+    // sequences 50.6 -> 43.9, 4096 -> 4096 at 1 token 6.5 -> 6.1, 11008 -> 4096 at 8 tokens 14.0 -> 12.9).  A layer alone keeps the common
+    // kernel with more than eight tokens (4096 -> 4096 at 16 tokens 8.5 and 9.0, 4096 -> 11008 12.7 and 13.4) and for long rows of a CTA or
+    // two per multiprocessor (11008 -> 4096 at 4 tokens 11.9 and 12.6).
+    const int ctas = (row_ctas + rot_ctas) * groups;
+    const bool common = sibs.n == 0 && (pairs || (deep && ctas > sm_count() / 2 + 4 && ctas <= 2 * sm_count()));
+    auto by_tokens = [&](auto staged_c, auto kind_c, const auto& siblings_of) -> cudaError_t {
+        constexpr bool S = decltype(staged_c)::value;
+        constexpr int K = decltype(kind_c)::value;
+        using SIBS = std::decay_t<decltype(siblings_of)>;
+        static unsigned long long done[5] = {};
+        if constexpr (K != kRowsPlain)
+            if (common) return launch(prologue_kernel<S, SIBS, K, 0>, siblings_of, &done[4]);
+        if (tpr == 8) return launch(prologue_kernel<S, SIBS, K, 8>, siblings_of, &done[3]);
+        if (tpr == 4) return launch(prologue_kernel<S, SIBS, K, 4>, siblings_of, &done[2]);
+        if (tpr == 2) return launch(prologue_kernel<S, SIBS, K, 2>, siblings_of, &done[1]);
+        return launch(prologue_kernel<S, SIBS, K, 1>, siblings_of, &done[0]);
+    };
+    auto by_kind = [&](const auto& siblings_of) -> cudaError_t {
+        using std::integral_constant;
+        if (pairs) return by_tokens(std::true_type{}, integral_constant<int, kRowsPaired>{}, siblings_of);
+        if (deep) return staged ? by_tokens(std::true_type{}, integral_constant<int, kRowsDeep>{}, siblings_of)
+                                : by_tokens(std::false_type{}, integral_constant<int, kRowsDeep>{}, siblings_of);
+        return staged ? by_tokens(std::true_type{}, integral_constant<int, kRowsPlain>{}, siblings_of)
+                      : by_tokens(std::false_type{}, integral_constant<int, kRowsPlain>{}, siblings_of);
+    };
+    if (sibs.n == 0 && !sibs.own_rows && option(LOPRO_OPT_ONE_KERNEL_SET) != 1) return by_kind(NoPrologueSiblings{});
+    return by_kind(sibs);
 }
 
 cudaError_t launch_lowrank_down(const lopro_desc& d, const __half* B, int r_pad, const __nv_bfloat16* x,

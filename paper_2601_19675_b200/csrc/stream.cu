@@ -352,7 +352,7 @@ constexpr int kWideWarps = 32;
 constexpr int kWideThreads = kWideWarps * 32;
 
 // Partial sums of the 16 step warps of a tile, red[step][token][row] with padded strides: the four token pairs of
-// a warp's store fall into different banks, and so do the four partial sums that a thread adds afterwards.
+// a warp's store fall into different banks, and so do the rows that a warp adds up afterwards.
 constexpr int kRedTok = 36;                 // floats between tokens
 constexpr int kRedStep = 8 * kRedTok + 8;   // floats between steps
 
@@ -494,16 +494,15 @@ stream_wide_kernel(const StreamParams p_in, const __grid_constant__ SIBS sibs) {
         red[step * kRedStep + tk * kRedTok + rl] = yacc[0][i];
     }
     __syncthreads();
-    // four threads per output: each adds four of the 16 partial sums, two shuffles finish
-    {
-        const int o = tid >> 2, part = tid & 3;
-        const int tk = o >> 5, rl = o & 31;
-        const float* src = red + part * kRedStep + tk * kRedTok + rl;
-        float sum = (src[0] + src[4 * kRedStep]) + (src[8 * kRedStep] + src[12 * kRedStep]);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-        if (part == 0 && tk < tc && rl < n_rt * 16) {
-            const size_t idx = (size_t)tk * p.ldy + (size_t)rt0 * 16 + rl;
+    // a warp per token, a row per lane: the token's rows of the tile are one piece of 64 (128) bytes
+    if (warp < tc) {
+        const float* src = red + warp * kRedTok + lane;
+        float part[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) part[q] = (src[q * kRedStep] + src[(q + 4) * kRedStep]) + (src[(q + 8) * kRedStep] + src[(q + 12) * kRedStep]);
+        const float sum = (part[0] + part[1]) + (part[2] + part[3]);
+        if (lane < n_rt * 16) {
+            const size_t idx = (size_t)warp * p.ldy + (size_t)rt0 * 16 + lane;
             if (p.out_f32) reinterpret_cast<float*>(p.y)[idx] = sum;
             else reinterpret_cast<__nv_bfloat16*>(p.y)[idx] = __float2bfloat16_rn(sum);
         }
