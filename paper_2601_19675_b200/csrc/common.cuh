@@ -174,7 +174,8 @@ struct Lr8Args {
 cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __half* B, int r_pad,
                             const __nv_bfloat16* x, int64_t ldx, unsigned char* act_image, __half* t, int t_pad,
                             int* status, int T, cudaStream_t s, const ImageOut* img = nullptr,
-                            const PrologueSiblings* siblings = nullptr, const Lr8Args* lr8 = nullptr);
+                            const PrologueSiblings* siblings = nullptr, const Lr8Args* lr8 = nullptr,
+                            bool other_product = false);   // not for the kernels of stream.cu, warps.cu and tall.cu
 // Plain rotated activations, 64-column sums and t (the general path's outputs) -> operand image.
 cudaError_t launch_image_convert(const lopro_desc& d, const __nv_bfloat16* xrot, const float* s64, int s64_ld,
                                  const __half* t, int r_pad, const ImageOut& img, int T, cudaStream_t s);

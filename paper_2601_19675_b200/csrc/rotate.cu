@@ -445,7 +445,7 @@ __device__ __forceinline__ void select_prologue_sibling(const PrologueSiblings& 
 enum { kRowsPlain, kRowsPaired, kRowsDeep };
 // TPR: tokens of a row CTA, 0 where they are an argument (one kernel for all, with the registers of eight).
 template <bool STAGED, typename SIBS, int KIND, int TPR>
-__global__ void __launch_bounds__(256, KIND == kRowsPlain ? 1 : 2)
+__global__ void __launch_bounds__(256, KIND == kRowsPlain && TPR > 0 ? 1 : 2)
 prologue_kernel(const __nv_bfloat16* __restrict__ x0, int64_t ldx, const int32_t* __restrict__ perm0,
                 const __half* __restrict__ B0, unsigned char* __restrict__ act_image0, __half* __restrict__ t0,
                 int* __restrict__ status, int n, int b_i, int b_h, float inv_sqrt_bh, int r_pad, int t_pad, int T_grid,
@@ -635,7 +635,7 @@ bool prologue_supported(const lopro_desc& d, int T) {
 cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __half* B, int r_pad,
                             const __nv_bfloat16* x, int64_t ldx, unsigned char* act_image, __half* t, int t_pad,
                             int* status, int T, cudaStream_t s, const ImageOut* img_out, const PrologueSiblings* siblings,
-                            const Lr8Args* lr8_args) {
+                            const Lr8Args* lr8_args, bool other_product) {
     const float inv = (float)(1.0 / sqrt((double)d.block_size));
     ImageOut img = {};
     if (img_out != nullptr) img = *img_out;
@@ -695,16 +695,17 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
     // next launch find room beside it (with kernels of their own throughout: decoder layer 4096, 4 sequences 69.4 -> 60.3 us, 2048, 6
     // sequences 50.6 -> 43.9, 4096 -> 4096 at 1 token 6.5 -> 6.1, 11008 -> 4096 at 8 tokens 14.0 -> 12.9).  A layer alone keeps the common
     // kernel with more than eight tokens (4096 -> 4096 at 16 tokens 8.5 and 9.0, 4096 -> 11008 12.7 and 13.4) and for long rows of a CTA or
-    // two per multiprocessor (11008 -> 4096 at 4 tokens 11.9 and 12.6).
+    // two per multiprocessor (11008 -> 4096 at 4 tokens 11.9 and 12.6).  So do the products whose CTAs leave no room for others anyhow:
+    // vector-quantized layers 4096 -> 4096 at 2 and 4 tokens 12.2 and 13.4 us, 12.3 and 12.6 (others gain up to 2.5 percent).
     const int ctas = (row_ctas + rot_ctas) * groups;
-    const bool common = sibs.n == 0 && (pairs || (deep && ctas > sm_count() / 2 + 4 && ctas <= 2 * sm_count()));
+    const bool common = other_product || img.ximg != nullptr ||
+                        (sibs.n == 0 && (pairs || (deep && ctas > sm_count() / 2 + 4 && ctas <= 2 * sm_count())));
     auto by_tokens = [&](auto staged_c, auto kind_c, const auto& siblings_of) -> cudaError_t {
         constexpr bool S = decltype(staged_c)::value;
         constexpr int K = decltype(kind_c)::value;
         using SIBS = std::decay_t<decltype(siblings_of)>;
         static unsigned long long done[5] = {};
-        if constexpr (K != kRowsPlain)
-            if (common) return launch(prologue_kernel<S, SIBS, K, 0>, siblings_of, &done[4]);
+        if (common) return launch(prologue_kernel<S, SIBS, K, 0>, siblings_of, &done[4]);
         if (tpr == 8) return launch(prologue_kernel<S, SIBS, K, 8>, siblings_of, &done[3]);
         if (tpr == 4) return launch(prologue_kernel<S, SIBS, K, 4>, siblings_of, &done[2]);
         if (tpr == 2) return launch(prologue_kernel<S, SIBS, K, 2>, siblings_of, &done[1]);

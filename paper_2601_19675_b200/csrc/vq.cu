@@ -599,7 +599,8 @@ lopro_status lopro_vq_linear_fwd(const lopro_vq_desc* desc, const void* packed, 
     const int t_pad = round_up_int(T, 8);
     if (records) {
         if (launch_prologue(sd, (const int32_t*)(blob + L.off_perm), (const __half*)(blob + L.off_b), L.r_pad,
-                            (const __nv_bfloat16*)x_bf16, ldx, ws + W.off_xrot, tbuf, t_pad, status, T, s) != cudaSuccess)
+                            (const __nv_bfloat16*)x_bf16, ldx, ws + W.off_xrot, tbuf, t_pad, status, T, s, nullptr, nullptr, nullptr,
+                            true) != cudaSuccess)
             return LOPRO_ERR_CUDA;
     } else {
         // the rotation kernels that write no column sums do not reset the status word themselves in every form: clear it here
