@@ -91,7 +91,7 @@ def time_oracle_stack(T, budget_s):
 # the kernels as committed (profiles/: the commands; counters re-read after the last change of each kernel, as ncu
 # prints them, i.e. to 10 kB); null for workloads without a capture.
 NCU_TRAFFIC = {("cfg2_T8", "stream_wide_kernel"): 9290000, ("cfg2_T32", "stream_kernel"): 9490000,
-               ("cfg4_T16", "tall_kernel"): 82610000, ("cfg3_T2048", "prefill_pair_kernel"): 60700000}
+               ("cfg4_T16", "run_kernel or tall_kernel"): 81680000, ("cfg3_T2048", "prefill_pair_kernel"): 60700000}
 METRIC = "quantized-linear fwd tokens/s"
 UNIT = "tokens/s"
 
@@ -551,11 +551,7 @@ def measure(args, name, steps, warmup, rank, world, local, dev, dist, with_e2e=T
     """Builds the workload, times `steps` steps (each a whole number of passes lasting at least args.step_ms) and
     returns the bench record."""
     import torch
-    from paper_2601_19675_b200 import lopro
     w = Workload(args, name, rank, dev)
-    # the stack alternates single-layer and grouped forwards: one set of kernel variants for both (see the switch's
-    # description in lopro.h); every other workload launches single layers only and keeps the default
-    lopro.configure(lopro.OPT_ONE_KERNEL_SET, 1 if w.cfg == "cfg5" else 0)
     stream = torch.cuda.Stream(device=dev)
     with torch.cuda.stream(stream):
         w.verify_pass()
@@ -628,7 +624,7 @@ def measure(args, name, steps, warmup, rank, world, local, dev, dist, with_e2e=T
     value = w.tokens_per_pass * passes * world / (ms_per_step * 1e-3)
     per_forward_s = ms_per_pass * 1e-3 / w.forwards
     # ("tall": none of the workloads is a layer that runs of row tiles take)
-    kernel = " + ".join({"stream": "stream_kernel", "wide": "stream_wide_kernel", "tall": "tall_kernel", "general": "decode_kernel",
+    kernel = " + ".join({"stream": "stream_kernel", "wide": "stream_wide_kernel", "tall": "run_kernel or tall_kernel", "general": "decode_kernel",
                          "prefill": "prefill_pair_kernel" if w.T >= 512 else "prefill_kernel",
                          "rowblock": "rowblock_kernel"}.get(n, n) for n in w.paths)
     note = ("duration = step time / layer forwards (includes the prologue kernels of each forward): an upper bound on the "
@@ -662,9 +658,6 @@ def measure(args, name, steps, warmup, rank, world, local, dev, dist, with_e2e=T
                           d2h_bytes_per_step=w.d2h, steps=e2e_steps,
                           note="one pass per step through the host-buffer entry point (pinned host x in, host y out)")
     rec["_workload"] = w
-    if w.cfg == "cfg5":
-        rec["config"]["one_kernel_set"] = 1
-        lopro.configure(lopro.OPT_ONE_KERNEL_SET, 0)
     return rec
 
 

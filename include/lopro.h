@@ -130,10 +130,10 @@ enum {
                                       their parameters, and which kernel a layer with many rows takes does not depend on
                                       who shares its launch: those that alone could go in runs of row tiles always take the
                                       persistent kernel.  By default a single-layer forward launches variants without
-                                      that table (0.15-0.4 us less per launch of a small layer); a caller that
-                                      alternates single and grouped forwards -- a decoder stack -- then alternates
-                                      between two copies of every kernel, which costs more than the table does
-                                      (measured: 4 % of a 224-layer decode step).  Such callers set this switch. */
+                                      that table (0.15-0.4 us less per launch of a small layer).  For callers that
+                                      want a layer's sums to be the same alone and in a group; it costs speed (the
+                                      224 linears of a 32-layer decoder at 1 and 32 tokens 1.34 -> 1.58 and
+                                      2.83 -> 2.88 ms).                                                           */
     LOPRO_OPT_NO_CTA_PAIRS = 6,  /* 1: the prefill kernel never pairs two CTAs on a tile (tcgen05 cta_group::2)   */
     LOPRO_OPT_COUNT = 7
 };
@@ -244,9 +244,10 @@ LOPRO_API lopro_status lopro_linear_fwd(const lopro_desc* desc, const void* pack
  * measure; the paper's Appendix A.3 lists the steps, not their grouping into launches).
  *   LOPRO_PATH_STREAM   2 launches: prologue (permutation, rotation, B x) + streaming product, T <= 32
  *   LOPRO_PATH_WIDE     the same with the 32-warp variant of the streaming kernel (T <= 8, all of K in the ring)
- *   LOPRO_PATH_TALL     the same with a kernel for layers with many output rows: the persistent streaming kernel or, for
- *                       up to 16 tokens where the rows make even waves of short runs, the streaming kernel with longer
- *                       runs of rows per CTA (not with LOPRO_OPT_ONE_KERNEL_SET)
+ *   LOPRO_PATH_TALL     the same with a kernel for layers with many output rows: one that gives every warp a run of the
+ *                       layer's weights, the persistent streaming kernel or, for up to 16 tokens where the rows make
+ *                       even waves of short runs, the streaming kernel with longer runs of rows per CTA (the last not
+ *                       with LOPRO_OPT_ONE_KERNEL_SET)
  *   LOPRO_PATH_GENERAL  rotation, B x, register-ring product (any shape the descriptor allows)
  *   LOPRO_PATH_PREFILL  rotation, B x (2 launches), tcgen05 product (one CTA per tile, or two with a launch more
  *                       where the last wave's tiles are cut along K), T > 32

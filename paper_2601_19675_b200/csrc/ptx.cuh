@@ -183,8 +183,8 @@ __device__ __forceinline__ void expand_codes(uint32_t (&a)[16], const uint32_t (
 // 14 per tile step, 3 bits: 10 instead of 15).  kOdd is a power of two and comes off with the rows' scale, exactly.  The
 // operands of those rows reach 140 (2 bits) and 184 (3 bits) instead of 131 and 135: the products of one step leave the fp32
 // range where its 64 |x~| add up to 1.8e36 or more (2.5e36 with operands up to 135).  The loops these
-// serve are bound by instruction issue with the integer pipe next; with the packed multiply-adds below 8192 -> 28672 at 2 bits,
-// 16 tokens 51.4 -> 48.8 us, eight experts 4096 -> 14336 at 2 bits 81.4 -> 76.3, 11008 -> 4096 at 3 bits, 5 tokens 14.5 -> 14.0.
+// serve are bound by instruction issue with the integer pipe next; with the packed multiply-adds below, in the kernels that ran them
+// then, 8192 -> 28672 at 2 bits, 16 tokens 51.4 -> 48.8 us (tall.cu), 11008 -> 4096 at 3 bits, 5 tokens 14.5 -> 14.0 (stream.cu).
 template <int BITS>
 struct OddRows {
     static constexpr float factor = BITS == 4 ? 1.0f : (BITS == 2 ? 4.0f : 8.0f);

@@ -638,9 +638,9 @@ bool plan_layout(const lopro_desc& d, StreamPlan* pl, int r_pad, int ng, int kto
 // K has eight stages or more, and with 8 tokens at most: 8192 -> 28672, 2 bits, rank 32, block 128, 4 tokens 37.9 and 34.0,
 // 16 tokens 41.7 and 46.1.  With less than a whole stage of K some of the sixteen warps have no step at all; with nine tokens and
 // more, runs of up to four tiles, which the persistent kernel takes as one group, then stay there (512 -> 8192, 2 bits, 9 tokens
-// 5.8 and 6.0; with five tiles 512 -> 11008, 12 tokens 8.7 and 8.2).  Layers that share a launch stay with the persistent kernel:
-// three layers 4096 -> 4096 alone gained (13.8 and 12.2), the decoder layer of one sequence around them lost (85.1 and 89.4; the
-// reason is not known).
+// 5.8 and 6.0; with five tiles 512 -> 11008, 12 tokens 8.7 and 8.2).  Layers that share a launch never go in runs of row tiles, and
+// layers of many tile steps per multiprocessor go in runs of tile steps per warp instead (warps.cu; the lines between the three are in
+// launch_tall).
 bool plan_run(const lopro_desc& d, int T, StreamPlan* pl, int* ctas) {
     if (T < 1 || T > 16) return false;
     pl->nt = T <= 8 ? 1 : 2;
