@@ -221,7 +221,9 @@ __device__ __forceinline__ void run_body(const RunParams& p, const int2 cta) {
             mbar_expect_tx(bar0 + 8u * (uint32_t)q, bytes);
             bulk_g2s(smem0 + p.off_x + (uint32_t)(q * p.x_bytes), p.act + (size_t)(stage0 + q) * p.t_pad * kActRecord, bytes, bar0 + 8u * (uint32_t)q);
         }
-        if (warp == kWarps - 1 && p.r_pad > 0) {  // low-rank intermediate of the live tokens
+        // low-rank intermediate of the live tokens, where this CTA adds up a tile: nobody else waits for it, and no CTA may leave with
+        // a copy into its shared memory under way (a cluster with one tile: its second CTA adds up none)
+        if (warp == kWarps - 1 && p.r_pad > 0 && rank < my_cnt) {
             const uint32_t t_bytes = (uint32_t)(min(kTok, p.T) * p.r_pad * 2);
             mbar_expect_tx(tbar, t_bytes);
             bulk_g2s(smem0 + p.off_t, p.t, t_bytes, tbar);

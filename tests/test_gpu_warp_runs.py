@@ -74,6 +74,14 @@ def test_siblings_of_unequal_rows(n, T):
     _check_group(layers, descs, blobs, synth.activations(T, n, seed=T + 50, outlier_frac=0.01), rows=rows, shared=True, bit_equal=False)
 
 
+def test_a_sibling_of_one_row_tile_beside_pairs_of_ctas():
+    # the second CTA of the pair that shares the small layer's K adds up no tile: it has no use for the low-rank intermediate, and
+    # must not leave with a copy of it under way
+    layers, descs, blobs = _siblings(4096, (4096, 4096, 16), 4, 128, 128, 32, seed=32)
+    rows = np.unique(np.concatenate([np.arange(16), np.random.default_rng(1).integers(0, 4096, 30)]))
+    _check_group(layers, descs, blobs, synth.activations(32, 4096, seed=3, outlier_frac=0.01), rows=rows, shared=True, bit_equal=False)
+
+
 @pytest.mark.parametrize("counts", [[1, 9, 8, 0, 16, 3], [2] * 8, [9, 1] * 4])
 def test_experts_of_one_and_of_two_token_tiles(counts):
     # in a launch shaped for up to 16 rows the experts with at most eight run the loop of one token tile
