@@ -267,6 +267,27 @@ typedef enum {
 } lopro_path;
 LOPRO_API int32_t lopro_linear_fwd_path(const lopro_desc* desc, int32_t T, int32_t* launches);
 
+/* The product kernel of the launch that serves T <= 32 tokens of one layer in LOPRO_LAYOUT_FRAGMENT (n_layers = 1), of siblings
+ * that share a launch (lopro_linear_fwd_group) or, with `rows`, of up to eight experts with rows[i] >= 1 rows each that share
+ * one (lopro_linear_fwd_experts; every desc the same, T ignored): the paths above tell the launches, this the kernel, for tests
+ * and benchmarks that must know what they ran (no counterpart in the paper).
+ *   LOPRO_PRODUCT_STREAM      runs of up to four row tiles, one wave            (csrc/stream.cu)
+ *   LOPRO_PRODUCT_WIDE        the same, 32 warps                                (csrc/stream.cu)
+ *   LOPRO_PRODUCT_PERSISTENT  persistent CTAs, one ring across tile groups      (csrc/tall.cu)
+ *   LOPRO_PRODUCT_ROW_RUNS    longer runs of row tiles, one or two even waves   (csrc/stream.cu)
+ *   LOPRO_PRODUCT_STEP_RUNS   every warp on a run of tile steps of its own      (csrc/warps.cu)
+ * form (five entries, may be NULL), for the last: token tiles, tile steps of a batch, batches of a warp's ring, CTAs that
+ * share K, most row tiles of such CTAs; zeros for the others.  Returns 0 where no such launch serves the call. */
+typedef enum {
+    LOPRO_PRODUCT_STREAM = 1,
+    LOPRO_PRODUCT_WIDE = 2,
+    LOPRO_PRODUCT_PERSISTENT = 3,
+    LOPRO_PRODUCT_ROW_RUNS = 4,
+    LOPRO_PRODUCT_STEP_RUNS = 5
+} lopro_product;
+LOPRO_API int32_t lopro_product_kernel(int32_t n_layers, const lopro_desc* const* descs, const int32_t* rows, int32_t T,
+                                       int32_t* form);
+
 /* Forward of several SIBLING layers that read the same activations -- the q/k/v projections of an attention block,
  * the gate/up projections of an MLP: y_i[t] = A_i (B_i x[t]) + W^_i (Q^T P_i^T x[t]), each layer with its own
  * permutation (Eq. 5 depends on the layer's residual and Hessian), low-rank factors and codes.  The paper names the

@@ -403,10 +403,24 @@ static bool use_tall(const lopro_desc& d, int T, long long total_rows = 0) {
 }
 // Sibling layers that share their launches: the persistent kernel when their rows together make more than one wave of
 // the per-group kernel (three 4096-row projections do, each alone does not).
-static bool group_uses_tall(int32_t n, const lopro_desc* const* descs, int32_t T) {
+static long long group_rows(int32_t n, const lopro_desc* const* descs) {
     long long rows = 0;
     for (int i = 0; i < n; ++i) rows += descs[i]->d_out;
-    return use_tall(*descs[0], T, rows);
+    return rows;
+}
+
+// The product kernel of a small-batch launch (LOPRO_PRODUCT_*) over the layer and its siblings, whose rows together are total_rows.
+static int product_of(const lopro_desc& d, int T, long long total_rows = 0, const StreamSiblingArgs* more = nullptr) {
+    return use_tall(d, T, total_rows) ? tall_product(d, T, more) : stream_product(d, T, more);
+}
+static cudaError_t launch_product(int product, const lopro_desc& d, const uint8_t* blob, const BlobLayout& L, const uint8_t* ws,
+                                  const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s, int t0 = 0,
+                                  const StreamSiblingArgs* more = nullptr) {
+    switch (product) {
+        case LOPRO_PRODUCT_STEP_RUNS: return launch_warp_runs(d, blob, L, ws, W, y, ldy, out_dtype, T, s, t0, more);
+        case LOPRO_PRODUCT_PERSISTENT: return launch_tall(d, blob, L, ws, W, y, ldy, out_dtype, T, s, t0, more);
+        default: return launch_stream(d, blob, L, ws, W, y, ldy, out_dtype, T, s, t0, more, product == LOPRO_PRODUCT_ROW_RUNS);
+    }
 }
 
 // Token counts a little above the small-batch range run as ONE prologue plus chunks of kDecodeMaxT tokens through the
@@ -458,7 +472,7 @@ int32_t lopro_linear_fwd_path(const lopro_desc* desc, int32_t T, int32_t* launch
         path = use_tall(*desc, kDecodeMaxT) ? LOPRO_PATH_TALL : LOPRO_PATH_STREAM;
         n = 1 + chunks;
     } else if (prologue_supported(*desc, T) && stream_supported(*desc, T)) {
-        path = use_tall(*desc, T) ? LOPRO_PATH_TALL : (stream_uses_wide(*desc, T) ? LOPRO_PATH_WIDE : LOPRO_PATH_STREAM);
+        path = use_tall(*desc, T) ? LOPRO_PATH_TALL : (product_of(*desc, T) == LOPRO_PRODUCT_WIDE ? LOPRO_PATH_WIDE : LOPRO_PATH_STREAM);
         n = 2;
     } else {
         const int pre = (T > kDecodeMaxT && prefill_supported(*desc, T) && rotate_lowrank_supported(*desc, T))
@@ -551,9 +565,8 @@ lopro_status lopro_linear_fwd(const lopro_desc* desc, const void* packed, const 
         for (int c = 0; c < chunks; ++c) {
             const int t0 = c * kDecodeMaxT, tc = T - t0 < kDecodeMaxT ? T - t0 : kDecodeMaxT;
             void* yc = (uint8_t*)y + (size_t)t0 * ldy * esz;
-            const cudaError_t e = use_tall(*desc, tc) ? launch_tall(*desc, blob, L, ws, W, yc, ldy, out_dtype, tc, s, t0)
-                                                      : launch_stream(*desc, blob, L, ws, W, yc, ldy, out_dtype, tc, s, t0);
-            if (e != cudaSuccess) return LOPRO_ERR_CUDA;
+            if (launch_product(product_of(*desc, tc), *desc, blob, L, ws, W, yc, ldy, out_dtype, tc, s, t0) != cudaSuccess)
+                return LOPRO_ERR_CUDA;
         }
         return LOPRO_OK;
     }
@@ -562,9 +575,7 @@ lopro_status lopro_linear_fwd(const lopro_desc* desc, const void* packed, const 
         if (launch_prologue(*desc, perm, B, L.r_pad, (const __nv_bfloat16*)x_bf16, ldx, ws + W.off_xrot,
                             (__half*)(ws + W.off_t), W.t_pad, status, T, s, nullptr, nullptr, &lr8) != cudaSuccess)
             return LOPRO_ERR_CUDA;
-        const cudaError_t e = use_tall(*desc, T) ? launch_tall(*desc, blob, L, ws, W, y, ldy, out_dtype, T, s)
-                                                 : launch_stream(*desc, blob, L, ws, W, y, ldy, out_dtype, T, s);
-        if (e != cudaSuccess) return LOPRO_ERR_CUDA;
+        if (launch_product(product_of(*desc, T), *desc, blob, L, ws, W, y, ldy, out_dtype, T, s) != cudaSuccess) return LOPRO_ERR_CUDA;
         return LOPRO_OK;
     }
     const void* a_f16 = nullptr;  // the up factor where it is not the blob's section
@@ -628,7 +639,7 @@ static bool group_shares_launches(int32_t n, const lopro_desc* const* descs, int
         if (!prologue_supported(d, T)) return false;
     }
     // all siblings through the persistent kernel (by their rows together) or all through the per-group kernel
-    if (!group_uses_tall(n, descs, T))
+    if (!use_tall(d0, T, group_rows(n, descs)))
         for (int i = 0; i < n; ++i)
             if (!stream_supported(*descs[i], T)) return false;
     return true;
@@ -735,9 +746,8 @@ lopro_status lopro_linear_fwd_group(int32_t n_layers, const lopro_desc* const* d
                         L[0].r_pad, (const __nv_bfloat16*)x_bf16, ldx, ws + W.off_xrot, (__half*)(ws + W.off_t), W.t_pad,
                         (int*)(ws + W.off_status), T, s, nullptr, &ps) != cudaSuccess)
         return LOPRO_ERR_CUDA;
-    const cudaError_t e = group_uses_tall(n_layers, descs, T)
-                              ? launch_tall(d0, blob0, L[0], ws, W, y[0], ldy[0], out_dtype, T, s, 0, &ss)
-                              : launch_stream(d0, blob0, L[0], ws, W, y[0], ldy[0], out_dtype, T, s, 0, &ss);
+    const int product = product_of(d0, T, group_rows(n_layers, descs), &ss);
+    const cudaError_t e = launch_product(product, d0, blob0, L[0], ws, W, y[0], ldy[0], out_dtype, T, s, 0, &ss);
     return e == cudaSuccess ? LOPRO_OK : LOPRO_ERR_CUDA;
 }
 
@@ -871,11 +881,43 @@ lopro_status lopro_linear_fwd_experts(const lopro_desc* desc, int32_t n_experts,
                             (int*)(ws0 + W.off_status), max_rows, s, nullptr, &ps) != cudaSuccess)
             return LOPRO_ERR_CUDA;
         void* y0 = rows_of_y(row_offsets[ids[0]]);
-        const cudaError_t err = use_tall(d, max_rows) ? launch_tall(d, blob0, L, ws0, W, y0, ldy, out_dtype, max_rows, s, 0, &ss)
-                                                      : launch_stream(d, blob0, L, ws0, W, y0, ldy, out_dtype, max_rows, s, 0, &ss);
-        if (err != cudaSuccess) return LOPRO_ERR_CUDA;
+        const int product = product_of(d, max_rows, 0, &ss);
+        if (launch_product(product, d, blob0, L, ws0, W, y0, ldy, out_dtype, max_rows, s, 0, &ss) != cudaSuccess) return LOPRO_ERR_CUDA;
     }
     return LOPRO_OK;
+}
+
+int32_t lopro_product_kernel(int32_t n_layers, const lopro_desc* const* descs, const int32_t* rows, int32_t T, int32_t* form) {
+    if (form) memset(form, 0, 5 * sizeof(int32_t));
+    if (n_layers < 1 || n_layers > kMaxSiblings || !descs) return 0;
+    for (int i = 0; i < n_layers; ++i)
+        if (!descs[i] || check_desc(*descs[i]) != LOPRO_OK) return 0;
+    const lopro_desc& d = *descs[0];
+    StreamSiblingArgs ss = {};
+    ss.n = n_layers - 1;
+    for (int i = 1; i < n_layers; ++i) ss.d_out[i - 1] = descs[i]->d_out;
+    long long total_rows = 0;
+    if (rows) {
+        ss.own_rows = 1;
+        T = 0;
+        for (int i = 0; i < n_layers; ++i) {
+            if (rows[i] < 1 || memcmp(descs[i], &d, sizeof(d)) != 0) return 0;
+            ss.T_of[i] = rows[i];
+            if (rows[i] > T) T = rows[i];
+        }
+        if (!experts_share_launches(d, T)) return 0;
+    } else if (n_layers > 1) {
+        if (!group_shares_launches(n_layers, descs, T)) return 0;
+        total_rows = group_rows(n_layers, descs);
+    } else {
+        const int path = T <= kDecodeMaxT ? lopro_linear_fwd_path(&d, T, nullptr) : 0;
+        if (path != LOPRO_PATH_STREAM && path != LOPRO_PATH_WIDE && path != LOPRO_PATH_TALL) return 0;
+    }
+    const StreamSiblingArgs* more = rows || n_layers > 1 ? &ss : nullptr;
+    const int product = product_of(d, T, total_rows, more);
+    int32_t how[5];
+    if (form && product == LOPRO_PRODUCT_STEP_RUNS && warp_run_steps(d, T, more, how) > 0) memcpy(form, how, sizeof(how));
+    return product;
 }
 
 size_t lopro_host_staging_bytes(const lopro_desc* desc, int32_t T, int32_t out_dtype) {

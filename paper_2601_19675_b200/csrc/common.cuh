@@ -193,7 +193,6 @@ cudaError_t launch_decode(const lopro_desc& d, const uint8_t* blob, const BlobLa
                           const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s);
 // Small-batch forward (T <= 32) after launch_prologue: bulk-copy ring, one CTA per 32 output rows.
 bool stream_supported(const lopro_desc& d, int T);
-bool stream_uses_wide(const lopro_desc& d, int T);  // the 32-warp variant of the kernel will run
 // `more`: sibling layers of a grouped launch (same descriptor but for d_out; each with its own blob, workspace
 // region laid out like W, and output) whose row tiles are appended to the grid.
 struct StreamSiblingArgs {
@@ -210,23 +209,27 @@ struct StreamSiblingArgs {
     int T_of[kMaxSiblings];
 };
 cudaError_t launch_stream(const lopro_desc& d, const uint8_t* blob, const BlobLayout& L, const uint8_t* ws,
-                          const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s, int t0 = 0,
-                          const StreamSiblingArgs* more = nullptr, bool in_runs = false);
-// The same kernel for a taller layer alone, in one or two even waves of longer runs of row tiles.
+                          const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s, int t0,
+                          const StreamSiblingArgs* more, bool in_runs);
+// The product kernel (LOPRO_PRODUCT_*) of a launch that the persistent kernel would not take (the first) or would (the second).
+int stream_product(const lopro_desc& d, int T, const StreamSiblingArgs* more);
+int tall_product(const lopro_desc& d, int T, const StreamSiblingArgs* more);
+// in_runs: the same kernel for a taller layer alone, in one or two even waves of longer runs of row tiles.
 bool run_supported(const lopro_desc& d, int T);
 
 // Small-batch forward for tall layers after launch_prologue: persistent CTAs, one ring across tile groups.
 bool tall_supported(const lopro_desc& d, int T, long long total_rows = 0);  // total_rows: of all siblings sharing the launch
 cudaError_t launch_tall(const lopro_desc& d, const uint8_t* blob, const BlobLayout& L, const uint8_t* ws,
-                        const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s, int t0 = 0,
-                        const StreamSiblingArgs* more = nullptr);
+                        const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s, int t0,
+                        const StreamSiblingArgs* more);
 
 // The same where the activations, or a half of them, fit shared memory: every warp on a run of tile steps of its own.  The first
-// answers how many 16 x 64 tile steps a CTA gets at most, 0 where the kernel does not take the layers, and how many CTAs share K.
-int warp_run_steps(const lopro_desc& d, int T, const StreamSiblingArgs* more, int* cluster);
+// answers how many 16 x 64 tile steps a CTA gets at most, 0 where the kernel does not take the layers, and the form of the launch
+// (as lopro_product_kernel reports it).
+int warp_run_steps(const lopro_desc& d, int T, const StreamSiblingArgs* more, int32_t (&form)[5]);
 cudaError_t launch_warp_runs(const lopro_desc& d, const uint8_t* blob, const BlobLayout& L, const uint8_t* ws,
-                             const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s, int t0 = 0,
-                             const StreamSiblingArgs* more = nullptr);
+                             const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s, int t0,
+                             const StreamSiblingArgs* more);
 
 // t = B x on the tensor cores for many tokens; `partial` holds lowrank_mma_scratch_bytes of fp32 K-slice sums.
 int lowrank_mma_slices(const lopro_desc& d, int T, bool compact = false);

@@ -672,14 +672,24 @@ static bool wide_variant(const lopro_desc& d, const StreamPlan& pl) {
            pl.off_stage_x == 2 * kStageSteps * 128 * d.bits;  // the variant's compile-time stage geometry
 }
 
-bool stream_uses_wide(const lopro_desc& d, int T) {
-    StreamPlan pl;
-    return plan_stream(d, T, &pl) && wide_variant(d, pl);
-}
-
 bool stream_supported(const lopro_desc& d, int T) {
     StreamPlan pl;
     return plan_stream(d, T, &pl);
+}
+
+int stream_product(const lopro_desc& d, int T, const StreamSiblingArgs* more) {
+    StreamPlan pl;
+    if (!plan_stream(d, T, &pl)) return 0;
+    if (wide_variant(d, pl)) return LOPRO_PRODUCT_WIDE;
+    // A layer alone of up to eight tokens whose K does not fit the 32-warp kernel, with at most one row tile per multiprocessor (half
+    // of them idle here: 8192 -> 1024, 4 tokens 9.4 and 8.0 us, 8192 -> 2048 9.3 and 8.4) or rows of ten stages and more (11008 -> 4096,
+    // 1 token 12.1 and 11.7, 3 bits with the FP8 record, 5 tokens 14.1 and 13.6): every warp on a run of its own.  Shorter rows of more
+    // tiles are as fast here (8192 -> 4096, 8 tokens 11.0 and 10.9, 2 bits 9.0 and 9.6).
+    int32_t form[5];
+    if (more == nullptr && T <= 8 && option(LOPRO_OPT_NO_TALL) != 1 && option(LOPRO_OPT_ONE_KERNEL_SET) != 1 &&
+        (d.d_out / 16 <= sm_count() || d.d_in >= 10240) && warp_run_steps(d, T, nullptr, form) > 0 && form[3] == 1)
+        return LOPRO_PRODUCT_STEP_RUNS;
+    return LOPRO_PRODUCT_STREAM;
 }
 
 cudaError_t launch_stream(const lopro_desc& d, const uint8_t* blob, const BlobLayout& L, const uint8_t* ws,
@@ -727,14 +737,6 @@ cudaError_t launch_stream(const lopro_desc& d, const uint8_t* blob, const BlobLa
         }
     }
     const bool wide = wide_variant(d, pl);
-    // A layer alone of up to eight tokens whose K does not fit the 32-warp kernel, with at most one row tile per multiprocessor (half
-    // of them idle here: 8192 -> 1024, 4 tokens 9.4 and 8.0 us, 8192 -> 2048 9.3 and 8.4) or rows of ten stages and more (11008 -> 4096,
-    // 1 token 12.1 and 11.7, 3 bits with the FP8 record, 5 tokens 14.1 and 13.6): every warp on a run of its own.  Shorter rows of more
-    // tiles are as fast here (8192 -> 4096, 8 tokens 11.0 and 10.9, 2 bits 9.0 and 9.6).
-    int cluster = 1;
-    if (!in_runs && !wide && more == nullptr && T <= 8 && option(LOPRO_OPT_NO_TALL) != 1 && option(LOPRO_OPT_ONE_KERNEL_SET) != 1 &&
-        (d.d_out / 16 <= sm_count() || d.d_in >= 10240) && warp_run_steps(d, T, nullptr, &cluster) > 0 && cluster == 1)
-        return launch_warp_runs(d, blob, L, ws, W, y, ldy, out_dtype, T, s, t0);
     const int rows_per_cta = wide ? 32 : pl.rt * 16;
     int grid = (d.d_out + rows_per_cta - 1) / rows_per_cta;
     // sibling layers: the CTAs of each follow those of the one before

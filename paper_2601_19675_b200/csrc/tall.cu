@@ -473,17 +473,11 @@ bool tall_supported(const lopro_desc& d, int T, long long total_rows) {
     return plan_tall(d, T, &pl, total_rows);
 }
 
-cudaError_t launch_tall(const lopro_desc& d, const uint8_t* blob, const BlobLayout& L, const uint8_t* ws,
-                        const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s, int t0,
-                        const StreamSiblingArgs* more) {
-    TallPlan pl;
-    long long total_rows = d.d_out;
-    if (more != nullptr)
-        for (int i = 0; i < more->n; ++i) total_rows += more->d_out[i];
+int tall_product(const lopro_desc& d, int T, const StreamSiblingArgs* more) {
     const bool alone = more == nullptr || more->n == 0, one_set = option(LOPRO_OPT_ONE_KERNEL_SET) == 1;
     const bool row_runs = run_supported(d, T);
-    int cluster = 1;
-    if (const int steps = warp_run_steps(d, T, more, &cluster)) {
+    int32_t form[5];
+    if (const int steps = warp_run_steps(d, T, more, form)) {
         // Every warp on a run of its own wherever the activations fit.  Against this kernel: 8192 -> 28672, 2 bits, 1 token 39.0 and
         // 29.2 us, 4096 -> 28672, 3 bits, 9 tokens 25.0 and 22.4, 1024 -> 28672, 8 tokens 12.5 and 9.0, 32 tokens 21.9 and 14.4, 512 -> 8192,
         // 32 tokens 9.4 and 7.6, eight experts of the 2-bit layer 69.8 and 52.9; two layers 1024 -> 2816 of 16 tokens (48 tile steps per
@@ -497,17 +491,26 @@ cudaError_t launch_tall(const lopro_desc& d, const uint8_t* blob, const BlobLayo
         int least = T <= 8 ? 1 : (T <= 16 ? 64 : 1);
         // (activations beyond 64 records of token and stage arrive too late: 8192 -> 8192, 2 bits, 9 tokens 16.3 and 16.9)
         if (row_runs && alone) least = T * ((d.d_in + 1023) / 1024) > 64 ? 1 << 30 : (T <= 8 ? 288 : 200);
-        if (cluster > 1) least = T <= 8 ? 640 : (T <= 16 ? 464 : 160);
+        if (form[3] > 1) least = T <= 8 ? 640 : (T <= 16 ? 464 : 160);
         bool take = steps >= least && !(one_set && row_runs);
         for (int i = 0; one_set && i < (alone ? 0 : more->n); ++i) {
             lopro_desc di = d;
             di.d_out = more->d_out[i];
             take = take && !run_supported(di, T);
         }
-        if (take) return launch_warp_runs(d, blob, L, ws, W, y, ldy, out_dtype, T, s, t0, more);
+        if (take) return LOPRO_PRODUCT_STEP_RUNS;
     }
     // (a caller that asks for one set of kernels gets the one that sibling layers use)
-    if (alone && !one_set && row_runs) return launch_stream(d, blob, L, ws, W, y, ldy, out_dtype, T, s, t0, more, true);
+    return alone && !one_set && row_runs ? LOPRO_PRODUCT_ROW_RUNS : LOPRO_PRODUCT_PERSISTENT;
+}
+
+cudaError_t launch_tall(const lopro_desc& d, const uint8_t* blob, const BlobLayout& L, const uint8_t* ws,
+                        const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s, int t0,
+                        const StreamSiblingArgs* more) {
+    TallPlan pl;
+    long long total_rows = d.d_out;
+    if (more != nullptr)
+        for (int i = 0; i < more->n; ++i) total_rows += more->d_out[i];
     if (!plan_tall(d, T, &pl, total_rows)) return cudaErrorInvalidValue;
     TallParams p;
     p.codes = blob + L.off[LOPRO_SEC_CODES];

@@ -552,10 +552,14 @@ cudaError_t launch_run_bits(const RunParams& p, const RunSiblings& sibs, const R
 
 }  // namespace
 
-int warp_run_steps(const lopro_desc& d, int T, const StreamSiblingArgs* more, int* cluster) {
+int warp_run_steps(const lopro_desc& d, int T, const StreamSiblingArgs* more, int32_t (&form)[5]) {
     RunPlan pl;
     if (!plan_run(d, T, more, &pl)) return 0;
-    *cluster = pl.cluster;
+    form[0] = pl.nt;
+    form[1] = pl.per;
+    form[2] = pl.depth;
+    form[3] = pl.cluster;
+    form[4] = pl.most;
     return pl.most * (d.d_in / 64) / pl.cluster;
 }
 

@@ -33,7 +33,7 @@ SYMBOLS = ["lopro_version", "lopro_status_str", "lopro_check_desc", "lopro_packe
            "lopro_block_add_rmsnorm", "lopro_block_rope_append", "lopro_block_attention_workspace_bytes",
            "lopro_block_attention_decode", "lopro_block_silu_mul", "lopro_experts_workspace_bytes",
            "lopro_linear_fwd_experts_path", "lopro_linear_fwd_experts", "lopro_vq_packed_bytes", "lopro_vq_workspace_bytes",
-           "lopro_vq_pack", "lopro_vq_linear_fwd"]
+           "lopro_vq_pack", "lopro_vq_linear_fwd", "lopro_product_kernel"]
 
 
 class Desc(ctypes.Structure):
@@ -106,6 +106,8 @@ def lib():
         dpp = ctypes.POINTER(ctypes.POINTER(Desc))
         L.lopro_group_workspace_bytes.restype = sz
         L.lopro_group_workspace_bytes.argtypes = [i32, dpp, i32]
+        L.lopro_product_kernel.restype = i32
+        L.lopro_product_kernel.argtypes = [i32, dpp, ctypes.POINTER(i32), i32, ctypes.POINTER(i32)]
         L.lopro_linear_fwd_group_path.restype = i32
         L.lopro_linear_fwd_group_path.argtypes = [i32, dpp, i32, ctypes.POINTER(i32)]
         L.lopro_linear_fwd_group.restype = ctypes.c_int
@@ -556,6 +558,19 @@ def _desc_array(descs):
 
 def group_workspace_bytes(descs, T):
     return int(lib().lopro_group_workspace_bytes(len(descs), _desc_array(descs), int(T)))
+
+
+PRODUCT_STREAM, PRODUCT_WIDE, PRODUCT_PERSISTENT, PRODUCT_ROW_RUNS, PRODUCT_STEP_RUNS = 1, 2, 3, 4, 5
+
+
+def product_kernel(descs, T=0, rows=None):
+    """(kernel, form) of the product launch that serves T <= 32 tokens of one layer, of siblings or, with rows, of experts of
+    rows[i] rows each that share a launch; kernel 0 = no such launch.  form: (token tiles, tile steps of a batch, batches of a
+    warp's ring, CTAs that share K, most row tiles of such CTAs) of PRODUCT_STEP_RUNS, zeros for the others."""
+    form = (ctypes.c_int32 * 5)()
+    n = None if rows is None else (ctypes.c_int32 * len(rows))(*[int(r) for r in rows])
+    kernel = lib().lopro_product_kernel(len(descs), _desc_array(descs), n, int(T), form)
+    return int(kernel), tuple(form)
 
 
 def linear_fwd_group_path(descs, T):

@@ -110,6 +110,27 @@ def test_forward_path_query_names_the_small_batch_and_general_paths():
     assert lopro.linear_fwd_path(bad, 8)[0] == 0
 
 
+def test_product_query_names_the_kernel_of_a_small_batch_launch():
+    def desc(n, m, bits=4, **kw):
+        return lopro.make_desc(n, m, bits, 128, 128, rank=32, **kw)
+
+    none = (0,) * 5
+    d = desc(4096, 4096)
+    assert lopro.product_kernel([d], 8) == (lopro.PRODUCT_WIDE, none)
+    assert lopro.product_kernel([d], 16) == (lopro.PRODUCT_STREAM, none)
+    assert lopro.product_kernel([d], 32) == (lopro.PRODUCT_PERSISTENT, none)
+    assert lopro.product_kernel([desc(5120, 5120)], 2) == (lopro.PRODUCT_ROW_RUNS, none)
+    # 148 multiprocessors without a device: 688 row tiles, five at most
+    assert lopro.product_kernel([desc(4096, 11008)], 8) == (lopro.PRODUCT_STEP_RUNS, (1, 4, 3, 1, 5))
+    assert lopro.product_kernel([d, d, d], 32) == (lopro.PRODUCT_STEP_RUNS, (4, 2, 3, 2, 11))
+    assert lopro.product_kernel([desc(4096, 14336)] * 4, rows=[3, 1, 8, 2])[0] == lopro.PRODUCT_STEP_RUNS
+    # nothing of the kind: other token counts, layouts and layers, a group that shares no launch, an expert without rows
+    for descs, T, rows in (([d], 0, None), ([d], 33, None), ([desc(4096, 4096, layout=lopro.LAYOUT_ROWBLOCK)], 8, None),
+                           ([desc(4096, 4096, 5)], 8, None), ([d, desc(4096, 4096, 3)], 8, None), ([d, d], 0, [4, 0]),
+                           ([d, desc(4096, 4096, 3)], 0, [4, 4]), ([d] * 9, 8, None)):
+        assert lopro.product_kernel(descs, T, rows) == (0, none)
+
+
 def test_null_and_bad_arguments_are_rejected_before_any_cuda_call():
     import ctypes
     L = lopro.lib()
