@@ -118,8 +118,10 @@ enum {
  * initial value of each is read once per process from the environment variable of the same name
  * (LOPRO_NO_WIDE=1, ...); 0 = default behaviour. */
 enum {
-    LOPRO_OPT_NO_WIDE = 0,       /* 1: never the 32-warp variant of the streaming kernel                       */
-    LOPRO_OPT_NO_TALL = 1,       /* 1: never the kernels for layers with many rows (persistent, runs of row tiles) */
+    LOPRO_OPT_NO_WIDE = 0,       /* 1: never the 32-warp variant of the streaming kernel (its layers take the 16-warp
+                                     one, those of at most one row tile per multiprocessor runs of tile steps)     */
+    LOPRO_OPT_NO_TALL = 1,       /* 1: the streaming kernel for every layer: neither the kernels for layers with many
+                                     rows (persistent, runs of row tiles) nor, for any, runs of tile steps          */
     LOPRO_OPT_NO_CHUNKS = 2,     /* 1: token counts above 32 always take the tensor-core (prefill) kernel      */
     LOPRO_OPT_NO_TCGEN05 = 3,    /* 1: never the tcgen05 prefill kernel (general register-ring product)        */
     LOPRO_OPT_PREFILL_PAIRS = 4, /* >= 0: number of two-block row tiles of the prefill grid; where two CTAs share a
@@ -135,7 +137,8 @@ enum {
                                       224 linears of a 32-layer decoder at 1 and 32 tokens 1.34 -> 1.58 and
                                       2.83 -> 2.88 ms).                                                           */
     LOPRO_OPT_NO_CTA_PAIRS = 6,  /* 1: the prefill kernel never pairs two CTAs on a tile (tcgen05 cta_group::2)   */
-    LOPRO_OPT_COUNT = 7
+    LOPRO_OPT_NO_STEP_RUNS = 7,  /* 1: never runs of tile steps per warp (LOPRO_PRODUCT_STEP_RUNS)                  */
+    LOPRO_OPT_COUNT = 8
 };
 /* Sets one switch for the whole process (not thread-safe against forwards running on other host threads).
  * Returns LOPRO_ERR_INVALID_ARG for an unknown option. */

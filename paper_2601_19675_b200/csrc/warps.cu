@@ -554,7 +554,7 @@ cudaError_t launch_run_bits(const RunParams& p, const RunSiblings& sibs, const R
 
 int warp_run_steps(const lopro_desc& d, int T, const StreamSiblingArgs* more, int32_t (&form)[5]) {
     RunPlan pl;
-    if (!plan_run(d, T, more, &pl)) return 0;
+    if (option(LOPRO_OPT_NO_STEP_RUNS) == 1 || !plan_run(d, T, more, &pl)) return 0;
     form[0] = pl.nt;
     form[1] = pl.per;
     form[2] = pl.depth;

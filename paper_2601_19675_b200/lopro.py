@@ -178,7 +178,8 @@ def _calls():
     return _native
 
 
-OPT_NO_WIDE, OPT_NO_TALL, OPT_NO_CHUNKS, OPT_NO_TCGEN05, OPT_PREFILL_PAIRS, OPT_ONE_KERNEL_SET, OPT_NO_CTA_PAIRS = range(7)
+OPT_NO_WIDE, OPT_NO_TALL, OPT_NO_CHUNKS, OPT_NO_TCGEN05, OPT_PREFILL_PAIRS, OPT_ONE_KERNEL_SET, OPT_NO_CTA_PAIRS, \
+    OPT_NO_STEP_RUNS = range(8)
 
 
 def configure(option, value):

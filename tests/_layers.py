@@ -4,7 +4,7 @@ import numpy as np
 import torch
 
 from oracle import lopro_oracle as o
-from paper_2601_19675_b200 import lopro, synth
+from paper_2601_19675_b200 import synth
 
 
 def random_layer_np(d_in, d_out, bits, group_size, rank, seed=0):
@@ -42,11 +42,3 @@ def device_bf16_to_f64(t):
     """Device bf16 tensor -> fp64 numpy via its bit patterns (no torch arithmetic)."""
     bits = t.contiguous().view(torch.int16).cpu().numpy().view(np.uint16)
     return o.bf16_bits_to_f64(bits)
-
-
-def takes_runs_of_row_tiles(d, blob, x):
-    """Whether a tall layer's forward takes the kernel of row-tile runs and not the persistent one, which it always takes under
-    the switch for one kernel set: the two add a row's products in different orders, and each does so in the same one always."""
-    y = lopro.linear_fwd(d, blob, x, lopro.OUT_F32)
-    with lopro.configured(lopro.OPT_ONE_KERNEL_SET, 1):
-        return not torch.equal(lopro.linear_fwd(d, blob, x, lopro.OUT_F32), y)

@@ -85,8 +85,8 @@ def test_attention_projections_of_the_stack_at_full_size(T):
     n = 4096
     layers, descs, blobs = _siblings(n, (4096, 4096, 4096), 4, 128, 128, 32, seed=T)
     rows = np.unique(np.concatenate([[0, 15, 16, 4095, 2048], np.random.default_rng(T).integers(0, 4096, size=24)]))
-    # together the three projections make more than one wave of the per-group kernel, so the group runs through the
-    # persistent kernel while each layer alone does not: same products, another order of summation
+    # together the three projections make more than one wave of the per-group kernel, so the group runs through another
+    # kernel than each layer alone: same products, another order of summation
     _check_group(layers, descs, blobs, synth.activations(T, n, seed=T + 1), rows=rows, shared=True, bit_equal=False)
     with lopro.configured(lopro.OPT_NO_TALL, 1):
         _check_group(layers, descs, blobs, synth.activations(T, n, seed=T + 1), rows=rows, shared=True)
@@ -105,7 +105,11 @@ def test_sibling_layers_through_the_persistent_kernel(T, bits, g, extra):
     ms = tuple(_persistent_rows(e) for e in extra)
     layers, descs, blobs = _siblings(n, ms, bits, g, 128, r, seed=T + bits)
     assert all(lopro.linear_fwd_path(d, T)[0] == lopro.PATH_TALL for d in descs)
-    _check_group(layers, descs, blobs, synth.activations(T, n, seed=T + 50, outlier_frac=0.01), shared=True, bit_equal=False)
+    x_bits = synth.activations(T, n, seed=T + 50, outlier_frac=0.01)
+    with lopro.configured(lopro.OPT_NO_STEP_RUNS, 1):
+        assert lopro.product_kernel(descs, T)[0] == lopro.PRODUCT_PERSISTENT
+        _check_group(layers, descs, blobs, x_bits, shared=True, bit_equal=False)
+    _check_group(layers, descs, blobs, x_bits, shared=True, bit_equal=False)
 
 
 @pytest.mark.parametrize("T", [1, 8, 16])
