@@ -129,13 +129,14 @@ enum {
                                      = none, at most 16; -1: chosen by the library                              */
     LOPRO_OPT_ONE_KERNEL_SET = 5, /* 1: single-layer forwards launch the same kernel variants as grouped ones
                                       (lopro_linear_fwd_group / _experts), which carry a table of sibling layers in
-                                      their parameters, and which kernel a layer with many rows takes does not depend on
-                                      who shares its launch: those that alone could go in runs of row tiles always take the
-                                      persistent kernel.  By default a single-layer forward launches variants without
-                                      that table (0.15-0.4 us less per launch of a small layer).  For callers that
-                                      want a layer's sums to be the same alone and in a group; it costs speed (the
-                                      224 linears of a 32-layer decoder at 1 and 32 tokens 1.34 -> 1.58 and
-                                      2.83 -> 2.88 ms).                                                           */
+                                      their parameters, and layers with many rows always take the persistent kernel, alone
+                                      and in a group: never runs of row tiles or of tile steps.  A layer's sums are then
+                                      taken in one order alone and in a group as long as the runs of rows of a CTA are a
+                                      multiple of the kernel's groups of four row tiles (two with more than 16 tokens) in
+                                      both; elsewhere, and between layers that need the persistent kernel only together,
+                                      they differ in the order of fp32 sums.  By default a single-layer forward launches
+                                      variants without that table (0.15-0.4 us less per launch of a small layer).  The
+                                      switch costs speed, most in groups.                                          */
     LOPRO_OPT_NO_CTA_PAIRS = 6,  /* 1: the prefill kernel never pairs two CTAs on a tile (tcgen05 cta_group::2)   */
     LOPRO_OPT_NO_STEP_RUNS = 7,  /* 1: never runs of tile steps per warp (LOPRO_PRODUCT_STEP_RUNS)                  */
     LOPRO_OPT_COUNT = 8

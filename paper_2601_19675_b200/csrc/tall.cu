@@ -474,8 +474,10 @@ bool tall_supported(const lopro_desc& d, int T, long long total_rows) {
 }
 
 int tall_product(const lopro_desc& d, int T, const StreamSiblingArgs* more) {
-    const bool alone = more == nullptr || more->n == 0, one_set = option(LOPRO_OPT_ONE_KERNEL_SET) == 1;
-    const bool row_runs = run_supported(d, T);
+    // A caller that asks for one set of kernels gets this one alone and in a group: how long the runs are of a CTA that shares
+    // its launch decides, for the other two, which of them is the faster one and, for runs of tile steps, where a row's sum is cut.
+    if (option(LOPRO_OPT_ONE_KERNEL_SET) == 1) return LOPRO_PRODUCT_PERSISTENT;
+    const bool row_runs = (more == nullptr || more->n == 0) && run_supported(d, T);
     int32_t form[5];
     if (const int steps = warp_run_steps(d, T, more, form)) {
         // Every warp on a run of its own wherever the activations fit.  Against this kernel: 8192 -> 28672, 2 bits, 1 token 39.0 and
@@ -486,22 +488,13 @@ int tall_product(const lopro_desc& d, int T, const StreamSiblingArgs* more) {
         // 11008 at 16 (160) 9.7 and 9.9, 2048 -> 8192 at 4 (128) 6.7 and 7.3.  Two CTAs that share K pay another 2 us: 4096 -> 11008 at 32
         // tokens (320 steps) 23.8 and 19.8, 3072 -> 8192 at 24 (168) 15.5 and 13.3, 4096 -> 4096 at 32 (128) 12.2 and 13.4; 8192 -> 28672,
         // 2 bits, 16 tokens (1600) 48.8 and 42, 5120 -> 13824 at 16 (480) 19.9 and 18.7, 8192 -> 8192 at 16 (448) 17.3 and 18.1.
-        // One set of kernels must not depend on who shares the launch: layers that alone may go in runs of row tiles then stay with
-        // this kernel.
         int least = T <= 8 ? 1 : (T <= 16 ? 64 : 1);
         // (activations beyond 64 records of token and stage arrive too late: 8192 -> 8192, 2 bits, 9 tokens 16.3 and 16.9)
-        if (row_runs && alone) least = T * ((d.d_in + 1023) / 1024) > 64 ? 1 << 30 : (T <= 8 ? 288 : 200);
+        if (row_runs) least = T * ((d.d_in + 1023) / 1024) > 64 ? 1 << 30 : (T <= 8 ? 288 : 200);
         if (form[3] > 1) least = T <= 8 ? 640 : (T <= 16 ? 464 : 160);
-        bool take = steps >= least && !(one_set && row_runs);
-        for (int i = 0; one_set && i < (alone ? 0 : more->n); ++i) {
-            lopro_desc di = d;
-            di.d_out = more->d_out[i];
-            take = take && !run_supported(di, T);
-        }
-        if (take) return LOPRO_PRODUCT_STEP_RUNS;
+        if (steps >= least) return LOPRO_PRODUCT_STEP_RUNS;
     }
-    // (a caller that asks for one set of kernels gets the one that sibling layers use)
-    return alone && !one_set && row_runs ? LOPRO_PRODUCT_ROW_RUNS : LOPRO_PRODUCT_PERSISTENT;
+    return row_runs ? LOPRO_PRODUCT_ROW_RUNS : LOPRO_PRODUCT_PERSISTENT;
 }
 
 cudaError_t launch_tall(const lopro_desc& d, const uint8_t* blob, const BlobLayout& L, const uint8_t* ws,

@@ -523,7 +523,7 @@ cudaError_t launch_run_ks(const RunParams& p, const SIBS& sibs, const RunPlan& p
 
 template <int BITS, int NT, int PER, int D, bool CLUSTER>
 cudaError_t launch_run_c(const RunParams& p, const RunSiblings& sibs, const RunPlan& pl, cudaStream_t s) {
-    return sibs.n == 0 && option(LOPRO_OPT_ONE_KERNEL_SET) != 1 ? launch_run_ks<BITS, NT, PER, D, CLUSTER, NoRunSiblings>(p, NoRunSiblings{}, pl, s)
+    return sibs.n == 0 ? launch_run_ks<BITS, NT, PER, D, CLUSTER, NoRunSiblings>(p, NoRunSiblings{}, pl, s)
                        : launch_run_ks<BITS, NT, PER, D, CLUSTER, RunSiblings>(p, sibs, pl, s);
 }
 template <int BITS, int NT, int PER, int D>

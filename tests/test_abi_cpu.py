@@ -1,5 +1,6 @@
 """Host-only checks of the C ABI: the library loads without a GPU, exports every symbol the header
 declares, validates descriptors, and sizes the blob by the storage accounting of Eq. 13."""
+import itertools
 import os
 import re
 
@@ -108,6 +109,18 @@ def test_forward_path_query_names_the_small_batch_and_general_paths():
     assert lopro.linear_fwd_path(lopro.make_desc(4096, 4096, 4, 128, 1024, identity_cols=0, rank=0), 8)[1] == 2
     bad = lopro.make_desc(4096, 4096, 5, 128, 128, rank=32)
     assert lopro.linear_fwd_path(bad, 8)[0] == 0
+
+
+def test_one_kernel_set_takes_one_kernel_alone_and_in_a_group():
+    # wherever the persistent kernel takes a layer alone, it takes the layer in a group and among experts too
+    persistent = (lopro.PRODUCT_PERSISTENT, (0,) * 5)
+    with lopro.configured(lopro.OPT_ONE_KERNEL_SET, 1):
+        for n, m, bits in itertools.product((512, 1024, 3072, 4096, 8192), (4096, 5120, 11008, 28672), (2, 3, 4)):
+            d = lopro.make_desc(n, m, bits, 64, 64, rank=32)
+            for T in (1, 8, 9, 16, 17, 32):
+                if lopro.linear_fwd_path(d, T)[0] == lopro.PATH_TALL:
+                    assert lopro.product_kernel([d], T) == lopro.product_kernel([d, d], T) == persistent
+                    assert lopro.product_kernel([d, d], rows=[T, 1]) == persistent
 
 
 def test_product_query_names_the_kernel_of_a_small_batch_launch():

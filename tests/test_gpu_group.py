@@ -112,14 +112,16 @@ def test_sibling_layers_through_the_persistent_kernel(T, bits, g, extra):
     _check_group(layers, descs, blobs, x_bits, shared=True, bit_equal=False)
 
 
-@pytest.mark.parametrize("T", [1, 8, 16])
-def test_one_kernel_set_gives_single_layers_the_sums_of_a_group(T):
-    # four row tiles per multiprocessor and layer: a CTA owns four alone and eight in the group of two, i.e. whole groups of
-    # four tiles either way, so the persistent kernel adds a row's products in one order -- and another kernel would not
-    n, m = 1024, 16 * 4 * torch.cuda.get_device_properties(0).multi_processor_count
+@pytest.mark.parametrize("T,per_sm", [(1, 4), (8, 4), (16, 4), (1, 8), (7, 12), (16, 8), (17, 2), (24, 4), (32, 8)])
+def test_one_kernel_set_gives_single_layers_the_sums_of_a_group(T, per_sm):
+    # four (eight, twelve) row tiles per multiprocessor and layer: a CTA owns four alone and eight in the group of two, i.e. whole
+    # groups of four tiles (two with more than 16 tokens) either way, so the persistent kernel adds a row's products in one
+    # order -- and another kernel would not
+    n, m = 1024, 16 * per_sm * torch.cuda.get_device_properties(0).multi_processor_count
     layers, descs, blobs = _siblings(n, (m, m), 4, 128, 128, 16, seed=T)
     x = bf16_bits_to_device(synth.activations(T, n, seed=T + 3))
     with lopro.configured(lopro.OPT_ONE_KERNEL_SET, 1):
+        assert lopro.product_kernel(descs, T)[0] == lopro.product_kernel(descs[:1], T)[0] == lopro.PRODUCT_PERSISTENT
         together = lopro.linear_fwd_group(descs, blobs, x, lopro.OUT_F32)
         for d, blob, y in zip(descs, blobs, together):
             assert torch.equal(lopro.linear_fwd(d, blob, x, lopro.OUT_F32), y)
