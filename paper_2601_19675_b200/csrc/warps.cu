@@ -434,12 +434,15 @@ struct RunPlan {
     int cta0[kMaxSiblings];
 };
 
-// The persistent CTAs are shared out in proportion to the layers' row tiles (at least one CTA each), a tile with two token tiles
-// counting one and a half: the first CTA (cluster) of layers 1 .. n and, returned, the most tiles of one.
-int share_ctas(const lopro_desc& d, const StreamSiblingArgs* more, int grid, int* cta0) {
+// The persistent CTAs are shared out in proportion to the layers' row tiles (at least one CTA each): the first CTA (cluster) of layers
+// 1 .. n and, returned, the most tiles of one.  mixed: experts of up to eight rows run the loop of one token tile beside others that run
+// that of two; a tile of the latter counts one and a half.  (Where every layer runs one loop this share left the smaller experts behind:
+// 2048 -> 5632, 4 bits, eight experts of 20 and 4 rows 38.0 us and with even shares 33.8; 8192 -> 5632, 2 bits, 12 and 4 rows, two CTAs
+// sharing K, 73.3 and 60.4.)
+int share_ctas(const lopro_desc& d, const StreamSiblingArgs* more, int grid, bool mixed, int* cta0) {
     const int n = more != nullptr ? more->n : 0;
     auto tiles = [&](int i) { return (i == 0 ? d.d_out : more->d_out[i - 1]) / 16; };
-    auto cost = [&](int i) { return (long long)tiles(i) * (more != nullptr && more->own_rows && more->T_of[i] <= 8 ? 2 : 3); };
+    auto cost = [&](int i) { return (long long)tiles(i) * (mixed && more->T_of[i] <= 8 ? 2 : 3); };
     long long all = 0, before = 0;
     for (int i = 0; i <= n; ++i) all += cost(i);
     int most = 0, from = 0;
@@ -470,7 +473,7 @@ bool plan_run(const lopro_desc& d, int T, const StreamSiblingArgs* more, RunPlan
         pl->cluster = c;
         pl->units = sm_count() / c;
         if (more != nullptr && more->n + 1 > pl->units) continue;
-        pl->most = share_ctas(d, more, pl->units, pl->cta0);
+        pl->most = share_ctas(d, more, pl->units, more != nullptr && more->own_rows && pl->nt == 2 && c == 1, pl->cta0);
         for (const auto& f : forms[pl->nt == 4]) {
             pl->per = f[0];
             pl->depth = f[1];

@@ -123,6 +123,22 @@ def test_one_kernel_set_takes_one_kernel_alone_and_in_a_group():
                     assert lopro.product_kernel([d, d], rows=[T, 1]) == persistent
 
 
+def test_experts_share_ctas_by_the_loop_that_each_runs():
+    # four or eight experts of 352 row tiles on 148 multiprocessors.  Where one of them has more than 16 rows all run the loop of
+    # four token tiles, where none has more than eight that of one: an even share.  Shaped for up to 16 rows, those of up to eight
+    # run the loop of one token tile beside the others, except where two CTAs share K
+    def most(n, m, bits, rows):
+        kernel, form = lopro.product_kernel([lopro.make_desc(n, m, bits, 64, 128, rank=16)] * len(rows), rows=rows)
+        assert kernel == lopro.PRODUCT_STEP_RUNS
+        return form[3:]
+
+    assert most(2048, 5632, 4, [20, 4] * 4) == most(2048, 5632, 4, [20] * 8) == (1, 20)      # 18 CTAs at least
+    assert most(4096, 5632, 2, [20, 4] * 2) == most(4096, 5632, 2, [20] * 4) == (2, 20)      # 18 pairs
+    assert most(2048, 5632, 4, [8, 1] * 4) == most(2048, 5632, 4, [12] * 8) == (1, 20)
+    assert most(2048, 5632, 4, [12, 4] * 4) == (1, 24)                                       # 15 and 22
+    assert most(8192, 5632, 2, [12, 4] * 4) == most(8192, 5632, 2, [12] * 8) == (2, 40)
+
+
 def test_product_query_names_the_kernel_of_a_small_batch_launch():
     def desc(n, m, bits=4, **kw):
         return lopro.make_desc(n, m, bits, 128, 128, rank=32, **kw)
