@@ -6,6 +6,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "prologue_rule.h"
 #include "ptx.cuh"
 #include "rotate_body.cuh"
 #include "rotate_mma.cuh"
@@ -644,45 +645,18 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
     Lr8Args lr8 = {};
     if (lr8_args != nullptr) lr8 = *lr8_args;
     cudaLaunchConfig_t cfg = {};
-    // tokens per row CTA: as few as it takes to fill the SMs
-    const int live = T < 8 ? T : 8;
-    int tpr = 8;
-    // (measured: with one group of tokens a CTA per (row, token) is best -- 256 CTAs for cfg2 --, with several
-    // groups about one CTA per SM)
-    const int want = T <= 8 ? 256 : 120;
-    while (tpr > 1 && r_pad * ((live + tpr - 1) / tpr) * ((T + 7) / 8) * (1 + sibs.n) < want) tpr >>= 1;
-    const int groups = (T + 7) / 8;
-    int row_ctas = d.rank > 0 ? r_pad * ((live + tpr - 1) / tpr) : 0;
-    // rotation: a token's row of x is staged in shared memory and gathered from there; with very few (token,
-    // chunk) pairs the gather straight from global memory, warp = token, is as fast (measured: 6.1 against 6.3 us
-    // per layer forward for one token and 4096 columns, 15.4 against 16.9 us for 8 tokens and 11008 columns)
-    const int nchunks = (d.d_in + 255) / 256;
-    const bool staged = nchunks * live * groups > 64;
-    // More than eight tokens: two rows of B per CTA and half the tokens (as many CTAs as before), or all eight tokens where
-    // that leaves more than one CTA per multiprocessor and all loads of x are in flight at once: fewer reads of x.  Whole
-    // forwards with one row, two rows and half the tokens, two rows and all of them: 2048 -> 1024, 128 rows, 32 tokens 11.9 us,
-    // 11.3, 10.6; 16 tokens (128 CTAs in the last form) 6.8, 6.5, 7.4; 4096 -> 4096, 64 rows, 32 tokens 14.3, 13.5, 13.4.  A
-    // kernel of its own: it takes other numbers of registers.
-    const bool pairs = staged && groups > 1 && tpr >= 4 && lr8.V == nullptr && (size_t)d.d_in * 2 <= 48 * 1024;
-    if (pairs) {
-        if (tpr == 8 && d.d_in <= 4096 && row_ctas * groups * (1 + sibs.n) > 2 * sm_count()) row_ctas /= 2;
-        else tpr /= 2;
-    }
-    // Few tokens of long rows: the passes over a row in flight together (11008 -> 4096 at 8 tokens 13.7 -> 13.4 us for the whole
-    // forward, FP8 record at 5 tokens 14.9 -> 14.5, 8192 columns 9.2 -> 9.1; 5120 columns 10.8 -> 11.0, so not there; also a kernel
-    // of its own, for its registers).
-    const bool deep = groups == 1 && d.d_in >= 8192;
-    const int rot_ctas = staged ? live * ((nchunks + 7) / 8) : nchunks;
-    cfg.gridDim = dim3(row_ctas + rot_ctas, (T + 7) / 8, 1 + sibs.n);
+    const int rp = d.rank > 0 ? r_pad : 0;
+    const PrologueShape sh = prologue_shape(d.d_in, rp, T, 1 + sibs.n, lr8.V != nullptr, other_product || img.ximg != nullptr, sm_count());
+    const int tpr = sh.tpr;
+    cfg.gridDim = dim3(sh.row_ctas + sh.rot_ctas, sh.groups, 1 + sibs.n);
     cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = staged ? (size_t)d.d_in * 2 : 0;
+    cfg.dynamicSmemBytes = sh.staged ? (size_t)d.d_in * 2 : 0;
     cfg.stream = s;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    const int rp = d.rank > 0 ? r_pad : 0;
     auto launch = [&](auto kernel, const auto& siblings_of, unsigned long long* done) -> cudaError_t {
         if (cfg.dynamicSmemBytes > 48 * 1024) {   // a row of x beyond the default limit
             const cudaError_t e = ensure_dynamic_smem(kernel, kPrologueMaxSmem, done);
@@ -691,21 +665,12 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
         return cudaLaunchKernelEx(&cfg, kernel, x, ldx, perm, B, act_image, t, status, d.d_in, d.identity_cols, d.block_size, inv, rp,
                                   t_pad, T, tpr, img, siblings_of, lr8);
     };
-    // A kernel per number of tokens of a row CTA: with one or two it takes 44 to 72 registers instead of 98 to 128, and the CTAs of the
-    // next launch find room beside it (with kernels of their own throughout: decoder layer 4096, 4 sequences 69.4 -> 60.3 us, 2048, 6
-    // sequences 50.6 -> 43.9, 4096 -> 4096 at 1 token 6.5 -> 6.1, 11008 -> 4096 at 8 tokens 14.0 -> 12.9).  A layer alone keeps the common
-    // kernel with more than eight tokens (4096 -> 4096 at 16 tokens 8.5 and 9.0, 4096 -> 11008 12.7 and 13.4) and for long rows of a CTA or
-    // two per multiprocessor (11008 -> 4096 at 4 tokens 11.9 and 12.6).  So do the products whose CTAs leave no room for others anyhow:
-    // vector-quantized layers 4096 -> 4096 at 2 and 4 tokens 12.2 and 13.4 us, 12.3 and 12.6 (others gain up to 2.5 percent).
-    const int ctas = (row_ctas + rot_ctas) * groups;
-    const bool common = other_product || img.ximg != nullptr ||
-                        (sibs.n == 0 && (pairs || (deep && ctas > sm_count() / 2 + 4 && ctas <= 2 * sm_count())));
     auto by_tokens = [&](auto staged_c, auto kind_c, const auto& siblings_of) -> cudaError_t {
         constexpr bool S = decltype(staged_c)::value;
         constexpr int K = decltype(kind_c)::value;
         using SIBS = std::decay_t<decltype(siblings_of)>;
         static unsigned long long done[5] = {};
-        if (common) return launch(prologue_kernel<S, SIBS, K, 0>, siblings_of, &done[4]);
+        if (sh.common) return launch(prologue_kernel<S, SIBS, K, 0>, siblings_of, &done[4]);
         if (tpr == 8) return launch(prologue_kernel<S, SIBS, K, 8>, siblings_of, &done[3]);
         if (tpr == 4) return launch(prologue_kernel<S, SIBS, K, 4>, siblings_of, &done[2]);
         if (tpr == 2) return launch(prologue_kernel<S, SIBS, K, 2>, siblings_of, &done[1]);
@@ -713,11 +678,11 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
     };
     auto by_kind = [&](const auto& siblings_of) -> cudaError_t {
         using std::integral_constant;
-        if (pairs) return by_tokens(std::true_type{}, integral_constant<int, kRowsPaired>{}, siblings_of);
-        if (deep) return staged ? by_tokens(std::true_type{}, integral_constant<int, kRowsDeep>{}, siblings_of)
-                                : by_tokens(std::false_type{}, integral_constant<int, kRowsDeep>{}, siblings_of);
-        return staged ? by_tokens(std::true_type{}, integral_constant<int, kRowsPlain>{}, siblings_of)
-                      : by_tokens(std::false_type{}, integral_constant<int, kRowsPlain>{}, siblings_of);
+        if (sh.pairs) return by_tokens(std::true_type{}, integral_constant<int, kRowsPaired>{}, siblings_of);
+        if (sh.deep) return sh.staged ? by_tokens(std::true_type{}, integral_constant<int, kRowsDeep>{}, siblings_of)
+                                      : by_tokens(std::false_type{}, integral_constant<int, kRowsDeep>{}, siblings_of);
+        return sh.staged ? by_tokens(std::true_type{}, integral_constant<int, kRowsPlain>{}, siblings_of)
+                         : by_tokens(std::false_type{}, integral_constant<int, kRowsPlain>{}, siblings_of);
     };
     if (sibs.n == 0 && !sibs.own_rows && option(LOPRO_OPT_ONE_KERNEL_SET) != 1) return by_kind(NoPrologueSiblings{});
     return by_kind(sibs);

@@ -67,6 +67,15 @@ def test_sibling_layers_share_two_launches(T, bits, g, ms):
     _check_group(layers, descs, blobs, synth.activations(T, n, seed=T + 40, outlier_frac=0.01), shared=True)
 
 
+@pytest.mark.parametrize("n,count,r,T", [(512, 4, 16, 16), (1024, 3, 96, 8), (1024, 3, 96, 5), (4096, 2, 128, 1), (4096, 2, 128, 3),
+                                         (4096, 8, 32, 1), (8192, 2, 128, 8), (8192, 2, 128, 4), (8192, 2, 64, 2), (2048, 3, 32, 16),
+                                         (4096, 3, 32, 32), (2048, 3, 16, 14)])
+def test_row_ctas_of_sibling_layers(n, count, r, T):
+    # the low-rank rows of all siblings in one launch: one, two, four and eight tokens per CTA, two rows per CTA, long rows
+    layers, descs, blobs = _siblings(n, (64, 80, 48, 16, 32, 64, 16, 96)[:count], 4, 64, 64, r, seed=T + r)
+    _check_group(layers, descs, blobs, synth.activations(T, n, seed=T + 60, outlier_frac=0.01), shared=True, bit_equal=n < 8192)
+
+
 def test_groups_that_cannot_share_run_layer_by_layer():
     n = 1024
     # different ranks: no shared launches, same results
