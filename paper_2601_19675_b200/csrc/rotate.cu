@@ -444,9 +444,10 @@ __device__ __forceinline__ void select_prologue_sibling(const PrologueSiblings& 
 
 // KIND of the row CTAs: kRowsPlain, kRowsPaired (two rows of B each), kRowsDeep (few tokens, long rows).
 enum { kRowsPlain, kRowsPaired, kRowsDeep };
-// TPR: tokens of a row CTA, 0 where they are an argument (one kernel for all, with the registers of eight).
+// TPR: tokens of a row CTA, 0 where they are an argument (one kernel for all, with the registers of eight: 96 to 128, none spilled; no
+// bound on the CTAs of a multiprocessor, since one of two made it spill and one of one took 134 to 168).
 template <bool STAGED, typename SIBS, int KIND, int TPR>
-__global__ void __launch_bounds__(256, KIND == kRowsPlain && TPR > 0 ? 1 : 2)
+__global__ void __launch_bounds__(256, TPR == 0 ? 0 : (KIND == kRowsPlain ? 1 : 2))
 prologue_kernel(const __nv_bfloat16* __restrict__ x0, int64_t ldx, const int32_t* __restrict__ perm0,
                 const __half* __restrict__ B0, unsigned char* __restrict__ act_image0, __half* __restrict__ t0,
                 int* __restrict__ status, int n, int b_i, int b_h, float inv_sqrt_bh, int r_pad, int t_pad, int T_grid,
@@ -479,8 +480,8 @@ prologue_kernel(const __nv_bfloat16* __restrict__ x0, int64_t ldx, const int32_t
         if constexpr (TPR > 0) rows(std::integral_constant<int, TPR>{});
         else if (tpr == 8) rows(std::integral_constant<int, 8>{});
         else if (tpr == 4) rows(std::integral_constant<int, 4>{});
-        else if (tpr == 2) rows(std::integral_constant<int, 2>{});
-        else rows(std::integral_constant<int, 1>{});
+        else if (KIND == kRowsPaired || tpr == 2) rows(std::integral_constant<int, 2>{});
+        else if constexpr (KIND != kRowsPaired) rows(std::integral_constant<int, 1>{});
         return;
     }
 

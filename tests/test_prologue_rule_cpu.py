@@ -2,10 +2,13 @@
 range of widths, ranks, token counts and layers of a launch."""
 import itertools
 import os
+import re
 import subprocess
 from collections import namedtuple
 
 import pytest
+
+from paper_2601_19675_b200 import build
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2601_19675_b200", "csrc")
@@ -51,3 +54,25 @@ def test_row_ctas_cover_every_row_and_token_once(shapes):
 def test_a_row_cta_has_no_loop_for_tokens_that_are_absent(shapes):
     for a, s in shapes.items():
         assert s.tpr < 2 * min(a.T, 8)
+
+
+@pytest.fixture(scope="module")
+def kernels(tmp_path_factory):
+    """{(staged, siblings, kind, tokens of a row CTA): (registers, bytes spilled)} of the prologue kernels, as the assembler reports."""
+    obj = tmp_path_factory.mktemp("obj") / "rotate.o"
+    run = [build._nvcc(), *build.NVCC_FLAGS, "-Xptxas", "-v", "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-c",
+           os.path.join(CSRC, "rotate.cu"), "-o", str(obj)]
+    text = subprocess.run(run, check=True, capture_output=True, text=True).stderr
+    found = {}
+    for name, stores, loads, regs in re.findall(r"entry function '(\S*prologue_kernel\S*)'.*?(\d+) bytes spill stores, (\d+) bytes spill loads"
+                                                r".*?Used (\d+) registers", text, re.S):
+        staged, none, kind, tpr = re.search(r"prologue_kernelILb([01])E\S*?(No)?PrologueSiblingsELi(\d)ELi(\d)E", name).groups()
+        found[int(staged), none is None, ("plain", "paired", "deep")[int(kind)], int(tpr)] = (int(regs), int(stores) + int(loads))
+    assert found
+    return found
+
+
+def test_the_common_prologue_kernels_spill_nothing_and_run_two_to_a_multiprocessor(kernels):
+    for name, (regs, spilled) in kernels.items():
+        if name[3] == 0:
+            assert spilled == 0 and regs <= 128, name
