@@ -57,6 +57,12 @@ inline PrologueShape prologue_shape(int d_in, int r_pad, int T, int layers, bool
     // vector-quantized layers 4096 -> 4096 at 2 and 4 tokens 12.2 and 13.4 us, 12.3 and 12.6 (others gain up to 2.5 percent).
     const int ctas = (s.row_ctas + s.rot_ctas) * s.groups;
     s.common = other_product || (layers == 1 && (s.pairs || (s.deep && ctas > sms / 2 + 4 && ctas <= 2 * sms)));
+    // The loop of eight tokens by itself takes 165 registers, so that a multiprocessor holds one CTA, against two of the common kernel:
+    // only where the last row CTA of the launch is among the first that start (the rotation's CTAs come after the rows' and end soon).
+    // 4096 -> 4096, FP8 record, 16 tokens by itself and in common: rank 64 (the last row CTA is number 144) 10.1 us and 10.5, 80 (176)
+    // 11.6 and 10.6, 128 (272) 12.7 and 11.1; 512 -> 4096, 32 tokens, rank 32 (134) 6.9 and 7.4, 64 (262) 8.5 and 7.9; three layers
+    // 4096 -> 4096, rank 128, 8 tokens 17.9 and 16.2.  With two rows of B per CTA and for long rows it has nothing over the common kernel.
+    if (s.tpr == 8 && (s.pairs || s.deep || ctas * layers - s.rot_ctas > sms)) s.common = true;
     return s;
 }
 

@@ -672,7 +672,8 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
         using SIBS = std::decay_t<decltype(siblings_of)>;
         static unsigned long long done[5] = {};
         if (sh.common) return launch(prologue_kernel<S, SIBS, K, 0>, siblings_of, &done[4]);
-        if (tpr == 8) return launch(prologue_kernel<S, SIBS, K, 8>, siblings_of, &done[3]);
+        if constexpr (K == kRowsPlain)
+            if (tpr == 8) return launch(prologue_kernel<S, SIBS, K, 8>, siblings_of, &done[3]);
         if (tpr == 4) return launch(prologue_kernel<S, SIBS, K, 4>, siblings_of, &done[2]);
         if (tpr == 2) return launch(prologue_kernel<S, SIBS, K, 2>, siblings_of, &done[1]);
         return launch(prologue_kernel<S, SIBS, K, 1>, siblings_of, &done[0]);

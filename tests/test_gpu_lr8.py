@@ -176,6 +176,18 @@ def test_forward_with_the_fp8_record(T, bits, g, r, m):
     _check(d, layer, rec, synth.activations(T, n, seed=T + 1, outlier_frac=0.01), rows=rows)
 
 
+@pytest.mark.parametrize("n,r,T", [(2048, 64, 9), (2048, 64, 16), (2048, 80, 16), (4096, 48, 24), (8192, 16, 1), (8192, 64, 5), (8192, 128, 8),
+                                   (11008, 16, 5)])
+def test_row_ctas_with_the_fp8_record(n, r, T):
+    # the low-rank rows: eight tokens per CTA by a kernel of its own and by the common one, long rows
+    m = 48
+    layer = random_layer_np(n, m, 4, 128, 0, seed=T + r)
+    rec = synth.lowrank_record(m, n, r, seed=T + r)
+    rec["sigma"] = synth.f32_to_f16_bits(np.float32(40.0) * o.f16_bits_to_f64(rec["sigma"]).astype(np.float32))
+    d = lopro.make_desc(n, m, 4, 128, 128, rank=r, lowrank_format=lopro.LOWRANK_FP8)
+    _check(d, layer, rec, synth.activations(T, n, seed=T + 1, outlier_frac=0.01))
+
+
 @pytest.mark.parametrize("n,m,bits,g,r,T", [(1024, 256, 4, 128, 16, 300), (2048, 400, 3, 64, 33, 130), (1024, 384, 2, 64, 128, 700)])
 def test_many_tokens_with_the_fp8_record_run_on_the_tensor_core_kernels(n, m, bits, g, r, T):
     # the record is folded into fp16 factors in the workspace (one more launch), then the same kernels as for a folded layer

@@ -56,6 +56,15 @@ def test_a_row_cta_has_no_loop_for_tokens_that_are_absent(shapes):
         assert s.tpr < 2 * min(a.T, 8)
 
 
+def test_the_loop_of_eight_tokens_by_itself_runs_where_every_row_cta_starts_at_once(shapes):
+    # (it leaves room for one CTA per multiprocessor); rows come before rotation within a layer and group of eight tokens
+    own = {a: s for a, s in shapes.items() if s.tpr == 8 and not s.common}
+    assert own
+    for a, s in own.items():
+        assert (s.row_ctas + s.rot_ctas) * s.groups * a.layers - s.rot_ctas <= SMS
+        assert not s.pairs and not s.deep
+
+
 @pytest.fixture(scope="module")
 def kernels(tmp_path_factory):
     """{(staged, siblings, kind, tokens of a row CTA): (registers, bytes spilled)} of the prologue kernels, as the assembler reports."""
