@@ -49,14 +49,21 @@ inline PrologueShape prologue_shape(int d_in, int r_pad, int T, int layers, bool
     // of its own, for its registers).
     s.deep = s.groups == 1 && d_in >= 8192;
     s.rot_ctas = s.staged ? live * ((nchunks + 7) / 8) : nchunks;
-    // A kernel per number of tokens of a row CTA: with one or two it takes 44 to 72 registers instead of 98 to 128, and the CTAs of the
+    // A kernel per number of tokens of a row CTA: with one or two it takes 54 to 92 registers instead of 96 to 128, and the CTAs of the
     // next launch find room beside it (with kernels of their own throughout: decoder layer 4096, 4 sequences 69.4 -> 60.3 us, 2048, 6
-    // sequences 50.6 -> 43.9, 4096 -> 4096 at 1 token 6.5 -> 6.1, 11008 -> 4096 at 8 tokens 14.0 -> 12.9).  A layer alone keeps the common
-    // kernel with more than eight tokens (4096 -> 4096 at 16 tokens 8.5 and 9.0, 4096 -> 11008 12.7 and 13.4) and for long rows of a CTA or
-    // two per multiprocessor (11008 -> 4096 at 4 tokens 11.9 and 12.6).  So do the products whose CTAs leave no room for others anyhow:
-    // vector-quantized layers 4096 -> 4096 at 2 and 4 tokens 12.2 and 13.4 us, 12.3 and 12.6 (others gain up to 2.5 percent).
+    // sequences 50.6 -> 43.9, 4096 -> 4096 at 1 token 6.5 -> 6.1, 11008 -> 4096 at 8 tokens 14.0 -> 12.9).  The common kernel stays
+    //  * for two rows of B per CTA and a layer alone (4096 -> 4096 at 16 tokens 8.5 and 9.0, 4096 -> 11008 12.7 and 13.4);
+    //  * for long rows of the FP8 record: 11008 -> 4096 at 1, 2, 3, 4 and 5 tokens, ranks 16 to 64, 12.5 to 14.0 us and 13.0 to 14.3 alone,
+    //    within one percent either way as part of a decoder layer.  With folded factors it gains as much on most long rows alone (8192 to
+    //    14336 columns, 1 to 4 tokens 0 to 4 percent; at 8 tokens it loses as often), but costs the layer around it more: decoder
+    //    layer 4096 of 1 and 4 sequences 63.9 us and 65.5, 60.3 and 62.2, 3072 with a gate of 10240 at 2 sequences 51.4 and 53.4;
+    //  * in front of products whose CTAs leave no room for others anyhow: vector-quantized layers 4096 -> 4096 at 2 and 4 tokens
+    //    12.2 and 13.4 us, 12.3 and 12.6 (others gain up to 2.5 percent).
+    // Layers alone that lose by their own kernels, and win as part of a decoder layer: one or two tokens whose product goes in runs of
+    // row tiles (5120 -> 5120, rank 64, 2 tokens 8.9 and 9.3; decoder layer 5120 80.9 and 77.6), 9 to 16 tokens of rank 16 (512 -> 4096,
+    // 16 tokens 4.6 and 5.2; decoder layer 1024 of 16 sequences 37.8 and 36.8, 4096 of 12 84.2 and 80.5).
     const int ctas = (s.row_ctas + s.rot_ctas) * s.groups;
-    s.common = other_product || (layers == 1 && (s.pairs || (s.deep && ctas > sms / 2 + 4 && ctas <= 2 * sms)));
+    s.common = other_product || (s.pairs && layers == 1) || (s.deep && fp8);
     // The loop of eight tokens by itself takes 165 registers, so that a multiprocessor holds one CTA, against two of the common kernel:
     // only where the last row CTA of the launch is among the first that start (the rotation's CTAs come after the rows' and end soon).
     // 4096 -> 4096, FP8 record, 16 tokens by itself and in common: rank 64 (the last row CTA is number 144) 10.1 us and 10.5, 80 (176)

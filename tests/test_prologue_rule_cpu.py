@@ -65,6 +65,12 @@ def test_the_loop_of_eight_tokens_by_itself_runs_where_every_row_cta_starts_at_o
         assert not s.pairs and not s.deep
 
 
+def test_the_kernel_of_long_rows_does_not_depend_on_how_many_ctas_there_are(shapes):
+    for a, s in shapes.items():
+        if s.deep and s.tpr < 8 and not a.other:
+            assert s.common == bool(a.fp8)
+
+
 @pytest.fixture(scope="module")
 def kernels(tmp_path_factory):
     """{(staged, siblings, kind, tokens of a row CTA): (registers, bytes spilled)} of the prologue kernels, as the assembler reports."""
