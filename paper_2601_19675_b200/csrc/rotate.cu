@@ -670,13 +670,19 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
         constexpr bool S = decltype(staged_c)::value;
         constexpr int K = decltype(kind_c)::value;
         using SIBS = std::decay_t<decltype(siblings_of)>;
+        // (no layer alone has two rows of B per CTA in a kernel of its own; those have two tokens at least, and rows that are long and
+        // not staged two at most)
+        constexpr bool own = K != kRowsPaired || !std::is_same_v<SIBS, NoPrologueSiblings>;
         static unsigned long long done[5] = {};
-        if (sh.common) return launch(prologue_kernel<S, SIBS, K, 0>, siblings_of, &done[4]);
-        if constexpr (K == kRowsPlain)
-            if (tpr == 8) return launch(prologue_kernel<S, SIBS, K, 8>, siblings_of, &done[3]);
-        if (tpr == 4) return launch(prologue_kernel<S, SIBS, K, 4>, siblings_of, &done[2]);
-        if (tpr == 2) return launch(prologue_kernel<S, SIBS, K, 2>, siblings_of, &done[1]);
-        return launch(prologue_kernel<S, SIBS, K, 1>, siblings_of, &done[0]);
+        if constexpr (own && K == kRowsPlain)
+            if (!sh.common && tpr == 8) return launch(prologue_kernel<S, SIBS, K, 8>, siblings_of, &done[3]);
+        if constexpr (own && (S || K != kRowsDeep))
+            if (!sh.common && tpr == 4) return launch(prologue_kernel<S, SIBS, K, 4>, siblings_of, &done[2]);
+        if constexpr (own)
+            if (!sh.common && tpr == 2) return launch(prologue_kernel<S, SIBS, K, 2>, siblings_of, &done[1]);
+        if constexpr (own && K != kRowsPaired)
+            if (!sh.common && tpr == 1) return launch(prologue_kernel<S, SIBS, K, 1>, siblings_of, &done[0]);
+        return launch(prologue_kernel<S, SIBS, K, 0>, siblings_of, &done[4]);
     };
     auto by_kind = [&](const auto& siblings_of) -> cudaError_t {
         using std::integral_constant;

@@ -91,3 +91,13 @@ def test_the_common_prologue_kernels_spill_nothing_and_run_two_to_a_multiprocess
     for name, (regs, spilled) in kernels.items():
         if name[3] == 0:
             assert spilled == 0 and regs <= 128, name
+
+
+def test_every_prologue_kernel_is_reached_and_every_shape_has_one(shapes, kernels):
+    # the table of siblings is also what experts alone and layers under the switch for one kernel set carry
+    reached = set()
+    for a, s in shapes.items():
+        kind = "paired" if s.pairs else ("deep" if s.deep else "plain")
+        for table in ({True} if a.layers > 1 else {False, True}):
+            reached.add((s.staged, table, kind, 0 if s.common else s.tpr))
+    assert reached == set(kernels)
