@@ -681,13 +681,15 @@ int stream_product(const lopro_desc& d, int T, const StreamSiblingArgs* more) {
     StreamPlan pl;
     if (!plan_stream(d, T, &pl)) return 0;
     if (wide_variant(d, pl)) return LOPRO_PRODUCT_WIDE;
-    // A layer alone of up to eight tokens whose K does not fit the 32-warp kernel, with at most one row tile per multiprocessor (half
-    // of them idle here: 8192 -> 1024, 4 tokens 9.4 and 8.0 us, 8192 -> 2048 9.3 and 8.4) or rows of ten stages and more (11008 -> 4096,
-    // 1 token 12.1 and 11.7, 3 bits with the FP8 record, 5 tokens 14.1 and 13.6): every warp on a run of its own.  Shorter rows of more
-    // tiles are as fast here (8192 -> 4096, 8 tokens 11.0 and 10.9, 2 bits 9.0 and 9.6).
+    // A layer alone of up to eight tokens whose K does not fit the 32-warp kernel: every warp on a run of its own with at most one row
+    // tile per multiprocessor (half of them idle here: 8192 -> 1024, 4 tokens 9.4 and 8.0 us, 8192 -> 2048 9.3 and 8.4), with up to four
+    // tokens (to 4096 rows, 1 and 2 tokens: 7168 columns 10.1 and 9.7, 10.1 and 10.0, 8192 10.3 and 9.4, 10.4 and 9.6, 10240 11.5 and 10.6,
+    // 12.2 and 11.6; 4 tokens 10.2 and 10.2, 10.6 and 10.4, 12.2 and 12.1) and with rows of more than ten stages (11008 -> 4096 at 5 and 8
+    // tokens 12.6 and 12.4, 13.0 and 12.9, 2 bits 12.4 and 12.0).  Five to eight tokens of shorter rows are faster here: 7168 columns, 5
+    // tokens 10.2 and 10.7, 9216, 8 tokens 11.5 and 12.0, 10240, 8 tokens 12.5 and 13.4.
     int32_t form[5];
     if (more == nullptr && T <= 8 && option(LOPRO_OPT_NO_TALL) != 1 && option(LOPRO_OPT_ONE_KERNEL_SET) != 1 &&
-        (d.d_out / 16 <= sm_count() || d.d_in >= 10240) && warp_run_steps(d, T, nullptr, form) > 0 && form[3] == 1)
+        (d.d_out / 16 <= sm_count() || T <= 4 || d.d_in > 10240) && warp_run_steps(d, T, nullptr, form) > 0 && form[3] == 1)
         return LOPRO_PRODUCT_STEP_RUNS;
     return LOPRO_PRODUCT_STREAM;
 }

@@ -139,6 +139,14 @@ def test_experts_share_ctas_by_the_loop_that_each_runs():
     assert most(8192, 5632, 2, [12, 4] * 4) == most(8192, 5632, 2, [12] * 8) == (2, 40)
 
 
+@pytest.mark.parametrize("n,m,bits,T,kernel", [(10240, 4096, 4, 8, "STREAM"), (10240, 3072, 4, 8, "STREAM"), (9216, 4096, 4, 6, "STREAM"),
+                                               (7168, 4096, 4, 5, "STREAM"), (10240, 4096, 4, 4, "STEP_RUNS"), (8192, 4096, 4, 1, "STEP_RUNS"),
+                                               (7168, 4096, 4, 2, "STEP_RUNS"), (11008, 4096, 3, 5, "STEP_RUNS"), (6144, 4096, 4, 2, "WIDE"),
+                                               (8192, 2048, 4, 8, "STEP_RUNS")])
+def test_long_rows_of_one_wave_take_the_kernel_measured_faster(n, m, bits, T, kernel):
+    assert lopro.product_kernel([lopro.make_desc(n, m, bits, 128, 128, rank=32)], T)[0] == getattr(lopro, "PRODUCT_" + kernel)
+
+
 def test_product_query_names_the_kernel_of_a_small_batch_launch():
     def desc(n, m, bits=4, **kw):
         return lopro.make_desc(n, m, bits, 128, 128, rank=32, **kw)

@@ -65,9 +65,10 @@ def test_runs_of_tile_steps(n, per_sm, extra, bits, g, r, T, form):
     assert (y - y_short).abs().max().item() <= 2e-5 * y_short.abs().max().item()
 
 
-@pytest.mark.parametrize("n,m,bits,T", [(11008, 320, 4, 1), (10240, 2400, 3, 4), (8192, 1024, 4, 8), (11008, 16, 4, 7)])
+@pytest.mark.parametrize("n,m,bits,T", [(11008, 320, 4, 1), (10240, 2400, 3, 4), (8192, 1024, 4, 8), (11008, 16, 4, 7),
+                                        (7424, 2416, 4, 2), (9216, 2400, 3, 4)])
 def test_long_rows_of_few_tiles(n, m, bits, T):
-    # fewer row tiles than multiprocessors, some CTAs without any
+    # fewer row tiles than multiprocessors, some CTAs without any, and a few tiles more
     layer = random_layer_np(n, m, bits, 128, 32, seed=n + m)
     d = lopro.make_desc(n, m, bits, 128, 128, identity_cols=128, rank=32)
     assert lopro.linear_fwd_path(d, T)[0] == lopro.PATH_STREAM and lopro.product_kernel([d], T)[0] == lopro.PRODUCT_STEP_RUNS
