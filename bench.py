@@ -91,9 +91,21 @@ def time_oracle_stack(T, budget_s):
 # the kernels as committed (profiles/: the commands; counters re-read after the last change of each kernel, as ncu
 # prints them, i.e. to 10 kB); null for workloads without a capture.
 NCU_TRAFFIC = {("cfg2_T8", "stream_wide_kernel"): 9290000, ("cfg2_T32", "stream_kernel"): 9490000,
-               ("cfg4_T16", "run_kernel or tall_kernel"): 81680000, ("cfg3_T2048", "prefill_pair_kernel"): 60700000}
+               ("cfg4_T16", "run_kernel"): 81680000, ("cfg3_T2048", "prefill_pair_kernel"): 60700000}
 METRIC = "quantized-linear fwd tokens/s"
 UNIT = "tokens/s"
+
+
+def product_kernels(calls, T):
+    """Names of the product kernels of the small-batch calls (descs, ...), as the library reports them; none for other paths."""
+    from paper_2601_19675_b200 import lopro
+    names = {lopro.PRODUCT_STREAM: "stream_kernel", lopro.PRODUCT_WIDE: "stream_wide_kernel", lopro.PRODUCT_PERSISTENT: "tall_kernel",
+             lopro.PRODUCT_ROW_RUNS: "stream_kernel", lopro.PRODUCT_STEP_RUNS: "run_kernel"}
+    found = set()
+    for descs, *_ in calls:
+        together = lopro.product_kernel(descs, T)[0]
+        found.update([together] if together else [lopro.product_kernel([d], T)[0] for d in descs])
+    return sorted({names[k] for k in found if k})
 
 
 def algorithmic_bytes(c, T, lowrank="f16"):
@@ -623,10 +635,9 @@ def measure(args, name, steps, warmup, rank, world, local, dev, dist, with_e2e=T
     ms_per_pass = ms_per_step / passes
     value = w.tokens_per_pass * passes * world / (ms_per_step * 1e-3)
     per_forward_s = ms_per_pass * 1e-3 / w.forwards
-    # ("tall": none of the workloads is a layer that runs of row tiles take)
-    kernel = " + ".join({"stream": "stream_kernel", "wide": "stream_wide_kernel", "tall": "run_kernel or tall_kernel", "general": "decode_kernel",
-                         "prefill": "prefill_pair_kernel" if w.T >= 512 else "prefill_kernel",
-                         "rowblock": "rowblock_kernel"}.get(n, n) for n in w.paths)
+    kernel = " + ".join(product_kernels(w.calls, w.T) or
+                        [{"general": "decode_kernel", "prefill": "prefill_pair_kernel" if w.T >= 512 else "prefill_kernel",
+                          "rowblock": "rowblock_kernel"}.get(n, n) for n in w.paths])
     note = ("duration = step time / layer forwards (includes the prologue kernels of each forward): an upper bound on the "
             "product kernel's own duration, a lower bound on `achieved`")
     if getattr(w, "block", False):

@@ -119,7 +119,7 @@ enum {
  * (LOPRO_NO_WIDE=1, ...); 0 = default behaviour. */
 enum {
     LOPRO_OPT_NO_WIDE = 0,       /* 1: never the 32-warp variant of the streaming kernel (its layers take the 16-warp
-                                     one, those of at most one row tile per multiprocessor runs of tile steps)     */
+                                     one or runs of tile steps, as layers alone whose K does not fit it do)        */
     LOPRO_OPT_NO_TALL = 1,       /* 1: the streaming kernel for every layer: neither the kernels for layers with many
                                      rows (persistent, runs of row tiles) nor, for any, runs of tile steps          */
     LOPRO_OPT_NO_CHUNKS = 2,     /* 1: token counts above 32 always take the tensor-core (prefill) kernel      */
@@ -246,12 +246,13 @@ LOPRO_API lopro_status lopro_linear_fwd(const lopro_desc* desc, const void* pack
 /* Which kernels lopro_linear_fwd runs for this layer and token count on the current device (an
  * implementation detail of this library, exposed so that tests and benchmarks can name what they
  * measure; the paper's Appendix A.3 lists the steps, not their grouping into launches).
- *   LOPRO_PATH_STREAM   2 launches: prologue (permutation, rotation, B x) + streaming product, T <= 32
+ *   LOPRO_PATH_STREAM   2 launches: prologue (permutation, rotation, B x) + streaming product, T <= 32 (for layers alone whose
+ *                       K does not fit the 32-warp variant also the kernel that gives every warp a run of the weights)
  *   LOPRO_PATH_WIDE     the same with the 32-warp variant of the streaming kernel (T <= 8, all of K in the ring)
  *   LOPRO_PATH_TALL     the same with a kernel for layers with many output rows: one that gives every warp a run of the
  *                       layer's weights, the persistent streaming kernel or, for up to 16 tokens where the rows make
- *                       even waves of short runs, the streaming kernel with longer runs of rows per CTA (the last not
- *                       with LOPRO_OPT_ONE_KERNEL_SET)
+ *                       even waves of short runs, the streaming kernel with longer runs of rows per CTA (with
+ *                       LOPRO_OPT_ONE_KERNEL_SET always the persistent one)
  *   LOPRO_PATH_GENERAL  rotation, B x, register-ring product (any shape the descriptor allows)
  *   LOPRO_PATH_PREFILL  rotation, B x (2 launches), tcgen05 product (one CTA per tile, or two with a launch more
  *                       where the last wave's tiles are cut along K), T > 32

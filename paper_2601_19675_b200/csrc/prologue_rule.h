@@ -51,7 +51,8 @@ inline PrologueShape prologue_shape(int d_in, int r_pad, int T, int layers, bool
     s.rot_ctas = s.staged ? live * ((nchunks + 7) / 8) : nchunks;
     // A kernel per number of tokens of a row CTA: with one or two it takes 54 to 92 registers instead of 96 to 128, and the CTAs of the
     // next launch find room beside it (with kernels of their own throughout: decoder layer 4096, 4 sequences 69.4 -> 60.3 us, 2048, 6
-    // sequences 50.6 -> 43.9, 4096 -> 4096 at 1 token 6.5 -> 6.1, 11008 -> 4096 at 8 tokens 14.0 -> 12.9).  The common kernel stays
+    // sequences 50.6 -> 43.9, 11008 -> 4096 at 8 tokens 14.0 -> 12.9, graphs of 4096 -> 4096 at 1 token 6.5 -> 6.1; the same by single
+    // calls, where the two launches cost the host more than that, 5.8 and 6.0).  The common kernel stays
     //  * for two rows of B per CTA and a layer alone (4096 -> 4096 at 16 tokens 8.5 and 9.0, 4096 -> 11008 12.7 and 13.4);
     //  * for long rows of the FP8 record: 11008 -> 4096 at 1, 2, 3, 4 and 5 tokens, ranks 16 to 64, 12.5 to 14.0 us and 13.0 to 14.3 alone,
     //    within one percent either way as part of a decoder layer.  With folded factors it gains as much on most long rows alone (8192 to

@@ -640,7 +640,7 @@ bool plan_layout(const lopro_desc& d, StreamPlan* pl, int r_pad, int ng, int kto
 // more, runs of up to four tiles, which the persistent kernel takes as one group, then stay there (512 -> 8192, 2 bits, 9 tokens
 // 5.8 and 6.0; with five tiles 512 -> 11008, 12 tokens 8.7 and 8.2).  Layers that share a launch never go in runs of row tiles, and
 // layers of many tile steps per multiprocessor go in runs of tile steps per warp instead (warps.cu; the lines between the three are in
-// launch_tall).
+// tall_product).
 bool plan_run(const lopro_desc& d, int T, StreamPlan* pl, int* ctas) {
     if (T < 1 || T > 16) return false;
     pl->nt = T <= 8 ? 1 : 2;

@@ -3,9 +3,9 @@
 // "U (Sigma Y)" of Appendix A.3, summed as in Eq. 8), after the prologue kernel that writes the
 // rotated activations x~ (as the stage image), their 64-column sums and t = B x.
 //
-// Up to 16 tokens most such layers go elsewhere (launch_tall): every warp on a run of tile steps of its own where the activations
-// fit shared memory (warps.cu), runs of row tiles for a layer alone with few steps per CTA (plan_run in stream.cu).  More tokens, longer
-// rows and, where callers ask for one set of kernels, the layers that alone might go in runs of row tiles run here.
+// Most such layers go elsewhere (tall_product): every warp on a run of tile steps of its own where the activations, or a half of them, fit
+// shared memory (warps.cu), runs of row tiles for a layer alone of up to 16 tokens with few steps per CTA (plan_run in stream.cu).  Here run
+// an odd number of steps per row, activations that do not fit, few steps per CTA and, where callers ask for one set of kernels, all of them.
 //
 // Persistent: one CTA per SM, each owning a contiguous run of 16-row tiles (the runs differ by at
 // most one tile) and walking it in groups of up to four tiles (two with 32 tokens).  A producer warp keeps one ring of

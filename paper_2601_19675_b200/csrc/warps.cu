@@ -11,10 +11,12 @@
 // shared with four busy warps; four producers or copies issued by the last warp of a stage were slower still.)  The activations of all of K are fetched once and stay.  A warp that leaves a tile, or ends, puts its
 // sums of the tile into shared memory; when all are done, a warp per tile adds them in order, with the low-rank term.
 //
-// What bounds it: the integer pipe (expansion: two cycles per instruction and scheduler) and the legacy tensor pipe (eight per
-// m16n8k16), which share the way out of a scheduler: twice the integer instructions plus eight times the products of a tile step
-// is what a loop without any overhead takes (one token tile, 2 bits: 44 + 32 against 74 cycles measured; two, 4 bits: 56 + 64 and 116).
-// 4096 -> 28672, 2 bits, 1 token: 75 instructions per tile step, of which 49 are the step itself, issue slots 57 percent busy.
+// What bounds it: instruction issue with little to hide latency behind, four warps per scheduler.  Twice the integer instructions
+// (expansion: two cycles per instruction and scheduler) plus eight times the products (m16n8k16 on the legacy tensor pipe), which share
+// the way out of a scheduler, are what no loop over these operands gets below: 44 + 32 = 76 cycles per tile step at 2 bits and one token
+// tile, 44 + 64 = 108 at two, 56 + 32 = 88 and 56 + 128 = 184 at 4 bits and one and four.  Instructions per step over the share of busy
+// issue slots, way in and out included: 4096 -> 28672, 2 bits, 1 token 126 cycles (75 instructions, of which 49 are the step), eight
+// experts 4096 -> 14336 97, 8192 -> 28672, 2 bits, 16 tokens 173, 4096 -> 11008, 4 bits, 8 tokens 202 (20 steps per warp), 32 tokens 408.
 //
 // Arithmetic as in stream.cu: sum_k s (c_k - z) x~_k = s (sum_k (128 + c_k) x~_k - (128 + z) sum_k x~_k),
 // exact bf16 operands 128 + c_k on the tensor cores (rows gq + 8 of a tile: see expand_codes_by_rows), fp32 accumulation,
