@@ -414,6 +414,13 @@ static long long group_rows(int32_t n, const lopro_desc* const* descs) {
 static int product_of(const lopro_desc& d, int T, long long total_rows = 0, const StreamSiblingArgs* more = nullptr) {
     return use_tall(d, T, total_rows) ? tall_product(d, T, more) : stream_product(d, T, more);
 }
+// The same for a layer alone, 0 where the small-batch kernels do not take the call.  No plan more than it takes: host time counts in a
+// call of one small layer, which waits for two launches of 2.8 us (another plan and device query: 0.5 percent of 4096 -> 4096 at 1 token).
+static int single_product(const lopro_desc& d, int T) {
+    if (!prologue_supported(d, T)) return 0;
+    if (use_tall(d, T)) return stream_supported(d, T) ? tall_product(d, T, nullptr) : 0;
+    return stream_product(d, T, nullptr);
+}
 static cudaError_t launch_product(int product, const lopro_desc& d, const uint8_t* blob, const BlobLayout& L, const uint8_t* ws,
                                   const WorkspaceLayout& W, void* y, int64_t ldy, int out_dtype, int T, cudaStream_t s, int t0 = 0,
                                   const StreamSiblingArgs* more = nullptr) {
@@ -472,8 +479,8 @@ int32_t lopro_linear_fwd_path(const lopro_desc* desc, int32_t T, int32_t* launch
     if (const int chunks = small_batch_chunks(*desc, T)) {
         path = use_tall(*desc, kDecodeMaxT) ? LOPRO_PATH_TALL : LOPRO_PATH_STREAM;
         n = 1 + chunks;
-    } else if (prologue_supported(*desc, T) && stream_supported(*desc, T)) {
-        path = use_tall(*desc, T) ? LOPRO_PATH_TALL : (product_of(*desc, T) == LOPRO_PRODUCT_WIDE ? LOPRO_PATH_WIDE : LOPRO_PATH_STREAM);
+    } else if (const int product = single_product(*desc, T)) {
+        path = use_tall(*desc, T) ? LOPRO_PATH_TALL : (product == LOPRO_PRODUCT_WIDE ? LOPRO_PATH_WIDE : LOPRO_PATH_STREAM);
         n = 2;
     } else {
         const int pre = (T > kDecodeMaxT && prefill_supported(*desc, T) && rotate_lowrank_supported(*desc, T))
@@ -571,12 +578,12 @@ lopro_status lopro_linear_fwd(const lopro_desc* desc, const void* packed, const 
         }
         return LOPRO_OK;
     }
-    if (prologue_supported(*desc, T) && stream_supported(*desc, T)) {
+    if (const int product = single_product(*desc, T)) {
         // small batch: prologue + streaming kernel, chained by programmatic launches
         if (launch_prologue(*desc, perm, B, L.r_pad, (const __nv_bfloat16*)x_bf16, ldx, ws + W.off_xrot,
                             (__half*)(ws + W.off_t), W.t_pad, status, T, s, nullptr, nullptr, &lr8) != cudaSuccess)
             return LOPRO_ERR_CUDA;
-        if (launch_product(product_of(*desc, T), *desc, blob, L, ws, W, y, ldy, out_dtype, T, s) != cudaSuccess) return LOPRO_ERR_CUDA;
+        if (launch_product(product, *desc, blob, L, ws, W, y, ldy, out_dtype, T, s) != cudaSuccess) return LOPRO_ERR_CUDA;
         return LOPRO_OK;
     }
     const void* a_f16 = nullptr;  // the up factor where it is not the blob's section

@@ -16,7 +16,7 @@ struct PrologueShape {
 };
 
 // r_pad: padded rank (0: no low-rank term); layers: of the launch; fp8: the FP8 low-rank record; other_product: not in front of the
-// kernels of stream.cu, warps.cu and tall.cu; sms: multiprocessors.
+// kernels of stream.cu, warps.cu and tall.cu; sms: multiprocessors (read only where a row CTA has eight tokens, i.e. with five and more).
 inline PrologueShape prologue_shape(int d_in, int r_pad, int T, int layers, bool fp8, bool other_product, int sms) {
     PrologueShape s;
     const int live = T < 8 ? T : 8, nchunks = (d_in + 255) / 256;

@@ -647,7 +647,9 @@ cudaError_t launch_prologue(const lopro_desc& d, const int32_t* perm, const __ha
     if (lr8_args != nullptr) lr8 = *lr8_args;
     cudaLaunchConfig_t cfg = {};
     const int rp = d.rank > 0 ? r_pad : 0;
-    const PrologueShape sh = prologue_shape(d.d_in, rp, T, 1 + sibs.n, lr8.V != nullptr, other_product || img.ximg != nullptr, sm_count());
+    // (the number of multiprocessors, a query of the device, counts only with eight tokens per row CTA: from five tokens on)
+    const PrologueShape sh = prologue_shape(d.d_in, rp, T, 1 + sibs.n, lr8.V != nullptr, other_product || img.ximg != nullptr,
+                                            T > 4 ? sm_count() : 0);
     const int tpr = sh.tpr;
     cfg.gridDim = dim3(sh.row_ctas + sh.rot_ctas, sh.groups, 1 + sibs.n);
     cfg.blockDim = dim3(256);

@@ -51,6 +51,11 @@ def test_row_ctas_cover_every_row_and_token_once(shapes):
         assert s.row_ctas == a.r_pad // rows * -(-min(a.T, 8) // s.tpr)
 
 
+def test_the_number_of_multiprocessors_counts_from_five_tokens_on(shapes):
+    # the launch asks the device for it there only
+    assert all(s.tpr < 8 for a, s in shapes.items() if a.T <= 4)
+
+
 def test_a_row_cta_has_no_loop_for_tokens_that_are_absent(shapes):
     for a, s in shapes.items():
         assert s.tpr < 2 * min(a.T, 8)
