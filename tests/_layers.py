@@ -4,7 +4,7 @@ import numpy as np
 import torch
 
 from oracle import lopro_oracle as o
-from paper_2601_19675_b200 import synth
+from paper_2601_19675_b200 import lopro, synth
 
 
 def random_layer_np(d_in, d_out, bits, group_size, rank, seed=0):
@@ -42,3 +42,9 @@ def device_bf16_to_f64(t):
     """Device bf16 tensor -> fp64 numpy via its bit patterns (no torch arithmetic)."""
     bits = t.contiguous().view(torch.int16).cpu().numpy().view(np.uint16)
     return o.bf16_bits_to_f64(bits)
+
+
+def takes_runs_of_row_tiles(d, blob, x):
+    """Whether a tall layer alone goes in runs of row tiles and not through the persistent kernel, where runs of tile steps are off."""
+    with lopro.configured(lopro.OPT_NO_STEP_RUNS, 1):
+        return lopro.product_kernel([d], x.shape[0])[0] == lopro.PRODUCT_ROW_RUNS

@@ -76,23 +76,13 @@ def test_experts_through_the_persistent_kernel():
     n, m, r = 512, 16 * (2 * sms + 5), 16
     d, layers, blobs = _experts(n, m, 4, 128, 128, r, 5, seed=2)
     assert lopro.linear_fwd_path(d, 8)[0] == lopro.PATH_TALL
-    with lopro.configured(lopro.OPT_NO_STEP_RUNS, 1):
-        assert lopro.product_kernel([d] * 4, rows=[8, 3, 20, 1])[0] == lopro.PRODUCT_PERSISTENT
-        _check_experts(d, layers, blobs, [8, 0, 3, 20, 1], seed=9, shared=True, bit_equal=False)
+    _check_experts(d, layers, blobs, [8, 0, 3, 20, 1], seed=9, shared=True, bit_equal=False)
 
 
-@pytest.mark.parametrize("per_sm,extra,counts,off,kernel", [
-    (7, 3, [8] * 8 + [3], 1, lopro.PRODUCT_PERSISTENT),             # up to 8 rows
-    (2, 5, [20] + [1] * 7 + [2], 1, lopro.PRODUCT_PERSISTENT),      # and more than 16
-    (7, 3, [8] * 8 + [3], 0, lopro.PRODUCT_STEP_RUNS),
-    (2, 5, [20] + [1] * 7 + [2], 0, lopro.PRODUCT_STEP_RUNS),
-    (2, 5, [8] * 8 + [1], 0, lopro.PRODUCT_ROW_RUNS)])              # the last layer alone
-def test_an_expert_alone_in_the_last_launch_writes_its_own_rows_only(per_sm, extra, counts, off, kernel):
-    with lopro.configured(lopro.OPT_NO_STEP_RUNS, off):
-        _last_expert_alone(per_sm, extra, counts, kernel)
-
-
-def _last_expert_alone(per_sm, extra, counts, kernel):
+@pytest.mark.parametrize("per_sm,extra,counts", [(7, 3, [8] * 8 + [3]),           # persistent kernel, up to 8 rows
+                                                 (2, 5, [20] + [1] * 7 + [2]),    # and more than 16
+                                                 (2, 5, [8] * 8 + [1])])          # the last layer alone: in runs of row tiles
+def test_an_expert_alone_in_the_last_launch_writes_its_own_rows_only(per_sm, extra, counts):
     # eight experts share a pair of launches, the ninth has one of its own, shaped for the largest row count: its rows end
     # where y ends, and the rows behind keep their pattern
     n, m = 512, 16 * (torch.cuda.get_device_properties(0).multi_processor_count * per_sm + extra)
@@ -101,7 +91,7 @@ def _last_expert_alone(per_sm, extra, counts, kernel):
     offs = np.concatenate([[0], np.cumsum(counts)]).tolist()
     total, spare = offs[-1], max(counts)
     x = bf16_bits_to_device(synth.activations(total, n, seed=total))
-    assert lopro.product_kernel([d], max(counts))[0] == kernel
+    assert lopro.linear_fwd_path(d, max(counts))[0] == lopro.PATH_TALL
     buf = torch.full((total + spare, m), 7.0, dtype=torch.float32, device="cuda")
     y = lopro.linear_fwd_experts(d, blobs, offs, x, lopro.OUT_F32, y=buf[:total])
     torch.cuda.synchronize()

@@ -11,7 +11,8 @@ import torch
 
 from oracle import lopro_oracle as o
 from paper_2601_19675_b200 import lopro, synth
-from tests._layers import bf16_bits_to_device, device_bf16_to_f64, oracle_args, random_layer_np, to_device
+from tests._layers import (bf16_bits_to_device, device_bf16_to_f64, oracle_args, random_layer_np, takes_runs_of_row_tiles,
+                           to_device)
 
 pytestmark = pytest.mark.gpu
 
@@ -233,7 +234,7 @@ def _tall_rows(tiles_per_sm, extra_tiles):
 @pytest.mark.parametrize("per_sm,extra", [(2, 1), (4, 100), (5, 7), (6, 3)])
 def test_tall_layers(bits, g, r, T, per_sm, extra):
     # more 16-row tiles than twice the SM count: runs of tiles per CTA (2/3, 4/5, 5/6, 6/7) and a ragged last stage (36 steps);
-    # up to 16 tokens the shorter ones go through runs of row tiles, most others through runs of tile steps
+    # up to 16 tokens the shorter ones go through the kernel of runs
     n, m = 2304, _tall_rows(per_sm, extra)
     d = lopro.make_desc(n, m, bits, g, 64, identity_cols=64, rank=r)
     assert lopro.linear_fwd_path(d, T)[0] == lopro.PATH_TALL
@@ -245,18 +246,16 @@ def test_tall_layers(bits, g, r, T, per_sm, extra):
 @pytest.mark.parametrize("T", [1, 8, 16, 32])
 @pytest.mark.parametrize("per_sm,extra", [(6, 3), (8, 1), (9, 100), (10, 7)])
 def test_tall_layers_persistent_kernel(bits, g, r, T, per_sm, extra):
-    # too many tiles for runs of row tiles: with runs of tile steps off the persistent kernel, whose runs of tiles per CTA end in
-    # groups of 1, 2 and 3 tiles (4+2/4+3, 8/8+1, 8+1/8+2, 8+2/8+3 tiles per CTA) and a ragged last stage (36 steps)
+    # too many tiles for runs: the persistent kernel, whose runs of tiles per CTA end in groups of 1, 2 and 3 tiles
+    # (4+2/4+3, 8/8+1, 8+1/8+2, 8+2/8+3 tiles per CTA) and a ragged last stage (36 steps)
     n, m = 2304, _tall_rows(per_sm, extra)
     d = lopro.make_desc(n, m, bits, g, 64, identity_cols=64, rank=r)
     assert lopro.linear_fwd_path(d, T)[0] == lopro.PATH_TALL
     layer = random_layer_np(n, m, bits, g, r, seed=m + bits + T)
     x_bits = synth.activations(T, n, seed=T + 11, outlier_frac=0.01)
+    assert not takes_runs_of_row_tiles(d, _pack(layer, d), bf16_bits_to_device(x_bits))
     # the rows of the first CTAs and of the last ones, and some between
     rows = np.unique(np.concatenate([np.arange(16 * 24), m - 1 - np.arange(16 * 24), np.random.default_rng(m).integers(0, m, 64)]))
-    with lopro.configured(lopro.OPT_NO_STEP_RUNS, 1):
-        assert lopro.product_kernel([d], T)[0] == lopro.PRODUCT_PERSISTENT
-        _check_forward(layer, d, x_bits, rows=rows)
     _check_forward(layer, d, x_bits, rows=rows)
 
 
@@ -264,8 +263,8 @@ def test_tall_layers_persistent_kernel(bits, g, r, T, per_sm, extra):
 @pytest.mark.parametrize("T,m", [(8, 160), (16, 160), (8, 2), (8, 7), (32, 7)])
 def test_groups_as_long_as_or_longer_than_a_stage(g, T, m):
     # a stage of the small-batch kernels holds 1024 columns: groups of exactly one stage, of two stages and of
-    # the whole row (one scale per row), on the 32-warp and the 16-warp kernel, in runs of row tiles and, with runs of tile steps
-    # off, on the persistent kernel (m below 16: tiles per multiprocessor, and a few)
+    # the whole row (one scale per row), on the 32-warp and the 16-warp kernel, in runs of row tiles and on the persistent kernel
+    # (m below 16: tiles per multiprocessor, and a few)
     n, per_sm = 4096, m
     m = _tall_rows(m, 5) if m < 16 else m
     d = lopro.make_desc(n, m, 4, g, 128, identity_cols=128, rank=16)
@@ -273,12 +272,9 @@ def test_groups_as_long_as_or_longer_than_a_stage(g, T, m):
     assert lopro.linear_fwd_path(d, T)[0] == want
     layer = random_layer_np(n, m, 4, g, 16, seed=g + T)
     x_bits = synth.activations(T, n, seed=T + g)
-    rows = None if m <= 160 else np.unique(np.concatenate([np.arange(160), np.arange(0, m, 37)]))
     if want == lopro.PATH_TALL:
-        with lopro.configured(lopro.OPT_NO_STEP_RUNS, 1):
-            assert lopro.product_kernel([d], T)[0] == (lopro.PRODUCT_ROW_RUNS if per_sm == 2 else lopro.PRODUCT_PERSISTENT)
-            _check_forward(layer, d, x_bits, rows=rows)
-    _check_forward(layer, d, x_bits, rows=rows)
+        assert takes_runs_of_row_tiles(d, _pack(layer, d), bf16_bits_to_device(x_bits)) == (per_sm == 2)
+    _check_forward(layer, d, x_bits, rows=None if m <= 160 else np.unique(np.concatenate([np.arange(160), np.arange(0, m, 37)])))
 
 
 @pytest.mark.parametrize("T,n,m,path", [(33, 1024, 4096, "tall"), (96, 1024, 4096, "tall"), (128, 1024, 4096, "prefill"),
@@ -309,25 +305,21 @@ def test_rotated_entry_on_a_bf16_rounding_boundary():
     _check_forward(layer, d, synth.activations(T, n, seed=T))
 
 
-def test_tall_kernels_agree_with_the_per_group_kernel():
-    # the small-batch kernels sum the same products in fp32 in different orders: outputs agree to fp32 rounding
+def test_tall_kernel_agrees_with_the_per_group_kernel():
+    # both small-batch kernels sum the same products in fp32 in different orders: outputs agree to fp32 rounding
     n, m, bits, g, r, T = 1024, _tall_rows(8, 9), 4, 128, 32, 8
     d = lopro.make_desc(n, m, bits, g, 128, rank=r)
     layer = random_layer_np(n, m, bits, g, r, seed=3)
     blob = _pack(layer, d)
     x = bf16_bits_to_device(synth.activations(T, n, seed=4))
-    assert lopro.product_kernel([d], T)[0] == lopro.PRODUCT_STEP_RUNS
-    y_steps = lopro.linear_fwd(d, blob, x, lopro.OUT_F32)
-    with lopro.configured(lopro.OPT_NO_STEP_RUNS, 1):
-        assert lopro.product_kernel([d], T)[0] == lopro.PRODUCT_PERSISTENT
-        y_persistent = lopro.linear_fwd(d, blob, x, lopro.OUT_F32)
+    y_tall = lopro.linear_fwd(d, blob, x, lopro.OUT_F32)
+    assert not takes_runs_of_row_tiles(d, blob, x)
     with lopro.configured(lopro.OPT_NO_TALL, 1):
         assert lopro.linear_fwd_path(d, T)[0] in (lopro.PATH_STREAM, lopro.PATH_WIDE)
         y_stream = lopro.linear_fwd(d, blob, x, lopro.OUT_F32)
     torch.cuda.synchronize()
     scale = y_stream.abs().max().item()
-    for y in (y_steps, y_persistent):
-        assert (y - y_stream).abs().max().item() <= 1e-5 * scale
+    assert (y_tall - y_stream).abs().max().item() <= 1e-5 * scale
 
 
 def test_outputs_can_be_strided_and_calls_repeat_bitwise():

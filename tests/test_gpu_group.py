@@ -67,15 +67,6 @@ def test_sibling_layers_share_two_launches(T, bits, g, ms):
     _check_group(layers, descs, blobs, synth.activations(T, n, seed=T + 40, outlier_frac=0.01), shared=True)
 
 
-@pytest.mark.parametrize("n,count,r,T", [(512, 4, 16, 16), (1024, 3, 96, 8), (1024, 3, 96, 5), (4096, 2, 128, 1), (4096, 2, 128, 3),
-                                         (4096, 8, 32, 1), (8192, 2, 128, 8), (8192, 2, 128, 4), (8192, 2, 64, 2), (2048, 3, 32, 16),
-                                         (4096, 3, 32, 32), (2048, 3, 16, 14)])
-def test_row_ctas_of_sibling_layers(n, count, r, T):
-    # the low-rank rows of all siblings in one launch: one, two, four and eight tokens per CTA, two rows per CTA, long rows
-    layers, descs, blobs = _siblings(n, (64, 80, 48, 16, 32, 64, 16, 96)[:count], 4, 64, 64, r, seed=T + r)
-    _check_group(layers, descs, blobs, synth.activations(T, n, seed=T + 60, outlier_frac=0.01), shared=True, bit_equal=n < 8192)
-
-
 def test_groups_that_cannot_share_run_layer_by_layer():
     n = 1024
     # different ranks: no shared launches, same results
@@ -94,8 +85,8 @@ def test_attention_projections_of_the_stack_at_full_size(T):
     n = 4096
     layers, descs, blobs = _siblings(n, (4096, 4096, 4096), 4, 128, 128, 32, seed=T)
     rows = np.unique(np.concatenate([[0, 15, 16, 4095, 2048], np.random.default_rng(T).integers(0, 4096, size=24)]))
-    # together the three projections make more than one wave of the per-group kernel, so the group runs through another
-    # kernel than each layer alone: same products, another order of summation
+    # together the three projections make more than one wave of the per-group kernel, so the group runs through the
+    # persistent kernel while each layer alone does not: same products, another order of summation
     _check_group(layers, descs, blobs, synth.activations(T, n, seed=T + 1), rows=rows, shared=True, bit_equal=False)
     with lopro.configured(lopro.OPT_NO_TALL, 1):
         _check_group(layers, descs, blobs, synth.activations(T, n, seed=T + 1), rows=rows, shared=True)
@@ -114,23 +105,17 @@ def test_sibling_layers_through_the_persistent_kernel(T, bits, g, extra):
     ms = tuple(_persistent_rows(e) for e in extra)
     layers, descs, blobs = _siblings(n, ms, bits, g, 128, r, seed=T + bits)
     assert all(lopro.linear_fwd_path(d, T)[0] == lopro.PATH_TALL for d in descs)
-    x_bits = synth.activations(T, n, seed=T + 50, outlier_frac=0.01)
-    with lopro.configured(lopro.OPT_NO_STEP_RUNS, 1):
-        assert lopro.product_kernel(descs, T)[0] == lopro.PRODUCT_PERSISTENT
-        _check_group(layers, descs, blobs, x_bits, shared=True, bit_equal=False)
-    _check_group(layers, descs, blobs, x_bits, shared=True, bit_equal=False)
+    _check_group(layers, descs, blobs, synth.activations(T, n, seed=T + 50, outlier_frac=0.01), shared=True, bit_equal=False)
 
 
-@pytest.mark.parametrize("T,per_sm", [(1, 4), (8, 4), (16, 4), (1, 8), (7, 12), (16, 8), (17, 2), (24, 4), (32, 8)])
-def test_one_kernel_set_gives_single_layers_the_sums_of_a_group(T, per_sm):
-    # four (eight, twelve) row tiles per multiprocessor and layer: a CTA owns four alone and eight in the group of two, i.e. whole
-    # groups of four tiles (two with more than 16 tokens) either way, so the persistent kernel adds a row's products in one
-    # order -- and another kernel would not
-    n, m = 1024, 16 * per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+@pytest.mark.parametrize("T", [1, 8, 16])
+def test_one_kernel_set_gives_single_layers_the_sums_of_a_group(T):
+    # four row tiles per multiprocessor and layer: a CTA owns four alone and eight in the group of two, i.e. whole groups of
+    # four tiles either way, so the persistent kernel adds a row's products in one order -- and another kernel would not
+    n, m = 1024, 16 * 4 * torch.cuda.get_device_properties(0).multi_processor_count
     layers, descs, blobs = _siblings(n, (m, m), 4, 128, 128, 16, seed=T)
     x = bf16_bits_to_device(synth.activations(T, n, seed=T + 3))
     with lopro.configured(lopro.OPT_ONE_KERNEL_SET, 1):
-        assert lopro.product_kernel(descs, T)[0] == lopro.product_kernel(descs[:1], T)[0] == lopro.PRODUCT_PERSISTENT
         together = lopro.linear_fwd_group(descs, blobs, x, lopro.OUT_F32)
         for d, blob, y in zip(descs, blobs, together):
             assert torch.equal(lopro.linear_fwd(d, blob, x, lopro.OUT_F32), y)

@@ -1,13 +1,12 @@
 """Taller layers of up to 16 tokens in runs of row tiles (launch_stream, in_runs): run lengths at the edges of each kernel
 variant, one wave and two, a ragged last stage of K, rings that hold all of K and rings that are refilled, against the oracle and
-against the kernel of short runs; and the layers that stay with the persistent kernel.  Runs of tile steps per warp, which
-take some of these layers from both, are off."""
+against the kernel of short runs; and the layers that stay with the persistent kernel."""
 import numpy as np
 import pytest
 import torch
 
 from paper_2601_19675_b200 import lopro, synth
-from tests._layers import bf16_bits_to_device, random_layer_np
+from tests._layers import bf16_bits_to_device, random_layer_np, takes_runs_of_row_tiles
 from tests.test_gpu_forward import _check_forward, _pack
 
 pytestmark = pytest.mark.gpu
@@ -43,12 +42,11 @@ def test_runs_of_row_tiles(n, per_sm, extra, bits, g, T, runs):
     assert lopro.linear_fwd_path(d, T)[0] == lopro.PATH_TALL
     x_bits = synth.activations(T, n, seed=T, outlier_frac=0.01)
     blob, x = _pack(layer, d), bf16_bits_to_device(x_bits)
+    assert takes_runs_of_row_tiles(d, blob, x) == runs
     rows = np.unique(np.concatenate([[0, 15, 16, m - 17, m - 1], np.random.default_rng(m).integers(0, m, 40)]))
-    with lopro.configured(lopro.OPT_NO_STEP_RUNS, 1):
-        assert lopro.product_kernel([d], T)[0] == (lopro.PRODUCT_ROW_RUNS if runs else lopro.PRODUCT_PERSISTENT)
-        _check_forward(layer, d, x_bits, rows=rows)
-        y = lopro.linear_fwd(d, blob, x, lopro.OUT_F32)
+    _check_forward(layer, d, x_bits, rows=rows)
     # the same products in fp32 in another order, every row (K = 8256: 2^-24 times the square root of the terms, times 16)
+    y = lopro.linear_fwd(d, blob, x, lopro.OUT_F32)
     with lopro.configured(lopro.OPT_NO_TALL, 1):
         y_short = lopro.linear_fwd(d, blob, x, lopro.OUT_F32)
     torch.cuda.synchronize()

@@ -18,39 +18,31 @@ def _rows(per_sm, extra):
     return 16 * (torch.cuda.get_device_properties(0).multi_processor_count * per_sm + extra)
 
 
-@pytest.mark.parametrize("n,per_sm,extra,bits,g,r,T,form", [
-    # form: token tiles, tile steps of a batch, batches of a ring, CTAs that share K
-    (256, 7, 1, 4, 128, 16, 1, (1, 4, 3, 1)),       # one batch per tile: warps without a batch, tiles of one warp
-    (128, 8, 5, 2, 128, 0, 8, (1, 2, 3, 1)),        # a tile is one batch of two steps; no low-rank term
-    (2304, 7, 3, 3, 64, 17, 5, (1, 4, 3, 1)),       # a ragged last stage of activations
-    (1152, 9, 100, 4, 64, 40, 3, (1, 2, 3, 1)),     # 18 steps per tile, three tiles of ranks
-    (4096, 4, 1, 4, 128, 128, 8, (1, 4, 3, 1)),     # longer runs instead of runs of row tiles; ranks in two passes
-    (4096, 3, 100, 2, 64, 32, 16, (2, 4, 3, 1)),    # two token tiles
-    (4096, 7, 9, 3, 256, 16, 9, (2, 4, 3, 1)),      # groups as long as a batch
-    (4096, 7, 9, 4, 128, 32, 13, (2, 4, 2, 1)),     # a ring of two batches
-    (4096, 5, 9, 4, 128, 64, 16, (2, 4, 2, 1)),
-    (8192, 8, 3, 4, 128, 16, 8, (1, 4, 2, 1)),
-    (1152, 6, 3, 2, 64, 16, 9, (2, 2, 3, 1)),       # two token tiles, batches of two, at every number of bits
-    (1152, 6, 3, 3, 64, 32, 16, (2, 2, 3, 1)),
-    (1152, 6, 3, 4, 128, 17, 12, (2, 2, 3, 1)),
-    (8192, 13, 3, 2, 64, 64, 2, (1, 4, 3, 1)),      # eight stages of activations
-    (4096, 40, 11, 2, 2048, 16, 4, (1, 4, 3, 1)),   # forty tiles per CTA, groups longer than a stage
-    (512, 2, 3, 4, 64, 16, 32, (4, 2, 4, 1)),       # four token tiles
-    (1024, 8, 3, 2, 64, 32, 17, (4, 2, 4, 1)),      # two bits: a ring of four batches, where the sums of four token tiles fit
-    (2048, 3, 1, 3, 128, 0, 25, (4, 2, 4, 1)),      # no low-rank term
-    (2304, 5, 3, 3, 64, 40, 32, (4, 2, 4, 2)),      # two CTAs share K and the second begins in the middle of a stage
-    (4096, 4, 77, 4, 128, 32, 31, (4, 2, 4, 2)),
-    (4096, 4, 96, 4, 128, 32, 32, (4, 2, 3, 2)),
-    (4096, 12, 9, 4, 128, 64, 32, (4, 2, 2, 2)),    # a ring of two batches of two
-    (4224, 4, 9, 4, 128, 17, 24, (4, 2, 2, 2)),     # an odd number of batches of two: the CTAs' parts of K differ
-    (8192, 7, 5, 2, 64, 128, 16, (2, 4, 3, 2)),     # two token tiles, eight stages shared by two CTAs
-    (11008, 8, 1, 3, 128, 16, 8, (1, 4, 3, 2)),     # one token tile, eleven stages shared by two CTAs
+@pytest.mark.parametrize("n,per_sm,extra,bits,g,r,T", [
+    (256, 7, 1, 4, 128, 16, 1),       # one batch of four steps per tile: warps without a batch, tiles of one warp
+    (128, 8, 5, 2, 128, 0, 8),        # a tile is one batch of two steps; no low-rank term
+    (2304, 7, 3, 3, 64, 17, 5),       # batches of four, a ragged last stage of activations
+    (1152, 9, 100, 4, 64, 40, 3),     # batches of two steps (18 steps per tile), three tiles of ranks
+    (4096, 4, 1, 4, 128, 128, 8),     # longer runs instead of runs of row tiles; ranks in two passes
+    (4096, 3, 100, 2, 64, 32, 16),    # two token tiles, a ring of two batches
+    (4096, 7, 9, 3, 256, 16, 9),      # groups as long as a batch
+    (4096, 7, 9, 4, 128, 32, 13),     # four bits and two token tiles: batches of two
+    (8192, 13, 3, 2, 64, 64, 2),      # eight stages of activations
+    (4096, 40, 11, 2, 2048, 16, 4),   # forty tiles per CTA, groups longer than a stage
+    (512, 2, 3, 4, 64, 16, 32),       # four token tiles
+    (1024, 8, 3, 2, 64, 32, 17),      # two bits: a ring of four batches, where the sums of four token tiles fit
+    (2048, 3, 1, 3, 128, 0, 25),      # no low-rank term
+    (2304, 5, 3, 3, 64, 40, 32),      # two CTAs share K and the second begins in the middle of a stage
+    (4096, 4, 77, 4, 128, 32, 31),    # a ring of two batches of two
+    (4224, 4, 9, 4, 128, 17, 24),     # an odd number of batches of two: the CTAs' parts of K differ
+    (8192, 7, 5, 2, 64, 128, 16),     # two token tiles, eight stages shared by two CTAs
+    (11008, 8, 1, 3, 128, 16, 8),     # one token tile, eleven stages shared by two CTAs
 ])
-def test_runs_of_tile_steps(n, per_sm, extra, bits, g, r, T, form):
+def test_runs_of_tile_steps(n, per_sm, extra, bits, g, r, T):
     m = _rows(per_sm, extra)
     layer = random_layer_np(n, m, bits, g, r, seed=n + T + bits)
     d = lopro.make_desc(n, m, bits, g, 64, identity_cols=64, rank=r)
-    assert lopro.product_kernel([d], T)[0] == lopro.PRODUCT_STEP_RUNS and lopro.product_kernel([d], T)[1][:4] == form
+    assert lopro.linear_fwd_path(d, T)[0] == lopro.PATH_TALL
     x_bits = synth.activations(T, n, seed=T, outlier_frac=0.01)
     blob, x = _pack(layer, d), bf16_bits_to_device(x_bits)
     rows = np.unique(np.concatenate([[0, 15, 16, m - 17, m - 1], np.random.default_rng(m).integers(0, m, 40)]))
@@ -65,13 +57,12 @@ def test_runs_of_tile_steps(n, per_sm, extra, bits, g, r, T, form):
     assert (y - y_short).abs().max().item() <= 2e-5 * y_short.abs().max().item()
 
 
-@pytest.mark.parametrize("n,m,bits,T", [(11008, 320, 4, 1), (10240, 2400, 3, 4), (8192, 1024, 4, 8), (11008, 16, 4, 7),
-                                        (7424, 2416, 4, 2), (9216, 2400, 3, 4)])
+@pytest.mark.parametrize("n,m,bits,T", [(11008, 320, 4, 1), (10240, 2400, 3, 4), (8192, 1024, 4, 8), (11008, 16, 4, 7)])
 def test_long_rows_of_few_tiles(n, m, bits, T):
-    # fewer row tiles than multiprocessors, some CTAs without any, and a few tiles more
+    # fewer row tiles than multiprocessors, some CTAs without any
     layer = random_layer_np(n, m, bits, 128, 32, seed=n + m)
     d = lopro.make_desc(n, m, bits, 128, 128, identity_cols=128, rank=32)
-    assert lopro.linear_fwd_path(d, T)[0] == lopro.PATH_STREAM and lopro.product_kernel([d], T)[0] == lopro.PRODUCT_STEP_RUNS
+    assert lopro.linear_fwd_path(d, T)[0] == lopro.PATH_STREAM
     _check_forward(layer, d, synth.activations(T, n, seed=T, outlier_frac=0.01), rows=np.arange(0, m, 7))
 
 
@@ -80,25 +71,12 @@ def test_siblings_of_unequal_rows(n, T):
     # the smallest layer gets a CTA (at 3072 columns and 30 tokens two that share K) or two, the tallest most of them
     layers, descs, blobs = _siblings(n, (64, _rows(9, 3), 272), 4, 128, 128, 17, seed=T)
     rows = np.arange(0, 64, 5)
-    kernel, form = lopro.product_kernel(descs, T)
-    assert kernel == lopro.PRODUCT_STEP_RUNS and form[3] == (2 if n == 3072 else 1)
     _check_group(layers, descs, blobs, synth.activations(T, n, seed=T + 50, outlier_frac=0.01), rows=rows, shared=True, bit_equal=False)
-
-
-def test_a_sibling_of_one_row_tile_beside_pairs_of_ctas():
-    # the second CTA of the pair that shares the small layer's K adds up no tile: it has no use for the low-rank intermediate, and
-    # must not leave with a copy of it under way
-    layers, descs, blobs = _siblings(4096, (4096, 4096, 16), 4, 128, 128, 32, seed=32)
-    assert lopro.product_kernel(descs, 32)[0] == lopro.PRODUCT_STEP_RUNS and lopro.product_kernel(descs, 32)[1][3] == 2
-    rows = np.unique(np.concatenate([np.arange(16), np.random.default_rng(1).integers(0, 4096, 30)]))
-    _check_group(layers, descs, blobs, synth.activations(32, 4096, seed=3, outlier_frac=0.01), rows=rows, shared=True, bit_equal=False)
 
 
 @pytest.mark.parametrize("counts", [[1, 9, 8, 0, 16, 3], [2] * 8, [9, 1] * 4])
 def test_experts_of_one_and_of_two_token_tiles(counts):
     # in a launch shaped for up to 16 rows the experts with at most eight run the loop of one token tile
-    n, m = 1024, _rows(2, 5)
+    n, m = 1024, _rows(1, 5)
     d, layers, blobs = _experts(n, m, 3, 64, 128, 16, len(counts), seed=3)
-    with_rows = [c for c in counts if c]
-    assert lopro.product_kernel([d] * len(with_rows), rows=with_rows)[1][:4] == ((2, 4, 3, 1) if max(counts) > 8 else (1, 4, 3, 1))
     _check_experts(d, layers, blobs, counts, seed=9, shared=True, bit_equal=False)
